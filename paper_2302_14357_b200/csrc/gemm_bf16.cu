@@ -512,6 +512,19 @@ int make_tmap_bf16(CUtensorMap* out, const void* base, uint64_t rows, uint64_t K
   return r == CUDA_SUCCESS ? TW_OK : TW_ERR_CUDA;
 }
 
+int make_tmap_f32(CUtensorMap* out, const float* base, uint64_t rows, uint64_t K, uint64_t ld, uint32_t box_rows) {
+  EncodeTiledFn fn = encode_fn();
+  if (!fn || (K % 4) != 0 || (ld % 4) != 0 || (reinterpret_cast<uintptr_t>(base) & 15) != 0 || box_rows > 256 || rows == 0) return TW_ERR_ARG;
+  cuuint64_t dims[2] = {K, rows};
+  cuuint64_t strides[1] = {ld * 4};
+  cuuint32_t box[2] = {32, box_rows};
+  cuuint32_t estr[2] = {1, 1};
+  CUresult r = fn(out, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, const_cast<float*>(base), dims, strides, box, estr,
+                  CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                  CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+  return r == CUDA_SUCCESS ? TW_OK : TW_ERR_CUDA;
+}
+
 int gemm_bf16_setup() {
   cudaError_t e1 = cudaFuncSetAttribute(gemm_bf16_kernel<256, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Cfg<256>::kSmem);
   cudaError_t e2 = cudaFuncSetAttribute(gemm_bf16_kernel<128, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Cfg<128>::kSmem);

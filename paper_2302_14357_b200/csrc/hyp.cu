@@ -694,6 +694,8 @@ __device__ __forceinline__ float sigmoidf_acc(float x) { return 1.f / (1.f + exp
 __global__ void lstm_pointwise_kernel(const float* gates, const int* pw_new, const int* pw_par,
                                       const int* n_dev, int n_max, const float* hc_in, float* hc_out,
                                       int L, int l, int Hd) {
+  pdl_wait();
+  pdl_trigger();
   const int n = n_dev ? *n_dev : n_max;
   const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= (long long)n * Hd) return;
@@ -737,8 +739,8 @@ void launch_lstm_pointwise(const float* gates, const int* idx_out, const int* id
                            int n_max, const float* hc_in, float* hc_out, int L, int l, int Hd, cudaStream_t st) {
   if (n_max <= 0) return;
   const long long tot = (long long)n_max * Hd;
-  lstm_pointwise_kernel<<<(unsigned)((tot + 255) / 256), 256, 0, st>>>(gates, idx_out, idx_in, n_dev, n_max, hc_in,
-                                                                      hc_out, L, l, Hd);
+  launch_pdl(lstm_pointwise_kernel, dim3((unsigned)((tot + 255) / 256)), dim3(256), 0, st, gates, idx_out, idx_in, n_dev, n_max, hc_in,
+             hc_out, L, l, Hd);
 }
 
 }  // namespace tw

@@ -1,132 +1,254 @@
 // fp32 (TW_MODE_F32) stage kernels: SIMT GEMM, joiner contraction, log-softmax, Eq. 3-7.
 // This is the accuracy path: plain FFMA accumulation and libm tanhf/expf/logf, no fast-math.
+#include <atomic>
+
 #include "topn.cuh"
+#include "bf16_path.cuh"
+#include "sm100.cuh"
 #include "tw_internal.cuh"
 
 namespace tw {
 
 namespace {
 
-constexpr int BM = 64, BN = 64, BK = 16, LDS = BM + 4;
+// ---------------------------------------------------------------------------------------------
+// SIMT fp32 GEMM.  The rows of a decode step are few (tens to hundreds) and K is long, so a CTA owns a short, wide tile
+// (16 rows x 256 columns) and its eight warps split every K block between them: each accumulates the whole tile over its
+// eighth of K, and the partial tiles are summed in a fixed order at the end.  Where such tiles leave SMs idle, a cluster
+// of two or four CTAs splits K once more and sums over distributed shared memory.  A lane holds 16 x NJ outputs: shared
+// memory delivers one register per lane and cycle to the whole SM, so the 16 + 8 operand registers of a k take 96 of
+// the 128 cycles in which the four schedulers issue its FMAs (with 8 x 8 outputs it would be 64 of 64).  The 64-column
+// tiles (NJ = 2) are for narrow matrices.
+// Only eight warps fit beside that many accumulators, so nothing but FMAs and operand reads may take issue slots: the
+// weights arrive by TMA (128-byte swizzle: the 16-byte reads along K of eight neighbouring rows hit distinct banks), the
+// rows of A by bulk copies, four blocks of 32 ahead, each block sent for by another warp, and the warps meet on the
+// ring's mbarriers only.  The weights of the first blocks are asked for before the wait for the kernel ahead.
+// Bound by FFMA issue: on a B200 register-only FFMA loops reach 51 of the nominal 74 TFLOP/s; measured here 27 us for
+// 112 x 2560 x 1280 and 26 us for 435 x 1024 x 640 (77 and 59 us with 64 x 64 tiles, 4 x 4 outputs a thread, whole K).
+constexpr int TM = 16, BK = 32, kStagesF = 6, kAhead = kStagesF - 2, kWarpsF = 8, kThreadsF = 32 * kWarpsF;
+template <int NJ> struct F32Smem {
+  static constexpr size_t kB = (size_t)32 * NJ * BK * 4, kA = (size_t)TM * BK * 4;
+  static constexpr size_t kOps = kStagesF * (kB + kA), kRed = (size_t)kWarpsF * TM * 32 * NJ * 4;
+  static constexpr size_t kTotal = (kOps > kRed ? kOps : kRed) + 1024 + 2 * kStagesF * 8;
+};
 
 struct GemmParams {
   GemmOperand op[2];
   GemmOut out;
   const int* M_dev;
+  int M_scale;        // rows = *M_dev * M_scale
   int M_max, N;
   // joiner mode
   JoinerRows jr;
   const float* W_out;
   const float* b_out;
   float* z;
+  int* err;           // raised by a wait that gave up
 };
 
-__device__ __forceinline__ void load4(const float* p, int k, int K, bool valid, float v[4]) {
-  if (!valid) { v[0] = v[1] = v[2] = v[3] = 0.f; return; }
-  if (k + 3 < K && ((reinterpret_cast<uintptr_t>(p + k) & 15) == 0)) {
-    float4 q = *reinterpret_cast<const float4*>(p + k);
-    v[0] = q.x; v[1] = q.y; v[2] = q.z; v[3] = q.w;
-  } else {
+__device__ __forceinline__ float4 load4(const float* p, int k, int K) {
+  if (k + 3 < K && ((reinterpret_cast<uintptr_t>(p + k) & 15) == 0)) return *reinterpret_cast<const float4*>(p + k);
+  float v[4];
 #pragma unroll
-    for (int i = 0; i < 4; ++i) v[i] = (k + i < K) ? p[k + i] : 0.f;
-  }
+  for (int i = 0; i < 4; ++i) v[i] = (k + i < K) ? p[k + i] : 0.f;
+  return make_float4(v[0], v[1], v[2], v[3]);
 }
+__device__ __forceinline__ float act_f32(float x, int act) { return act == TW_ACT_RELU ? fmaxf(x, 0.f) : tanhf(x); }
 
-// MODE 0: plain / gathered rows, one or two operand pairs.  MODE 1: joiner rows, A = tanh(E + Pp).
-template <int MODE>
-__global__ void __launch_bounds__(256) gemm_f32_kernel(GemmParams p) {
-  __shared__ __align__(16) float As[BK][LDS];
-  __shared__ __align__(16) float Bs[BK][LDS];
-
-  int M;
-  if (MODE == 1) {
-    int R = p.jr.R_dev ? *p.jr.R_dev : p.jr.R_max;
-    M = R * p.jr.S;
-  } else {
-    M = p.M_dev ? *p.M_dev : p.M_max;
-  }
-  const int m0 = blockIdx.y * BM, n0 = blockIdx.x * BN;
-  if (m0 >= M) return;
+// MODE 0: plain / gathered rows, one or two operand pairs.  MODE 1: joiner rows, A = act(E + Pp) formed on the way.
+// VEC: K is a multiple of 4 and every row starts on a 16-byte boundary (TMA and bulk copies); otherwise the warps copy
+// the operands element by element.
+template <int MODE, int NJ, bool VEC>
+__global__ void __launch_bounds__(kThreadsF, 1)
+gemm_f32_kernel(const __grid_constant__ CUtensorMap tm0, const __grid_constant__ CUtensorMap tm1, GemmParams p) {
+  using namespace sm100;
+  using Sm = F32Smem<NJ>;
+  extern __shared__ uint8_t smem_raw[];
+  constexpr int BN = 32 * NJ;                                // lane: all 16 rows, columns lane + 32 j
+  uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
+  float* sm_f32 = reinterpret_cast<float*>(smem);            // the partial tiles, once the operands are done with
+  uint8_t* sB = smem;                                        // [kStagesF][BN][BK], swizzled
+  uint8_t* sA = smem + kStagesF * Sm::kB;                    // [kStagesF][TM][BK]
+  uint64_t* full = reinterpret_cast<uint64_t*>(smem + (Sm::kOps > Sm::kRed ? Sm::kOps : Sm::kRed));
+  uint64_t* empty = full + kStagesF;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int m0 = blockIdx.y * TM, n0 = blockIdx.x * BN;
   const int N = (MODE == 1) ? p.jr.V : p.N;
+  const int K0 = (MODE == 1) ? p.jr.J : p.op[0].K, K1 = (MODE == 1) ? 0 : p.op[1].K;
+  const int nb0 = (K0 + BK - 1) / BK, nb_all = nb0 + (K1 + BK - 1) / BK;
+  const int split = gridDim.z, part = blockIdx.z;            // the CTAs of a cluster share K
+  const int b_lo = nb_all * part / split, nb = nb_all * (part + 1) / split - b_lo;
+  constexpr bool kBulkA = VEC && MODE == 0;
 
-  const int tid = threadIdx.x;
-  const int lrow = tid >> 2, kq = (tid & 3) * 4;
-  const int tx = tid & 15, ty = tid >> 4;
+  if (tid == 0) {
+    for (int s = 0; s < kStagesF; ++s) { mbar_init(&full[s], VEC ? (MODE == 0 ? 2 : 1 + kWarpsF) : kWarpsF); mbar_init(&empty[s], kWarpsF); }
+    fence_barrier_init();
+  }
+  if (kBulkA && ((K0 | K1) & (BK - 1)) != 0)                 // what a short last block leaves in A meets zeros of B: it has to be a number
+    for (int i = tid; i < kStagesF * TM * BK / 4; i += kThreadsF) reinterpret_cast<float4*>(sA)[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+  fence_proxy_async_smem();
+  __syncthreads();
+  auto send_B = [&](int i) {               // one thread: the weights of block i
+    const int blk = b_lo + i, s = i % kStagesF;
+    mbar_expect_tx(&full[s], (uint32_t)Sm::kB);
+    tma_load_2d(sB + s * Sm::kB, blk < nb0 ? &tm0 : &tm1, &full[s], (blk < nb0 ? blk : blk - nb0) * BK, n0);
+  };
+  const int pre = nb < kAhead ? nb : kAhead;
+  if (VEC && tid == 0) for (int i = 0; i < pre; ++i) send_B(i);   // constant weights: ahead of the wait
+  pdl_wait();
+  pdl_trigger();
+  int M;
+  if (MODE == 1) M = (p.jr.R_dev ? *p.jr.R_dev : p.jr.R_max) * p.jr.S;
+  else M = p.M_dev ? *p.M_dev * p.M_scale : p.M_max;
+  if (m0 >= M) {                           // no rows here: only the copies already under way have to be waited for
+    if (VEC && tid == 0)
+      for (int i = 0; i < pre; ++i) {
+        for (int c = 1; c < (MODE == 0 ? 2 : 1 + kWarpsF); ++c) mbar_arrive(&full[i]);
+        mbar_wait(&full[i], 0, p.err);
+      }
+    return;
+  }
 
-  float acc[4][4];
-#pragma unroll
-  for (int i = 0; i < 4; ++i)
-#pragma unroll
-    for (int j = 0; j < 4; ++j) acc[i][j] = 0.f;
-
-  const int nops = (MODE == 1) ? 1 : (p.op[1].K > 0 ? 2 : 1);
-  for (int o = 0; o < nops; ++o) {
-    const float* arow = nullptr;   // MODE 0: A row; MODE 1: E row
-    const float* prow = nullptr;   // MODE 1: Pp row
-    bool avalid = false;
+  const int lrow = kBulkA ? (lane & 15) : (tid >> 4);        // the row of A this thread looks after
+  const float* arow = nullptr;
+  const float* prow = nullptr;             // MODE 0: the row of the second operand; MODE 1: the Pp row
+  if (m0 + lrow < M) {
     const int m = m0 + lrow;
-    int K;
-    const float* Bmat;
-    long long ldB;
     if (MODE == 1) {
-      K = p.jr.J; Bmat = p.W_out; ldB = p.jr.J;
-      if (m < M) {
-        int r = m / p.jr.S, t = m - r * p.jr.S;
-        int sl = p.jr.row_slen ? p.jr.row_slen[r] : p.jr.S;
-        if (t < sl) {
-          avalid = true;
-          arow = p.jr.E + (long long)(p.jr.row_e0[r] + t) * K;
-          prow = p.jr.Pp + (long long)(p.jr.row_p ? p.jr.row_p[r] : r) * K;
-        }
+      const int r = m / p.jr.S, t = m - r * p.jr.S;
+      const int sl = p.jr.row_slen ? p.jr.row_slen[r] : p.jr.S;
+      if (t < sl) {
+        arow = p.jr.E + (long long)(p.jr.row_e0[r] + t) * K0;
+        prow = p.jr.Pp + (long long)(p.jr.row_p ? p.jr.row_p[r] : r) * K0;
       }
     } else {
-      const GemmOperand& op = p.op[o];
-      K = op.K; Bmat = op.B; ldB = op.ldB;
-      if (m < M) {
-        avalid = true;
-        arow = op.A + (long long)(op.idx ? op.idx[m] : m) * op.ldA;
-      }
-    }
-    const int n = n0 + lrow;
-    const bool bvalid = n < N;
-    const float* brow = Bmat + (long long)(bvalid ? n : 0) * ldB;
-
-    for (int k0 = 0; k0 < K; k0 += BK) {
-      float a[4], b[4];
-      load4(arow, k0 + kq, K, avalid, a);
-      if (MODE == 1) {
-        float q[4];
-        load4(prow, k0 + kq, K, avalid, q);
-#pragma unroll
-        for (int i = 0; i < 4; ++i) a[i] = (avalid && k0 + kq + i < K) ? (p.jr.act == TW_ACT_RELU ? fmaxf(a[i] + q[i], 0.f) : tanhf(a[i] + q[i])) : 0.f;
-      }
-      load4(brow, k0 + kq, K, bvalid, b);
-#pragma unroll
-      for (int i = 0; i < 4; ++i) { As[kq + i][lrow] = a[i]; Bs[kq + i][lrow] = b[i]; }
-      __syncthreads();
-#pragma unroll
-      for (int k = 0; k < BK; ++k) {
-        float4 av = *reinterpret_cast<const float4*>(&As[k][ty * 4]);
-        float4 bv = *reinterpret_cast<const float4*>(&Bs[k][tx * 4]);
-        float aa[4] = {av.x, av.y, av.z, av.w}, bb[4] = {bv.x, bv.y, bv.z, bv.w};
-#pragma unroll
-        for (int i = 0; i < 4; ++i)
-#pragma unroll
-          for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(aa[i], bb[j], acc[i][j]);
-      }
-      __syncthreads();
+      arow = p.op[0].A + (long long)(p.op[0].idx ? p.op[0].idx[m] : m) * p.op[0].ldA;
+      if (K1 > 0) prow = p.op[1].A + (long long)(p.op[1].idx ? p.op[1].idx[m] : m) * p.op[1].ldA;
     }
   }
-
+  // the rows of A of block i (bulk copies: one warp; else: the whole CTA forms them, and copies B if it has to)
+  auto send_A = [&](int i) {
+    const int blk = b_lo + i, s = i % kStagesF;
+    const bool second = blk >= nb0;
+    const int k = (second ? blk - nb0 : blk) * BK, kn = min(BK, (second ? K1 : K0) - k);
+    if (lane == 0) mbar_expect_tx(&full[s], (uint32_t)(min(TM, M - m0) * kn * 4));
+    __syncwarp();
+    if (lane < TM && arow != nullptr)
+      bulk_load(sA + s * Sm::kA + lane * (BK * 4), (second ? prow : arow) + k, (uint32_t)kn * 4u, &full[s]);
+  };
+  auto form = [&](int i) {
+    const int blk = b_lo + i, s = i % kStagesF;
+    const bool second = blk >= nb0;
+    const int k0 = (second ? blk - nb0 : blk) * BK, K = second ? K1 : K0;
 #pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    const int m = m0 + ty * 4 + i;
-    if (m >= M) continue;
+    for (int u = 0; u < 2; ++u) {          // two elements of A per thread
+      const int k = k0 + (tid & 15) * 2 + u;
+      float v = 0.f;
+      if (arow != nullptr && k < K) v = MODE == 1 ? act_f32(arow[k] + prow[k], p.jr.act) : (second ? prow : arow)[k];
+      reinterpret_cast<float*>(sA + s * Sm::kA)[lrow * BK + (tid & 15) * 2 + u] = v;
+    }
+    if (!VEC) {
+      const float* Bm = (MODE == 1) ? p.W_out : (second ? p.op[1].B : p.op[0].B);
+      const long long ld = (MODE == 1) ? p.jr.J : (second ? p.op[1].ldB : p.op[0].ldB);
+      for (int e = tid; e < BN * BK; e += kThreadsF) {
+        const int r = e / BK, kk = e % BK;
+        const float v = (n0 + r < N && k0 + kk < K) ? Bm[(n0 + r) * ld + k0 + kk] : 0.f;
+        reinterpret_cast<float*>(sB + s * Sm::kB)[r * BK + (((kk >> 2) ^ (r & 7)) << 2) + (kk & 3)] = v;
+      }
+    }
+    __syncwarp();
+    if (lane == 0) mbar_arrive(&full[s]);
+  };
+  for (int i = 0; i < pre; ++i) {
+    if (!kBulkA) form(i);
+    else if (warp == i % kWarpsF) send_A(i);
+  }
+
+  float acc[TM][NJ];
+#pragma unroll
+  for (int i = 0; i < TM; ++i)
+#pragma unroll
+    for (int j = 0; j < NJ; ++j) acc[i][j] = 0.f;
+  bool ok = true;
+  uint32_t st = 0, ph = 0;                 // stage and phase of block blk
+#pragma unroll 1
+  for (int blk = 0; blk < nb && ok; ++blk) {
+    const int nxt = blk + kAhead;
+    if (nxt < nb && (!kBulkA || warp == nxt % kWarpsF)) {
+      const int use = nxt / kStagesF;
+      if (use > 0) ok = mbar_wait(&empty[nxt % kStagesF], (use - 1) & 1, p.err);
+      if (!ok) break;
+      if (VEC && lane == 0 && (kBulkA || warp == 0)) send_B(nxt);
+      if (kBulkA) send_A(nxt); else form(nxt);
+    }
+    ok = mbar_wait(&full[st], ph, p.err);
+    if (!ok) break;
+    const float* a = reinterpret_cast<const float*>(sA + st * Sm::kA) + warp * 4;
+    const uint8_t* b = sB + st * Sm::kB + lane * (BK * 4) + ((warp ^ (lane & 7)) << 4);
+    float4 av[TM];
+#pragma unroll
+    for (int i = 0; i < TM; ++i) av[i] = *reinterpret_cast<const float4*>(a + i * BK);
+#pragma unroll
+    for (int j = 0; j < NJ; ++j) {
+      const float4 bv = *reinterpret_cast<const float4*>(b + j * (32 * BK * 4));
+#pragma unroll
+      for (int i = 0; i < TM; ++i) acc[i][j] = fmaf(av[i].x, bv.x, acc[i][j]);
+#pragma unroll
+      for (int i = 0; i < TM; ++i) acc[i][j] = fmaf(av[i].y, bv.y, acc[i][j]);
+#pragma unroll
+      for (int i = 0; i < TM; ++i) acc[i][j] = fmaf(av[i].z, bv.z, acc[i][j]);
+#pragma unroll
+      for (int i = 0; i < TM; ++i) acc[i][j] = fmaf(av[i].w, bv.w, acc[i][j]);
+    }
+    __syncwarp();
+    if (lane == 0) mbar_arrive(&empty[st]);
+    if (++st == kStagesF) { st = 0; ph ^= 1; }
+  }
+
+  // ---- the warps' partial tiles, summed in the order of K; [kWarpsF][TM][BN] in the operands' place
+  __syncthreads();                         // every block has been waited for: nothing is on its way into shared memory
+#pragma unroll
+  for (int i = 0; i < TM; ++i)
+#pragma unroll
+    for (int j = 0; j < NJ; ++j) sm_f32[(warp * TM + i) * BN + lane + 32 * j] = acc[i][j];
+  __syncthreads();
+  auto part_sum = [&](int at) {
+    float4 v = *reinterpret_cast<const float4*>(&sm_f32[at]);
+#pragma unroll
+    for (int w = 1; w < kWarpsF; ++w) {
+      const float4 u = *reinterpret_cast<const float4*>(&sm_f32[w * TM * BN + at]);
+      v.x += u.x; v.y += u.y; v.z += u.z; v.w += u.w;
+    }
+    return v;
+  };
+  if (split > 1) {                         // this CTA's sums in place; each CTA then finishes its share of the tile
+#pragma unroll
+    for (int i = 0; i < NJ / 2; ++i) {
+      const int at = (tid + i * kThreadsF) * 4;
+      *reinterpret_cast<float4*>(&sm_f32[at]) = part_sum(at);
+    }
+    sm100::cluster_sync_all();
+  }
+  const int chunks = TM * BN / 4 / split;  // of four columns
+  for (int i = tid; i < chunks; i += kThreadsF) {
+    const int c = part * chunks + i, rr = c / (BN / 4), cc = (c - rr * (BN / 4)) * 4;
+    const int m = m0 + rr, n = n0 + cc;
+    if (m >= M || n >= N) continue;
+    float4 v;
+    if (split == 1) {
+      v = part_sum(c * 4);
+    } else {
+      v = make_float4(0.f, 0.f, 0.f, 0.f);
+      for (int q = 0; q < split; ++q) {
+        const float4 u = sm100::ld_cluster_f32x4(sm100::map_to_cta(sm100::smem_u32(&sm_f32[c * 4]), (uint32_t)q));
+        v.x += u.x; v.y += u.y; v.z += u.z; v.w += u.w;
+      }
+    }
     float* crow;
     const float* bias;
     if (MODE == 1) {
-      int r = m / p.jr.S, t = m - r * p.jr.S;
-      int sl = p.jr.row_slen ? p.jr.row_slen[r] : p.jr.S;
+      const int r = m / p.jr.S, t = m - r * p.jr.S;
+      const int sl = p.jr.row_slen ? p.jr.row_slen[r] : p.jr.S;
       if (t >= sl) continue;
       crow = p.z + (long long)m * N;
       bias = p.b_out;
@@ -134,10 +256,38 @@ __global__ void __launch_bounds__(256) gemm_f32_kernel(GemmParams p) {
       crow = p.out.C + (long long)(p.out.oidx ? p.out.oidx[m] : m) * p.out.ldC;
       bias = p.out.bias;
     }
+    if (n + 3 < N && ((reinterpret_cast<uintptr_t>(crow + n) & 15) == 0)) {
+      if (bias) { v.x += bias[n]; v.y += bias[n + 1]; v.z += bias[n + 2]; v.w += bias[n + 3]; }
+      *reinterpret_cast<float4*>(crow + n) = v;
+    } else {
+      const float o[4] = {v.x, v.y, v.z, v.w};
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const int n = n0 + tx * 4 + j;
-      if (n < N) crow[n] = acc[i][j] + (bias ? bias[n] : 0.f);
+      for (int j = 0; j < 4; ++j) if (n + j < N) crow[n + j] = o[j] + (bias ? bias[n + j] : 0.f);
+    }
+  }
+  if (split > 1) sm100::cluster_sync_all();          // nobody leaves while a cluster mate still reads its sums
+}
+
+// the joiner's operand act(E + Pp) of every (row, frame) as float32 [R S, J]: a joiner with many column tiles forms it
+// once instead of once per column tile (rows of padding frames are left as they are: nothing reads their products)
+__global__ void __launch_bounds__(256) joiner_A_f32_kernel(JoinerRows jr, float* __restrict__ A) {
+  pdl_wait();
+  pdl_trigger();
+  const int M = (jr.R_dev ? *jr.R_dev : jr.R_max) * jr.S;
+  const int m = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;      // a warp per row
+  if (m >= M) return;
+  const int r = m / jr.S, t = m - r * jr.S;
+  if (t >= (jr.row_slen ? jr.row_slen[r] : jr.S)) return;
+  const float* e = jr.E + (long long)(jr.row_e0[r] + t) * jr.J;
+  const float* q = jr.Pp + (long long)(jr.row_p ? jr.row_p[r] : r) * jr.J;
+  float* dst = A + (long long)m * jr.J;
+  for (int k = lane * 4; k < jr.J; k += 128) {
+    const float4 ev = load4(e, k, jr.J), pv = load4(q, k, jr.J);
+    const float v[4] = {act_f32(ev.x + pv.x, jr.act), act_f32(ev.y + pv.y, jr.act), act_f32(ev.z + pv.z, jr.act), act_f32(ev.w + pv.w, jr.act)};
+    if (k + 3 < jr.J && ((reinterpret_cast<uintptr_t>(dst + k) & 15) == 0)) {
+      *reinterpret_cast<float4*>(dst + k) = make_float4(v[0], v[1], v[2], v[3]);
+    } else {
+      for (int i = 0; i < 4 && k + i < jr.J; ++i) dst[k + i] = v[i];
     }
   }
 }
@@ -302,23 +452,80 @@ __global__ void rows_from_groups_kernel(const int* row_group, const int* seg_len
 
 }  // namespace
 
+namespace {
+bool row_aligned(const float* base, long long ld) { return (reinterpret_cast<uintptr_t>(base) & 15) == 0 && (ld & 3) == 0; }
+
+template <int MODE, int NJ, bool VEC>
+void launch_gemm_one(const GemmParams& p, long long M_max, int N, cudaStream_t st) {
+  static std::atomic<unsigned long long> ready{0};           // devices whose copy of the kernel has its shared-memory limit raised
+  int dev = 0;
+  cudaGetDevice(&dev);
+  const unsigned long long bit = 1ull << (dev & 63);
+  if (dev > 63 || !(ready.load(std::memory_order_acquire) & bit)) {
+    cudaFuncSetAttribute(gemm_f32_kernel<MODE, NJ, VEC>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)F32Smem<NJ>::kTotal);
+    ready.fetch_or(bit, std::memory_order_release);
+  }
+  const long long mt = (M_max + TM - 1) / TM, nt = (N + 32 * NJ - 1) / (32 * NJ);
+  // K shared by two or four CTAs while the tiles of the largest row count leave SMs idle (a step mostly has fewer rows
+  // than its maximum) and every CTA keeps four blocks of K
+  const int nb = MODE == 1 ? (p.jr.J + BK - 1) / BK : (p.op[0].K + BK - 1) / BK + (p.op[1].K + BK - 1) / BK;
+  const unsigned split = (mt * nt <= 40 && nb >= 16) ? 4 : ((mt * nt <= 110 && nb >= 8) ? 2 : 1);
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)nt, (unsigned)mt, split); cfg.blockDim = dim3(kThreadsF);
+  cfg.dynamicSmemBytes = F32Smem<NJ>::kTotal; cfg.stream = st;
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = 1; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = split;
+  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[1].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr; cfg.numAttrs = g_pdl_on ? 2 : 1;
+  CUtensorMap tm0 = {}, tm1 = {};
+  if (VEC) {
+    const GemmOperand b0 = MODE == 1 ? GemmOperand{nullptr, nullptr, 0, p.W_out, p.jr.J, p.jr.J} : p.op[0];
+    make_tmap_f32(&tm0, b0.B, N, b0.K, b0.ldB, 32 * NJ);
+    if (p.op[1].K > 0) make_tmap_f32(&tm1, p.op[1].B, N, p.op[1].K, p.op[1].ldB, 32 * NJ);
+  }
+  cudaLaunchKernelEx(&cfg, gemm_f32_kernel<MODE, NJ, VEC>, tm0, tm1, p);
+}
+template <int MODE>
+void launch_gemm_tiles(const GemmParams& p, bool vec, long long M_max, int N, cudaStream_t st) {
+  if (N <= 128) {
+    if (vec) launch_gemm_one<MODE, 2, true>(p, M_max, N, st); else launch_gemm_one<MODE, 2, false>(p, M_max, N, st);
+  } else {
+    if (vec) launch_gemm_one<MODE, 8, true>(p, M_max, N, st); else launch_gemm_one<MODE, 8, false>(p, M_max, N, st);
+  }
+}
+}  // namespace
+
 void launch_gemm_f32(const GemmOperand& op1, const GemmOperand& op2, const GemmOut& out,
                      const int* M_dev, int M_max, int N, cudaStream_t st) {
   if (M_max <= 0 || N <= 0) return;
   GemmParams p{};
-  p.op[0] = op1; p.op[1] = op2; p.out = out; p.M_dev = M_dev; p.M_max = M_max; p.N = N;
-  dim3 grid((N + BN - 1) / BN, (M_max + BM - 1) / BM);
-  gemm_f32_kernel<0><<<grid, 256, 0, st>>>(p);
+  p.op[0] = op1; p.op[1] = op2; p.out = out; p.M_dev = M_dev; p.M_scale = 1; p.M_max = M_max; p.N = N; p.err = out.err;
+  auto ok = [](const GemmOperand& o) { return o.K == 0 || ((o.K & 3) == 0 && row_aligned(o.A, o.ldA) && row_aligned(o.B, o.ldB)); };
+  launch_gemm_tiles<0>(p, ok(op1) && ok(op2), M_max, N, st);
 }
 
-void launch_joiner_f32(const JoinerRows& rows, const float* W_out, const float* b_out, float* z,
-                       cudaStream_t st) {
-  if (rows.R_max <= 0) return;
+int launch_joiner_f32(const JoinerRows& rows, const float* W_out, const float* b_out, float* z, float* A_buf, int* err, cudaStream_t st) {
+  if (rows.R_max <= 0) return 0;
   GemmParams p{};
+  p.err = err;
+  const long long M_max = (long long)rows.R_max * rows.S;
+  // tanhf costs as much as some 25 FFMAs, so forming the operand anew in every column tile adds about 40 % to the
+  // contraction: a separate pass as soon as there is more than one wave of tiles (below, its launch costs more)
+  const long long tiles = (M_max + TM - 1) / TM * ((rows.V + 63) / 64);
+  const bool vec = (rows.J & 3) == 0 && row_aligned(W_out, rows.J);
+  if (A_buf != nullptr && tiles > 148) {
+    launch_pdl(joiner_A_f32_kernel, dim3((unsigned)((M_max + 7) / 8)), dim3(256), 0, st, rows, A_buf);
+    p.op[0] = GemmOperand{A_buf, nullptr, rows.J, W_out, rows.J, rows.J};
+    p.out = GemmOut{z, nullptr, rows.V, b_out};
+    p.M_dev = rows.R_dev; p.M_scale = rows.S; p.M_max = (int)M_max; p.N = rows.V;
+    launch_gemm_tiles<0>(p, vec, M_max, rows.V, st);
+    return 2;
+  }
   p.jr = rows; p.W_out = W_out; p.b_out = b_out; p.z = z;
-  long long M_max = (long long)rows.R_max * rows.S;
-  dim3 grid((rows.V + BN - 1) / BN, (unsigned)((M_max + BM - 1) / BM));
-  gemm_f32_kernel<1><<<grid, 256, 0, st>>>(p);
+  launch_gemm_tiles<1>(p, vec, M_max, rows.V, st);
+  return 1;
 }
 
 void launch_log_softmax(const JoinerRows& rows, int blank, float* z, cudaStream_t st) {

@@ -11,8 +11,9 @@ constexpr long long kScratchFloats = TW_NOALLOC_MAX_ELEMS;   // R * S * V of log
 constexpr int kMaxRows = TW_NOALLOC_MAX_ROWS;
 constexpr int kMaxDevices = 64;
 
-// [0, kScratchFloats): log J;  then kMaxRows ints of first-frame rows;  then kMaxRows ints of lengths.
-static __device__ __align__(256) float g_noalloc_scratch[kScratchFloats + 2 * kMaxRows];
+// [0, kScratchFloats): log J;  then kMaxRows ints of first-frame rows;  then kMaxRows ints of lengths;  then
+// the error word of the bounded waits.
+static __device__ __align__(256) float g_noalloc_scratch[kScratchFloats + 2 * kMaxRows + 1];
 
 std::mutex g_mu;
 float* g_scratch_addr[kMaxDevices] = {};
@@ -60,7 +61,7 @@ extern "C" int tw_joiner_expand_noalloc(const float* W_out, const float* b_out, 
   JoinerRows jr{};
   jr.E = E_seg; jr.row_e0 = row_e0; jr.Pp = Pp; jr.row_p = nullptr; jr.row_slen = row_slen;
   jr.R_dev = nullptr; jr.R_max = R; jr.S = S; jr.J = J; jr.V = V; jr.act = joiner_act;
-  launch_joiner_f32(jr, W_out, b_out, logp, st);
+  launch_joiner_f32(jr, W_out, b_out, logp, nullptr, row_slen + kMaxRows, st);
   launch_log_softmax(jr, blank, logp, st);
   launch_expand_f32(logp, ld_old, row_slen, nullptr, R, S, V, blank, out_ldphi, out_ldnb, out_la, nullptr,
                     nullptr, CandOut{}, st);

@@ -89,7 +89,7 @@ void enqueue_predictor(tw_handle* h, const int* tok, const float* hc_in, const i
   GemmOperand none{};
   if (h->pred_kind == TW_PRED_STATELESS) {
     GemmOperand a{h->emb, tok, h->emb_dim, h->W_p, h->P, h->P};
-    GemmOut o{Pp_out, idx_out, h->J, nullptr};
+    GemmOut o{Pp_out, idx_out, h->J, nullptr, h->bf.err};
     launch_gemm_f32(a, none, o, n_dev, n_max, h->J, st);
     *launches += 1;
     return;
@@ -127,7 +127,7 @@ void enqueue_predictor(tw_handle* h, const int* tok, const float* hc_in, const i
     const float* hp = hc_in + (long long)l * 2 * Hd;
     GemmOperand xo{x, xi, xld, h->W_ih[l], xk, xk};
     GemmOperand ro{hp, idx_in, stride, h->W_hh[l], Hd, Hd};
-    GemmOut o{h->gates, nullptr, 4 * Hd, h->b_l[l]};
+    GemmOut o{h->gates, nullptr, 4 * Hd, h->b_l[l], h->bf.err};
     launch_gemm_f32(xo, ro, o, n_dev, n_max, 4 * Hd, st);
     // pointwise: c' = sigma(f) c + sigma(i) tanh(g), h' = sigma(o) tanh(c')
     launch_lstm_pointwise(h->gates, idx_out, idx_in, n_dev, n_max, hc_in, hc_out, L, l, Hd, st);
@@ -135,7 +135,7 @@ void enqueue_predictor(tw_handle* h, const int* tok, const float* hc_in, const i
   }
   const float* top = hc_out + (long long)(L - 1) * 2 * Hd;
   GemmOperand to{top, idx_out, stride, h->W_p, h->P, h->P};
-  GemmOut o{Pp_out, idx_out, h->J, nullptr};
+  GemmOut o{Pp_out, idx_out, h->J, nullptr, h->bf.err};
   launch_gemm_f32(to, none, o, n_dev, n_max, h->J, st);
   *launches += 1;
 }
@@ -171,7 +171,7 @@ void enqueue_project(tw_handle* h, const void* enc, int rows, float* E, cudaStre
   } else {
     GemmOperand a{enc32, nullptr, h->D_enc, h->W_e, h->D_enc, h->D_enc};
     GemmOperand none{};
-    GemmOut o{E, nullptr, h->J, nullptr};
+    GemmOut o{E, nullptr, h->J, nullptr, h->bf.err};
     launch_gemm_f32(a, none, o, nullptr, rows, h->J, st);
     *launches += 1;
   }
@@ -181,8 +181,6 @@ void enqueue_project(tw_handle* h, const void* enc, int rows, float* E, cudaStre
 int build_bf16(tw_handle* h) {
   if ((h->D_enc % 8) || (h->J % 8) || (h->P % 8) || (h->emb_dim % 8) || (h->Hd % 8)) return TW_ERR_ARG;
   TW_TRY(gemm_bf16_setup());
-  TW_TRY(dev_alloc(h, &h->bf.err, (size_t)1));
-  TW_CUDA(h, cudaMemset(h->bf.err, 0, sizeof(int)));
   TW_TRY(make_bf16_mat(h, &h->bf.W_e, h->W_e, h->J, h->D_enc, false, true));
   TW_TRY(make_bf16_mat(h, &h->bf.W_out, h->W_out, h->V, h->J, false, true));
   TW_TRY(make_bf16_mat(h, &h->bf.enc, nullptr, (long long)h->max_batch * h->max_T, h->D_enc, true, false));
@@ -206,7 +204,7 @@ int build_bf16(tw_handle* h) {
       TW_TRY(dev_alloc(h, &h->bf.EmbProj, (size_t)h->V * G4));
       GemmOperand a{h->emb, nullptr, h->emb_dim, h->W_ih[0], h->emb_dim, h->emb_dim};
       GemmOperand none{};
-      GemmOut o{tmp, nullptr, G4, h->b_l[0]};
+      GemmOut o{tmp, nullptr, G4, h->b_l[0], h->bf.err};
       launch_gemm_f32(a, none, o, nullptr, h->V, G4, 0);
       launch_permute_cols_f32(tmp, perm_dev, h->V, G4, h->bf.EmbProj, 0);
       TW_CUDA(h, cudaDeviceSynchronize());
@@ -346,6 +344,7 @@ int build_workspace(tw_handle* h) {
   TW_TRY(dev_alloc(h, &hs.ldnb, R * h->V));
   TW_TRY(dev_alloc(h, &hs.logp, R * S * h->V));
   TW_TRY(dev_alloc(h, &h->E, (nb * h->max_T + 1) * h->J));   // + one dump row for frames a streamed chunk does not hold
+  if (h->mode == TW_MODE_F32) TW_TRY(dev_alloc(h, &h->A_f32, R * S * h->J));
   if (h->mode == TW_MODE_F32 && h->dtype == TW_BF16) TW_TRY(dev_alloc(h, &h->enc_f32, nb * h->max_T * h->D_enc));
   TW_TRY(dev_alloc(h, &h->stream_oidx, nb * h->max_T));
   TW_TRY(dev_alloc(h, &h->zero_len, nb));
@@ -357,6 +356,9 @@ int build_workspace(tw_handle* h) {
 }
 
 int init_impl(tw_handle* h, const tw_model* m, const tw_config* c) {
+  TW_TRY(dev_alloc(h, &h->bf.err, (size_t)1));
+  TW_CUDA(h, cudaMemset(h->bf.err, 0, sizeof(int)));
+  PdlScope plain(false);                     // kernels that fetch weights ahead of their wait run right behind the ones that write them
   h->D_enc = m->D_enc; h->P = m->P; h->J = m->J; h->V = m->V; h->blank = m->blank;
   h->pred_kind = m->pred_kind; h->emb_dim = m->emb_dim; h->joiner_act = m->joiner_act;
   h->dtype = m->dtype; h->esize = m->dtype == TW_BF16 ? 2 : 4;
@@ -391,11 +393,11 @@ int init_impl(tw_handle* h, const tw_model* m, const tw_config* c) {
     // gets a row of its own after the vocabulary's, which serves the empty prefix.
     TW_TRY(dev_alloc(h, &h->PpTab, (size_t)(h->V + 1) * h->J));
     GemmOperand a{h->emb, nullptr, h->emb_dim, h->W_p, h->P, h->P};
-    GemmOut o{h->PpTab, nullptr, h->J, nullptr};
+    GemmOut o{h->PpTab, nullptr, h->J, nullptr, h->bf.err};
     launch_gemm_f32(a, none, o, nullptr, h->V, h->J, 0);
     if (init_out) {
       GemmOperand a1{init_out, nullptr, h->P, h->W_p, h->P, h->P};
-      GemmOut o1{h->PpTab + (size_t)h->V * h->J, nullptr, h->J, nullptr};
+      GemmOut o1{h->PpTab + (size_t)h->V * h->J, nullptr, h->J, nullptr, h->bf.err};
       launch_gemm_f32(a1, none, o1, nullptr, 1, h->J, 0);
       h->hs.empty_row = h->hs_fused.empty_row = h->V;
     }
@@ -408,7 +410,7 @@ int init_impl(tw_handle* h, const tw_model* m, const tw_config* c) {
       else { TW_TRY(dev_alloc(h, &h->init_hc, nhc)); TW_CUDA(h, cudaMemset(h->init_hc, 0, nhc * sizeof(float))); }
       const float* out = init_out ? init_out : h->init_hc + (size_t)(h->L - 1) * 2 * h->Hd;
       GemmOperand a1{out, nullptr, h->P, h->W_p, h->P, h->P};
-      GemmOut o1{h->init_Pp, nullptr, h->J, nullptr};
+      GemmOut o1{h->init_Pp, nullptr, h->J, nullptr, h->bf.err};
       launch_gemm_f32(a1, none, o1, nullptr, 1, h->J, 0);
     } else {
       // one step on the blank token from an all-zero state
@@ -501,8 +503,7 @@ void enqueue_joiner_logits(tw_handle* h, const JoinerRows& rows, float* logp, cu
     gemm_bf16(h, h->bf.A_join, h->bf.W_out, M_dev, rows.R_max * rows.S, logp, nullptr, rows.V, h->b_out, st);
     *launches += 2;
   } else {
-    launch_joiner_f32(rows, h->W_out, h->b_out, logp, st);
-    *launches += 1;
+    *launches += launch_joiner_f32(rows, h->W_out, h->b_out, logp, h->A_f32, h->bf.err, st);
   }
 }
 }  // namespace tw

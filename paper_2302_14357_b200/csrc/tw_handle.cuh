@@ -27,6 +27,7 @@ struct tw_handle {
   tw::HypState hs{};
   tw::HypState hs_fused{};    // same arrays, but log J is not materialised (fused joiner path)
   float* E = nullptr;         // projected encoder frames [max_batch * max_T, J]
+  float* A_f32 = nullptr;     // TW_MODE_F32: the joiner's operand [R_max * S, J]
   float* gates = nullptr;     // LSTM gate pre-activations [R_max, 4 Hd]
   int *stage_e0 = nullptr, *stage_slen = nullptr;   // [R_max] scratch of the stage entry points
   int* stream_oidx = nullptr;   // [max_batch * max_T] destination rows of a pushed chunk's frames
@@ -42,7 +43,7 @@ struct tw_handle {
     tw::Bf16Mat Htop;                                     // [R_max, Hd]
     float* bias_perm[tw::kMaxLayers] = {};   // LSTM biases in the interleaved gate order (layers > 0)
     float* EmbProj = nullptr;   // [V, 4Hd] = emb W_ih[0]^T + b[0]: layer 0's input half, one row per token
-    int* err = nullptr;                                   // device error word of the bounded waits
+    int* err = nullptr;                                   // device error word of the bounded waits (both modes)
     // fused joiner + softmax + Eq. 3-7 + selection (logits stay in tensor memory)
     bool fused_ok = false, fused_on = false, no_max = false;
     float zbound = 0.f;                                   // bound of |logit| behind no_max

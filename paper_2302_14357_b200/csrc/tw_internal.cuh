@@ -76,6 +76,7 @@ struct GemmOut {
   const int* oidx;
   long long ldC;
   const float* bias;  // optional [N]
+  int* err;           // device word, raised by a wait that gave up
 };
 
 // M may come from device memory (M_dev != nullptr): CTAs beyond it exit.
@@ -101,9 +102,10 @@ struct JoinerRows {
   unsigned long long* skipped = nullptr;
 };
 // z[(r,t), k] = sum_j tanh(E[e0[r]+t, j] + Pp[p[r], j]) * W_out[k, j] + b_out[k]; rows of padding
-// frames (t >= slen) are left untouched.
-void launch_joiner_f32(const JoinerRows& rows, const float* W_out, const float* b_out, float* z,
-                       cudaStream_t st);
+// frames (t >= slen) hold no result.  A_buf: optional scratch [R_max S, J] for the operand, so that it is formed once and
+// not once per column tile (nullptr: never).  err: device word, raised by a wait that gave up.  Returns the number of kernels launched.
+int launch_joiner_f32(const JoinerRows& rows, const float* W_out, const float* b_out, float* z, float* A_buf,
+                      int* err, cudaStream_t st);
 // in place: z[(r,t), :] -> log softmax; padding frames get (0 at blank, -inf elsewhere)
 void launch_log_softmax(const JoinerRows& rows, int blank, float* z, cudaStream_t st);
 // Per-row candidates of ChooseNBestExpansions: the row's best N non-blank tokens, best first
