@@ -292,6 +292,39 @@ __global__ void __launch_bounds__(256) joiner_A_f32_kernel(JoinerRows jr, float*
   }
 }
 
+// C[m, n] = sum_k A[m, k] B[n, k] + bias[n] for the tables that tw_init builds from the weights: every product is
+// accumulated over k in ascending order by one thread, so that a table's values do not depend on how a tile is split
+// (a table feeds every later step; the decode-time kernel above is free to choose its split).  64 x 64 tiles, 4 x 4 a thread.
+__global__ void __launch_bounds__(256) gemm_f32_table_kernel(const float* __restrict__ A, const float* __restrict__ B, const float* __restrict__ bias,
+                                                             float* __restrict__ C, int M, int N, int K) {
+  __shared__ __align__(16) float As[16][68], Bs[16][68];
+  const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4, m0 = blockIdx.y * 64, n0 = blockIdx.x * 64;
+  float acc[4][4] = {};
+  for (int k0 = 0; k0 < K; k0 += 16) {
+    for (int i = tid; i < 64 * 16; i += 256) {
+      const int r = i >> 4, k = i & 15;
+      As[k][r] = (m0 + r < M && k0 + k < K) ? A[(long long)(m0 + r) * K + k0 + k] : 0.f;
+      Bs[k][r] = (n0 + r < N && k0 + k < K) ? B[(long long)(n0 + r) * K + k0 + k] : 0.f;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int k = 0; k < 16; ++k) {
+      const float4 a = *reinterpret_cast<const float4*>(&As[k][ty * 4]), b = *reinterpret_cast<const float4*>(&Bs[k][tx * 4]);
+      const float aa[4] = {a.x, a.y, a.z, a.w}, bb[4] = {b.x, b.y, b.z, b.w};
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(aa[i], bb[j], acc[i][j]);
+    }
+    __syncthreads();
+  }
+  for (int i = 0; i < 4; ++i)
+    for (int j = 0; j < 4; ++j) {
+      const int m = m0 + ty * 4 + i, n = n0 + tx * 4 + j;
+      if (m < M && n < N) C[(long long)m * N + n] = acc[i][j] + (bias ? bias[n] : 0.f);
+    }
+}
+
 __device__ __forceinline__ float warp_max(float v) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, o));
@@ -504,6 +537,10 @@ void launch_gemm_f32(const GemmOperand& op1, const GemmOperand& op2, const GemmO
   p.op[0] = op1; p.op[1] = op2; p.out = out; p.M_dev = M_dev; p.M_scale = 1; p.M_max = M_max; p.N = N; p.err = out.err;
   auto ok = [](const GemmOperand& o) { return o.K == 0 || ((o.K & 3) == 0 && row_aligned(o.A, o.ldA) && row_aligned(o.B, o.ldB)); };
   launch_gemm_tiles<0>(p, ok(op1) && ok(op2), M_max, N, st);
+}
+
+void launch_gemm_f32_table(const float* A, const float* B, const float* bias, float* C, int M, int N, int K, cudaStream_t st) {
+  gemm_f32_table_kernel<<<dim3((N + 63) / 64, (M + 63) / 64), 256, 0, st>>>(A, B, bias, C, M, N, K);
 }
 
 int launch_joiner_f32(const JoinerRows& rows, const float* W_out, const float* b_out, float* z, float* A_buf, int* err, cudaStream_t st) {

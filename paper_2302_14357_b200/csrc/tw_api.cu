@@ -202,10 +202,7 @@ int build_bf16(tw_handle* h) {
       float* tmp = nullptr;
       TW_CUDA(h, cudaMalloc((void**)&tmp, (size_t)h->V * G4 * sizeof(float)));
       TW_TRY(dev_alloc(h, &h->bf.EmbProj, (size_t)h->V * G4));
-      GemmOperand a{h->emb, nullptr, h->emb_dim, h->W_ih[0], h->emb_dim, h->emb_dim};
-      GemmOperand none{};
-      GemmOut o{tmp, nullptr, G4, h->b_l[0], h->bf.err};
-      launch_gemm_f32(a, none, o, nullptr, h->V, G4, 0);
+      launch_gemm_f32_table(h->emb, h->W_ih[0], h->b_l[0], tmp, h->V, G4, h->emb_dim, 0);
       launch_permute_cols_f32(tmp, perm_dev, h->V, G4, h->bf.EmbProj, 0);
       TW_CUDA(h, cudaDeviceSynchronize());
       cudaFree(tmp);
@@ -385,20 +382,15 @@ int init_impl(tw_handle* h, const tw_model* m, const tw_config* c) {
   if (h->mode == TW_MODE_BF16) TW_TRY(build_bf16(h));
 
   int launches = 0;
-  GemmOperand none{};
   float* init_out = nullptr;                 // InitPredictor's output as given by the caller (Sec. 3.2), float32
   if (m->pred_init_out) TW_TRY(copy_weight(h, &init_out, m->pred_init_out, (size_t)h->P));
   if (h->pred_kind == TW_PRED_STATELESS) {
     // W_p emb[k] for every token: the joiner rows index this table by their last token.  A given initial output
     // gets a row of its own after the vocabulary's, which serves the empty prefix.
     TW_TRY(dev_alloc(h, &h->PpTab, (size_t)(h->V + 1) * h->J));
-    GemmOperand a{h->emb, nullptr, h->emb_dim, h->W_p, h->P, h->P};
-    GemmOut o{h->PpTab, nullptr, h->J, nullptr, h->bf.err};
-    launch_gemm_f32(a, none, o, nullptr, h->V, h->J, 0);
+    launch_gemm_f32_table(h->emb, h->W_p, nullptr, h->PpTab, h->V, h->J, h->P, 0);
     if (init_out) {
-      GemmOperand a1{init_out, nullptr, h->P, h->W_p, h->P, h->P};
-      GemmOut o1{h->PpTab + (size_t)h->V * h->J, nullptr, h->J, nullptr, h->bf.err};
-      launch_gemm_f32(a1, none, o1, nullptr, 1, h->J, 0);
+      launch_gemm_f32_table(init_out, h->W_p, nullptr, h->PpTab + (size_t)h->V * h->J, 1, h->J, h->P, 0);
       h->hs.empty_row = h->hs_fused.empty_row = h->V;
     }
   } else {
@@ -409,9 +401,7 @@ int init_impl(tw_handle* h, const tw_model* m, const tw_config* c) {
       if (m->pred_init_state) TW_TRY(copy_weight(h, &h->init_hc, m->pred_init_state, nhc));
       else { TW_TRY(dev_alloc(h, &h->init_hc, nhc)); TW_CUDA(h, cudaMemset(h->init_hc, 0, nhc * sizeof(float))); }
       const float* out = init_out ? init_out : h->init_hc + (size_t)(h->L - 1) * 2 * h->Hd;
-      GemmOperand a1{out, nullptr, h->P, h->W_p, h->P, h->P};
-      GemmOut o1{h->init_Pp, nullptr, h->J, nullptr, h->bf.err};
-      launch_gemm_f32(a1, none, o1, nullptr, 1, h->J, 0);
+      launch_gemm_f32_table(out, h->W_p, nullptr, h->init_Pp, 1, h->J, h->P, 0);
     } else {
       // one step on the blank token from an all-zero state
       float* zero = nullptr; int* tok = nullptr;

@@ -83,6 +83,9 @@ struct GemmOut {
 void launch_gemm_f32(const GemmOperand& op1, const GemmOperand& op2, const GemmOut& out,
                      const int* M_dev, int M_max, int N, cudaStream_t st);
 
+// C[m, n] = sum_k A[m, k] B[n, k] (+ bias[n]), dense, each product summed in ascending k: the tables tw_init builds
+void launch_gemm_f32_table(const float* A, const float* B, const float* bias, float* C, int M, int N, int K, cudaStream_t st);
+
 // Joiner rows: hypothesis row r covers frames E[row_e0[r] + t], t < row_slen[r], and the projected
 // predictor output Pp[row_p[r]].
 struct JoinerRows {
