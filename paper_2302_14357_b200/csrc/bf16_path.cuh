@@ -96,7 +96,7 @@ void launch_joiner_A_bf16(const JoinerRows& rows, __nv_bfloat16* A, cudaStream_t
 struct FusedJoinerParams {
   const int* R_dev; int R_max;       // hypothesis rows (device count optional; written before the operand kernel ahead of this
                                      // one was launched, and not by it: the kernel reads it ahead of its wait)
-  int S, V, K, blank, CL;            // CL = V / 256 CTAs per cluster; K = J
+  int S, V, K, blank, CL;            // K = J; CL = V / (columns per CTA) CTAs per cluster, filled in by launch_fused_joiner
   int no_max;                        // logits are bounded by zbound (at most 40): softmax sums need no maximum search
   float zbound;                      // max_k (|W_out[k, :]|_1 + |b_out[k]|) >= |z| (tanh joiner); used when no_max
   const float* bias;                 // b_out [V]
@@ -104,7 +104,7 @@ struct FusedJoinerParams {
   const int* row_slen;               // [R] (nullptr: S)
   float* ldphi; float* la; float* lse;   // [R], [R][S], [R][S]
   float* ldnb;                       // [R][V] delta_nb as a probability ratio, NOT its log (0 at the blank column)
-  float* dmax;                       // optional [R][V / 32]: the largest delta_nb of every 32-column chunk of every row
+  float* dmax;                       // optional [R][V / fused_joiner_chunk]: the largest delta_nb of every chunk of columns of every row
                                      // (written by the instances that sum over frames with shuffles: fused_joiner_writes_maxima)
   int* err;
   int hat;                           // factorised output (JoinerRows::hat); log2_tau = log2 of the blank threshold
@@ -117,7 +117,15 @@ bool fused_joiner_eligible(int S, int V, int J);
 bool fused_joiner_specialised(int S);
 bool fused_joiner_writes_maxima(int S);   // the instance for this segment size fills FusedJoinerParams::dmax   // a kernel instance with this segment size compiled in exists
 long long fused_joiner_A_rows(int R_max, int S);      // rows of the tile-layout A operand
-int fused_joiner_setup(int CL, int S, int* max_clusters);
+// Columns of the vocabulary per CTA: 256 shares an operand tile between the fewest CTAs, but a step with few row tiles then
+// leaves most SMs idle.  With 64 or 128 a tile's contraction and epilogue get shorter (B = 32, V = 1024, S = 3: four tiles
+// on 64 instead of 16 CTAs; 16.2 -> 14.9 ms per decode of 400 frames), as long as its cluster (V / columns CTAs, at most 16)
+// fits and the tiles of this row count are one round of resident clusters; a step mostly has some fewer rows than its
+// maximum, hence the 4/5.
+int fused_joiner_columns(int R_max, int S, const int max_clusters[3]);
+inline int fused_joiner_chunk(int columns) { return columns == 64 ? 16 : 32; }     // columns per entry of FusedJoinerParams::dmax
+// max_clusters[i]: clusters the device keeps resident with 64 << i columns per CTA (0: no such cluster)
+int fused_joiner_setup(int V, int S, int max_clusters[3]);
 // max_k (sum_j |W_out[k, j]| + |b_out[k]|): bound of |z| since |tanh| <= 1; written to *out (device)
 void launch_logit_bound(const __nv_bfloat16* W, const float* bias, int V, int J, float* out, cudaStream_t st);
 // dst[r, k] = log src[r * ld_src + k] (log 0 = -inf) for r < R, k < V; dst rows have V columns (dst may be src when
@@ -129,8 +137,8 @@ void launch_joiner_A_tiled(const JoinerRows& rows, __nv_bfloat16* A, cudaStream_
 // the same for the rows of a decode step (utterance b's rows are row_off[b] .. + nA[b] - 1, all on one segment)
 void launch_joiner_A_tiled_utt(const JoinerRows& rows, const int* row_off, const int* nA, int B, __nv_bfloat16* A,
                                cudaStream_t st);
-int launch_fused_joiner(const CUtensorMap& tmA, const CUtensorMap& tmB256, const FusedJoinerParams& p,
-                        int max_clusters, cudaStream_t st);
+int launch_fused_joiner(const Bf16Mat& A, const Bf16Mat& W, const FusedJoinerParams& p, int columns, const int max_clusters[3],
+                        cudaStream_t st);
 // adds log J(t, parent row, token) to A_ld of the hypotheses created in this step
 void launch_survivor_ld(const HypState& hs, int B, int T, const __nv_bfloat16* A, const __nv_bfloat16* W, const float* bias,
                         const float* lse, cudaStream_t st);

@@ -179,14 +179,18 @@ __global__ void __launch_bounds__(2 * kStepThreads) hyp_step_kernel(HypState hs)
       const double base = hs.A_ls[b * kMaxBeam + h];
       // a lower bound of the N-th best value: the N-th largest of the 32 lane maxima (distinct elements)
       const int nchunk = V >> 5;
-      const float* cmax = (hs.dnb_max != nullptr && (V & 31) == 0 && nchunk <= 128) ? hs.dnb_max + (long long)(r0 + h) * nchunk : nullptr;
+      const bool pairs = hs.dnb_chunk == 16;     // maxima of 16 columns: two make a chunk's
+      const float* cmax = (hs.dnb_max != nullptr && (V & 31) == 0 && nchunk <= 128) ? hs.dnb_max + (long long)(r0 + h) * (pairs ? 2 * nchunk : nchunk) : nullptr;
       float lmax = 0.f;
       float m4[4] = {0.f, 0.f, 0.f, 0.f};        // with chunk maxima: those of chunks lane, lane + 32, lane + 64, lane + 96
       if (cmax != nullptr) {
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
           const int c = lane + 32 * u;
-          if (c < nchunk) m4[u] = __ldg(cmax + c);
+          if (c < nchunk) {
+            if (pairs) { const float2 m2 = __ldg(reinterpret_cast<const float2*>(cmax) + c); m4[u] = fmaxf(m2.x, m2.y); }
+            else m4[u] = __ldg(cmax + c);
+          }
           lmax = fmaxf(lmax, m4[u]);
         }
       } else {

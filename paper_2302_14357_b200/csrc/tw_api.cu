@@ -222,8 +222,7 @@ int build_bf16(tw_handle* h) {
   // fused joiner: needs S frames of a hypothesis inside one warp and V split into 256-column CTAs
   h->bf.Vp = (h->V + 255) / 256 * 256;
   if (fused_joiner_eligible(h->S, h->bf.Vp, h->J)) {
-    h->bf.CL = h->bf.Vp / 256;
-    int s = fused_joiner_setup(h->bf.CL, h->S, &h->bf.max_clusters);
+    int s = fused_joiner_setup(h->bf.Vp, h->S, h->bf.max_clusters);
     if (s == TW_OK) {
       if (h->bf.Vp == h->V) {
         h->bf.W_out_pad = h->bf.W_out; h->bf.bias_pad = h->b_out; h->bf.ldnb_pad = h->hs.ldnb;
@@ -243,9 +242,9 @@ int build_bf16(tw_handle* h) {
       TW_CUDA(h, cudaMemcpy(&bound, bound_dev, sizeof(float), cudaMemcpyDeviceToHost));
       h->bf.no_max = (bound <= 40.f) && h->joiner_act == TW_ACT_TANH;   // the bound needs |act| <= 1
       h->bf.zbound = bound;
-      TW_TRY(make_bf16_mat(h, &h->bf.A_tiled, nullptr, fused_joiner_A_rows(h->R_max, h->S), h->J, true, false));
+      TW_TRY(make_bf16_mat(h, &h->bf.A_tiled, nullptr, fused_joiner_A_rows(h->R_max, h->S), h->J, true, true));
       TW_TRY(dev_alloc(h, &h->bf.lse, (size_t)h->R_max * h->S));
-      TW_TRY(dev_alloc(h, &h->bf.dmax, (size_t)h->R_max * (h->bf.Vp / 32)));
+      TW_TRY(dev_alloc(h, &h->bf.dmax, (size_t)h->R_max * (h->bf.Vp / 16)));
       TW_TRY(scan_select_setup());
       h->bf.fused_ok = true;
       // default: on for the segment sizes with a specialised kernel instance; the generic instance is
@@ -467,12 +466,12 @@ int enqueue_joiner_fused(tw_handle* h, const JoinerRows& rows, const float* ld_o
   if (ldnb == nullptr) ldnb = h->bf.ldnb_pad;   // a caller's buffer has V columns: only with an unpadded vocabulary
   FusedJoinerParams fp{};
   fp.R_dev = rows.R_dev; fp.R_max = rows.R_max; fp.S = rows.S; fp.V = h->bf.Vp; fp.K = rows.J; fp.blank = h->blank;
-  fp.CL = h->bf.CL; fp.no_max = h->bf.no_max ? 1 : 0; fp.zbound = h->bf.zbound; fp.bias = h->bf.bias_pad; fp.ld_old = ld_old; fp.row_slen = rows.row_slen;
+  fp.no_max = h->bf.no_max ? 1 : 0; fp.zbound = h->bf.zbound; fp.bias = h->bf.bias_pad; fp.ld_old = ld_old; fp.row_slen = rows.row_slen;
   fp.ldphi = ldphi; fp.la = la; fp.lse = h->bf.lse; fp.ldnb = ldnb; fp.err = h->bf.err; fp.clear_word = clear_word;
   fp.dmax = (ldnb == h->bf.ldnb_pad && fused_joiner_writes_maxima(rows.S)) ? h->bf.dmax : nullptr;   // the chunk maxima belong to the handle's own delta_nb buffer
   fp.early_w = utt_B > 0 ? 0 : 1;       // (measured: beside the per-utterance operand kernel the early loads cost 6 % at c2, S = 10)
   fp.hat = rows.hat; fp.log2_tau = rows.log_tau * 1.4426950408889634f; fp.skipped = rows.skipped;
-  TW_TRY(launch_fused_joiner(h->bf.A_tiled.as_A, h->bf.W_out_pad.as_B256, fp, h->bf.max_clusters, st));
+  TW_TRY(launch_fused_joiner(h->bf.A_tiled, h->bf.W_out_pad, fp, fused_joiner_columns(rows.R_max, rows.S, h->bf.max_clusters), h->bf.max_clusters, st));
   if (mark_fn) mark_fn(h, 2, st);       // the fused kernel alone
   *launches += 2;
   if (cand.n != nullptr) {      // ChooseNBestExpansions, first stage: the rows' N best tokens
@@ -641,7 +640,11 @@ int tw_set_profiling(tw_handle* h, int on) {
 int tw_get_stats(const tw_handle* h, tw_stats* out) {
   if (!h || !out) return TW_ERR_ARG;
   *out = h->stats;
-  out->fused_clusters = h->bf.fused_ok ? h->bf.max_clusters : 0;
+  out->fused_clusters = 0;
+  if (h->bf.fused_ok) {
+    const int nc = fused_joiner_columns(h->R_max, h->S, h->bf.max_clusters);
+    out->fused_clusters = h->bf.max_clusters[nc == 64 ? 0 : (nc == 128 ? 1 : 2)];
+  }
   out->fused_on = (h->mode == TW_MODE_BF16 && h->bf.fused_on) ? 1 : 0;
   return TW_OK;
 }

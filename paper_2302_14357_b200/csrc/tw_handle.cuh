@@ -47,15 +47,15 @@ struct tw_handle {
     // fused joiner + softmax + Eq. 3-7 + selection (logits stay in tensor memory)
     bool fused_ok = false, fused_on = false, no_max = false;
     float zbound = 0.f;                                   // bound of |logit| behind no_max
-    int CL = 0, max_clusters = 0;
-    // The fused kernel splits the vocabulary into 256-column CTAs.  A vocabulary that is not a multiple of 256 is
+    int max_clusters[3] = {0, 0, 0};                      // fused_joiner_setup
+    // The fused kernel splits the vocabulary between CTAs of up to 256 columns.  A vocabulary that is not a multiple of 256 is
     // padded for it: Vp columns, the added rows of W_out zero and their bias -1e30 (probability 0, never a
     // candidate).  Vp == V: the padded objects below are the plain ones.
     int Vp = 0;
     tw::Bf16Mat W_out_pad;
     float* bias_pad = nullptr;
     float* ldnb_pad = nullptr;                            // [R_max, Vp]
-    float* dmax = nullptr;                                // [R_max, Vp / 32] chunk maxima of delta_nb (fused decode path)
+    float* dmax = nullptr;                                // [R_max, Vp / 16 or / 32] chunk maxima of delta_nb (fused decode path)
     tw::Bf16Mat A_tiled;                                  // A operand in the fused kernel's tile layout
     float* lse = nullptr;                                 // [R_max, S]
   } bf;

@@ -138,3 +138,12 @@ def test_fused_joiner_padded_vocabulary_every_element(S, R, rounds):
     the paper's models (Sec. 4.1): the stage returns the 501 real columns.  One tile per cluster, and four."""
     cfg = tw_synth.get_config("p1")
     _run(cfg, S=S, N=16, R=R, G=R // 10, seed=40 + S, min_rounds=rounds)
+
+
+@pytest.mark.parametrize("name,S,R", [("c1", 3, 1), ("c1", 2, 17), ("c1", 5, 140), ("c2", 10, 100), ("c2", 3, 640), ("p1", 4, 33), ("p1", 1, 700),
+                                      ("p1", 5, 160), ("c1", 8, 49)])
+def test_fused_joiner_few_tiles_every_element(name, S, R):
+    """One round of clusters whose CTAs own 64 or 128 columns of the vocabulary, the last tile with one to four of its lane
+    quarters in use (S = 3: ten hypotheses to a quarter, one row fills one quarter, 17 rows of S = 2 two of them)."""
+    cfg = tw_synth.get_config(name)
+    _run(cfg, S=S, N=5, R=R, G=max(1, R // 8), seed=60 + S + R, min_rounds=0)
