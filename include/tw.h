@@ -289,7 +289,7 @@ int tw_joiner_expand_noalloc(const float* W_out, const float* b_out, int32_t J, 
 
 /* TW_MODE_BF16 only: switches between the fused joiner (joiner, softmax and Eq. 3-7 in one kernel, logits
  * kept in tensor memory; available when S <= 32 and V <= 4096, a vocabulary that is not a multiple of 256
- * being padded internally with columns of probability 0; the default for S in {1..5, 8, 10}) and the
+ * being padded internally with columns of probability 0; the default wherever it is available) and the
  * staged kernels that pass the logits through device memory.  Both compute the same quantities.
  * TW_ERR_STATE if the fused kernel is not available for this handle. */
 int tw_set_fused(tw_handle* h, int on);

@@ -105,7 +105,6 @@ struct FusedJoinerParams {
   float* ldphi; float* la; float* lse;   // [R], [R][S], [R][S]
   float* ldnb;                       // [R][V] delta_nb as a probability ratio, NOT its log (0 at the blank column)
   float* dmax;                       // optional [R][V / fused_joiner_chunk]: the largest delta_nb of every chunk of columns of every row
-                                     // (written by the instances that sum over frames with shuffles: fused_joiner_writes_maxima)
   int* err;
   int hat;                           // factorised output (JoinerRows::hat); log2_tau = log2 of the blank threshold
   float log2_tau;
@@ -114,8 +113,6 @@ struct FusedJoinerParams {
   int early_w;                       // 1: the W_out tiles of the first ring stages are asked for ahead of the wait for the operand kernel
 };
 bool fused_joiner_eligible(int S, int V, int J);
-bool fused_joiner_specialised(int S);
-bool fused_joiner_writes_maxima(int S);   // the instance for this segment size fills FusedJoinerParams::dmax   // a kernel instance with this segment size compiled in exists
 long long fused_joiner_A_rows(int R_max, int S);      // rows of the tile-layout A operand
 // Columns of the vocabulary per CTA: 256 shares an operand tile between the fewest CTAs, but a step with few row tiles then
 // leaves most SMs idle.  With 64 or 128 a tile's contraction and epilogue get shorter (B = 32, V = 1024, S = 3: four tiles
@@ -123,7 +120,9 @@ long long fused_joiner_A_rows(int R_max, int S);      // rows of the tile-layout
 // fits and the tiles of this row count are one round of resident clusters; a step mostly has some fewer rows than its
 // maximum, hence the 4/5.
 int fused_joiner_columns(int R_max, int S, const int max_clusters[3]);
-inline int fused_joiner_chunk(int columns) { return columns == 64 ? 16 : 32; }     // columns per entry of FusedJoinerParams::dmax
+bool fused_joiner_writes_maxima(int S);   // the instance for this segment size fills FusedJoinerParams::dmax
+// columns per entry of FusedJoinerParams::dmax (segments of 11 to 16 frames are summed 16 columns at a time)
+inline int fused_joiner_chunk(int columns, int S) { return columns == 64 || (S > 10 && S <= 16) ? 16 : 32; }
 // max_clusters[i]: clusters the device keeps resident with 64 << i columns per CTA (0: no such cluster)
 int fused_joiner_setup(int V, int S, int max_clusters[3]);
 // max_k (sum_j |W_out[k, j]| + |b_out[k]|): bound of |z| since |tanh| <= 1; written to *out (device)

@@ -38,7 +38,7 @@ constexpr int kColGroups = 4;                // epilogue warps per TMEM lane qua
 constexpr int kEpiWarps = 4 * kColGroups, kEpiThreads = 32 * kEpiWarps;
 constexpr int kThreadsFused = 64 + kEpiThreads;
 constexpr uint32_t kABytes = BM * BK * 2, kAQuarter = kABytes / 4;
-// longer segments (S = 5, 8, 10): the sum over a hypothesis's frames goes through a per-warp staging tile in shared
+// longer segments (S >= 5): the sum over a hypothesis's frames goes through a per-warp staging tile in shared
 // memory, 16 columns at a time (row = TMEM lane, odd pitch: conflict-free row-per-lane writes)
 constexpr int kStagePitch = 17;
 
@@ -72,26 +72,12 @@ __device__ __forceinline__ float logaddexp2_fast(float a, float b) {
   return mx + lg2f(1.f + ex2f(d));
 }
 
-// sum over the S lanes [lane, lane + S) of x, valid in lanes whose window stays inside the warp.
-// ST > 0: segment size known at compile time (plain unrolled shuffles); ST == 0: any S <= 32.
-template <int ST>
-__device__ __forceinline__ float window_sum(float x, int S) {
-  if (ST > 0 && ST <= 4) {
-    float total = x;
+// sum over the S lanes [lane, lane + S) of x, valid in lanes whose window stays inside the warp
+template <int S>
+__device__ __forceinline__ float window_sum(float x) {
+  float total = x;
 #pragma unroll
-    for (int d = 1; d < ST; ++d) total += __shfl_down_sync(0xffffffffu, x, d);
-    return total;
-  }
-  // doubling: windows of 1, 2, 4, ... lanes; the set bits of S pick the pieces (unrolled when S is known)
-  const int SS = ST > 0 ? ST : S;
-  float total = 0.f, cur = x;
-  int off = 0;
-#pragma unroll
-  for (int size = 1; size <= 32; size <<= 1) {
-    if (size > SS) break;
-    if (SS & size) { total += (off == 0) ? cur : __shfl_down_sync(0xffffffffu, cur, off); off += size; }   // the first piece is the lane's own
-    if (2 * size <= SS) cur += __shfl_down_sync(0xffffffffu, cur, size);
-  }
+  for (int d = 1; d < S; ++d) total += __shfl_down_sync(0xffffffffu, x, d);
   return total;
 }
 

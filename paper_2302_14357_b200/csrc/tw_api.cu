@@ -247,9 +247,7 @@ int build_bf16(tw_handle* h) {
       TW_TRY(dev_alloc(h, &h->bf.dmax, (size_t)h->R_max * (h->bf.Vp / 16)));
       TW_TRY(scan_select_setup());
       h->bf.fused_ok = true;
-      // default: on for the segment sizes with a specialised kernel instance; the generic instance is
-      // currently slower than the staged kernels
-      h->bf.fused_on = fused_joiner_specialised(h->S);
+      h->bf.fused_on = true;
     }
   }
   h->hs.defer_rows = 0;

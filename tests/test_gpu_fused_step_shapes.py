@@ -147,3 +147,12 @@ def test_fused_joiner_few_tiles_every_element(name, S, R):
     quarters in use (S = 3: ten hypotheses to a quarter, one row fills one quarter, 17 rows of S = 2 two of them)."""
     cfg = tw_synth.get_config(name)
     _run(cfg, S=S, N=5, R=R, G=max(1, R // 8), seed=60 + S + R, min_rounds=0)
+
+
+@pytest.mark.parametrize("name,S,R,rounds", [("c2", 20, 700, 3), ("c2", 13, 1100, 3), ("c1", 6, 37, 0), ("p1", 7, 90, 0), ("c1", 9, 500, 0), ("p1", 11, 70, 0),
+                                             ("c1", 16, 33, 0), ("p1", 17, 5, 0), ("c1", 32, 410, 3), ("p1", 32, 3, 0)])
+def test_fused_joiner_long_segments_every_element(name, S, R, rounds):
+    """S = 6, 7, 9 (instances of their own), 11 to 16 (two hypotheses to a warp) and 17 to 32 (one), at the ends of those ranges,
+    with ragged segments; one quarter of a tile up to several rounds."""
+    cfg = tw_synth.get_config(name)
+    _run(cfg, S=S, N=10, R=R, G=max(1, R // 8), seed=90 + S, min_rounds=rounds)
