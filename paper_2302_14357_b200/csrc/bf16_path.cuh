@@ -94,8 +94,8 @@ void launch_joiner_A_bf16(const JoinerRows& rows, __nv_bfloat16* A, cudaStream_t
 
 // ---- fused joiner + softmax + Eq. 3-7 + candidate selection (fused_joiner.cu) ------------------
 struct FusedJoinerParams {
-  const int* R_dev; int R_max;       // hypothesis rows (device count optional; written before the operand kernel ahead of this
-                                     // one was launched, and not by it: the kernel reads it ahead of its wait)
+  const int* R_dev; int R_max;       // hypothesis rows (device count optional), or as many as the B utterances' list sizes nA
+  const int* nA; int B;              // add up to (nA != nullptr); older than the operand kernel ahead, and read ahead of the wait
   int S, V, K, blank, CL;            // K = J; CL = V / (columns per CTA) CTAs per cluster, filled in by launch_fused_joiner
   int no_max;                        // logits are bounded by zbound (at most 40): softmax sums need no maximum search
   float zbound;                      // max_k (|W_out[k, :]|_1 + |b_out[k]|) >= |z| (tanh joiner); used when no_max
@@ -136,6 +136,17 @@ void launch_joiner_A_tiled(const JoinerRows& rows, __nv_bfloat16* A, cudaStream_
 // the same for the rows of a decode step (utterance b's rows are row_off[b] .. + nA[b] - 1, all on one segment)
 void launch_joiner_A_tiled_utt(const JoinerRows& rows, const int* row_off, const int* nA, int B, __nv_bfloat16* A,
                                cudaStream_t st);
+// The operand of a small decode step.  The kernel also completes the new hypotheses' frame distributions (Eq. 5, from the
+// previous step's operand A_prev and softmax normalisers lse) and numbers the rows of the step, ahead of its wait for the
+// kernel before it (early != 0: that kernel is not hyp_step_kernel).
+struct StepPrep {
+  HypState hs;
+  const __nv_bfloat16* A_prev; const __nv_bfloat16* W; const float* bias; const float* lse;
+  int B, T, early;
+};
+bool step_prep_inside(int R_max, int S);              // whether a decode step of this size takes that kernel
+void launch_joiner_A_step(const JoinerRows& rows, const StepPrep& sp, __nv_bfloat16* A, cudaStream_t st, const void* pf_base,
+                          long long pf_bytes);
 int launch_fused_joiner(const Bf16Mat& A, const Bf16Mat& W, const FusedJoinerParams& p, int columns, const int max_clusters[3],
                         cudaStream_t st);
 // adds log J(t, parent row, token) to A_ld of the hypotheses created in this step

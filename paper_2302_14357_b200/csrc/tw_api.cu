@@ -242,7 +242,14 @@ int build_bf16(tw_handle* h) {
       TW_CUDA(h, cudaMemcpy(&bound, bound_dev, sizeof(float), cudaMemcpyDeviceToHost));
       h->bf.no_max = (bound <= 40.f) && h->joiner_act == TW_ACT_TANH;   // the bound needs |act| <= 1
       h->bf.zbound = bound;
-      TW_TRY(make_bf16_mat(h, &h->bf.A_tiled, nullptr, fused_joiner_A_rows(h->R_max, h->S), h->J, true, true));
+      // (the second operand buffer is for decode steps small enough to complete the previous one inside the operand kernel;
+      // a batch may have any size up to max_batch)
+      const long long rows0 = fused_joiner_A_rows(h->R_max, h->S);
+      long long rows1 = 128;
+      for (int b = h->max_batch; b >= 1; --b)
+        if (step_prep_inside(b * h->N, h->S)) { rows1 = fused_joiner_A_rows(b * h->N, h->S); break; }
+      TW_TRY(make_bf16_mat(h, &h->bf.A_tiled[0], nullptr, rows0, h->J, true, true));
+      TW_TRY(make_bf16_mat(h, &h->bf.A_tiled[1], nullptr, rows1, h->J, true, true));
       TW_TRY(dev_alloc(h, &h->bf.lse, (size_t)h->R_max * h->S));
       TW_TRY(dev_alloc(h, &h->bf.dmax, (size_t)h->R_max * (h->bf.Vp / 16)));
       TW_TRY(scan_select_setup());
@@ -447,38 +454,37 @@ void enqueue_scan(tw_handle* h, const JoinerRows& rows, const float* ld_old, flo
   }
 }
 
-// Fused path: joiner, softmax, Eq. 3-7 and per-row candidates with the logits kept in tensor memory
+// Fused path: joiner, softmax and Eq. 3-7 with the logits kept in tensor memory
 int enqueue_joiner_fused(tw_handle* h, const JoinerRows& rows, const float* ld_old, float* ldphi, float* ldnb,
-                         float* la, const CandOut& cand, cudaStream_t st, int* launches, StageMarkFn mark_fn,
-                         bool plain_first, int utt_B, int* clear_word) {
-  {
-    PdlScope first(plain_first ? false : g_pdl_on);
-    if (utt_B > 0) launch_joiner_A_tiled_utt(rows, h->hs.row_off, h->hs.nA, utt_B, h->bf.A_tiled.ptr, st);
-    else {
-      // a small model's weights stay in L2 between two steps by themselves; a large one's W_out is asked for again
-      const long long wbytes = (long long)h->bf.W_out_pad.rows * h->bf.W_out_pad.K * 2;
-      launch_joiner_A_tiled(rows, h->bf.A_tiled.ptr, st, wbytes >= (4ll << 20) ? h->bf.W_out_pad.ptr : nullptr, wbytes);
-    }
+                         float* la, cudaStream_t st, int* launches, StageMarkFn mark_fn, int step_B, const StepPrep* prep, int* clear_word) {
+  // a small model's weights stay in L2 between two steps by themselves; a large one's W_out is asked for again
+  const long long wbytes = (long long)h->bf.W_out_pad.rows * h->bf.W_out_pad.K * 2;
+  const void* pf = wbytes >= (4ll << 20) ? h->bf.W_out_pad.ptr : nullptr;
+  // long segments: the operand kernel that reads a segment's frames and an utterance's predictor rows once
+  // (measured: c4, S = 10, 554 -> 522..532 ms per decode; no gain at S = 3 or 5)
+  const bool per_utterance = step_B > 0 && prep == nullptr && rows.S >= 8;
+  const Bf16Mat& A = h->bf.A_tiled[prep ? h->bf.par : 0];
+  if (prep) {
+    launch_joiner_A_step(rows, *prep, A.ptr, st, pf, wbytes);
+  } else {
+    // a decode step's operand kernel has two predecessors (the side branch's join): plain stream ordering
+    PdlScope first(step_B > 0 ? false : g_pdl_on);
+    if (per_utterance) launch_joiner_A_tiled_utt(rows, h->hs.row_off, h->hs.nA, step_B, A.ptr, st);
+    else launch_joiner_A_tiled(rows, A.ptr, st, pf, wbytes);
   }
   if (mark_fn) mark_fn(h, 3, st);       // operand preparation is booked with the elementwise stages
   if (ldnb == nullptr) ldnb = h->bf.ldnb_pad;   // a caller's buffer has V columns: only with an unpadded vocabulary
   FusedJoinerParams fp{};
   fp.R_dev = rows.R_dev; fp.R_max = rows.R_max; fp.S = rows.S; fp.V = h->bf.Vp; fp.K = rows.J; fp.blank = h->blank;
+  if (prep) { fp.nA = h->hs.nA; fp.B = step_B; }
   fp.no_max = h->bf.no_max ? 1 : 0; fp.zbound = h->bf.zbound; fp.bias = h->bf.bias_pad; fp.ld_old = ld_old; fp.row_slen = rows.row_slen;
   fp.ldphi = ldphi; fp.la = la; fp.lse = h->bf.lse; fp.ldnb = ldnb; fp.err = h->bf.err; fp.clear_word = clear_word;
   fp.dmax = (ldnb == h->bf.ldnb_pad && fused_joiner_writes_maxima(rows.S)) ? h->bf.dmax : nullptr;   // the chunk maxima belong to the handle's own delta_nb buffer
-  fp.early_w = utt_B > 0 ? 0 : 1;       // (measured: beside the per-utterance operand kernel the early loads cost 6 % at c2, S = 10)
+  fp.early_w = per_utterance ? 0 : 1;   // (measured: beside the per-utterance operand kernel the early loads cost 6 % at c2, S = 10)
   fp.hat = rows.hat; fp.log2_tau = rows.log_tau * 1.4426950408889634f; fp.skipped = rows.skipped;
-  TW_TRY(launch_fused_joiner(h->bf.A_tiled, h->bf.W_out_pad, fp, fused_joiner_columns(rows.R_max, rows.S, h->bf.max_clusters), h->bf.max_clusters, st));
+  TW_TRY(launch_fused_joiner(A, h->bf.W_out_pad, fp, fused_joiner_columns(rows.R_max, rows.S, h->bf.max_clusters), h->bf.max_clusters, st));
   if (mark_fn) mark_fn(h, 2, st);       // the fused kernel alone
   *launches += 2;
-  if (cand.n != nullptr) {      // ChooseNBestExpansions, first stage: the rows' N best tokens
-    ScanSelectArgs a{};
-    a.R_dev = rows.R_dev; a.R_max = rows.R_max; a.S = rows.S; a.V = h->bf.Vp; a.blank = h->blank;
-    a.cand = cand; a.dnb_in = ldnb; a.dnb_linear = 1;
-    launch_scan_select(a, true, st);
-    *launches += 1;
-  }
   return TW_OK;
 }
 
