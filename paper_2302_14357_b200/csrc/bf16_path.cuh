@@ -94,8 +94,8 @@ void launch_joiner_A_bf16(const JoinerRows& rows, __nv_bfloat16* A, cudaStream_t
 
 // ---- fused joiner + softmax + Eq. 3-7 + candidate selection (fused_joiner.cu) ------------------
 struct FusedJoinerParams {
-  const int* R_dev; int R_max;       // hypothesis rows (device count optional), or as many as the B utterances' list sizes nA
-  const int* nA; int B;              // add up to (nA != nullptr); older than the operand kernel ahead, and read ahead of the wait
+  const int* R_dev; int R_max;       // hypothesis rows (device count optional; written before the kernel ahead of this one was
+                                     // launched, and not by it: it is read ahead of the wait)
   int S, V, K, blank, CL;            // K = J; CL = V / (columns per CTA) CTAs per cluster, filled in by launch_fused_joiner
   int no_max;                        // logits are bounded by zbound (at most 40): softmax sums need no maximum search
   float zbound;                      // max_k (|W_out[k, :]|_1 + |b_out[k]|) >= |z| (tanh joiner); used when no_max
@@ -109,6 +109,7 @@ struct FusedJoinerParams {
   int hat;                           // factorised output (JoinerRows::hat); log2_tau = log2 of the blank threshold
   float log2_tau;
   unsigned long long* skipped;       // optional counter of the (row, frame) pairs blank thresholding left out
+  int *clear_word2, *steps_word;     // with clear_word, optional: a second word to clear, a count of the passes that had rows
   int* clear_word;                   // optional: one device word the kernel sets to 0 once its predecessors have finished
   int early_w;                       // 1: the W_out tiles of the first ring stages are asked for ahead of the wait for the operand kernel
 };
@@ -136,17 +137,21 @@ void launch_joiner_A_tiled(const JoinerRows& rows, __nv_bfloat16* A, cudaStream_
 // the same for the rows of a decode step (utterance b's rows are row_off[b] .. + nA[b] - 1, all on one segment)
 void launch_joiner_A_tiled_utt(const JoinerRows& rows, const int* row_off, const int* nA, int B, __nv_bfloat16* A,
                                cudaStream_t st);
-// The operand of a small decode step.  The kernel also completes the new hypotheses' frame distributions (Eq. 5, from the
-// previous step's operand A_prev and softmax normalisers lse) and numbers the rows of the step, ahead of its wait for the
-// kernel before it (early != 0: that kernel is not hyp_step_kernel).
-struct StepPrep {
-  HypState hs;
-  const __nv_bfloat16* A_prev; const __nv_bfloat16* W; const float* bias; const float* lse;
-  int B, T, early;
+// The output projection of the new hypotheses (M_dev entries of the work list, at most M) with the joiner's operand rows
+// formed from it (pred_out.cu): Pp row pw_new[m], and for frame t of the segment of utterance b = pw_bi[m] / kMaxBeam the
+// operand row of joiner row row_off[b] + pw_bi[m] % kMaxBeam.
+struct WpOperandParams {
+  const int* M_dev; int M, N, K;     // N = J, K = the predictor's output width
+  const int* pw_new; const int* pw_bi;
+  const int* row_off; const int* t0; const int* slen;    // per utterance
+  const float* E; int T, S, act;     // projected frames: row b * T + t
+  float* Pp; __nv_bfloat16* A;
+  const char* pf_base; long long pf_bytes;               // optional: a constant matrix to ask into L2
+  int* err;
 };
-bool step_prep_inside(int R_max, int S);              // whether a decode step of this size takes that kernel
-void launch_joiner_A_step(const JoinerRows& rows, const StepPrep& sp, __nv_bfloat16* A, cudaStream_t st, const void* pf_base,
-                          long long pf_bytes);
+int wp_operand_setup();
+void launch_wp_operand(const Bf16Mat& A, const Bf16Mat& W, const WpOperandParams& p, cudaStream_t st);
+
 int launch_fused_joiner(const Bf16Mat& A, const Bf16Mat& W, const FusedJoinerParams& p, int columns, const int max_clusters[3],
                         cudaStream_t st);
 // adds log J(t, parent row, token) to A_ld of the hypotheses created in this step

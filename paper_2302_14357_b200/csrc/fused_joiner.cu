@@ -23,7 +23,7 @@
 #include <map>
 #include <mutex>
 
-#include "bf16_path.cuh"
+#include "operand.cuh"
 #include "sm100.cuh"
 
 namespace tw {

@@ -8,7 +8,7 @@
 // stage kernels work on values relative to the row's score, which stay small.
 #include <cuda_bf16.h>
 
-#include "tw_internal.cuh"
+#include "operand.cuh"
 #include "sm100.cuh"
 
 namespace tw {
@@ -63,6 +63,27 @@ __device__ void turn_over(const HypState& hs, int b) {
   }
 }
 
+// own_rows, behind a turn_over: claims the joiner rows of the carried hypotheses and writes their tables and operand rows.
+// Called by the whole CTA.
+__device__ void carry_rows(const HypState& hs, int b) {
+  __shared__ int s_r0;
+  __syncthreads();                           // what turn_over wrote
+  const int n = hs.nA[b], sl = hs.slen[b], t0 = hs.t0[b], S = hs.S, J = hs.J, per = J >> 3;
+  if (threadIdx.x == 0) { s_r0 = atomicAdd(hs.rows_next, n); hs.row_off[b] = s_r0; }
+  __syncthreads();
+  const int r0 = s_r0;
+  if (threadIdx.x < n) hs.row_slen[r0 + threadIdx.x] = sl;
+  for (int i = threadIdx.x; i < n * S; i += blockDim.x) hs.row_ld[(long long)r0 * S + i] = (i % S) == 0 ? 0.f : -INFINITY;   // all mass on the first frame
+  for (int c = threadIdx.x; c < n * sl * per; c += blockDim.x) {
+    const int pair = c / per, x = (c - pair * per) * 8, hh = pair / sl, t = pair - hh * sl;
+    const float* e = hs.E + ((long long)b * hs.E_T + t0 + t) * J + x;
+    const float* pp = hs.slot_Pp + ((long long)b * hs.capSlot + hs.A_slot[b * kMaxBeam + hh]) * J + x;
+    *reinterpret_cast<uint4*>(static_cast<__nv_bfloat16*>(hs.A_next) + operand_row(r0 + hh, t, S) * J + x) =
+        act8(*reinterpret_cast<const float4*>(e), *reinterpret_cast<const float4*>(e + 4), *reinterpret_cast<const float4*>(pp),
+             *reinterpret_cast<const float4*>(pp + 4), hs.act);
+  }
+}
+
 __global__ void __launch_bounds__(kThreads) hyp_init_kernel(HypState hs, const int* lengths, int T) {
   const int b = blockIdx.x;
   const long long gs = (long long)b * hs.capSlot;   // slot 0 holds the empty hypothesis
@@ -87,7 +108,10 @@ __global__ void __launch_bounds__(kThreads) hyp_init_kernel(HypState hs, const i
     for (int i = threadIdx.x; i < hs.J; i += blockDim.x) hs.slot_Pp[gs * hs.J + i] = hs.init_Pp[i];
   }
   __syncthreads();
-  if (hs.len[b] > 0) turn_over(hs, b);
+  if (hs.len[b] > 0) {
+    turn_over(hs, b);
+    if (hs.own_rows) carry_rows(hs, b);
+  }
 }
 
 constexpr int kStepThreads = 512;   // 16 warps: one per hypothesis of list A
@@ -103,7 +127,7 @@ __device__ __forceinline__ unsigned long long order_key(double x) {
 }
 
 __global__ void __launch_bounds__(2 * kStepThreads) hyp_step_kernel(HypState hs) {
-  __shared__ int s_nB, s_hasthr, s_nkeep, s_wbase;
+  __shared__ int s_hasthr, s_nkeep, s_wbase, s_rbase;
   __shared__ int s_found[kMaxBeam], s_touched[kMaxBeam], s_carry[kMaxBeam];
   __shared__ double s_Als[kMaxBeam], s_Adone[kMaxBeam];
   __shared__ int s_Aslot[kMaxBeam], s_Alen[kMaxBeam];
@@ -157,7 +181,13 @@ __global__ void __launch_bounds__(2 * kStepThreads) hyp_step_kernel(HypState hs)
   const int N = hs.N, S = hs.S, V = hs.V;
 
   if (tid < kMaxBeam) { s_Als[tid] = ld_Als; s_Aslot[tid] = ld_Aslot; s_Adone[tid] = ld_Adone; s_carry[tid] = ld_carry; }
-  if (tid == 0) { hs.calls[b] += 1; hs.joins[b] += slen; }
+  if (tid == 0) {
+    hs.calls[b] += 1; hs.joins[b] += slen;
+    if (hs.own_rows) {                      // totals of the pass
+      atomicAdd(reinterpret_cast<unsigned long long*>(hs.rows_total), (unsigned long long)H);
+      atomicAdd(reinterpret_cast<unsigned long long*>(hs.rows_total) + 1, (unsigned long long)(H * slen));
+    }
+  }
   // With in-kernel selection the CTA has 32 warps: warps 16..31 select (one row each) while warps 0..15 merge the
   // blank expansions into list B and find the threshold; the two halves meet at the barrier before the ranking.
   // Until then the merging half synchronises on a named barrier of its own.
@@ -370,7 +400,6 @@ __global__ void __launch_bounds__(2 * kStepThreads) hyp_step_kernel(HypState hs)
   if (tid == 0) {
     int nB = nB0;
     for (int q = 0; q < H; ++q) nB += (s_found[q] < 0);
-    s_nB = nB;
     hs.nB[b] = nB;
   }
   if (warp < 16) sync_merge();
@@ -477,9 +506,51 @@ __global__ void __launch_bounds__(2 * kStepThreads) hyp_step_kernel(HypState hs)
       hs.nA[b] = nk; hs.n_new[b] = nk;
       s_wbase = (hs.inline_gather && nk > 0) ? atomicAdd(&hs.scalars[kScNPred], nk) : 0;   // this utterance's work-list entries
     }
+    if (lane == 1 && hs.own_rows && nk > 0) { const int r = atomicAdd(hs.rows_next, nk); s_rbase = r; hs.row_off[b] = r; }
   }
   __syncthreads();
   const int nk = s_nkeep;
+
+  // ---- own_rows: log J(t, k) of the kept expansions, a warp per (expansion, frame), the last warps first (the first ones
+  // write the new lists below); their joiner rows' frame distributions relative to their scores
+  if (hs.own_rows) {
+    const int J = hs.J;
+    for (int pair = (int)(blockDim.x >> 5) - 1 - warp; pair < nk * slen; pair += blockDim.x >> 5) {
+      const int i = pair / slen, t = pair - i * slen;
+      const int h = s_keep_h[i], k = s_keep_k[i];
+      const long long rt = (long long)(r0 + h) * S + t;
+      const __nv_bfloat16* arow = static_cast<const __nv_bfloat16*>(hs.A_cur) + operand_row(r0 + h, t, S) * J;
+      const __nv_bfloat16* wrow = static_cast<const __nv_bfloat16*>(hs.W_out) + (long long)k * J;
+      const float la = hs.la[rt], lse = hs.lse_j[rt], bias = hs.b_out[k];
+      float acc = 0.f;
+#pragma unroll 4
+      for (int x = lane * 8; x < J; x += 256) {
+        const uint4 av = *reinterpret_cast<const uint4*>(arow + x), wv = __ldg(reinterpret_cast<const uint4*>(wrow + x));
+        const __nv_bfloat162* a2 = reinterpret_cast<const __nv_bfloat162*>(&av);
+        const __nv_bfloat162* w2 = reinterpret_cast<const __nv_bfloat162*>(&wv);
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          const float2 af = __bfloat1622float2(a2[u]), wf = __bfloat1622float2(w2[u]);
+          acc = fmaf(af.x, wf.x, fmaf(af.y, wf.y, acc));
+        }
+      }
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+      if (lane == 0) {
+        const double d = s_Als[h] + (double)la + ((double)(acc + bias) - (double)lse), ls = s_keep_ls[i];
+        const float rel = d == -INFINITY ? -INFINITY : (float)(d - ls);
+        float* out = hs.row_ld + (long long)(s_rbase + i) * S;
+        if (!hs.mono) {
+          out[t] = rel;
+        } else {                            // emitted at frame t: continues at t + 1, or has left the segment
+          if (t == 0) out[0] = -INFINITY;
+          if (t + 1 < slen) out[t + 1] = rel;
+          else hs.A_done[b * kMaxBeam + i] = d;
+        }
+      }
+    }
+    if (tid < nk) hs.row_slen[s_rbase + tid] = slen;
+  }
 
   // ---- new list A (one warp per kept expansion): tokens, hash, frame distribution d_h(k) (Eq. 5)
   if (warp < nk) {
@@ -508,7 +579,7 @@ __global__ void __launch_bounds__(2 * kStepThreads) hyp_step_kernel(HypState hs)
         for (int l = 0; l < hs.L; ++l) sm100::prefetch_l2_bulk(pc + (long long)l * 2 * hs.Hd, (uint32_t)hs.Hd * 4u);
       }
       const int wrow = s_wbase + i;
-      if (wrow < hs.B * hs.N) { hs.pw_new[wrow] = (int)gn; hs.pw_par[wrow] = (int)gp; hs.pw_tok[wrow] = k; }
+      if (wrow < hs.B * hs.N) { hs.pw_new[wrow] = (int)gn; hs.pw_par[wrow] = (int)gp; hs.pw_tok[wrow] = k; hs.pw_bi[wrow] = b * kMaxBeam + i; }
       else hs.status[b] = TW_ERR_LIMIT;            // cannot happen: the list holds at most N entries per utterance
     }
     const long long r = r0 + h;
@@ -524,7 +595,9 @@ __global__ void __launch_bounds__(2 * kStepThreads) hyp_step_kernel(HypState hs)
       }
       return v;
     };
-    if (!hs.mono) {
+    if (hs.own_rows) {
+      // done above
+    } else if (!hs.mono) {
       for (int t = lane; t < S; t += 32) hs.A_ld[((long long)b * kMaxBeam + i) * S + t] = d_at(t);
     } else {
       // emitted at frame t: the hypothesis continues at frame t + 1, or has left the segment
@@ -560,7 +633,10 @@ __global__ void __launch_bounds__(2 * kStepThreads) hyp_step_kernel(HypState hs)
     }
   }
   // ---- list A empty: this segment is done ------------------------------------------------------
-  if (nk == 0 && hs.t0[b] + slen < hs.len[b]) turn_over(hs, b);
+  if (nk == 0 && hs.t0[b] + slen < hs.len[b]) {
+    turn_over(hs, b);
+    if (hs.own_rows) carry_rows(hs, b);
+  }
 }
 
 // One CTA: packs the live hypotheses of all utterances into joiner rows and the new hypotheses
@@ -666,7 +742,10 @@ __global__ void __launch_bounds__(kThreads) stream_advance_kernel(HypState hs, c
     s_go = (hs.nA[b] == 0 && hs.t0[b] + hs.slen[b] < len);
   }
   __syncthreads();
-  if (s_go) turn_over(hs, b);
+  if (s_go) {
+    turn_over(hs, b);
+    if (hs.own_rows) carry_rows(hs, b);
+  }
 }
 
 // ChooseNBest(B) at the end of the utterance, best first.

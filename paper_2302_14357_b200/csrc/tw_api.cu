@@ -85,7 +85,8 @@ void gemm_bf16(tw_handle* h, const Bf16Mat& A, const Bf16Mat& B, const int* M_de
 // output W_p g goes to row (idx_out ? idx_out[i] : i) of Pp_out.  State rows are [L][2][Hd].
 void enqueue_predictor(tw_handle* h, const int* tok, const float* hc_in, const int* idx_in, float* hc_out,
                        const int* idx_out, float* Pp_out, const int* n_dev, int n_max, cudaStream_t st,
-                       int* launches, const WorkListBuild* wl = nullptr, bool gathered = false) {
+                       int* launches, const WorkListBuild* wl = nullptr, bool gathered = false,
+                       const WpOperandParams* wo = nullptr) {
   GemmOperand none{};
   if (h->pred_kind == TW_PRED_STATELESS) {
     GemmOperand a{h->emb, tok, h->emb_dim, h->W_p, h->P, h->P};
@@ -115,7 +116,11 @@ void enqueue_predictor(tw_handle* h, const int* tok, const float* hc_in, const i
       if (!launch_gemm_lstm_wide(h->bf.X[l].as_A, h->bf.W_cat[l].as_B64, h->bf.W_cat[l].as_B32, p, st))
         launch_gemm_bf16(h->bf.X[l].as_A, h->bf.W_cat[l].as_B128, h->bf.W_cat[l].as_B256, p, st);
     }
-    gemm_bf16(h, h->bf.Htop, h->bf.W_p, n_dev, n_max, Pp_out, idx_out, h->J, nullptr, st, nullptr, nullptr, 0, /*m_early=*/1);
+    if (wo) {                             // the projection forms the joiner's operand too
+      launch_wp_operand(h->bf.Htop, h->bf.W_p, *wo, st);
+    } else {
+      gemm_bf16(h, h->bf.Htop, h->bf.W_p, n_dev, n_max, Pp_out, idx_out, h->J, nullptr, st, nullptr, nullptr, 0, /*m_early=*/1);
+    }
     *launches += L + (gathered ? 1 : 2);
     return;
   }
@@ -149,7 +154,8 @@ int enqueue_predictor_plain(tw_handle* h, const int* tokens, const float* state_
 // UpdatePredictorOutput for the work list the compaction kernel built (new slot, parent slot, token).
 // build_list: the compaction kernel did not run; the gather kernel derives the work list from the per-utterance
 // lists of new hypotheses itself (bf16 mode)
-void enqueue_predictor_slots(tw_handle* h, cudaStream_t st, int* launches, bool build_list = false, int B = 0) {
+void enqueue_predictor_slots(tw_handle* h, cudaStream_t st, int* launches, bool build_list = false, int B = 0,
+                             const WpOperandParams* wo = nullptr) {
   if (h->pred_kind == TW_PRED_STATELESS) return;   // the joiner reads W_p emb[last token] from a table
   const HypState& hs = h->hs;
   WorkListBuild wl{};
@@ -159,7 +165,7 @@ void enqueue_predictor_slots(tw_handle* h, cudaStream_t st, int* launches, bool 
   }
   const bool gathered = build_list && h->hs_fused.inline_gather != 0;
   enqueue_predictor(h, hs.pw_tok, hs.slot_hc, hs.pw_par, hs.slot_hc, hs.pw_new, hs.slot_Pp,
-                    hs.scalars + kScNPred, h->R_max, st, launches, build_list && !gathered ? &wl : nullptr, gathered);
+                    hs.scalars + kScNPred, h->R_max, st, launches, build_list && !gathered ? &wl : nullptr, gathered, wo);
 }
 
 // E = enc W_e^T for `rows` frames
@@ -181,13 +187,14 @@ void enqueue_project(tw_handle* h, const void* enc, int rows, float* E, cudaStre
 int build_bf16(tw_handle* h) {
   if ((h->D_enc % 8) || (h->J % 8) || (h->P % 8) || (h->emb_dim % 8) || (h->Hd % 8)) return TW_ERR_ARG;
   TW_TRY(gemm_bf16_setup());
+  TW_TRY(wp_operand_setup());
   TW_TRY(make_bf16_mat(h, &h->bf.W_e, h->W_e, h->J, h->D_enc, false, true));
   TW_TRY(make_bf16_mat(h, &h->bf.W_out, h->W_out, h->V, h->J, false, true));
   TW_TRY(make_bf16_mat(h, &h->bf.enc, nullptr, (long long)h->max_batch * h->max_T, h->D_enc, true, false));
   TW_TRY(make_bf16_mat(h, &h->bf.A_join, nullptr, (long long)h->R_max * h->S, h->J, true, false));
   if (h->pred_kind == TW_PRED_LSTM) {
     TW_TRY(make_bf16_mat(h, &h->bf.W_p, h->W_p, h->J, h->P, false, true));
-    TW_TRY(make_bf16_mat(h, &h->bf.Htop, nullptr, h->R_max, h->Hd, true, false));
+    TW_TRY(make_bf16_mat(h, &h->bf.Htop, nullptr, h->R_max, h->Hd, true, true));
     // Gate GEMM outputs are interleaved by hidden unit (column 4 j + g = gate g of unit j) so that the
     // LSTM cell can run in the GEMM epilogue: weight rows, biases and the table are permuted once here.
     const int G4 = 4 * h->Hd;
@@ -242,14 +249,9 @@ int build_bf16(tw_handle* h) {
       TW_CUDA(h, cudaMemcpy(&bound, bound_dev, sizeof(float), cudaMemcpyDeviceToHost));
       h->bf.no_max = (bound <= 40.f) && h->joiner_act == TW_ACT_TANH;   // the bound needs |act| <= 1
       h->bf.zbound = bound;
-      // (the second operand buffer is for decode steps small enough to complete the previous one inside the operand kernel;
-      // a batch may have any size up to max_batch)
-      const long long rows0 = fused_joiner_A_rows(h->R_max, h->S);
-      long long rows1 = 128;
-      for (int b = h->max_batch; b >= 1; --b)
-        if (step_prep_inside(b * h->N, h->S)) { rows1 = fused_joiner_A_rows(b * h->N, h->S); break; }
-      TW_TRY(make_bf16_mat(h, &h->bf.A_tiled[0], nullptr, rows0, h->J, true, true));
-      TW_TRY(make_bf16_mat(h, &h->bf.A_tiled[1], nullptr, rows1, h->J, true, true));
+      // two operand buffers: a step's operand is written while the previous step's is still read
+      for (Bf16Mat& a : h->bf.A_tiled)
+        TW_TRY(make_bf16_mat(h, &a, nullptr, &a == &h->bf.A_tiled[0] || h->S < 8 ? fused_joiner_A_rows(h->R_max, h->S) : 128, h->J, true, true));
       TW_TRY(dev_alloc(h, &h->bf.lse, (size_t)h->R_max * h->S));
       TW_TRY(dev_alloc(h, &h->bf.dmax, (size_t)h->R_max * (h->bf.Vp / 16)));
       TW_TRY(scan_select_setup());
@@ -325,7 +327,7 @@ int build_workspace(tw_handle* h) {
   TW_TRY(dev_alloc(h, &hs.new_par, nb * kMaxBeam));
   TW_TRY(dev_alloc(h, &hs.new_tok, nb * kMaxBeam));
   TW_TRY(dev_alloc(h, &hs.new_row, nb * kMaxBeam));
-  int** per_row[] = {&hs.row_b, &hs.row_e0, &hs.row_p, &hs.row_slen, &hs.pw_new, &hs.pw_par, &hs.pw_tok,
+  int** per_row[] = {&hs.row_b, &hs.row_e0, &hs.row_p, &hs.row_slen, &hs.pw_new, &hs.pw_par, &hs.pw_tok, &hs.pw_bi,
                      &h->stage_e0, &h->stage_slen};
   for (int** p : per_row) TW_TRY(dev_alloc(h, p, R));
   TW_TRY(dev_alloc(h, &hs.row_ld, R * S));
@@ -456,16 +458,16 @@ void enqueue_scan(tw_handle* h, const JoinerRows& rows, const float* ld_old, flo
 
 // Fused path: joiner, softmax and Eq. 3-7 with the logits kept in tensor memory
 int enqueue_joiner_fused(tw_handle* h, const JoinerRows& rows, const float* ld_old, float* ldphi, float* ldnb,
-                         float* la, cudaStream_t st, int* launches, StageMarkFn mark_fn, int step_B, const StepPrep* prep, int* clear_word) {
+                         float* la, cudaStream_t st, int* launches, StageMarkFn mark_fn, int step_B, int* clear_word, bool own_rows) {
   // a small model's weights stay in L2 between two steps by themselves; a large one's W_out is asked for again
   const long long wbytes = (long long)h->bf.W_out_pad.rows * h->bf.W_out_pad.K * 2;
   const void* pf = wbytes >= (4ll << 20) ? h->bf.W_out_pad.ptr : nullptr;
   // long segments: the operand kernel that reads a segment's frames and an utterance's predictor rows once
   // (measured: c4, S = 10, 554 -> 522..532 ms per decode; no gain at S = 3 or 5)
-  const bool per_utterance = step_B > 0 && prep == nullptr && rows.S >= 8;
-  const Bf16Mat& A = h->bf.A_tiled[prep ? h->bf.par : 0];
-  if (prep) {
-    launch_joiner_A_step(rows, *prep, A.ptr, st, pf, wbytes);
+  const bool per_utterance = step_B > 0 && rows.S >= 8;
+  const Bf16Mat& A = h->bf.A_tiled[own_rows ? h->bf.par : 0];
+  if (own_rows) {
+    *launches -= 1;
   } else {
     // a decode step's operand kernel has two predecessors (the side branch's join): plain stream ordering
     PdlScope first(step_B > 0 ? false : g_pdl_on);
@@ -476,9 +478,9 @@ int enqueue_joiner_fused(tw_handle* h, const JoinerRows& rows, const float* ld_o
   if (ldnb == nullptr) ldnb = h->bf.ldnb_pad;   // a caller's buffer has V columns: only with an unpadded vocabulary
   FusedJoinerParams fp{};
   fp.R_dev = rows.R_dev; fp.R_max = rows.R_max; fp.S = rows.S; fp.V = h->bf.Vp; fp.K = rows.J; fp.blank = h->blank;
-  if (prep) { fp.nA = h->hs.nA; fp.B = step_B; }
   fp.no_max = h->bf.no_max ? 1 : 0; fp.zbound = h->bf.zbound; fp.bias = h->bf.bias_pad; fp.ld_old = ld_old; fp.row_slen = rows.row_slen;
   fp.ldphi = ldphi; fp.la = la; fp.lse = h->bf.lse; fp.ldnb = ldnb; fp.err = h->bf.err; fp.clear_word = clear_word;
+  if (own_rows) { fp.clear_word2 = h->hs.scalars + kScRow0 + (h->bf.par ^ 1); fp.steps_word = h->hs.scalars + kScSteps; }
   fp.dmax = (ldnb == h->bf.ldnb_pad && fused_joiner_writes_maxima(rows.S)) ? h->bf.dmax : nullptr;   // the chunk maxima belong to the handle's own delta_nb buffer
   fp.early_w = per_utterance ? 0 : 1;   // (measured: beside the per-utterance operand kernel the early loads cost 6 % at c2, S = 10)
   fp.hat = rows.hat; fp.log2_tau = rows.log_tau * 1.4426950408889634f; fp.skipped = rows.skipped;

@@ -56,7 +56,7 @@ struct tw_handle {
     float* bias_pad = nullptr;
     float* ldnb_pad = nullptr;                            // [R_max, Vp]
     float* dmax = nullptr;                                // [R_max, Vp / 16 or / 32] chunk maxima of delta_nb (fused decode path)
-    tw::Bf16Mat A_tiled[2];                               // A operand in the fused kernel's tile layout; small decode steps take them in turn
+    tw::Bf16Mat A_tiled[2];                               // A operand in the fused kernel's tile layout; own_rows: the steps take them in turn
     int par = 0;                                          // the one the next step writes
     float* lse = nullptr;                                 // [R_max, S]
   } bf;
@@ -121,8 +121,8 @@ typedef void (*StageMarkFn)(tw_handle*, int, cudaStream_t);
 int enqueue_joiner_fused(tw_handle* h, const JoinerRows& rows, const float* ld_old, float* ldphi, float* ldnb,
                          float* la, cudaStream_t st, int* launches, StageMarkFn mark_fn = nullptr,
                          int step_B = 0,              // step_B > 0: the rows are a decode step's (hs.row_off, hs.nA of step_B utterances)
-                         const StepPrep* prep = nullptr,   // a small one: numbered and completed by the operand kernel
-                         int* clear_word = nullptr);  // a device word the fused kernel clears (FusedJoinerParams::clear_word)
+                         int* clear_word = nullptr,   // a device word the fused kernel clears (FusedJoinerParams::clear_word)
+                         bool own_rows = false);      // a decode step with HypState::own_rows: its operand rows are written already
 void enqueue_scan(tw_handle* h, const JoinerRows& rows, const float* ld_old, float* logp, float* ldphi,
                   float* ldnb, float* la, double* ldphi_d, double* la_d, const CandOut& cand, cudaStream_t st,
                   int* launches);

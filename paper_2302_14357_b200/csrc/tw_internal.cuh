@@ -143,7 +143,7 @@ void launch_rows_from_groups(const int* row_group, const int* seg_len, int R, in
 
 // ---------------------------------------------------------------------------------------------
 // Hypothesis state of a batch (structure of arrays in one device workspace).
-enum Scalar { kScR = 0, kScNPred = 1, kScActive = 2, kScSteps = 3, kScM = 4, kScCount = 8 };   // kScM = R * S
+enum Scalar { kScR = 0, kScNPred = 1, kScActive = 2, kScSteps = 3, kScM = 4, kScRow0 = 5, kScRow1 = 6, kScCount = 8 };   // kScM = R * S; kScRow0/1: HypState::own_rows
 
 struct HypState {
   int B, N, S, V, J, U_cap, I_max, blank;
@@ -187,6 +187,7 @@ struct HypState {
   int *row_off, *new_off;     // [B] first row / first work-list entry of each utterance
   // compacted predictor work list: [B*N]
   int *pw_new, *pw_par, *pw_tok;
+  int* pw_bi;                 // utterance * kMaxBeam + position in list A (written with inline_gather)
   int* scalars;           // [kScCount] device scalars
   long long* rows_total;  // [2]: sum over steps of rows R, and of rows x their segment's frames
   // stage outputs of the current step
@@ -208,6 +209,17 @@ struct HypState {
   // table far larger than L2) and every layer reads the parent's cell state; hyp_step_kernel, which is the first to
   // know tokens and parents, asks for both in L2 so that the GEMM's epilogue threads do not each wait on DRAM.
   const char* pf_table; int pf_row_bytes;
+  // own_rows != 0 (fused bf16 decode, LSTM predictor, S < 8, inline_gather): there is no kernel between hyp_step_kernel and
+  // the next pass's predictor that numbers the rows.  An utterance claims the joiner rows of its new list A by an atomic
+  // add on *rows_next (as it claims its work-list entries: the order varies from run to run, no result depends on it),
+  // and hyp_step_kernel itself completes their frame distributions (row_ld, Eq. 5: log J of the kept expansions from the
+  // pass's operand A_cur and W_out, S dot products of length J each) and writes the operand rows of hypotheses carried over
+  // a segment turn-over into A_next; those of new hypotheses are written with the predictor's output.
+  // rows_next is one of two words, in turn: the joiner kernel reads one and clears the other.
+  int own_rows; int* rows_next;
+  const float* E; int E_T, act;             // projected frames (row b * E_T + t) and the joiner's nonlinearity
+  const void* A_cur; void* A_next;          // operand of this pass / of the next one, bf16
+  const void* W_out; const float* b_out; const float* lse_j;
 };
 
 void launch_hyp_init(const HypState& hs, const int* lengths, int B, int T, cudaStream_t st);
