@@ -49,8 +49,8 @@ void launch_gemm_bf16(const CUtensorMap& tmA, const CUtensorMap& tmB128, const C
 
 // LSTM gate GEMM (epi == 1) as a single wave of one tile per CTA when 128 x 256 tiles would need a second,
 // nearly empty wave; returns false (nothing launched) when the shape does not call for it.
-// tmB64 / tmB32: maps of B with 64- and 32-row boxes
-bool launch_gemm_lstm_wide(const CUtensorMap& tmA, const CUtensorMap& tmB64, const CUtensorMap& tmB32,
+// tmA32: map of A with 32-row boxes; tmB64 / tmB32: maps of B with 64- and 32-row boxes
+bool launch_gemm_lstm_wide(const CUtensorMap& tmA, const CUtensorMap& tmA32, const CUtensorMap& tmB64, const CUtensorMap& tmB32,
                            const GemmBf16Params& p, cudaStream_t st);
 
 // A bf16 matrix with its tensor maps

@@ -257,10 +257,22 @@ gemm_bf16_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
 // over floor(#SM / row tiles) CTAs in units of 32 columns, so every CTA owns exactly one tile of up to
 // 320 columns (one tcgen05.mma of N <= 256 plus one of N <= 64 per K step, accumulators side by side in
 // TMEM) and the whole GEMM is one wave.  B is loaded in boxes of 64 (and one of 32) rows.
-constexpr int kWideMaxBN = 320, kWideStages = 4, kWideEpiWarps = 16;
-constexpr int kThreadsWide = 64 + 32 * kWideEpiWarps;
-constexpr uint32_t kWideABytes = BM * BK * 2, kWideBBytes = kWideMaxBN * BK * 2;
-constexpr size_t kWideSmem = (size_t)kWideStages * (kWideABytes + kWideBBytes) + 1024 + 256;
+// Two instances: 16 epilogue warps for tiles of up to 320 columns, one CTA per SM; 8 for tiles of up to 128 columns (small
+// steps), which takes less than half of an SM's shared memory, registers and tensor memory, so that the next kernel's CTAs
+// are resident beside it, past their set-up and with their first weight tiles already in shared memory when it ends.
+// The ring's stages are as large as the CTA's own tile needs (128 rows of A, its columns of B).  A row tile whose last lane
+// quarters have no rows fetches, in the small instance, only the quarters that do (what the MMA makes of stale operand rows
+// stays in their lanes).
+constexpr int kWideMaxStages = 8;
+constexpr uint32_t kWideABytes = BM * BK * 2;
+template <int EPIW>
+struct Wide {
+  static constexpr int kMaxBN = EPIW == 16 ? 320 : 128, kThreads = 64 + 32 * EPIW, kGroups = EPIW / 4;
+  static constexpr int kMaxChunks = (kMaxBN / 32 + kGroups - 1) / kGroups;      // chunks of 32 columns a warp can own (groups of 4 warps)
+  static constexpr uint32_t kTmem = EPIW == 16 ? 512 : 128;
+  static constexpr uint32_t kRing = EPIW == 16 ? 4 * (kWideABytes + kMaxBN * BK * 2) : 5 * (kWideABytes + 32 * BK * 2);
+  static constexpr size_t kSmem = (size_t)kRing + 1024 + 256;
+};
 
 // The LSTM cell on one CTA's accumulator tile: rows m0 .. m0 + 127, gate columns n0 .. n0 + 32 nu - 1 (TMEM columns
 // 0 .. 32 nu - 1).  Called by the 16 epilogue warps (warp = 2 .. 17).  Two things keep the part after the contraction
@@ -269,23 +281,33 @@ constexpr size_t kWideSmem = (size_t)kWideStages * (kWideABytes + kWideBBytes) +
 // those rows (128 bytes per thread and chunk, scattered) runs while the first operand tiles are still on their way,
 // and the MMA thread waits on acc_init for it.  (2) The parents' cell states of all of a warp's chunks are fetched
 // into registers during the contraction.  After it a chunk is one tensor-memory load, the cell and three stores.
-constexpr int kWideMaxChunks = (kWideMaxBN / 32 + 3) / 4;      // chunks of 32 columns a warp can own (groups of 4 warps)
+// M_late (the kernel ahead writes the row count, and M is its maximum): the row tables, which have M entries, are asked for
+// together with the count.
+template <int EPIW>
 __device__ __forceinline__ void lstm_tile_epilogue(const GemmBf16Params& p, uint32_t tmem_base, uint64_t* acc_full,
-                                                   uint64_t* acc_init, int M, int m0, int n0, int nu, int warp, int lane) {
+                                                   uint64_t* acc_init, int M, const int* M_late, int m0, int n0, int nu, int warp, int lane) {
+  constexpr int kWideMaxChunks = Wide<EPIW>::kMaxChunks, kWideEpiWarps = EPIW;
   // a row per thread; warp group grp takes the 32-column chunks grp, grp + 4, grp + 8
   const int ew = warp - 2, q = warp & 3, grp = ew >> 2;
   const int m = m0 + q * 32 + lane;
-  const bool live = m < M;                                   // tcgen05 accesses below are warp-wide: idle rows stay in the loops
+  bool live = m < M;                                         // tcgen05 accesses below are warp-wide: idle rows stay in the loops
+  const int i_in = (live && p.lstm.idx_in) ? p.lstm.idx_in[m] : m, i_out = (live && p.lstm.idx_out) ? p.lstm.idx_out[m] : m;
+  const int i_add = (live && p.addend && p.add_idx) ? p.add_idx[m] : m;
+  if (EPIW == 8 && M_late) {
+    const int M_now = *M_late;
+    if (m0 >= M_now) return;
+    live = m < M_now;
+  }
   const long long stride = (long long)p.lstm.L * 2 * p.lstm.Hd, lo = (long long)p.lstm.l * 2 * p.lstm.Hd;
   const float* cin = nullptr;
   const float* arow = nullptr;
   float* hout = nullptr;
   __nv_bfloat16* xrow = nullptr;
   if (live) {
-    cin = p.lstm.hc_in + (long long)(p.lstm.idx_in ? p.lstm.idx_in[m] : m) * stride + lo + p.lstm.Hd;
-    hout = p.lstm.hc_out + (long long)(p.lstm.idx_out ? p.lstm.idx_out[m] : m) * stride + lo;
+    cin = p.lstm.hc_in + (long long)i_in * stride + lo + p.lstm.Hd;
+    hout = p.lstm.hc_out + (long long)i_out * stride + lo;
     xrow = p.lstm.xnext + (long long)m * p.lstm.ld_xnext;
-    if (p.addend) arow = p.addend + (long long)(p.add_idx ? p.add_idx[m] : m) * p.ld_add;
+    if (p.addend) arow = p.addend + (long long)i_add * p.ld_add;
   }
   // 256-bit accesses when every row segment this kernel touches starts on a 32-byte boundary
   const bool wide_ok = (p.lstm.Hd & 7) == 0 &&
@@ -384,16 +406,16 @@ __device__ __forceinline__ void lstm_tile_epilogue(const GemmBf16Params& p, uint
     }
   }
 }
-__global__ void __launch_bounds__(kThreadsWide, 1)
-gemm_lstm_wide_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB64,
-                      const __grid_constant__ CUtensorMap tmB32, GemmBf16Params p) {
+template <int EPIW>
+__global__ void __launch_bounds__(Wide<EPIW>::kThreads, EPIW == 16 ? 1 : 2)
+gemm_lstm_wide_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmA32,
+                      const __grid_constant__ CUtensorMap tmB64, const __grid_constant__ CUtensorMap tmB32, GemmBf16Params p) {
+  using W = Wide<EPIW>;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
-  uint8_t* sA = smem;
-  uint8_t* sB = smem + kWideStages * kWideABytes;
-  uint64_t* full = reinterpret_cast<uint64_t*>(sB + kWideStages * kWideBBytes);
-  uint64_t* empty = full + kWideStages;
-  uint64_t* acc_full = empty + kWideStages;
+  uint64_t* full = reinterpret_cast<uint64_t*>(smem + W::kRing);
+  uint64_t* empty = full + kWideMaxStages;
+  uint64_t* acc_full = empty + kWideMaxStages;
   uint64_t* acc_init = acc_full + 1;        // the epilogue warps have written the accumulators' initial values
   uint32_t* tmem_holder = reinterpret_cast<uint32_t*>(acc_init + 1);
 
@@ -403,25 +425,26 @@ gemm_lstm_wide_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_cons
 
   if (threadIdx.x == 0) {
     prefetch_tensormap(&tmA);
+    if (EPIW == 8) prefetch_tensormap(&tmA32);
     prefetch_tensormap(&tmB64);
     prefetch_tensormap(&tmB32);
-    for (int s = 0; s < kWideStages; ++s) { mbar_init(&full[s], 1); mbar_init(&empty[s], 1); }
+    for (int s = 0; s < kWideMaxStages; ++s) { mbar_init(&full[s], EPIW == 8 ? 2 : 1); mbar_init(&empty[s], 1); }   // full, small instance: B's bytes and A's, each armed apart
     mbar_init(acc_full, 1);
-    mbar_init(acc_init, kWideEpiWarps);
+    mbar_init(acc_init, EPIW);
     fence_barrier_init();
     fence_proxy_async_smem();
   }
-  if (warp == 1) { tmem_alloc(tmem_holder, 512); tmem_relinquish(); }
+  if (warp == 1) { tmem_alloc(tmem_holder, W::kTmem); tmem_relinquish(); }
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem_base = *tmem_holder;
-  // the set-up above touched only this CTA: it may overlap the tail of the kernel that produces A and M
-  pdl_wait();
-  pdl_trigger();
-  // The split follows the row count of THIS launch: fewer row tiles than the grid was sized for give
-  // every row tile more CTAs, i.e. narrower and faster tiles (never wider than the host's bound).
-  const int M = p.M_dev ? (p.m_early ? M_pre : *p.M_dev) : p.M;
+  // The split follows the row count of THIS launch: fewer row tiles than the grid was sized for give every row tile more
+  // CTAs, i.e. narrower and faster tiles (never wider than the host's bound).  The small instance, where the kernel ahead
+  // writes the count (late), splits for the largest count: its tiles are narrow anyway, and so are known before the wait.
+  const bool late = EPIW == 8 && p.M_dev != nullptr && !p.m_early;
+  if (EPIW == 16) { pdl_wait(); pdl_trigger(); }      // the set-up touched only this CTA: it may overlap the tail of the kernel that produces A and M
+  const int M = (late || !p.M_dev) ? p.M : (p.m_early ? M_pre : *p.M_dev);
   const int m_tiles = M > 0 ? (M + BM - 1) / BM : 1;
   const int units = p.N >> 5;
   int n_split = (int)gridDim.x / m_tiles;
@@ -430,38 +453,65 @@ gemm_lstm_wide_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_cons
   const int m0 = mt * BM;
   const int ubase = units / n_split, urem = units - ubase * n_split;
   const int u0 = ns * ubase + (ns < urem ? ns : urem), nu = ubase + (ns < urem ? 1 : 0);
-  const int n0 = u0 * 32, w = nu * 32;                   // this CTA's columns [n0, n0 + w), w <= kWideMaxBN
-  if (w > kWideMaxBN && threadIdx.x == 0) atomicExch(p.err, 1);    // the host sizes the grid so that this cannot happen
-  const bool active = m0 < M && mt < m_tiles && w <= kWideMaxBN;   // an idle CTA skips the roles and only frees its TMEM
+  const int n0 = u0 * 32, w = nu * 32;                   // this CTA's columns [n0, n0 + w), w <= kMaxBN
+  if (w > W::kMaxBN && threadIdx.x == 0) atomicExch(p.err, 1);     // the host sizes the grid so that this cannot happen
+  const bool active = m0 < M && mt < m_tiles && w <= W::kMaxBN;    // an idle CTA skips the roles and only frees its TMEM
+  const uint32_t stage = kWideABytes + (uint32_t)w * (BK * 2);
+  const int nst = EPIW == 16 ? 4 : min((int)(W::kRing / stage), kWideMaxStages);
 
   if (!active) {
+    if (EPIW == 8) { pdl_wait(); pdl_trigger(); }
   } else if (warp == 0) {
+    const uint64_t keep = l2_policy_evict_last();          // the gate weights: read again by every step
+    auto send_B = [&](int kb, int s, uint32_t more = 0) {
+      mbar_expect_tx(&full[s], (uint32_t)w * (BK * 2) + more);
+      uint8_t* bdst = smem + s * stage + kWideABytes;
+      int r = 0;
+      for (; r + 64 <= w; r += 64) tma_load_2d_hint(bdst + r * (BK * 2), &tmB64, &full[s], kb * BK, n0 + r, keep);
+      if (r < w) tma_load_2d_hint(bdst + r * (BK * 2), &tmB32, &full[s], kb * BK, n0 + r, keep);
+    };
+    int npre = 0;
+    if (EPIW == 8) {
+      // the weights of the first stages ahead of the wait (with the wide tiles of a large step that measured slower: the
+      // kernel ahead is still pulling its own through L2)
+      npre = min(num_kb, nst);
+      if (lane == 0) for (int kb = 0; kb < npre; ++kb) send_B(kb, kb);
+      pdl_wait();
+      pdl_trigger();
+    }
     if (lane == 0) {
-      const uint64_t keep = l2_policy_evict_last();        // the gate weights: read again by every step
-      for (int kb = 0; kb < num_kb; ++kb) {
-        const int s = kb % kWideStages;
-        const uint32_t ph = (kb / kWideStages) & 1;
-        if (!mbar_wait(&empty[s], ph ^ 1, p.err)) break;
-        mbar_expect_tx(&full[s], kWideABytes + (uint32_t)w * (BK * 2));
-        tma_load_2d(sA + s * kWideABytes, &tmA, &full[s], kb * BK, m0);
-        uint8_t* bdst = sB + s * kWideBBytes;
-        int r = 0;
-        for (; r + 64 <= w; r += 64) tma_load_2d_hint(bdst + r * (BK * 2), &tmB64, &full[s], kb * BK, n0 + r, keep);
-        if (r < w) tma_load_2d_hint(bdst + r * (BK * 2), &tmB32, &full[s], kb * BK, n0 + r, keep);
+      const int rows = (late ? *p.M_dev : M) - m0;
+      const int nq = EPIW == 8 && rows < BM ? (rows + 31) >> 5 : 4;      // lane quarters with rows in them (the large instance fetches all)
+      const uint32_t a_bytes = (uint32_t)nq * (kWideABytes / 4);
+      int s = 0;
+      uint32_t ph = 0;
+      if (rows <= 0)                                         // late: no rows after all; only the copies under way have to be waited for
+        for (int kb = 0; kb < npre; ++kb) { mbar_arrive(&full[kb]); mbar_wait(&full[kb], 0, p.err); }
+      for (int kb = 0; kb < num_kb && rows > 0; ++kb) {
+        if (kb >= npre) {
+          if (!mbar_wait(&empty[s], ph ^ 1, p.err)) break;
+          send_B(kb, s, EPIW == 8 ? 0 : a_bytes);
+        }
+        if (EPIW == 8) mbar_expect_tx(&full[s], a_bytes);
+        uint8_t* adst = smem + s * stage;
+        if (nq == 4) tma_load_2d(adst, &tmA, &full[s], kb * BK, m0);
+        else for (int q = 0; q < nq; ++q) tma_load_2d(adst + q * (kWideABytes / 4), &tmA32, &full[s], kb * BK, m0 + 32 * q);
+        if (++s == nst) { s = 0; ph ^= 1; }
       }
     }
   } else if (warp == 1) {
-    if (lane == 0) {
+    if (EPIW == 8) { pdl_wait(); pdl_trigger(); }
+    if (lane == 0 && (!late || m0 < *p.M_dev)) {
       const int n1 = w <= 256 ? w : ((w >> 1) + 15) & ~15, n2 = w - n1;    // wider than one MMA: two of about equal width
       const uint32_t idesc1 = make_idesc_bf16(BM, n1), idesc2 = make_idesc_bf16(BM, n2);
       bool ok = mbar_wait(acc_init, 0, p.err);             // the accumulators hold bias + addend: accumulate onto them
+      int s = 0;
+      uint32_t ph = 0;
       for (int kb = 0; kb < num_kb && ok; ++kb) {
-        const int s = kb % kWideStages;
-        const uint32_t ph = (kb / kWideStages) & 1;
         ok = mbar_wait(&full[s], ph, p.err);
         if (!ok) break;
         tc_fence_after();
-        const uint32_t a_addr = smem_u32(sA + s * kWideABytes), b_addr = smem_u32(sB + s * kWideBBytes);
+        const uint32_t a_addr = smem_u32(smem + s * stage), b_addr = a_addr + kWideABytes;
 #pragma unroll
         for (int k = 0; k < BK / 16; ++k) {
           const uint64_t da = make_desc_k_sw128(a_addr + k * 32);
@@ -470,15 +520,17 @@ gemm_lstm_wide_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_cons
             umma_bf16(tmem_base + (uint32_t)n1, da, make_desc_k_sw128(b_addr + n1 * (BK * 2) + k * 32), idesc2, 1u);
         }
         umma_commit(&empty[s]);
+        if (++s == nst) { s = 0; ph ^= 1; }
       }
       if (ok) umma_commit(acc_full);
     }
   } else {
-    lstm_tile_epilogue(p, tmem_base, acc_full, acc_init, M, m0, n0, nu, warp, lane);
+    if (EPIW == 8) { pdl_wait(); pdl_trigger(); }
+    lstm_tile_epilogue<EPIW>(p, tmem_base, acc_full, acc_init, M, late ? p.M_dev : nullptr, m0, n0, nu, warp, lane);
   }
   tc_fence_before();
   __syncthreads();
-  if (warp == 1) tmem_dealloc(tmem_base, 512);
+  if (warp == 1) tmem_dealloc(tmem_base, W::kTmem);
 }
 
 typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
@@ -532,7 +584,8 @@ int gemm_bf16_setup() {
   cudaError_t e4 = cudaFuncSetAttribute(gemm_bf16_kernel<128, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Cfg<128>::kSmem);
   cudaError_t e6 = cudaFuncSetAttribute(gemm_bf16_kernel<64, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Cfg<64>::kSmem);
   if (e6 != cudaSuccess) return TW_ERR_CUDA;
-  cudaError_t e5 = cudaFuncSetAttribute(gemm_lstm_wide_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kWideSmem);
+  cudaError_t e5 = cudaFuncSetAttribute(gemm_lstm_wide_kernel<16>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Wide<16>::kSmem);
+  if (cudaFuncSetAttribute(gemm_lstm_wide_kernel<8>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Wide<8>::kSmem) != cudaSuccess) return TW_ERR_CUDA;
   return (e1 == cudaSuccess && e2 == cudaSuccess && e3 == cudaSuccess && e4 == cudaSuccess && e5 == cudaSuccess) ? TW_OK : TW_ERR_CUDA;
 }
 
@@ -546,7 +599,7 @@ static int sm_count() {
   return num_sms;
 }
 
-bool launch_gemm_lstm_wide(const CUtensorMap& tmA, const CUtensorMap& tmB64, const CUtensorMap& tmB32,
+bool launch_gemm_lstm_wide(const CUtensorMap& tmA, const CUtensorMap& tmA32, const CUtensorMap& tmB64, const CUtensorMap& tmB32,
                            const GemmBf16Params& p, cudaStream_t st) {
   if (p.epi != 1 || p.M <= 0 || p.N <= 0 || (p.N & 31) != 0) return false;
   const int num_sms = sm_count();
@@ -556,9 +609,15 @@ bool launch_gemm_lstm_wide(const CUtensorMap& tmA, const CUtensorMap& tmB64, con
   const int n_split = num_sms / mt;
   if (n_split < 1) return false;
   const int units = p.N >> 5;
-  if (((units + n_split - 1) / n_split) * 32 > kWideMaxBN) return false;
+  const int w = ((units + n_split - 1) / n_split) * 32;
+  if (w > Wide<16>::kMaxBN) return false;
+  // one or two row tiles at most: the small instance
+  if (mt <= 2 && w <= 64) {
+    launch_pdl(gemm_lstm_wide_kernel<8>, dim3(num_sms), dim3(Wide<8>::kThreads), Wide<8>::kSmem, st, tmA, tmA32, tmB64, tmB32, p);
+    return true;
+  }
   // one CTA per SM: the kernel splits the columns of each row tile over floor(grid / row tiles of this launch) CTAs
-  launch_pdl(gemm_lstm_wide_kernel, dim3(num_sms), dim3(kThreadsWide), kWideSmem, st, tmA, tmB64, tmB32, p);
+  launch_pdl(gemm_lstm_wide_kernel<16>, dim3(num_sms), dim3(Wide<16>::kThreads), Wide<16>::kSmem, st, tmA, tmA32, tmB64, tmB32, p);
   return true;
 }
 

@@ -19,14 +19,14 @@ constexpr int BM = 128, BK = 64, kCols = 16;       // kCols: accumulator columns
 
 template <int BN>
 struct WpCfg {
-  static constexpr int kStages = BN == 64 ? 8 : 10;
+  static constexpr int kStages = BN == 64 ? 8 : 5;          // BN = 32: half an SM, to be resident beside a gate GEMM's CTA
   static constexpr int kEpiWarps = 4 * (BN / kCols), kThreads = 64 + 32 * kEpiWarps;
   static constexpr uint32_t kABytes = BM * BK * 2, kBBytes = BN * BK * 2;
   static constexpr size_t kSmem = (size_t)kStages * (kABytes + kBBytes) + 1024 + 256;
 };
 
 template <int BN>
-__global__ void __launch_bounds__(WpCfg<BN>::kThreads, 1)
+__global__ void __launch_bounds__(WpCfg<BN>::kThreads, BN == 64 ? 1 : 2)
 wp_operand_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmA32, const __grid_constant__ CUtensorMap tmB,
                   WpOperandParams p) {
   using C = WpCfg<BN>;

@@ -113,7 +113,7 @@ void enqueue_predictor(tw_handle* h, const int* tok, const float* hc_in, const i
       p.m_early = l > 0;                      // the row count is older than the layer below, which runs ahead of this one
       p.lstm = LstmEpi{hc_in, idx_in, hc_out, idx_out, L, l, Hd,
                        (l + 1 < L) ? h->bf.X[l + 1].ptr : h->bf.Htop.ptr, (l + 1 < L) ? 2LL * Hd : (long long)Hd};
-      if (!launch_gemm_lstm_wide(h->bf.X[l].as_A, h->bf.W_cat[l].as_B64, h->bf.W_cat[l].as_B32, p, st))
+      if (!launch_gemm_lstm_wide(h->bf.X[l].as_A, h->bf.X[l].as_B32, h->bf.W_cat[l].as_B64, h->bf.W_cat[l].as_B32, p, st))
         launch_gemm_bf16(h->bf.X[l].as_A, h->bf.W_cat[l].as_B128, h->bf.W_cat[l].as_B256, p, st);
     }
     if (wo) {                             // the projection forms the joiner's operand too
@@ -215,13 +215,13 @@ int build_bf16(tw_handle* h) {
       cudaFree(tmp);
       TW_TRY(make_bf16_mat(h, &h->bf.W_cat[0], nullptr, G4, h->Hd, false, true));
       launch_gather_concat_bf16(h->W_hh[0], perm_dev, h->Hd, h->Hd, nullptr, nullptr, 0, 0, nullptr, G4, h->bf.W_cat[0].ptr, 0);
-      TW_TRY(make_bf16_mat(h, &h->bf.X[0], nullptr, h->R_max, h->Hd, true, false));
+      TW_TRY(make_bf16_mat(h, &h->bf.X[0], nullptr, h->R_max, h->Hd, true, true));
     }
     for (int l = 1; l < h->L; ++l) {
       TW_TRY(make_bf16_mat(h, &h->bf.W_cat[l], nullptr, G4, 2 * h->Hd, false, true));
       launch_gather_concat_bf16(h->W_ih[l], perm_dev, h->Hd, h->Hd, h->W_hh[l], perm_dev, h->Hd, h->Hd, nullptr, G4,
                                 h->bf.W_cat[l].ptr, 0);
-      TW_TRY(make_bf16_mat(h, &h->bf.X[l], nullptr, h->R_max, 2 * h->Hd, true, false));
+      TW_TRY(make_bf16_mat(h, &h->bf.X[l], nullptr, h->R_max, 2 * h->Hd, true, true));
       TW_TRY(dev_alloc(h, &h->bf.bias_perm[l], (size_t)G4));
       launch_permute_cols_f32(h->b_l[l], perm_dev, 1, G4, h->bf.bias_perm[l], 0);
     }
