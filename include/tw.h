@@ -151,8 +151,8 @@ int tw_destroy(tw_handle* h);
  *   out_scores [B, N]        float64 log p, descending; -inf for an unused slot
  *   out_status [B]           TW_OK, TW_ERR_LIMIT or TW_ERR_ARG per utterance
  * Every step of the inner loop (joiner over the segment, softmax, Eq. 3-7, AddAndMerge, threshold,
- * N-best expansions, predictor update) runs on the device; the host only enqueues batches of steps
- * and polls one completion word between batches.  The call synchronises `stream` before returning.
+ * N-best expansions, predictor update) runs on the device, and so does the loop's end; the host enqueues it
+ * and waits.  The call synchronises `stream` before returning.
  * Returns TW_ERR_LIMIT if any utterance hit a cap (outputs are still valid for the others),
  * TW_ERR_ARG if B > max_batch, T > max_T or a pointer is null.
  */
@@ -294,8 +294,8 @@ int tw_joiner_expand_noalloc(const float* W_out, const float* b_out, int32_t J, 
  * TW_ERR_STATE if the fused kernel is not available for this handle. */
 int tw_set_fused(tw_handle* h, int on);
 
-/* tw_decode replays its step body (16 device steps) as a CUDA graph, captured once per batch shape, on
- * a stream of the handle's own that is ordered after `stream`; tw_set_graph(h, 0) makes it enqueue the
+/* tw_decode runs its loop as a CUDA graph (a conditional node, a few device steps per iteration), captured once per batch
+ * shape, on a stream of the handle's own that is ordered after `stream`; tw_set_graph(h, 0) makes it enqueue the
  * kernels one by one on `stream` instead (as it also does while profiling is on).  Default: on. */
 int tw_set_graph(tw_handle* h, int on);
 

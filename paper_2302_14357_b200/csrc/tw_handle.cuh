@@ -73,14 +73,13 @@ struct tw_handle {
 
   int* host_flag = nullptr;   // pinned copy of the device scalars
 
-  // The step body (kStepsPerGraph device steps) is captured once per (B, T, joiner path) into a CUDA
-  // graph and replayed; it runs on a stream of the handle's own because the caller's may be the legacy
-  // default stream, which cannot be captured.
+  // The decode loop is captured once per (B, T, joiner path) into a CUDA graph and replayed; it runs on a stream of the
+  // handle's own because the caller's may be the legacy default stream, which cannot be captured.
   bool graph_on = true, graph_failed = false;
   cudaStream_t own_stream = nullptr;
   cudaEvent_t ev_order = nullptr;
   cudaGraphExec_t graph_exec = nullptr;
-  int graph_B = -1, graph_T = -1, graph_fused = -1, graph_launches = 0;
+  int graph_B = -1, graph_T = -1, graph_fused = -1, graph_launches = 0, graph_steps = 0;
   cudaEvent_t ev_poll = nullptr;
   // side branch of a decode step: the kernel that completes the new hypotheses' frame distributions and
   // writes the rows' row_ld runs on aux_stream beside the next pass's predictor kernels (fork after the
@@ -96,6 +95,7 @@ struct tw_handle {
     cudaStream_t st = nullptr;
     bool use_graph = false, active = false;
     long long issued = 0, max_steps = 0;
+    int loop_steps = 4;
     int launches = 0;
   } run;
 

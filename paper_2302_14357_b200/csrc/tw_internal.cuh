@@ -143,7 +143,7 @@ void launch_rows_from_groups(const int* row_group, const int* seg_len, int R, in
 
 // ---------------------------------------------------------------------------------------------
 // Hypothesis state of a batch (structure of arrays in one device workspace).
-enum Scalar { kScR = 0, kScNPred = 1, kScActive = 2, kScSteps = 3, kScM = 4, kScRow0 = 5, kScRow1 = 6, kScCount = 8 };   // kScM = R * S; kScRow0/1: HypState::own_rows
+enum Scalar { kScR = 0, kScNPred = 1, kScActive = 2, kScSteps = 3, kScM = 4, kScRow0 = 5, kScRow1 = 6, kScIter = 7, kScCount = 8 };   // kScM = R * S; kScRow0/1: HypState::own_rows
 
 struct HypState {
   int B, N, S, V, J, U_cap, I_max, blank;
@@ -221,6 +221,10 @@ struct HypState {
   const void* A_cur; void* A_next;          // operand of this pass / of the next one, bf16
   const void* W_out; const float* b_out; const float* lse_j;
 };
+
+// Last kernel of the decode loop's body (a conditional graph node): the body runs again while *rows != 0 and *err == 0, at most
+// max_iterations times in all; *iterations counts
+void launch_loop_cond(cudaGraphConditionalHandle handle, const int* rows, const int* err, int* iterations, int max_iterations, cudaStream_t st);
 
 void launch_hyp_init(const HypState& hs, const int* lengths, int B, int T, cudaStream_t st);
 void launch_hyp_step(const HypState& hs, int B, cudaStream_t st);
