@@ -474,6 +474,8 @@ __global__ void __launch_bounds__(256) expand_f32_kernel(const float* __restrict
 
 __global__ void rows_from_groups_kernel(const int* row_group, const int* seg_len, int R, int G, int S,
                                         int* row_e0, int* row_slen) {
+  pdl_wait();
+  pdl_trigger();
   int r = blockIdx.x * blockDim.x + threadIdx.x;
   if (r >= R) return;
   int g = row_group[r];
@@ -581,7 +583,7 @@ void launch_expand_f32(const float* logp, const float* ld_old, const int* row_sl
 void launch_rows_from_groups(const int* row_group, const int* seg_len, int R, int G, int S, int* row_e0,
                              int* row_slen, cudaStream_t st) {
   if (R <= 0) return;
-  rows_from_groups_kernel<<<(R + 255) / 256, 256, 0, st>>>(row_group, seg_len, R, G, S, row_e0, row_slen);
+  launch_pdl(rows_from_groups_kernel, dim3((R + 255) / 256), dim3(256), 0, st, row_group, seg_len, R, G, S, row_e0, row_slen);
 }
 
 }  // namespace tw

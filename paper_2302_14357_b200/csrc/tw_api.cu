@@ -41,12 +41,20 @@ int copy_weight(tw_handle* h, float** dst, const void* src, size_t count) {
   return TW_OK;
 }
 
-// Encoder frames of the caller's element type -> what the projection GEMM of this mode reads: the bf16 operand
-// buffer (TW_MODE_BF16) or float32 frames (TW_MODE_F32; the caller's own buffer when it is float32 already).
-const float* stage_frames(tw_handle* h, const void* enc, long long n, cudaStream_t st) {
+// Encoder frames of the caller's element type -> what the projection GEMM of this mode reads: float32 frames (TW_MODE_F32; the
+// caller's own buffer when it is float32 already), or nullptr and the bf16 operand in *A (TW_MODE_BF16; bf16 frames are read
+// where they are, through a tensor map of the caller's buffer, if that starts on a 16-byte boundary).
+const float* stage_frames(tw_handle* h, const void* enc, long long rows, Bf16Mat* A, cudaStream_t st) {
+  const long long n = rows * h->D_enc;
   if (h->mode == TW_MODE_BF16) {
-    if (h->dtype == TW_BF16) cudaMemcpyAsync(h->bf.enc.ptr, enc, (size_t)n * 2, cudaMemcpyDeviceToDevice, st);
-    else launch_f32_to_bf16(static_cast<const float*>(enc), h->bf.enc.ptr, n, st);
+    *A = h->bf.enc;
+    if (h->dtype == TW_BF16) {
+      if (make_tmap_bf16(&A->as_A, enc, (uint64_t)rows, (uint64_t)h->D_enc, 128) == TW_OK) return nullptr;
+      *A = h->bf.enc;
+      cudaMemcpyAsync(h->bf.enc.ptr, enc, (size_t)n * 2, cudaMemcpyDeviceToDevice, st);
+    } else {
+      launch_f32_to_bf16(static_cast<const float*>(enc), h->bf.enc.ptr, n, st);
+    }
     return nullptr;
   }
   if (h->dtype == TW_BF16) {
@@ -170,9 +178,10 @@ void enqueue_predictor_slots(tw_handle* h, cudaStream_t st, int* launches, bool 
 
 // E = enc W_e^T for `rows` frames
 void enqueue_project(tw_handle* h, const void* enc, int rows, float* E, cudaStream_t st, int* launches) {
-  const float* enc32 = stage_frames(h, enc, (long long)rows * h->D_enc, st);
+  Bf16Mat A;
+  const float* enc32 = stage_frames(h, enc, rows, &A, st);
   if (h->mode == TW_MODE_BF16) {
-    gemm_bf16(h, h->bf.enc, h->bf.W_e, nullptr, rows, E, nullptr, h->J, nullptr, st);
+    gemm_bf16(h, A, h->bf.W_e, nullptr, rows, E, nullptr, h->J, nullptr, st);
     *launches += 2;
   } else {
     GemmOperand a{enc32, nullptr, h->D_enc, h->W_e, h->D_enc, h->D_enc};
