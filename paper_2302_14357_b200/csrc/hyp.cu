@@ -63,6 +63,13 @@ __device__ void turn_over(const HypState& hs, int b) {
   }
 }
 
+// Row of a hypothesis in the projected predictor outputs: its slot, or (stateless predictor) its last token's row of the table
+__device__ __forceinline__ int pp_row(const HypState& hs, long long gs) {
+  if (!hs.stateless) return (int)gs;
+  const int ln = hs.slot_len[gs];
+  return ln > 0 ? hs.slot_tok[gs * hs.U_cap + ln - 1] : hs.empty_row;
+}
+
 // own_rows, behind a turn_over: claims the joiner rows of the carried hypotheses and writes their tables and operand rows.
 // Called by the whole CTA.
 __device__ void carry_rows(const HypState& hs, int b) {
@@ -73,7 +80,12 @@ __device__ void carry_rows(const HypState& hs, int b) {
   __syncthreads();
   const int r0 = s_r0;
   if (threadIdx.x < n) hs.row_slen[r0 + threadIdx.x] = sl;
+  if (hs.own_rows == 2 && threadIdx.x < n) {
+    hs.row_e0[r0 + threadIdx.x] = b * hs.E_T + t0;
+    hs.row_p[r0 + threadIdx.x] = pp_row(hs, (long long)b * hs.capSlot + hs.A_slot[b * kMaxBeam + threadIdx.x]);
+  }
   for (int i = threadIdx.x; i < n * S; i += blockDim.x) hs.row_ld[(long long)r0 * S + i] = (i % S) == 0 ? 0.f : -INFINITY;   // all mass on the first frame
+  if (hs.own_rows == 2) return;
   for (int c = threadIdx.x; c < n * sl * per; c += blockDim.x) {
     const int pair = c / per, x = (c - pair * per) * 8, hh = pair / sl, t = pair - hh * sl;
     const float* e = hs.E + ((long long)b * hs.E_T + t0 + t) * J + x;
@@ -504,7 +516,7 @@ __global__ void __launch_bounds__(2 * kStepThreads) hyp_step_kernel(HypState hs)
       if (passm != 0 && (capped || (passm & ~keepm) != 0)) hs.status[b] = TW_ERR_LIMIT;   // pass cap or token capacity
       s_nkeep = nk;
       hs.nA[b] = nk; hs.n_new[b] = nk;
-      s_wbase = (hs.inline_gather && nk > 0) ? atomicAdd(&hs.scalars[kScNPred], nk) : 0;   // this utterance's work-list entries
+      s_wbase = ((hs.inline_gather || hs.own_rows == 2) && nk > 0) ? atomicAdd(&hs.scalars[kScNPred], nk) : 0;   // this utterance's work-list entries
     }
     if (lane == 1 && hs.own_rows && nk > 0) { const int r = atomicAdd(hs.rows_next, nk); s_rbase = r; hs.row_off[b] = r; }
   }
@@ -513,7 +525,7 @@ __global__ void __launch_bounds__(2 * kStepThreads) hyp_step_kernel(HypState hs)
 
   // ---- own_rows: log J(t, k) of the kept expansions, a warp per (expansion, frame), the last warps first (the first ones
   // write the new lists below); their joiner rows' frame distributions relative to their scores
-  if (hs.own_rows) {
+  if (hs.own_rows == 1) {
     const int J = hs.J;
     for (int pair = (int)(blockDim.x >> 5) - 1 - warp; pair < nk * slen; pair += blockDim.x >> 5) {
       const int i = pair / slen, t = pair - i * slen;
@@ -549,8 +561,8 @@ __global__ void __launch_bounds__(2 * kStepThreads) hyp_step_kernel(HypState hs)
         }
       }
     }
-    if (tid < nk) hs.row_slen[s_rbase + tid] = slen;
   }
+  if (hs.own_rows && tid < nk) hs.row_slen[s_rbase + tid] = slen;
 
   // ---- new list A (one warp per kept expansion): tokens, hash, frame distribution d_h(k) (Eq. 5)
   if (warp < nk) {
@@ -595,13 +607,23 @@ __global__ void __launch_bounds__(2 * kStepThreads) hyp_step_kernel(HypState hs)
       }
       return v;
     };
-    if (hs.own_rows) {
+    if (hs.own_rows == 2 && lane == 0) {             // the joiner row's tables and the work-list entry
+      const int r = s_rbase + i, wrow = s_wbase + i;
+      hs.row_e0[r] = b * hs.E_T + hs.t0[b];
+      hs.row_p[r] = hs.stateless ? k : (int)gn;
+      hs.pw_new[wrow] = (int)gn; hs.pw_par[wrow] = (int)gp; hs.pw_tok[wrow] = k;
+    }
+    auto put_d = [&](int t, double d) {
+      if (hs.own_rows == 2) hs.row_ld[(long long)(s_rbase + i) * S + t] = d == -INFINITY ? -INFINITY : (float)(d - s_keep_ls[i]);
+      else hs.A_ld[((long long)b * kMaxBeam + i) * S + t] = d;
+    };
+    if (hs.own_rows == 1) {
       // done above
     } else if (!hs.mono) {
-      for (int t = lane; t < S; t += 32) hs.A_ld[((long long)b * kMaxBeam + i) * S + t] = d_at(t);
+      for (int t = lane; t < S; t += 32) put_d(t, d_at(t));
     } else {
       // emitted at frame t: the hypothesis continues at frame t + 1, or has left the segment
-      for (int t = lane; t < S; t += 32) hs.A_ld[((long long)b * kMaxBeam + i) * S + t] = t < slen ? d_at(t - 1) : -INFINITY;
+      for (int t = lane; t < S; t += 32) put_d(t, t < slen ? d_at(t - 1) : -INFINITY);
       if (lane == 0) hs.A_done[b * kMaxBeam + i] = d_at(slen - 1);
     }
   }

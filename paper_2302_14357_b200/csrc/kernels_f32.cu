@@ -391,7 +391,8 @@ __global__ void __launch_bounds__(256) expand_f32_kernel(const float* __restrict
                                                          const int* row_slen, const int* R_dev,
                                                          int R_max, int S, int V, int blank,
                                                          float* ldphi, float* ldnb, float* la_out,
-                                                         double* ldphi_d, double* la_d, CandOut cand) {
+                                                         double* ldphi_d, double* la_d, CandOut cand, StepWords words) {
+  update_step_words(words);
   __shared__ float la[kMaxSeg];
   __shared__ float s_wv[8][kMaxBeam];
   __shared__ int s_wk[8][kMaxBeam];
@@ -574,10 +575,10 @@ void launch_log_softmax(const JoinerRows& rows, int blank, float* z, cudaStream_
 
 void launch_expand_f32(const float* logp, const float* ld_old, const int* row_slen, const int* R_dev,
                        int R_max, int S, int V, int blank, float* ldphi, float* ldnb, float* la,
-                       double* ldphi_d, double* la_d, const CandOut& cand, cudaStream_t st) {
+                       double* ldphi_d, double* la_d, const CandOut& cand, cudaStream_t st, const StepWords& words) {
   if (R_max <= 0) return;
   expand_f32_kernel<<<R_max, 256, 0, st>>>(logp, ld_old, row_slen, R_dev, R_max, S, V, blank, ldphi,
-                                           ldnb, la, ldphi_d, la_d, cand);
+                                           ldnb, la, ldphi_d, la_d, cand, words);
 }
 
 void launch_rows_from_groups(const int* row_group, const int* seg_len, int R, int G, int S, int* row_e0,

@@ -49,6 +49,7 @@ __global__ void __launch_bounds__(kMaxT) scan_select_kernel(ScanSelectArgs a) {
 
   pdl_wait();
   pdl_trigger();
+  update_step_words(a.words);
   const int R = a.R_dev ? *a.R_dev : a.R_max;
   const int r = blockIdx.x;
   if (r >= R) return;

@@ -438,9 +438,6 @@ int init_impl(tw_handle* h, const tw_model* m, const tw_config* c) {
 
 namespace tw {
 void enqueue_joiner_logits(tw_handle* h, const JoinerRows& rows, float* logp, cudaStream_t st, int* launches);
-void enqueue_scan(tw_handle* h, const JoinerRows& rows, const float* ld_old, float* logp, float* ldphi,
-                  float* ldnb, float* la, double* ldphi_d, double* la_d, const CandOut& cand, cudaStream_t st,
-                  int* launches);
 void enqueue_joiner_expand_f32(tw_handle* h, const JoinerRows& rows, const float* ld_old, float* logp,
                                float* ldphi, float* ldnb, float* la, double* ldphi_d, double* la_d,
                                const CandOut& cand, cudaStream_t st, int* launches) {
@@ -451,16 +448,17 @@ void enqueue_joiner_expand_f32(tw_handle* h, const JoinerRows& rows, const float
 // softmax, Eq. 3-7 and the rows' candidates from the raw logits in `logp`
 void enqueue_scan(tw_handle* h, const JoinerRows& rows, const float* ld_old, float* logp, float* ldphi,
                   float* ldnb, float* la, double* ldphi_d, double* la_d, const CandOut& cand, cudaStream_t st,
-                  int* launches) {
+                  int* launches, const StepWords& words) {
   if (h->hs.lse != nullptr && !h->hat) {
     ScanSelectArgs a{logp, ld_old, rows.row_slen, rows.R_dev, rows.R_max, rows.S, rows.V, h->blank,
                      h->hs.lse, ldphi, ldnb, la, ldphi_d, la_d, cand};
+    a.words = words;
     launch_scan_select(a, h->mode == TW_MODE_BF16, st);
     *launches += 1;
   } else {
     launch_log_softmax(rows, h->blank, logp, st);        // factorised output and blank thresholding included (rows.hat)
     launch_expand_f32(logp, ld_old, rows.row_slen, rows.R_dev, rows.R_max, rows.S, rows.V, h->blank, ldphi,
-                      ldnb, la, ldphi_d, la_d, cand, st);
+                      ldnb, la, ldphi_d, la_d, cand, st, words);
     *launches += 2;
   }
 }

@@ -125,7 +125,7 @@ int enqueue_joiner_fused(tw_handle* h, const JoinerRows& rows, const float* ld_o
                          bool own_rows = false);      // a decode step with HypState::own_rows: its operand rows are written already
 void enqueue_scan(tw_handle* h, const JoinerRows& rows, const float* ld_old, float* logp, float* ldphi,
                   float* ldnb, float* la, double* ldphi_d, double* la_d, const CandOut& cand, cudaStream_t st,
-                  int* launches);
+                  int* launches, const StepWords& words = StepWords{});
 void enqueue_joiner_expand_f32(tw_handle* h, const JoinerRows& rows, const float* ld_old, float* logp,
                                float* ldphi, float* ldnb, float* la, double* ldphi_d, double* la_d,
                                const CandOut& cand, cudaStream_t st, int* launches);

@@ -116,12 +116,18 @@ void launch_log_softmax(const JoinerRows& rows, int blank, float* z, cudaStream_
 struct CandOut {
   float* v; int* k; int* n; int N;
 };
+// Words of a decode step with HypState::own_rows that the kernel behind the joiner's contraction looks after: it clears
+// the work list's length and the next pass's row count, and counts the pass if it has rows
+struct StepWords { int* clear1 = nullptr; int* clear2 = nullptr; int* steps = nullptr; const int* rows = nullptr; };
+__device__ __forceinline__ void update_step_words(const StepWords& w) {
+  if (w.clear1 != nullptr && blockIdx.x == 0 && threadIdx.x == 0) { *w.clear1 = 0; *w.clear2 = 0; if (*w.rows > 0) *w.steps += 1; }
+}
 // Eq. 3-7 from materialised log J; ldnb may be nullptr when only the candidates are wanted, and
 // cand.n may be nullptr when they are not
 void launch_expand_f32(const float* logp, const float* ld_old, const int* row_slen, const int* R_dev,
                        int R_max, int S, int V, int blank, float* ldphi, float* ldnb, float* la,
                        double* ldphi_d, double* la_d, const CandOut& cand,
-                       cudaStream_t st);   // float64 copies optional
+                       cudaStream_t st, const StepWords& words = StepWords{});   // float64 copies optional
 // Softmax + Eq. 3-7 + per-row candidates from RAW logits z [R, S, V] read once into shared memory
 // (scan_select.cu).  Every output pointer is optional.
 struct ScanSelectArgs {
@@ -132,6 +138,7 @@ struct ScanSelectArgs {
   CandOut cand;
   const float* dnb_in = nullptr;   // when set: [R, V] delta_nb values are given and only the selection runs
   int dnb_linear = 0;              // dnb_in holds probabilities (0 = none), candidates are returned as logs
+  StepWords words = {};
 };
 bool scan_select_fits(int S, int V);   // the row's S x V logits fit in shared memory
 int scan_select_setup();
@@ -215,7 +222,9 @@ struct HypState {
   // and hyp_step_kernel itself completes their frame distributions (row_ld, Eq. 5: log J of the kept expansions from the
   // pass's operand A_cur and W_out, S dot products of length J each) and writes the operand rows of hypotheses carried over
   // a segment turn-over into A_next; those of new hypotheses are written with the predictor's output.
-  // rows_next is one of two words, in turn: the joiner kernel reads one and clears the other.
+  // In TW_MODE_F32 own_rows == 2: the rows are claimed in the same way, and their tables and frame distributions are written
+  // from the log J at hand; that saves the compaction kernel.
+  // rows_next is one of two words, in turn: the joiner kernel (TW_MODE_F32: the scan kernel) reads one and clears the other.
   int own_rows; int* rows_next;
   const float* E; int E_T, act;             // projected frames (row b * E_T + t) and the joiner's nonlinearity
   const void* A_cur; void* A_next;          // operand of this pass / of the next one, bf16
