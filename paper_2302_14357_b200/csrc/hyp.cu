@@ -138,11 +138,17 @@ __device__ __forceinline__ unsigned long long order_key(double x) {
   return (u >> 63) ? ~u : (u | 0x8000000000000000ull);
 }
 
-__global__ void __launch_bounds__(2 * kStepThreads) hyp_step_kernel(HypState hs) {
+// tok_cap: capacity (tokens) of the dynamic shared memory's [N] token sequences of list A's hypotheses, 0: they stay in
+// global memory.  Every new hypothesis is a child of one of these, whose tokens the search below reads anyway.
+constexpr int kTokStageMax = 24 * 1024;
+__global__ void __launch_bounds__(2 * kStepThreads) hyp_step_kernel(HypState hs, int tok_cap) {
+  extern __shared__ int s_tok[];
   __shared__ int s_hasthr, s_nkeep, s_wbase, s_rbase;
   __shared__ int s_found[kMaxBeam], s_touched[kMaxBeam], s_carry[kMaxBeam];
   __shared__ double s_Als[kMaxBeam], s_Adone[kMaxBeam];
   __shared__ int s_Aslot[kMaxBeam], s_Alen[kMaxBeam];
+  __shared__ unsigned long long s_Ahash[kMaxBeam];
+  __shared__ double s_Bls[kMaxBeam];          // score of the entry of list B that a hypothesis merges with
   __shared__ double s_thr;
   __shared__ int s_ck[kMaxBeam * kMaxBeam];
   __shared__ double s_abs[kMaxBeam * kMaxBeam];
@@ -187,12 +193,54 @@ __global__ void __launch_bounds__(2 * kStepThreads) hyp_step_kernel(HypState hs)
   unsigned long long my_hash = 0;
   int my_len = 0;
   if (warp < H) { my_hash = hs.slot_hash[bS + my_slot]; my_len = hs.slot_len[bS + my_slot]; }
+  if (warp == 15 && H > 0) {
+    // ring cursor, pass counter and the best-N set of list B as the previous pass left it, by a warp that mostly has
+    // nothing to do in the search
+    const int nT = hs.nTop[b];
+    if (lane == 0) { s_cursor = hs.cursor[b]; s_iters = hs.iters[b]; s_nT0 = nT; }
+    if (lane < kMaxBeam) {
+      const int bt = hs.B_top[b * kMaxBeam + lane];
+      s_Btop[lane] = bt;
+      if (lane < nT) s_Btopls[lane] = hs.B_ls[bB + bt];       // before this pass's merges; touched entries are patched below
+    }
+  }
+  // ---- AddAndMerge, search: warp h looks for the tokens of A_h among the entries already in B.  It needs the lists only,
+  // so it runs ahead of the wait.  (Entries of A are distinct sequences, so two of them never merge with each other.)
+  if (warp < H) {
+    const int* ta = hs.slot_tok + (bS + my_slot) * hs.U_cap;
+    if (tok_cap > 0) for (int i = lane; i < my_len; i += 32) s_tok[warp * tok_cap + i] = ta[i];
+    int found = -1;
+    for (int base = 0; base < nB0 && found < 0; base += 32) {
+      const int e = base + lane;
+      const bool match = e < nB0 && (base == 0 ? (pre_hash == my_hash && pre_len == my_len)
+                                               : (hs.B_hash[bB + e] == my_hash && hs.B_len[bB + e] == my_len));
+      unsigned mask = __ballot_sync(0xffffffffu, match);
+      while (mask != 0 && found < 0) {
+        const int c = base + __ffs(mask) - 1;
+        mask &= mask - 1;
+        const int oslot = base == 0 ? __shfl_sync(0xffffffffu, pre_slot, c) : hs.B_slot[bB + c];
+        int diff = 0;                       // a 64-bit hash match is not proof: compare the tokens
+        if (oslot != my_slot) {
+          const int* tb = hs.slot_tok + (bS + oslot) * hs.U_cap;
+          for (int i = lane; i < my_len; i += 32) diff |= (ta[i] != tb[i]);
+        }
+        if (!__any_sync(0xffffffffu, diff)) found = c;
+      }
+    }
+    if (lane == 0) {
+      s_found[warp] = found; s_Alen[warp] = my_len; s_Ahash[warp] = my_hash;
+      s_Bls[warp] = found >= 0 ? hs.B_ls[bB + found] : 0.0;
+    }
+  }
+  if (tid < kMaxBeam) { s_Als[tid] = ld_Als; s_Aslot[tid] = ld_Aslot; s_Adone[tid] = ld_Adone; s_carry[tid] = ld_carry; }
   pdl_wait();                               // from here on: what the joiner kernel wrote (delta_phi, delta_nb, occupancies)
   pdl_trigger();
   if (H == 0) return;                       // idle (finished) utterance
   const int N = hs.N, S = hs.S, V = hs.V;
 
-  if (tid < kMaxBeam) { s_Als[tid] = ld_Als; s_Aslot[tid] = ld_Aslot; s_Adone[tid] = ld_Adone; s_carry[tid] = ld_carry; }
+  double dphi = 0.0;
+  if (tid < H) dphi = hs.ldphi_d ? hs.ldphi_d[r0 + tid] : (double)hs.ldphi[r0 + tid];
+  if (tid < kMaxBeam) s_sel[tid] = -1;
   if (tid == 0) {
     hs.calls[b] += 1; hs.joins[b] += slen;
     if (hs.own_rows) {                      // totals of the pass
@@ -349,62 +397,29 @@ __global__ void __launch_bounds__(2 * kStepThreads) hyp_step_kernel(HypState hs)
       }
     }
   }
-  if (warp == 15) {
-    // ring cursor, pass counter and the best-N set of list B as the previous pass left it: fetched now, by a
-    // warp that has nothing to do in the search, so that the later phases find them in shared memory
-    const int nT = hs.nTop[b];
-    if (lane == 0) { s_cursor = hs.cursor[b]; s_iters = hs.iters[b]; s_nT0 = nT; }
-    if (lane < kMaxBeam) {
-      const int bt = hs.B_top[b * kMaxBeam + lane];
-      s_Btop[lane] = bt;
-      if (lane < nT) s_Btopls[lane] = hs.B_ls[bB + bt];       // before this pass's merges; touched entries are patched below
-    }
-  }
-  if (warp < 16) sync_merge();
-
-  // ---- AddAndMerge, search: warp h looks for the tokens of A_h among the entries already in B.
-  // (Entries of A are distinct sequences, so two of them never merge with each other.)
-  if (warp < H) {
-    const int slot = my_slot;
-    const unsigned long long hh = my_hash;
-    const int ln = my_len;
-    const int* ta = hs.slot_tok + (bS + slot) * hs.U_cap;
-    int found = -1;
-    for (int base = 0; base < nB0 && found < 0; base += 32) {
-      const int e = base + lane;
-      const bool match = e < nB0 && (base == 0 ? (pre_hash == hh && pre_len == ln)
-                                               : (hs.B_hash[bB + e] == hh && hs.B_len[bB + e] == ln));
-      unsigned mask = __ballot_sync(0xffffffffu, match);
-      while (mask != 0 && found < 0) {
-        const int c = base + __ffs(mask) - 1;
-        mask &= mask - 1;
-        const int oslot = base == 0 ? __shfl_sync(0xffffffffu, pre_slot, c) : hs.B_slot[bB + c];
-        int diff = 0;                       // a 64-bit hash match is not proof: compare the tokens
-        if (oslot != slot) {
-          const int* tb = hs.slot_tok + (bS + oslot) * hs.U_cap;
-          for (int i = lane; i < ln; i += 32) diff |= (ta[i] != tb[i]);
-        }
-        if (!__any_sync(0xffffffffu, diff)) found = c;
-      }
-    }
-    if (lane == 0) { s_found[warp] = found; s_Alen[warp] = ln; }
+  if (!two_halves && tid >= kMaxBeam * kMaxBeam) {      // the rows' candidate lists, by the warps that merge nothing
+    const int c = tid - kMaxBeam * kMaxBeam, h = c / kMaxBeam, j = c % kMaxBeam;
+    const bool valid = h < H && j < hs.cand_n[r0 + h];
+    s_abs[c] = valid ? hs.A_ls[b * kMaxBeam + h] + (double)hs.cand_v[(long long)(r0 + h) * kMaxBeam + j] : -INFINITY;
+    s_ck[c] = valid ? hs.cand_k[(long long)(r0 + h) * kMaxBeam + j] : -1;
+    s_key[c] = order_key(s_abs[c]);
   }
   if (warp < 16) sync_merge();
   // ---- AddAndMerge, apply: sum into the matching entry or append (appends keep the order of A)
   if (tid < H) {
     const int h = tid;
     const int slot = s_Aslot[h];
-    double val = s_Als[h] + (hs.ldphi_d ? hs.ldphi_d[r0 + h] : (double)hs.ldphi[r0 + h]);
+    double val = s_Als[h] + dphi;
     val = logaddexp_d(val, s_Adone[h]);       // monotonic: plus what had already left the segment (else log 0)
     int e = s_found[h];
     if (e >= 0) {
-      val = logaddexp_d(hs.B_ls[bB + e], val);
+      val = logaddexp_d(s_Bls[h], val);       // (two hypotheses never merge with the same entry)
       hs.B_ls[bB + e] = val;
     } else {
       e = nB0;                              // capB = N * I_max bounds this by construction
       for (int q = 0; q < h; ++q) e += (s_found[q] < 0);
       hs.B_slot[bB + e] = slot; hs.B_ls[bB + e] = val;
-      hs.B_hash[bB + e] = hs.slot_hash[bS + slot]; hs.B_len[bB + e] = hs.slot_len[bS + slot];
+      hs.B_hash[bB + e] = s_Ahash[h]; hs.B_len[bB + e] = s_Alen[h];
     }
     s_touched[h] = e;
     s_tval[h] = val;
@@ -449,14 +464,6 @@ __global__ void __launch_bounds__(2 * kStepThreads) hyp_step_kernel(HypState hs)
   }
   // ---- ChooseNBestExpansions, second stage: the N best (h, k) over the rows' candidate lists, in
   // float64; order (score desc, h asc, k asc).  The lists are sorted by (score desc, k asc).
-  if (hs.dnb_sel == nullptr && tid < kMaxBeam * kMaxBeam) {
-    const int h = tid / kMaxBeam, j = tid % kMaxBeam;
-    const bool valid = h < H && j < hs.cand_n[r0 + h];
-    s_abs[tid] = valid ? s_Als[h] + (double)hs.cand_v[(long long)(r0 + h) * kMaxBeam + j] : -INFINITY;
-    s_ck[tid] = valid ? hs.cand_k[(long long)(r0 + h) * kMaxBeam + j] : -1;
-    s_key[tid] = order_key(s_abs[tid]);
-  }
-  if (tid < kMaxBeam) s_sel[tid] = -1;
   __syncthreads();
   if (tid < kMaxBeam * kMaxBeam && s_ck[tid] >= 0) {
     const unsigned long long mine = s_key[tid];
@@ -569,14 +576,14 @@ __global__ void __launch_bounds__(2 * kStepThreads) hyp_step_kernel(HypState hs)
     const int i = warp;
     const int h = s_keep_h[i], k = s_keep_k[i];
     const long long gp = bS + s_Aslot[h], gn = bS + s_keep_slot[i];
-    const int plen = hs.slot_len[gp];
-    const int* src = hs.slot_tok + gp * hs.U_cap;
+    const int plen = s_Alen[h];
+    const int* src = tok_cap > 0 ? s_tok + h * tok_cap : hs.slot_tok + gp * hs.U_cap;
     int* dst = hs.slot_tok + gn * hs.U_cap;
     for (int q = lane; q < plen; q += 32) dst[q] = src[q];
     if (lane == 0) {
       dst[plen] = k;
       hs.slot_len[gn] = plen + 1;
-      hs.slot_hash[gn] = hash_push(hs.slot_hash[gp], k);
+      hs.slot_hash[gn] = hash_push(s_Ahash[h], k);
       hs.new_slot[b * kMaxBeam + i] = (int)gn;
       hs.new_par[b * kMaxBeam + i] = (int)gp;
       hs.new_tok[b * kMaxBeam + i] = k;
@@ -822,7 +829,9 @@ void launch_hyp_init(const HypState& hs, const int* lengths, int B, int T, cudaS
   if (B > 0) hyp_init_kernel<<<B, kThreads, 0, st>>>(hs, lengths, T);
 }
 void launch_hyp_step(const HypState& hs, int B, cudaStream_t st) {
-  if (B > 0) launch_pdl(hyp_step_kernel, dim3(B), dim3(hs.dnb_sel ? 2 * kStepThreads : kStepThreads), 0, st, hs);
+  if (B <= 0) return;
+  const int tok_cap = hs.N * hs.U_cap * 4 <= kTokStageMax ? hs.U_cap : 0;
+  launch_pdl(hyp_step_kernel, dim3(B), dim3(hs.dnb_sel ? 2 * kStepThreads : kStepThreads), (size_t)hs.N * tok_cap * 4, st, hs, tok_cap);
 }
 void launch_compact(const HypState& hs, int B, int T, cudaStream_t st) {
   launch_pdl(compact_kernel, dim3(1), dim3(1024), 0, st, hs, B, T);
