@@ -800,29 +800,6 @@ __global__ void __launch_bounds__(kThreads) finish_kernel(HypState hs, int* out_
   if (threadIdx.x == 0) out_status[b] = hs.status[b];
 }
 
-__device__ __forceinline__ float sigmoidf_acc(float x) { return 1.f / (1.f + expf(-x)); }
-
-// c' = sigma(f) c + sigma(i) tanh(g);  h' = sigma(o) tanh(c')   (gate order i, f, g, o)
-__global__ void lstm_pointwise_kernel(const float* gates, const int* pw_new, const int* pw_par,
-                                      const int* n_dev, int n_max, const float* hc_in, float* hc_out,
-                                      int L, int l, int Hd) {
-  pdl_wait();
-  pdl_trigger();
-  const int n = n_dev ? *n_dev : n_max;
-  const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= (long long)n * Hd) return;
-  const int r = (int)(i / Hd), j = (int)(i - (long long)r * Hd);
-  const float* g = gates + (long long)r * 4 * Hd;
-  const long long stride = (long long)L * 2 * Hd;
-  const long long pin = (pw_par ? pw_par[r] : r) * stride + (long long)l * 2 * Hd;
-  const long long pout = (pw_new ? pw_new[r] : r) * stride + (long long)l * 2 * Hd;
-  const float c_prev = hc_in[pin + Hd + j];
-  const float c = sigmoidf_acc(g[Hd + j]) * c_prev + sigmoidf_acc(g[j]) * tanhf(g[2 * Hd + j]);
-  const float h = sigmoidf_acc(g[3 * Hd + j]) * tanhf(c);
-  hc_out[pout + j] = h;
-  hc_out[pout + Hd + j] = c;
-}
-
 }  // namespace
 
 void launch_hyp_init(const HypState& hs, const int* lengths, int B, int T, cudaStream_t st) {
@@ -849,12 +826,4 @@ void launch_finish(const HypState& hs, int B, int* out_tokens, int* out_lens, do
                    int* out_status, cudaStream_t st) {
   if (B > 0) finish_kernel<<<B, kThreads, 0, st>>>(hs, out_tokens, out_lens, out_scores, out_status);
 }
-void launch_lstm_pointwise(const float* gates, const int* idx_out, const int* idx_in, const int* n_dev,
-                           int n_max, const float* hc_in, float* hc_out, int L, int l, int Hd, cudaStream_t st) {
-  if (n_max <= 0) return;
-  const long long tot = (long long)n_max * Hd;
-  launch_pdl(lstm_pointwise_kernel, dim3((unsigned)((tot + 255) / 256)), dim3(256), 0, st, gates, idx_out, idx_in, n_dev, n_max, hc_in,
-             hc_out, L, l, Hd);
-}
-
 }  // namespace tw

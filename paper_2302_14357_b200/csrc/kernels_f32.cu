@@ -53,6 +53,7 @@ __device__ __forceinline__ float4 load4(const float* p, int k, int K) {
   for (int i = 0; i < 4; ++i) v[i] = (k + i < K) ? p[k + i] : 0.f;
   return make_float4(v[0], v[1], v[2], v[3]);
 }
+__device__ __forceinline__ float sigmoidf_acc(float x) { return 1.f / (1.f + expf(-x)); }
 __device__ __forceinline__ float act_f32(float x, int act) { return act == TW_ACT_RELU ? fmaxf(x, 0.f) : tanhf(x); }
 
 // MODE 0: plain / gathered rows, one or two operand pairs.  MODE 1: joiner rows, A = act(E + Pp) formed on the way.
@@ -243,6 +244,15 @@ gemm_f32_kernel(const __grid_constant__ CUtensorMap tm0, const __grid_constant__
         const float4 u = sm100::ld_cluster_f32x4(sm100::map_to_cta(sm100::smem_u32(&sm_f32[c * 4]), (uint32_t)q));
         v.x += u.x; v.y += u.y; v.z += u.z; v.w += u.w;
       }
+    }
+    if (MODE == 0 && p.out.lstm.hc_out != nullptr) {           // the four gates of hidden unit n / 4
+      const LstmF32& q = p.out.lstm;
+      const float4 b4 = *reinterpret_cast<const float4*>(p.out.bias + n);
+      const long long pin = (q.idx_in ? q.idx_in[m] : m) * q.stride + q.lo + (n >> 2), pout = (q.idx_out ? q.idx_out[m] : m) * q.stride + q.lo + (n >> 2);
+      const float cn = sigmoidf_acc(v.y + b4.y) * q.hc_in[pin + q.Hd] + sigmoidf_acc(v.x + b4.x) * tanhf(v.z + b4.z);
+      q.hc_out[pout] = sigmoidf_acc(v.w + b4.w) * tanhf(cn);
+      q.hc_out[pout + q.Hd] = cn;
+      continue;
     }
     float* crow;
     const float* bias;
@@ -473,6 +483,11 @@ __global__ void __launch_bounds__(256) expand_f32_kernel(const float* __restrict
   }
 }
 
+__global__ void permute_rows_f32_kernel(const float* __restrict__ src, const int* __restrict__ perm, long long rows, int cols, float* __restrict__ dst) {
+  const float* s = src + (long long)perm[blockIdx.x] * cols;
+  for (int c = threadIdx.x; c < cols; c += blockDim.x) dst[(long long)blockIdx.x * cols + c] = s[c];
+}
+
 __global__ void rows_from_groups_kernel(const int* row_group, const int* seg_len, int R, int G, int S,
                                         int* row_e0, int* row_slen) {
   pdl_wait();
@@ -579,6 +594,10 @@ void launch_expand_f32(const float* logp, const float* ld_old, const int* row_sl
   if (R_max <= 0) return;
   expand_f32_kernel<<<R_max, 256, 0, st>>>(logp, ld_old, row_slen, R_dev, R_max, S, V, blank, ldphi,
                                            ldnb, la, ldphi_d, la_d, cand, words);
+}
+
+void launch_permute_rows_f32(const float* src, const int* perm, long long rows, int cols, float* dst, cudaStream_t st) {
+  permute_rows_f32_kernel<<<(unsigned)rows, 256, 0, st>>>(src, perm, rows, cols, dst);
 }
 
 void launch_rows_from_groups(const int* row_group, const int* seg_len, int R, int G, int S, int* row_e0,

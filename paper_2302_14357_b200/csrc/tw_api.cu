@@ -140,11 +140,10 @@ void enqueue_predictor(tw_handle* h, const int* tok, const float* hc_in, const i
     const float* hp = hc_in + (long long)l * 2 * Hd;
     GemmOperand xo{x, xi, xld, h->W_ih[l], xk, xk};
     GemmOperand ro{hp, idx_in, stride, h->W_hh[l], Hd, Hd};
-    GemmOut o{h->gates, nullptr, 4 * Hd, h->b_l[l], h->bf.err};
+    GemmOut o{nullptr, nullptr, 0, h->b_l[l], h->bf.err};
+    o.lstm = LstmF32{hc_in, idx_in, hc_out, idx_out, stride, (long long)l * 2 * Hd, Hd};       // the cell in the epilogue
     launch_gemm_f32(xo, ro, o, n_dev, n_max, 4 * Hd, st);
-    // pointwise: c' = sigma(f) c + sigma(i) tanh(g), h' = sigma(o) tanh(c')
-    launch_lstm_pointwise(h->gates, idx_out, idx_in, n_dev, n_max, hc_in, hc_out, L, l, Hd, st);
-    *launches += 2;
+    *launches += 1;
   }
   const float* top = hc_out + (long long)(L - 1) * 2 * Hd;
   GemmOperand to{top, idx_out, stride, h->W_p, h->P, h->P};
@@ -155,6 +154,13 @@ void enqueue_predictor(tw_handle* h, const int* tok, const float* hc_in, const i
 
 int enqueue_predictor_plain(tw_handle* h, const int* tokens, const float* state_in, int R,
                             float* state_out, float* out_Pp, cudaStream_t st, int* launches) {
+  const size_t n = (size_t)R * h->L * 2 * h->Hd;
+  if (h->mode == TW_MODE_F32 && h->L > 0 && state_in < state_out + n && state_out < state_in + n) {
+    // a caller's state updated in place: the gate GEMM writes h while its other CTAs still read it, so it reads a copy
+    if (!h->state_copy) TW_TRY(dev_alloc(h, &h->state_copy, (size_t)h->R_max * h->L * 2 * h->Hd));
+    TW_CUDA(h, cudaMemcpyAsync(h->state_copy, state_in, n * sizeof(float), cudaMemcpyDeviceToDevice, st));
+    state_in = h->state_copy;
+  }
   enqueue_predictor(h, tokens, state_in, nullptr, state_out, nullptr, out_Pp, nullptr, R, st, launches);
   return TW_OK;
 }
@@ -330,7 +336,6 @@ int build_workspace(tw_handle* h) {
   if (!hs.stateless) {
     TW_TRY(dev_alloc(h, &hs.slot_hc, nslot * hs.L * 2 * hs.Hd));
     TW_TRY(dev_alloc(h, &hs.slot_Pp, nslot * h->J));
-    TW_TRY(dev_alloc(h, &h->gates, R * 4 * hs.Hd));
   }
   TW_TRY(dev_alloc(h, &hs.new_slot, nb * kMaxBeam));
   TW_TRY(dev_alloc(h, &hs.new_par, nb * kMaxBeam));
@@ -392,6 +397,26 @@ int init_impl(tw_handle* h, const tw_model* m, const tw_config* c) {
     TW_TRY(copy_weight(h, &h->W_ih[l], m->host_lstm_W_ih[l], (size_t)4 * h->Hd * in));
     TW_TRY(copy_weight(h, &h->W_hh[l], m->host_lstm_W_hh[l], (size_t)4 * h->Hd * h->Hd));
     TW_TRY(copy_weight(h, &h->b_l[l], m->host_lstm_b[l], (size_t)4 * h->Hd));
+  }
+  if (h->mode == TW_MODE_F32 && h->L > 0) {
+    // gate rows interleaved by hidden unit, so that the cell runs in the gate GEMM's epilogue
+    const int G4 = 4 * h->Hd;
+    std::vector<int> perm(G4);
+    for (int j = 0; j < h->Hd; ++j)
+      for (int g = 0; g < 4; ++g) perm[4 * j + g] = g * h->Hd + j;
+    int* perm_dev = nullptr;
+    TW_TRY(dev_alloc(h, &perm_dev, (size_t)G4));
+    TW_CUDA(h, cudaMemcpy(perm_dev, perm.data(), G4 * sizeof(int), cudaMemcpyHostToDevice));
+    for (int l = 0; l < h->L; ++l) {
+      float** w[3] = {&h->W_ih[l], &h->W_hh[l], &h->b_l[l]};
+      const int cols[3] = {l == 0 ? h->emb_dim : h->Hd, h->Hd, 1};
+      for (int i = 0; i < 3; ++i) {
+        float* dst = nullptr;
+        TW_TRY(dev_alloc(h, &dst, (size_t)G4 * cols[i]));
+        launch_permute_rows_f32(*w[i], perm_dev, G4, cols[i], dst, 0);
+        *w[i] = dst;
+      }
+    }
   }
   TW_TRY(build_workspace(h));
   if (h->mode == TW_MODE_BF16) TW_TRY(build_bf16(h));

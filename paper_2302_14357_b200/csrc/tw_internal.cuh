@@ -71,12 +71,18 @@ struct GemmOperand {
   int K;
 };
 
+// LSTM cell as the epilogue of a gate GEMM whose columns are interleaved by unit (column 4 j + g is gate g of hidden unit j, in
+// the order input, forget, cell, output): c' = sigma(f) c + sigma(i) tanh(g), h' = sigma(o) tanh(c').  c is read at
+// offset lo + Hd of state row (idx_in ? idx_in[m] : m) of hc_in, (h', c') go to lo and lo + Hd of row idx_out of hc_out.
+struct LstmF32 { const float* hc_in = nullptr; const int* idx_in = nullptr; float* hc_out = nullptr; const int* idx_out = nullptr; long long stride = 0, lo = 0; int Hd = 0; };
+
 struct GemmOut {
   float* C;           // row m written at C + (oidx ? oidx[m] : m) * ldC
   const int* oidx;
   long long ldC;
   const float* bias;  // optional [N]
   int* err;           // device word, raised by a wait that gave up
+  LstmF32 lstm = {};  // hc_out != nullptr: the cell instead of C
 };
 
 // M may come from device memory (M_dev != nullptr): CTAs beyond it exit.
@@ -249,9 +255,7 @@ void launch_stream_advance(const HypState& hs, const int* chunk_lens, int B, int
 void launch_finish(const HypState& hs, int B, int* out_tokens, int* out_lens, double* out_scores,
                    int* out_status, cudaStream_t st);
 
-// LSTM pointwise: gates [n, 4Hd] + c of row (idx_in ? idx_in[i] : i) of hc_in -> (h, c) of layer l in row
-// (idx_out ? idx_out[i] : i) of hc_out; state rows are [L][2][Hd]
-void launch_lstm_pointwise(const float* gates, const int* idx_out, const int* idx_in, const int* n_dev,
-                           int n_max, const float* hc_in, float* hc_out, int L, int l, int Hd, cudaStream_t st);
+// dst row r = src row perm[r]  (rows x cols float32)
+void launch_permute_rows_f32(const float* src, const int* perm, long long rows, int cols, float* dst, cudaStream_t st);
 
 }  // namespace tw
