@@ -506,7 +506,7 @@ int enqueue_joiner_fused(tw_handle* h, const JoinerRows& rows, const float* ld_o
     if (per_utterance) launch_joiner_A_tiled_utt(rows, h->hs.row_off, h->hs.nA, step_B, A.ptr, st);
     else launch_joiner_A_tiled(rows, A.ptr, st, pf, wbytes);
   }
-  if (mark_fn) mark_fn(h, 3, st);       // operand preparation is booked with the elementwise stages
+  if (mark_fn && !own_rows) mark_fn(h, 3, st);       // operand preparation is booked with the elementwise stages
   if (ldnb == nullptr) ldnb = h->bf.ldnb_pad;   // a caller's buffer has V columns: only with an unpadded vocabulary
   FusedJoinerParams fp{};
   fp.R_dev = rows.R_dev; fp.R_max = rows.R_max; fp.S = rows.S; fp.V = h->bf.Vp; fp.K = rows.J; fp.blank = h->blank;
