@@ -33,6 +33,7 @@ struct GemmBf16Params {
   int epi = 0;        // 0: store C (+ bias, + addend); 1: LSTM cell (C is not written)
   int m_early = 0;    // 1: *M_dev was written before the kernel launched ahead of this one began (not by that kernel):
                       // it is read during the set-up, ahead of the wait for that kernel
+  int beside = 0;     // 1: a kernel on another stream is expected to run beside this one
   LstmEpi lstm = {};
 };
 

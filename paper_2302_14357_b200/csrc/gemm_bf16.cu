@@ -611,8 +611,10 @@ bool launch_gemm_lstm_wide(const CUtensorMap& tmA, const CUtensorMap& tmA32, con
   const int units = p.N >> 5;
   const int w = ((units + n_split - 1) / n_split) * 32;
   if (w > Wide<16>::kMaxBN) return false;
-  // one or two row tiles at most: the small instance
-  if (mt <= 2 && w <= 64) {
+  // One or two row tiles at most: the small instance.  Up to five where another stream's kernel holds part of the SMs (p.beside):
+  // its CTAs find room beside that kernel's, those of the large instance wait for it (64 utterances at S = 20: 7 % per
+  // decode; without such a kernel the split for the largest count costs 2 % at 64 utterances, S = 3).
+  if ((mt <= 2 && w <= 64) || (p.beside && mt <= 5 && w <= 128)) {
     launch_pdl(gemm_lstm_wide_kernel<8>, dim3(num_sms), dim3(Wide<8>::kThreads), Wide<8>::kSmem, st, tmA, tmA32, tmB64, tmB32, p);
     return true;
   }

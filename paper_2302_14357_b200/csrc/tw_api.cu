@@ -118,6 +118,7 @@ void enqueue_predictor(tw_handle* h, const int* tok, const float* hc_in, const i
       if (l == 0) { p.addend = h->bf.EmbProj; p.add_idx = tok; p.ld_add = 4 * Hd; }   // W_ih[0] emb[tok] + b[0]: a table row
       else p.bias = h->bf.bias_perm[l];
       p.epi = 1;
+      p.beside = h->aux_pending ? 1 : 0;
       p.m_early = l > 0;                      // the row count is older than the layer below, which runs ahead of this one
       p.lstm = LstmEpi{hc_in, idx_in, hc_out, idx_out, L, l, Hd,
                        (l + 1 < L) ? h->bf.X[l + 1].ptr : h->bf.Htop.ptr, (l + 1 < L) ? 2LL * Hd : (long long)Hd};
