@@ -94,6 +94,11 @@ __device__ void carry_rows(const HypState& hs, int b) {
         act8(*reinterpret_cast<const float4*>(e), *reinterpret_cast<const float4*>(e + 4), *reinterpret_cast<const float4*>(pp),
              *reinterpret_cast<const float4*>(pp + 4), hs.act);
   }
+  // padding frames of a short segment: zeros, whatever an older pass left there (see pred_out.cu)
+  for (int c = threadIdx.x; c < n * (S - sl) * per; c += blockDim.x) {
+    const int pair = c / per, x = (c - pair * per) * 8, hh = pair / (S - sl), t = sl + pair - hh * (S - sl);
+    *reinterpret_cast<uint4*>(static_cast<__nv_bfloat16*>(hs.A_next) + operand_row(r0 + hh, t, S) * J + x) = make_uint4(0, 0, 0, 0);
+  }
 }
 
 __global__ void __launch_bounds__(kThreads) hyp_init_kernel(HypState hs, const int* lengths, int T) {

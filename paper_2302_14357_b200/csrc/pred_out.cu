@@ -4,8 +4,9 @@
 // What this saves is a kernel in the step's chain of dependent ones (the operand kernel: 4 us on a small step, 7 us with
 // 128 utterances at J = 1024, plus 2 to 4 us until it starts) and the round trip of Pp through L2.  Every frame is read
 // once per hypothesis: with longer segments that is L2-bound, and the per-utterance operand kernel stays.
-// The rows of hypotheses carried over a segment turn-over, which have no new Pp, are written elsewhere
-// (survivor_ld_kernel); rows of dead hypotheses and of padding frames keep older, finite contents, which the joiner masks.
+// The rows of hypotheses carried over a segment turn-over, which have no new Pp, are written by carry_rows (hyp.cu).  A live
+// hypothesis's rows of padding frames are written as zeros: the joiner multiplies their exponentials by 0, and an older pass
+// may have left a NaN there (an utterance with such frames must not reach its neighbours' sums).
 #include "operand.cuh"
 #include "sm100.cuh"
 
@@ -184,6 +185,10 @@ wp_operand_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
         ld_global_v8(e + (long long)t * p.N, x);
         if (two) ld_global_v8(e + (long long)t * p.N + 8, x + 8);
         frame(t, x);
+      }
+      for (int t = sl; t < p.S; ++t) {                        // padding frames (a last, short segment)
+        *reinterpret_cast<uint4*>(dst + (long long)t * p.N) = make_uint4(0, 0, 0, 0);
+        if (two) *reinterpret_cast<uint4*>(dst + (long long)t * p.N + 8) = make_uint4(0, 0, 0, 0);
       }
     }
     if (!waited) { pdl_wait(); pdl_trigger(); }
