@@ -85,8 +85,6 @@ gemm_f32_kernel(const __grid_constant__ CUtensorMap tm0, const __grid_constant__
     for (int s = 0; s < kStagesF; ++s) { mbar_init(&full[s], VEC ? (MODE == 0 ? 2 : 1 + kWarpsF) : kWarpsF); mbar_init(&empty[s], kWarpsF); }
     fence_barrier_init();
   }
-  if (kBulkA && ((K0 | K1) & (BK - 1)) != 0)                 // what a short last block leaves in A meets zeros of B: it has to be a number
-    for (int i = tid; i < kStagesF * TM * BK / 4; i += kThreadsF) reinterpret_cast<float4*>(sA)[i] = make_float4(0.f, 0.f, 0.f, 0.f);
   fence_proxy_async_smem();
   __syncthreads();
   auto send_B = [&](int i) {               // one thread: the weights of block i
@@ -132,6 +130,12 @@ gemm_f32_kernel(const __grid_constant__ CUtensorMap tm0, const __grid_constant__
     const int blk = b_lo + i, s = i % kStagesF;
     const bool second = blk >= nb0;
     const int k = (second ? blk - nb0 : blk) * BK, kn = min(BK, (second ? K1 : K0) - k);
+    if (kn < BK) {      // short last block: the rest meets zeros of B, and an infinity that an earlier block left there would make them NaN
+      if (lane < TM)
+        for (int x = kn; x < BK; x += 4) *reinterpret_cast<float4*>(sA + s * Sm::kA + (lane * BK + x) * 4) = make_float4(0.f, 0.f, 0.f, 0.f);
+      fence_proxy_async_smem();
+      __syncwarp();
+    }
     if (lane == 0) mbar_expect_tx(&full[s], (uint32_t)(min(TM, M - m0) * kn * 4));
     __syncwarp();
     if (lane < TM && arow != nullptr)

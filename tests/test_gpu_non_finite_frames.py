@@ -36,3 +36,18 @@ def test_nan_frames_stay_with_their_utterance(mode, S, short):
         for got, ref in zip(dec.decode(mixed, mixed_lens)[:4], want):
             for b in set(range(B)) - set(range(0, B, 3)):
                 np.testing.assert_array_equal(got.cpu().numpy()[b], ref[b])
+
+
+@pytest.mark.parametrize("D,rows", [(36, 40), (200, 3000), (204, 3000), (484, 3000), (256, 3000), (202, 300)])
+def test_an_infinite_element_stays_infinite_in_the_fp32_projection(D, rows):
+    """Row r of the frames has one infinite element, at column r mod D: every product with it is +-infinity and so is the sum,
+    whatever the length of the last block of K (D a multiple of 32, of 4, of 2)."""
+    from paper_2302_14357_b200.binding import TwDecoder, weights_from_synth
+    cfg = tw_synth.WorkloadConfig("inf", 4, 30, (7, 30), D, "stateless", 24, 0, 0, 48, 64, 3.0, 4, (3,), "f32", 11)
+    m = tw_synth.make_model(cfg)
+    dec = TwDecoder(weights_from_synth(m), N=4, S=3, mode=0, max_batch=1, max_T=3)
+    x = np.random.default_rng(D).standard_normal((rows, D)).astype(np.float32)
+    r = np.arange(rows)
+    x[r, r % D] = np.where(r % 2, np.inf, -np.inf)
+    got = dec.project_encoder(x).cpu().numpy()
+    np.testing.assert_array_equal(got, np.where(r % 2, 1.0, -1.0)[:, None] * np.sign(m.W_e[:, r % D].T) * np.inf)
