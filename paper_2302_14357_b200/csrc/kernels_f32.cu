@@ -73,8 +73,9 @@ gemm_f32_kernel(const __grid_constant__ CUtensorMap tm0, const __grid_constant__
   uint64_t* full = reinterpret_cast<uint64_t*>(smem + (Sm::kOps > Sm::kRed ? Sm::kOps : Sm::kRed));
   uint64_t* empty = full + kStagesF;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int m0 = blockIdx.y * TM, n0 = blockIdx.x * BN;
   const int N = (MODE == 1) ? p.jr.V : p.N;
+  const int n_tiles = (N + BN - 1) / BN;                     // row tiles by column tiles, all on grid.x (grid.y would end at 65535 row tiles)
+  const int m0 = (int)blockIdx.x / n_tiles * TM, n0 = (int)blockIdx.x % n_tiles * BN;
   const int K0 = (MODE == 1) ? p.jr.J : p.op[0].K, K1 = (MODE == 1) ? 0 : p.op[1].K;
   const int nb0 = (K0 + BK - 1) / BK, nb_all = nb0 + (K1 + BK - 1) / BK;
   const int split = gridDim.z, part = blockIdx.z;            // the CTAs of a cluster share K
@@ -526,7 +527,7 @@ void launch_gemm_one(const GemmParams& p, long long M_max, int N, cudaStream_t s
   const int nb = MODE == 1 ? (p.jr.J + BK - 1) / BK : (p.op[0].K + BK - 1) / BK + (p.op[1].K + BK - 1) / BK;
   const unsigned split = (mt * nt <= 40 && nb >= 16) ? 4 : ((mt * nt <= 110 && nb >= 8) ? 2 : 1);
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)nt, (unsigned)mt, split); cfg.blockDim = dim3(kThreadsF);
+  cfg.gridDim = dim3((unsigned)(nt * mt), 1, split); cfg.blockDim = dim3(kThreadsF);
   cfg.dynamicSmemBytes = F32Smem<NJ>::kTotal; cfg.stream = st;
   cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeClusterDimension;
