@@ -158,7 +158,6 @@ int enqueue_predictor_plain(tw_handle* h, const int* tokens, const float* state_
   const size_t n = (size_t)R * h->L * 2 * h->Hd;
   if (h->mode == TW_MODE_F32 && h->L > 0 && state_in < state_out + n && state_out < state_in + n) {
     // a caller's state updated in place: the gate GEMM writes h while its other CTAs still read it, so it reads a copy
-    if (!h->state_copy) TW_TRY(dev_alloc(h, &h->state_copy, (size_t)h->R_max * h->L * 2 * h->Hd));
     TW_CUDA(h, cudaMemcpyAsync(h->state_copy, state_in, n * sizeof(float), cudaMemcpyDeviceToDevice, st));
     state_in = h->state_copy;
   }
@@ -337,6 +336,7 @@ int build_workspace(tw_handle* h) {
   if (!hs.stateless) {
     TW_TRY(dev_alloc(h, &hs.slot_hc, nslot * hs.L * 2 * hs.Hd));
     TW_TRY(dev_alloc(h, &hs.slot_Pp, nslot * h->J));
+    if (h->mode == TW_MODE_F32) TW_TRY(dev_alloc(h, &h->state_copy, R * hs.L * 2 * hs.Hd));
   }
   TW_TRY(dev_alloc(h, &hs.new_slot, nb * kMaxBeam));
   TW_TRY(dev_alloc(h, &hs.new_par, nb * kMaxBeam));

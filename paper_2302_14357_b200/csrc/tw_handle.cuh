@@ -27,7 +27,7 @@ struct tw_handle {
   tw::HypState hs{};
   tw::HypState hs_fused{};    // same arrays, but log J is not materialised (fused joiner path)
   float* E = nullptr;         // projected encoder frames [max_batch * max_T, J]
-  float* state_copy = nullptr;   // TW_MODE_F32: tw_predictor_step in place (allocated on first use)
+  float* state_copy = nullptr;   // TW_MODE_F32: the parents' states of a tw_predictor_step in place [R_max, L, 2, Hd]
   float* A_f32 = nullptr;     // TW_MODE_F32: the joiner's operand [R_max * S, J]
   int *stage_e0 = nullptr, *stage_slen = nullptr;   // [R_max] scratch of the stage entry points
   int* stream_oidx = nullptr;   // [max_batch * max_T] destination rows of a pushed chunk's frames
