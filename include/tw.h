@@ -40,7 +40,9 @@ typedef enum {
   TW_ERR_CUDA = 3,   /* a CUDA call failed; tw_last_cuda_error() has the code           */
   TW_ERR_LIMIT = 4,  /* a safety cap was hit (per-utterance: see tw_decode out_status)  */
   TW_ERR_STATE = 5,  /* call not valid for this handle (e.g. stage needs another mode)  */
-  TW_ERR_TIMEOUT = 6 /* a bounded device-side wait gave up; results are not valid       */
+  TW_ERR_TIMEOUT = 6 /* a bounded device-side wait gave up; results are not valid.  A streaming session reports it from the
+                        call on in which it happened.  The stage calls return before their kernels have run: the next stage
+                        call on the handle reports it for them, once, and enqueues nothing */
 } tw_status;
 
 enum { TW_MODE_F32 = 0, TW_MODE_BF16 = 1 };   /* arithmetic of the decoder (tw_config::mode)                   */
@@ -275,7 +277,8 @@ int tw_predictor_step(tw_handle* h, const int32_t* tokens, const float* state_in
  * The first call on each device looks up the device address of the fixed array (with that device
  * current); make that first call outside any stream capture.
  * All calls on a device share the one array, which keeps whatever the previous call left in it.
- * Nothing in it has to start at zero: each call overwrites every element it later reads.  Two calls
+ * Nothing in it has to start at zero: each call overwrites every element it later reads.  If a bounded wait of the
+ * contraction gives up, out_ldphi of the rows concerned is NaN.  Two calls
  * that overlap on the GPU (different streams, or different host threads) race on the array and give
  * wrong results; serialise them.
  */

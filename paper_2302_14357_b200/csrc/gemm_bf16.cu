@@ -458,6 +458,7 @@ gemm_lstm_wide_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_cons
   const bool active = m0 < M && mt < m_tiles && w <= W::kMaxBN;    // an idle CTA skips the roles and only frees its TMEM
   const uint32_t stage = kWideABytes + (uint32_t)w * (BK * 2);
   const int nst = EPIW == 16 ? 4 : min((int)(W::kRing / stage), kWideMaxStages);
+  bool ok = true;                                        // every wait of the ring so far has ended in time
 
   if (!active) {
     if (EPIW == 8) { pdl_wait(); pdl_trigger(); }
@@ -489,7 +490,8 @@ gemm_lstm_wide_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_cons
         for (int kb = 0; kb < npre; ++kb) { mbar_arrive(&full[kb]); mbar_wait(&full[kb], 0, p.err); }
       for (int kb = 0; kb < num_kb && rows > 0; ++kb) {
         if (kb >= npre) {
-          if (!mbar_wait(&empty[s], ph ^ 1, p.err)) break;
+          ok = mbar_wait(&empty[s], ph ^ 1, p.err);
+          if (!ok) break;
           send_B(kb, s, EPIW == 8 ? 0 : a_bytes);
         }
         if (EPIW == 8) mbar_expect_tx(&full[s], a_bytes);
@@ -504,7 +506,7 @@ gemm_lstm_wide_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_cons
     if (lane == 0 && (!late || m0 < *p.M_dev)) {
       const int n1 = w <= 256 ? w : ((w >> 1) + 15) & ~15, n2 = w - n1;    // wider than one MMA: two of about equal width
       const uint32_t idesc1 = make_idesc_bf16(BM, n1), idesc2 = make_idesc_bf16(BM, n2);
-      bool ok = mbar_wait(acc_init, 0, p.err);             // the accumulators hold bias + addend: accumulate onto them
+      ok = mbar_wait(acc_init, 0, p.err);                  // the accumulators hold bias + addend: accumulate onto them
       int s = 0;
       uint32_t ph = 0;
       for (int kb = 0; kb < num_kb && ok; ++kb) {
@@ -529,7 +531,10 @@ gemm_lstm_wide_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_cons
     lstm_tile_epilogue<EPIW>(p, tmem_base, acc_full, acc_init, M, late ? p.M_dev : nullptr, m0, n0, nu, warp, lane);
   }
   tc_fence_before();
-  __syncthreads();
+  if (__syncthreads_or(!ok)) {
+    if (threadIdx.x == 0) drain_ring(full, kWideMaxStages, p.err);
+    __syncthreads();
+  }
   if (warp == 1) tmem_dealloc(tmem_base, W::kTmem);
 }
 

@@ -212,7 +212,13 @@ gemm_f32_kernel(const __grid_constant__ CUtensorMap tm0, const __grid_constant__
   }
 
   // ---- the warps' partial tiles, summed in the order of K; [kWarpsF][TM][BN] in the operands' place
-  __syncthreads();                         // every block has been waited for: nothing is on its way into shared memory
+  // Every block has been waited for: nothing is on its way into shared memory.  If a wait gave up, the sums of this CTA come
+  // out as NaN, and what may still be on its way is waited for (each wait ends after 1024 polls now that *err is set).
+  const bool bad = __syncthreads_or(!ok) != 0;
+  if (bad) {
+    if (VEC && tid == 0) drain_ring(full, kStagesF, p.err);
+    __syncthreads();
+  }
 #pragma unroll
   for (int i = 0; i < TM; ++i)
 #pragma unroll
@@ -225,6 +231,7 @@ gemm_f32_kernel(const __grid_constant__ CUtensorMap tm0, const __grid_constant__
       const float4 u = *reinterpret_cast<const float4*>(&sm_f32[w * TM * BN + at]);
       v.x += u.x; v.y += u.y; v.z += u.z; v.w += u.w;
     }
+    if (bad) v = make_float4(NAN, NAN, NAN, NAN);
     return v;
   };
   if (split > 1) {                         // this CTA's sums in place; each CTA then finishes its share of the tile
@@ -494,9 +501,10 @@ __global__ void permute_rows_f32_kernel(const float* __restrict__ src, const int
 }
 
 __global__ void rows_from_groups_kernel(const int* row_group, const int* seg_len, int R, int G, int S,
-                                        int* row_e0, int* row_slen) {
+                                        int* row_e0, int* row_slen, int* clear) {
   pdl_wait();
   pdl_trigger();
+  if (clear != nullptr && blockIdx.x == 0 && threadIdx.x == 0) *clear = 0;
   int r = blockIdx.x * blockDim.x + threadIdx.x;
   if (r >= R) return;
   int g = row_group[r];
@@ -606,9 +614,9 @@ void launch_permute_rows_f32(const float* src, const int* perm, long long rows, 
 }
 
 void launch_rows_from_groups(const int* row_group, const int* seg_len, int R, int G, int S, int* row_e0,
-                             int* row_slen, cudaStream_t st) {
+                             int* row_slen, int* clear, cudaStream_t st) {
   if (R <= 0) return;
-  launch_pdl(rows_from_groups_kernel, dim3((R + 255) / 256), dim3(256), 0, st, row_group, seg_len, R, G, S, row_e0, row_slen);
+  launch_pdl(rows_from_groups_kernel, dim3((R + 255) / 256), dim3(256), 0, st, row_group, seg_len, R, G, S, row_e0, row_slen, clear);
 }
 
 }  // namespace tw

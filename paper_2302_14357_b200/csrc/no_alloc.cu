@@ -55,9 +55,10 @@ extern "C" int tw_joiner_expand_noalloc(const float* W_out, const float* b_out, 
   int* row_e0 = reinterpret_cast<int*>(scratch + kScratchFloats);
   int* row_slen = row_e0 + kMaxRows;
   cudaStream_t st = (cudaStream_t)stream;
-  // every element of the scratch that is read below is written first by this call, so nothing left by
-  // an earlier call can leak in and nothing needs clearing
-  launch_rows_from_groups(row_group, seg_len, R, G, S, row_e0, row_slen, st);
+  // Every element of the scratch that is read below is written first by this call, so nothing left by an earlier call can
+  // leak in; the error word, which makes the contraction's waits give up early, is cleared.  A wait that gives up shows as
+  // NaN in the rows concerned.
+  launch_rows_from_groups(row_group, seg_len, R, G, S, row_e0, row_slen, row_slen + kMaxRows, st);
   JoinerRows jr{};
   jr.E = E_seg; jr.row_e0 = row_e0; jr.Pp = Pp; jr.row_p = nullptr; jr.row_slen = row_slen;
   jr.R_dev = nullptr; jr.R_max = R; jr.S = S; jr.J = J; jr.V = V; jr.act = joiner_act;
@@ -66,4 +67,16 @@ extern "C" int tw_joiner_expand_noalloc(const float* W_out, const float* b_out, 
   launch_expand_f32(logp, ld_old, row_slen, nullptr, R, S, V, blank, out_ldphi, out_ldnb, out_la, nullptr,
                     nullptr, CandOut{}, st);
   return cudaGetLastError() == cudaSuccess ? TW_OK : TW_ERR_CUDA;
+}
+
+// For the tests of the error path: puts `value` into the error word, as a wait that gave up would, and returns what it held
+// (-1: a CUDA call failed).  Synchronises the device.
+extern "C" int tw_test_noalloc_word(int32_t value) {
+  float* scratch = nullptr;
+  int old = -1;
+  if (scratch_for_current_device(&scratch) != TW_OK || cudaDeviceSynchronize() != cudaSuccess) return -1;
+  int* word = reinterpret_cast<int*>(scratch + kScratchFloats) + 2 * kMaxRows;
+  if (cudaMemcpy(&old, word, sizeof(int), cudaMemcpyDeviceToHost) != cudaSuccess) return -1;
+  if (cudaMemcpy(word, &value, sizeof(int), cudaMemcpyHostToDevice) != cudaSuccess) return -1;
+  return old;
 }

@@ -68,6 +68,7 @@ wp_operand_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
   const uint32_t tmem_base = *tmem_holder;
   const int m_tiles = (M + BM - 1) / BM, n_tiles = (p.N + BN - 1) / BN;
   const int num_tiles = m_tiles * n_tiles;     // a CTA past the last tile runs no loop iteration below
+  bool ok = true;                              // every wait of this thread so far has ended in time
 
   if (warp == 0) {
     int npre = 0;                              // W_p is a constant: the first tile's first stages ahead of the wait
@@ -83,7 +84,6 @@ wp_operand_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
     pdl_trigger();
     if (lane == 0) {
       uint32_t it = 0;
-      bool ok = true;
       for (int tile = blockIdx.x; tile < num_tiles && ok; tile += gridDim.x) {
         const int m0 = (tile / n_tiles) * BM, n0 = (tile % n_tiles) * BN;
         const int nq = min(4, (M - m0 + 31) >> 5);           // lane quarters with rows in them
@@ -108,7 +108,6 @@ wp_operand_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
     if (lane == 0) {
       constexpr uint32_t idesc = make_idesc_bf16(BM, BN);
       uint32_t it = 0, lt = 0;
-      bool ok = true;
       for (int tile = blockIdx.x; tile < num_tiles && ok; tile += gridDim.x, ++lt) {
         const uint32_t buf = lt & 1, aph = (lt >> 1) & 1;
         ok = mbar_wait(&acc_empty[buf], aph ^ 1, p.err);
@@ -132,7 +131,7 @@ wp_operand_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
   } else {
     const int q = warp & 3, grp = (warp - 2) >> 2;           // TMEM lane quarter, group of kCols columns
     uint32_t lt = 0;
-    bool ok = true, waited = false;
+    bool waited = false;
     for (int tile = blockIdx.x; tile < num_tiles && ok; tile += gridDim.x, ++lt) {
       const int m = (tile / n_tiles) * BM + q * 32 + lane, n = (tile % n_tiles) * BN + grp * kCols;
       const uint32_t buf = lt & 1, aph = (lt >> 1) & 1;
@@ -194,7 +193,10 @@ wp_operand_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
     if (!waited) { pdl_wait(); pdl_trigger(); }
   }
   tc_fence_before();
-  __syncthreads();
+  if (__syncthreads_or(!ok)) {
+    if (threadIdx.x == 0) drain_ring(full, C::kStages, p.err);
+    __syncthreads();
+  }
   if (warp == 1) tmem_dealloc(tmem_base, 2 * BN);
 }
 

@@ -62,6 +62,12 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, int* e
   return false;
 }
 
+// For a CTA that leaves because a wait gave up (*err is set): copies that it sent for may still be on their way into its shared
+// memory.  One thread waits for each of the ring's barriers, at most 1024 polls each.
+__device__ __forceinline__ void drain_ring(uint64_t* full, int stages, int* err) {
+  for (int s = 0; s < stages; ++s) { mbar_wait(&full[s], 0, err); mbar_wait(&full[s], 1, err); }
+}
+
 // ---- thread-block clusters --------------------------------------------------------------------
 __device__ __forceinline__ uint32_t cluster_ctarank() {
   uint32_t r;

@@ -305,6 +305,10 @@ int build_bf16(tw_handle* h) {
   return TW_OK;
 }
 
+// words of tw_handle::host_flag: the device scalars, then the counters of a decode (8-byte), then the stage calls' error word
+enum { kHostCounters = 16, kHostStageErr = 32, kHostWords = 64 };
+static_assert(kScCount <= kHostCounters, "scalars");
+
 int build_workspace(tw_handle* h) {
   HypState& hs = h->hs;
   const int B = h->max_batch, N = h->N, S = h->S;
@@ -369,13 +373,14 @@ int build_workspace(tw_handle* h) {
   TW_CUDA(h, cudaMemset(h->zero_len, 0, nb * sizeof(int)));
   TW_CUDA(h, cudaMemset(hs.scalars, 0, kScCount * sizeof(int)));
   TW_CUDA(h, cudaMemset(hs.rows_total, 0, 3 * sizeof(long long)));
-  TW_CUDA(h, cudaHostAlloc((void**)&h->host_flag, (kScCount + 4) * sizeof(long long), cudaHostAllocDefault));
+  h->bf.err = hs.scalars + kScErr;
+  TW_CUDA(h, cudaHostAlloc((void**)&h->host_flag, kHostWords * sizeof(int), cudaHostAllocMapped));
+  memset(h->host_flag, 0, kHostWords * sizeof(int));
+  TW_CUDA(h, cudaHostGetDevicePointer((void**)&h->stage_err, h->host_flag + kHostStageErr, 0));
   return TW_OK;
 }
 
 int init_impl(tw_handle* h, const tw_model* m, const tw_config* c) {
-  TW_TRY(dev_alloc(h, &h->bf.err, (size_t)1));
-  TW_CUDA(h, cudaMemset(h->bf.err, 0, sizeof(int)));
   PdlScope plain(false);                     // kernels that fetch weights ahead of their wait run right behind the ones that write them
   h->D_enc = m->D_enc; h->P = m->P; h->J = m->J; h->V = m->V; h->blank = m->blank;
   h->pred_kind = m->pred_kind; h->emb_dim = m->emb_dim; h->joiner_act = m->joiner_act;
@@ -457,7 +462,9 @@ int init_impl(tw_handle* h, const tw_model* m, const tw_config* c) {
   }
   TW_CUDA(h, cudaGetLastError());
   TW_CUDA(h, cudaDeviceSynchronize());
-  return TW_OK;
+  int err = 0;
+  TW_CUDA(h, cudaMemcpy(&err, h->bf.err, sizeof(int), cudaMemcpyDeviceToHost));
+  return err == 0 ? TW_OK : TW_ERR_TIMEOUT;
 }
 
 }  // namespace

@@ -43,7 +43,7 @@ struct tw_handle {
     tw::Bf16Mat Htop;                                     // [R_max, Hd]
     float* bias_perm[tw::kMaxLayers] = {};   // LSTM biases in the interleaved gate order (layers > 0)
     float* EmbProj = nullptr;   // [V, 4Hd] = emb W_ih[0]^T + b[0]: layer 0's input half, one row per token
-    int* err = nullptr;                                   // device error word of the bounded waits (both modes)
+    int* err = nullptr;                                   // error word of the bounded waits (both modes): hs.scalars[kScErr]; in a stage call, stage_err
     // fused joiner + softmax + Eq. 3-7 + selection (logits stay in tensor memory)
     bool fused_ok = false, fused_on = false, no_max = false;
     float zbound = 0.f;                                   // bound of |logit| behind no_max
@@ -71,7 +71,8 @@ struct tw_handle {
   int* st_chunk_lens = nullptr;                         // [kHostChunks][max_batch]
   double* st_scores = nullptr; int* st_status = nullptr;
 
-  int* host_flag = nullptr;   // pinned copy of the device scalars
+  int* host_flag = nullptr;   // pinned: copy of the device scalars, counters, and the word behind stage_err
+  int* stage_err = nullptr;   // error word of the stage calls' waits, in host memory: those calls do not synchronise, so the next one looks
 
   // The decode loop is captured once per (B, T, joiner path) into a CUDA graph and replayed; it runs on a stream of the
   // handle's own because the caller's may be the legacy default stream, which cannot be captured.

@@ -150,13 +150,14 @@ bool scan_select_fits(int S, int V);   // the row's S x V logits fit in shared m
 int scan_select_setup();
 void launch_scan_select(const ScanSelectArgs& a, bool fast_math, cudaStream_t st);
 // helper for the stage entry points: row_e0[r] = row_group[r] * S, row_slen[r] = seg_len[row_group[r]] clamped to
-// [0, S]; a row whose group is outside [0, G) becomes an empty row (length 0)
+// [0, S]; a row whose group is outside [0, G) becomes an empty row (length 0).  clear: optional device word set to 0
 void launch_rows_from_groups(const int* row_group, const int* seg_len, int R, int G, int S, int* row_e0,
-                             int* row_slen, cudaStream_t st);
+                             int* row_slen, int* clear, cudaStream_t st);
 
 // ---------------------------------------------------------------------------------------------
 // Hypothesis state of a batch (structure of arrays in one device workspace).
-enum Scalar { kScR = 0, kScNPred = 1, kScActive = 2, kScSteps = 3, kScM = 4, kScRow0 = 5, kScRow1 = 6, kScIter = 7, kScCount = 8 };   // kScM = R * S; kScRow0/1: HypState::own_rows
+// kScM = R * S; kScRow0/1: HypState::own_rows; kScErr: error word of a decode's bounded waits
+enum Scalar { kScR = 0, kScNPred = 1, kScActive = 2, kScSteps = 3, kScM = 4, kScRow0 = 5, kScRow1 = 6, kScIter = 7, kScErr = 8, kScCount = 9 };
 
 struct HypState {
   int B, N, S, V, J, U_cap, I_max, blank;
