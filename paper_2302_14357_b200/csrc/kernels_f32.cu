@@ -519,8 +519,9 @@ __global__ void rows_from_groups_kernel(const int* row_group, const int* seg_len
 namespace {
 bool row_aligned(const float* base, long long ld) { return (reinterpret_cast<uintptr_t>(base) & 15) == 0 && (ld & 3) == 0; }
 
+// false: no tensor map of the weights could be made, nothing was launched (a launch that fails is left to cudaGetLastError)
 template <int MODE, int NJ, bool VEC>
-void launch_gemm_one(const GemmParams& p, long long M_max, int N, cudaStream_t st) {
+bool launch_gemm_one(const GemmParams& p, long long M_max, int N, cudaStream_t st) {
   static std::atomic<unsigned long long> ready{0};           // devices whose copy of the kernel has its shared-memory limit raised
   int dev = 0;
   cudaGetDevice(&dev);
@@ -546,17 +547,18 @@ void launch_gemm_one(const GemmParams& p, long long M_max, int N, cudaStream_t s
   CUtensorMap tm0 = {}, tm1 = {};
   if (VEC) {
     const GemmOperand b0 = MODE == 1 ? GemmOperand{nullptr, nullptr, 0, p.W_out, p.jr.J, p.jr.J} : p.op[0];
-    make_tmap_f32(&tm0, b0.B, N, b0.K, b0.ldB, 32 * NJ);
-    if (p.op[1].K > 0) make_tmap_f32(&tm1, p.op[1].B, N, p.op[1].K, p.op[1].ldB, 32 * NJ);
+    if (make_tmap_f32(&tm0, b0.B, N, b0.K, b0.ldB, 32 * NJ) != TW_OK) return false;
+    if (p.op[1].K > 0 && make_tmap_f32(&tm1, p.op[1].B, N, p.op[1].K, p.op[1].ldB, 32 * NJ) != TW_OK) return false;
   }
   cudaLaunchKernelEx(&cfg, gemm_f32_kernel<MODE, NJ, VEC>, tm0, tm1, p);
+  return true;
 }
 template <int MODE>
 void launch_gemm_tiles(const GemmParams& p, bool vec, long long M_max, int N, cudaStream_t st) {
   if (N <= 128) {
-    if (vec) launch_gemm_one<MODE, 2, true>(p, M_max, N, st); else launch_gemm_one<MODE, 2, false>(p, M_max, N, st);
+    if (!vec || !launch_gemm_one<MODE, 2, true>(p, M_max, N, st)) launch_gemm_one<MODE, 2, false>(p, M_max, N, st);
   } else {
-    if (vec) launch_gemm_one<MODE, 8, true>(p, M_max, N, st); else launch_gemm_one<MODE, 8, false>(p, M_max, N, st);
+    if (!vec || !launch_gemm_one<MODE, 8, true>(p, M_max, N, st)) launch_gemm_one<MODE, 8, false>(p, M_max, N, st);
   }
 }
 }  // namespace

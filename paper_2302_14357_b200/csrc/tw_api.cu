@@ -16,6 +16,7 @@ namespace {
     cudaError_t e_ = (expr);                               \
     if (e_ != cudaSuccess) {                               \
       if (h) (h)->last_cuda = (int)e_;                     \
+      cudaGetLastError();   /* reported here, and not by a later call once more */ \
       return (e_ == cudaErrorMemoryAllocation) ? TW_ERR_ALLOC : TW_ERR_CUDA; \
     }                                                      \
   } while (0)
@@ -25,7 +26,7 @@ int dev_alloc(tw_handle* h, T** p, size_t count) {
   void* q = nullptr;
   if (count == 0) count = 1;
   cudaError_t e = cudaMalloc(&q, count * sizeof(T));
-  if (e != cudaSuccess) { h->last_cuda = (int)e; *p = nullptr; return TW_ERR_ALLOC; }
+  if (e != cudaSuccess) { h->last_cuda = (int)e; cudaGetLastError(); *p = nullptr; return TW_ERR_ALLOC; }
   h->dev_allocs.push_back(q);
   *p = static_cast<T*>(q);
   return TW_OK;
