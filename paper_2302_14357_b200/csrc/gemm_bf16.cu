@@ -616,10 +616,12 @@ bool launch_gemm_lstm_wide(const CUtensorMap& tmA, const CUtensorMap& tmA32, con
   const int units = p.N >> 5;
   const int w = ((units + n_split - 1) / n_split) * 32;
   if (w > Wide<16>::kMaxBN) return false;
-  // One or two row tiles at most: the small instance.  Up to five where another stream's kernel holds part of the SMs (p.beside):
-  // its CTAs find room beside that kernel's, those of the large instance wait for it (64 utterances at S = 20: 7 % per
-  // decode; without such a kernel the split for the largest count costs 2 % at 64 utterances, S = 3).
-  if ((mt <= 2 && w <= 64) || (p.beside && mt <= 5 && w <= 128)) {
+  // One or two row tiles at most: the small instance.  Where another stream's kernel holds part of the SMs (p.beside): wherever
+  // its 128 columns suffice.  Its CTAs find room beside that kernel's, those of the large instance wait for it (decodes at
+  // N = 10, large against small instance: H = 640, S = 20, three row tiles 9.80 -> 9.18 ms, five 11.7 -> 11.0, six 12.7 -> 11.9,
+  // seven, at the full 128 columns, 13.7 either way; H = 512, S = 8, six to nine 12.4 -> 11.8 .. 13.4 -> 13.1).  Without such
+  // a kernel the split for the largest count costs 2 % at five row tiles, S = 3.
+  if ((mt <= 2 && w <= 64) || (p.beside && w <= Wide<8>::kMaxBN)) {
     launch_pdl(gemm_lstm_wide_kernel<8>, dim3(num_sms), dim3(Wide<8>::kThreads), Wide<8>::kSmem, st, tmA, tmA32, tmB64, tmB32, p);
     return true;
   }

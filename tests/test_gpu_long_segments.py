@@ -56,9 +56,10 @@ def test_decode_matches_the_oracle_and_the_staged_kernels(S, B, V):
     _against_oracle(m, cfg, S, enc, lens, fused, range(min(B, 6)))
 
 
-@pytest.mark.parametrize("H,layers,B,S", [(640, 1, 32, 8), (640, 2, 64, 20), (1024, 2, 50, 8), (512, 3, 64, 13), (640, 1, 38, 10)])
+@pytest.mark.parametrize("H,layers,B,S", [(640, 1, 32, 8), (640, 2, 64, 20), (1024, 2, 50, 8), (512, 3, 64, 13), (640, 1, 38, 10),
+                                          (640, 1, 88, 8), (512, 1, 115, 10)])
 def test_gate_gemm_beside_the_side_branch(H, layers, B, S):
-    """Three to five row tiles (300 to 640 rows at N = 10), tiles of 64 to 128 gate columns, and lengths that empty whole row
+    """Three to nine row tiles (320 to 1150 rows at N = 10), tiles of 64 to 128 gate columns, and lengths that empty whole row
     tiles on the way: with the work list from hyp_step_kernel and from the gather kernel, as a graph and kernel by kernel."""
     cfg = _cfg(H, layers, 256, N=10)
     T = 2 * S + 3
