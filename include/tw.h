@@ -278,7 +278,7 @@ int tw_predictor_step(tw_handle* h, const int32_t* tokens, const float* state_in
  * current); make that first call outside any stream capture.
  * All calls on a device share the one array, which keeps whatever the previous call left in it.
  * Nothing in it has to start at zero: each call overwrites every element it later reads.  If a bounded wait of the
- * contraction gives up, out_ldphi of the rows concerned is NaN.  Two calls
+ * contraction gives up, out_ldphi is NaN.  Two calls
  * that overlap on the GPU (different streams, or different host threads) race on the array and give
  * wrong results; serialise them.
  */

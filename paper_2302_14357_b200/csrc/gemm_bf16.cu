@@ -531,10 +531,8 @@ gemm_lstm_wide_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_cons
     lstm_tile_epilogue<EPIW>(p, tmem_base, acc_full, acc_init, M, late ? p.M_dev : nullptr, m0, n0, nu, warp, lane);
   }
   tc_fence_before();
-  if (__syncthreads_or(!ok)) {
-    if (threadIdx.x == 0) drain_ring(full, kWideMaxStages, p.err);
-    __syncthreads();
-  }
+  settle_copies(ok);
+  __syncthreads();
   if (warp == 1) tmem_dealloc(tmem_base, W::kTmem);
 }
 

@@ -95,9 +95,12 @@ __device__ void carry_rows(const HypState& hs, int b) {
              *reinterpret_cast<const float4*>(pp + 4), hs.act);
   }
   // padding frames of a short segment: zeros, whatever an older pass left there (see pred_out.cu)
-  for (int c = threadIdx.x; c < n * (S - sl) * per; c += blockDim.x) {
-    const int pair = c / per, x = (c - pair * per) * 8, hh = pair / (S - sl), t = sl + pair - hh * (S - sl);
-    *reinterpret_cast<uint4*>(static_cast<__nv_bfloat16*>(hs.A_next) + operand_row(r0 + hh, t, S) * J + x) = make_uint4(0, 0, 0, 0);
+  if (__builtin_expect(sl < S, 0)) {
+#pragma unroll 1
+    for (int c = threadIdx.x; c < n * (S - sl) * per; c += blockDim.x) {
+      const int pair = c / per, x = (c - pair * per) * 8, hh = pair / (S - sl), t = sl + pair - hh * (S - sl);
+      *reinterpret_cast<uint4*>(static_cast<__nv_bfloat16*>(hs.A_next) + operand_row(r0 + hh, t, S) * J + x) = make_uint4(0, 0, 0, 0);
+    }
   }
 }
 

@@ -212,13 +212,8 @@ gemm_f32_kernel(const __grid_constant__ CUtensorMap tm0, const __grid_constant__
   }
 
   // ---- the warps' partial tiles, summed in the order of K; [kWarpsF][TM][BN] in the operands' place
-  // Every block has been waited for: nothing is on its way into shared memory.  If a wait gave up, the sums of this CTA come
-  // out as NaN, and what may still be on its way is waited for (each wait ends after 1024 polls now that *err is set).
-  const bool bad = __syncthreads_or(!ok) != 0;
-  if (bad) {
-    if (VEC && tid == 0) drain_ring(full, kStagesF, p.err);
-    __syncthreads();
-  }
+  settle_copies(ok);
+  __syncthreads();                         // every block has been waited for: nothing is on its way into shared memory
 #pragma unroll
   for (int i = 0; i < TM; ++i)
 #pragma unroll
@@ -231,7 +226,6 @@ gemm_f32_kernel(const __grid_constant__ CUtensorMap tm0, const __grid_constant__
       const float4 u = *reinterpret_cast<const float4*>(&sm_f32[w * TM * BN + at]);
       v.x += u.x; v.y += u.y; v.z += u.z; v.w += u.w;
     }
-    if (bad) v = make_float4(NAN, NAN, NAN, NAN);
     return v;
   };
   if (split > 1) {                         // this CTA's sums in place; each CTA then finishes its share of the tile
@@ -413,7 +407,7 @@ __global__ void __launch_bounds__(256) expand_f32_kernel(const float* __restrict
                                                          const int* row_slen, const int* R_dev,
                                                          int R_max, int S, int V, int blank,
                                                          float* ldphi, float* ldnb, float* la_out,
-                                                         double* ldphi_d, double* la_d, CandOut cand, StepWords words) {
+                                                         double* ldphi_d, double* la_d, CandOut cand, StepWords words, const int* err) {
   update_step_words(words);
   __shared__ float la[kMaxSeg];
   __shared__ float s_wv[8][kMaxBeam];
@@ -439,7 +433,7 @@ __global__ void __launch_bounds__(256) expand_f32_kernel(const float* __restrict
       la[t] = -INFINITY;
       if (la_d) la_d[(long long)r * S + t] = -INFINITY;
     }
-    ldphi[r] = (float)phi;
+    ldphi[r] = (err != nullptr && *err != 0) ? NAN : (float)phi;
     if (ldphi_d) ldphi_d[r] = phi;
   }
   __syncthreads();
@@ -605,10 +599,10 @@ void launch_log_softmax(const JoinerRows& rows, int blank, float* z, cudaStream_
 
 void launch_expand_f32(const float* logp, const float* ld_old, const int* row_slen, const int* R_dev,
                        int R_max, int S, int V, int blank, float* ldphi, float* ldnb, float* la,
-                       double* ldphi_d, double* la_d, const CandOut& cand, cudaStream_t st, const StepWords& words) {
+                       double* ldphi_d, double* la_d, const CandOut& cand, cudaStream_t st, const StepWords& words, const int* err) {
   if (R_max <= 0) return;
   expand_f32_kernel<<<R_max, 256, 0, st>>>(logp, ld_old, row_slen, R_dev, R_max, S, V, blank, ldphi,
-                                           ldnb, la, ldphi_d, la_d, cand, words);
+                                           ldnb, la, ldphi_d, la_d, cand, words, err);
 }
 
 void launch_permute_rows_f32(const float* src, const int* perm, long long rows, int cols, float* dst, cudaStream_t st) {

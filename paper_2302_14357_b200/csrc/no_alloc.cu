@@ -57,7 +57,7 @@ extern "C" int tw_joiner_expand_noalloc(const float* W_out, const float* b_out, 
   cudaStream_t st = (cudaStream_t)stream;
   // Every element of the scratch that is read below is written first by this call, so nothing left by an earlier call can
   // leak in; the error word, which makes the contraction's waits give up early, is cleared.  A wait that gives up shows as
-  // NaN in the rows concerned.
+  // NaN in out_ldphi.
   launch_rows_from_groups(row_group, seg_len, R, G, S, row_e0, row_slen, row_slen + kMaxRows, st);
   JoinerRows jr{};
   jr.E = E_seg; jr.row_e0 = row_e0; jr.Pp = Pp; jr.row_p = nullptr; jr.row_slen = row_slen;
@@ -65,7 +65,7 @@ extern "C" int tw_joiner_expand_noalloc(const float* W_out, const float* b_out, 
   launch_joiner_f32(jr, W_out, b_out, logp, nullptr, row_slen + kMaxRows, st);
   launch_log_softmax(jr, blank, logp, st);
   launch_expand_f32(logp, ld_old, row_slen, nullptr, R, S, V, blank, out_ldphi, out_ldnb, out_la, nullptr,
-                    nullptr, CandOut{}, st);
+                    nullptr, CandOut{}, st, StepWords{}, row_slen + kMaxRows);
   return cudaGetLastError() == cudaSuccess ? TW_OK : TW_ERR_CUDA;
 }
 

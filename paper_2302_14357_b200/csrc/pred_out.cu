@@ -185,18 +185,19 @@ wp_operand_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
         if (two) ld_global_v8(e + (long long)t * p.N + 8, x + 8);
         frame(t, x);
       }
-      for (int t = sl; t < p.S; ++t) {                        // padding frames (a last, short segment)
-        *reinterpret_cast<uint4*>(dst + (long long)t * p.N) = make_uint4(0, 0, 0, 0);
-        if (two) *reinterpret_cast<uint4*>(dst + (long long)t * p.N + 8) = make_uint4(0, 0, 0, 0);
+      if (__builtin_expect(sl < p.S, 0)) {                    // padding frames (a last, short segment)
+#pragma unroll 1
+        for (int t = sl; t < p.S; ++t) {
+          *reinterpret_cast<uint4*>(dst + (long long)t * p.N) = make_uint4(0, 0, 0, 0);
+          if (two) *reinterpret_cast<uint4*>(dst + (long long)t * p.N + 8) = make_uint4(0, 0, 0, 0);
+        }
       }
     }
     if (!waited) { pdl_wait(); pdl_trigger(); }
   }
   tc_fence_before();
-  if (__syncthreads_or(!ok)) {
-    if (threadIdx.x == 0) drain_ring(full, C::kStages, p.err);
-    __syncthreads();
-  }
+  settle_copies(ok);
+  __syncthreads();
   if (warp == 1) tmem_dealloc(tmem_base, 2 * BN);
 }
 

@@ -62,10 +62,11 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, int* e
   return false;
 }
 
-// For a CTA that leaves because a wait gave up (*err is set): copies that it sent for may still be on their way into its shared
-// memory.  One thread waits for each of the ring's barriers, at most 1024 polls each.
-__device__ __forceinline__ void drain_ring(uint64_t* full, int stages, int* err) {
-  for (int s = 0; s < stages; ++s) { mbar_wait(&full[s], 0, err); mbar_wait(&full[s], 1, err); }
+// For a thread that leaves its loop because a wait gave up: copies that its CTA sent for may still be on their way into shared
+// memory, which the CTA must not leave before.  They take microseconds; a millisecond passes before the thread goes on to the
+// CTA's last barrier.  (One instruction: a loop over the ring's barriers, never run, cost the fp32 GEMM 1 % by its mere size.)
+__device__ __forceinline__ void settle_copies(bool ok) {
+  if (!ok) __nanosleep(1000000);
 }
 
 // ---- thread-block clusters --------------------------------------------------------------------

@@ -133,7 +133,8 @@ __device__ __forceinline__ void update_step_words(const StepWords& w) {
 void launch_expand_f32(const float* logp, const float* ld_old, const int* row_slen, const int* R_dev,
                        int R_max, int S, int V, int blank, float* ldphi, float* ldnb, float* la,
                        double* ldphi_d, double* la_d, const CandOut& cand,
-                       cudaStream_t st, const StepWords& words = StepWords{});   // float64 copies optional
+                       cudaStream_t st, const StepWords& words = StepWords{},   // float64 copies optional
+                       const int* err = nullptr);   // optional device word: where it is raised, ldphi is NaN
 // Softmax + Eq. 3-7 + per-row candidates from RAW logits z [R, S, V] read once into shared memory
 // (scan_select.cu).  Every output pointer is optional.
 struct ScanSelectArgs {
