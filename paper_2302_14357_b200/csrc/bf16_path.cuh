@@ -43,6 +43,7 @@ int make_tmap_bf16(CUtensorMap* out, const void* base, uint64_t rows, uint64_t K
 // the same over a row-major float32 matrix with leading dimension ld, box = 32 x box_rows; K and ld multiples of 4
 int make_tmap_f32(CUtensorMap* out, const float* base, uint64_t rows, uint64_t K, uint64_t ld, uint32_t box_rows);
 int gemm_bf16_setup();
+int sm_count();    // SMs of the device
 // tmB128 / tmB256: maps of the same B matrix with 128- and 256-row boxes
 // tmB64 (optional): a map with 64-row boxes, used for small problems without an epilogue fusion
 void launch_gemm_bf16(const CUtensorMap& tmA, const CUtensorMap& tmB128, const CUtensorMap& tmB256,

@@ -1,4 +1,4 @@
-// Fused joiner + softmax + Eq. 3-7 + candidate selection for TW_MODE_BF16.  The [rows, V] logits live
+// Fused joiner + softmax + Eq. 3-7 for TW_MODE_BF16.  The [rows, V] logits live
 // only in tensor memory: a thread-block cluster of CL = V / NC CTAs (NC = 256, 128 or 64 columns each) owns a tile of 128
 // rows, CTA c holding columns [NC c, NC c + NC) of it in TMEM (two accumulator buffers, so the contraction of
 // the next row tile overlaps this tile's epilogue).
@@ -12,7 +12,7 @@
 //                 hypothesis (frames of a hypothesis are adjacent lanes of one warp): Eq. 3-5, 7
 //   epilogue B    delta_nb(k) = sum_t exp(la[t] - lse[t] + z[t, k]) (Eq. 6) by a segmented warp
 //                 reduction, written to device memory ([rows / S, V]: S times smaller than the logits);
-//                 the rows' N best tokens are then picked by the selection kernel of scan_select.cu
+//                 with, for some segment sizes, the maximum of every 16 or 32 columns; hyp_step_kernel picks the N best
 // Row layout: a tile holds 4 * (32 / S) hypotheses; hypothesis j of warp quarter q sits in TMEM lanes
 // 32 q + j S .. + S - 1 (one lane per frame); lanes past (32 / S) S are idle.
 //

@@ -592,7 +592,7 @@ int gemm_bf16_setup() {
   return (e1 == cudaSuccess && e2 == cudaSuccess && e3 == cudaSuccess && e4 == cudaSuccess && e5 == cudaSuccess) ? TW_OK : TW_ERR_CUDA;
 }
 
-static int sm_count() {
+int sm_count() {
   static int num_sms = 0;
   if (num_sms == 0) {
     int dev = 0;

@@ -722,7 +722,6 @@ __global__ void __launch_bounds__(1024) compact_kernel(HypState hs, int B, int T
       const int r = (chip ? (s_off[b] & 0xffff) : hs.row_off[b]) + h;
       const int slot = hs.A_slot[b * kMaxBeam + h];
       const long long gs = (long long)b * hs.capSlot + slot;
-      hs.row_b[r] = b;
       hs.row_e0[r] = b * T + hs.t0[b];
       hs.row_slen[r] = hs.slen[b];
       if (hs.stateless) {

@@ -23,8 +23,10 @@ namespace {
 // weights arrive by TMA (128-byte swizzle: the 16-byte reads along K of eight neighbouring rows hit distinct banks), the
 // rows of A by bulk copies, four blocks of 32 ahead, each block sent for by another warp, and the warps meet on the
 // ring's mbarriers only.  The weights of the first blocks are asked for before the wait for the kernel ahead.
-// Bound by FFMA issue: on a B200 register-only FFMA loops reach 51 of the nominal 74 TFLOP/s; measured here 27 us for
-// 112 x 2560 x 1280 and 26 us for 435 x 1024 x 640 (77 and 59 us with 64 x 64 tiles, 4 x 4 outputs a thread, whole K).
+// Measured: 27 us for 112 x 2560 x 1280 and 26 us for 435 x 1024 x 640 (77 and 59 us with 64 x 64 tiles, 4 x 4 outputs a
+// thread, whole K), 27 and 22 TFLOP/s, where register-only FFMA loops reach 51 of the nominal 74 on a B200.  By FFMA issue
+// alone the share of one CTA (16 x 256 x 640) would take 15 us at that rate; the rest is the way of the first blocks
+// into shared memory, the sum over warps and CTAs, and the SMs that the 140 and 112 CTAs leave idle.
 constexpr int TM = 16, BK = 32, kStagesF = 6, kAhead = kStagesF - 2, kWarpsF = 8, kThreadsF = 32 * kWarpsF;
 template <int NJ> struct F32Smem {
   static constexpr size_t kB = (size_t)32 * NJ * BK * 4, kA = (size_t)TM * BK * 4;
@@ -575,11 +577,14 @@ int launch_joiner_f32(const JoinerRows& rows, const float* W_out, const float* b
   GemmParams p{};
   p.err = err;
   const long long M_max = (long long)rows.R_max * rows.S;
-  // tanhf costs as much as some 25 FFMAs, so forming the operand anew in every column tile adds about 40 % to the
-  // contraction: a separate pass as soon as there is more than one wave of tiles (below, its launch costs more)
+  // The operand (a tanhf per element) formed anew in every column tile, or once in a pass of its own, which costs a launch and a
+  // round trip through L2: 1 to 2 us.  The pass from one 16 x 64 output tile per SM on, which is a quarter of that many CTAs
+  // for V > 128.  Measured, without / with it, tw_joiner_expand: V = 1024, J = 640: 129 GEMM rows 30.2 / 30.8 us, 192 26.8 /
+  // 27.6, 321 44.6 / 43.1, 768 70 / 64; V = 501: 480 27.5 / 28.0, 768 45.3 / 43.6; V = 4096, J = 1024: 33 42.5 / 42.8, 81
+  // 67.8 / 64.4; V = 128: 1536 13.6 / 12.1.
   const long long tiles = (M_max + TM - 1) / TM * ((rows.V + 63) / 64);
   const bool vec = (rows.J & 3) == 0 && row_aligned(W_out, rows.J);
-  if (A_buf != nullptr && tiles > 148) {
+  if (A_buf != nullptr && tiles > sm_count()) {
     launch_pdl(joiner_A_f32_kernel, dim3((unsigned)((M_max + 7) / 8)), dim3(256), 0, st, rows, A_buf);
     p.op[0] = GemmOperand{A_buf, nullptr, rows.J, W_out, rows.J, rows.J};
     p.out = GemmOut{z, nullptr, rows.V, b_out};

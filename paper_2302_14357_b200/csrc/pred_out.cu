@@ -204,7 +204,7 @@ wp_operand_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
 template <int BN>
 void launch_wp(const Bf16Mat& A, const CUtensorMap& tmB, const WpOperandParams& p, int mt, cudaStream_t st) {
   const int tiles = mt * ((p.N + BN - 1) / BN);
-  launch_pdl(wp_operand_kernel<BN>, dim3(tiles < 148 ? tiles : 148), dim3(WpCfg<BN>::kThreads), WpCfg<BN>::kSmem, st, A.as_A, A.as_B32, tmB, p);
+  launch_pdl(wp_operand_kernel<BN>, dim3(tiles < sm_count() ? tiles : sm_count()), dim3(WpCfg<BN>::kThreads), WpCfg<BN>::kSmem, st, A.as_A, A.as_B32, tmB, p);
 }
 
 }  // namespace
@@ -220,7 +220,7 @@ int wp_operand_setup() {
 void launch_wp_operand(const Bf16Mat& A, const Bf16Mat& W, const WpOperandParams& p, cudaStream_t st) {
   if (p.M <= 0) return;
   const int mt = (p.M + BM - 1) / BM;
-  if (mt * ((p.N + 63) / 64) <= 74) launch_wp<32>(A, W.as_B32, p, mt, st);
+  if (2 * mt * ((p.N + 63) / 64) <= sm_count()) launch_wp<32>(A, W.as_B32, p, mt, st);
   else launch_wp<64>(A, W.as_B64, p, mt, st);
 }
 

@@ -54,36 +54,13 @@ __global__ void __launch_bounds__(kMaxT) scan_select_kernel(ScanSelectArgs a) {
   const int r = blockIdx.x;
   if (r >= R) return;
   const int S = a.S, V = a.V, blank = a.blank;
-  const int sl = a.dnb_in ? 1 : (a.row_slen ? min(max(a.row_slen[r], 0), S) : S);
+  const int sl = a.row_slen ? min(max(a.row_slen[r], 0), S) : S;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int kT = blockDim.x, nwarps = kT >> 5;
-  const int gshift = kT >= 256 ? 4 : 3, ngroups = kT >> gshift;   // groups of 16 threads (8 in a 128-thread CTA): at least 16 groups
+  const int ngroups = kT >> 4;                         // groups of 16 threads: at least 16 groups
   const float* z = a.z + (long long)r * S * V;
 
   float tmax = -INFINITY;
-  if (a.dnb_in != nullptr) {
-    // selection only: the row of delta_nb values is given
-    const float* src = a.dnb_in + (long long)r * V;
-    if ((V & 3) == 0) {
-      for (int k = tid * 4; k < V; k += kT * 4) {
-        float4 v = *reinterpret_cast<const float4*>(src + k);
-        if (a.dnb_linear) {                                // order is the same as that of the logs
-          v.x = v.x > 0.f ? v.x : -INFINITY; v.y = v.y > 0.f ? v.y : -INFINITY;
-          v.z = v.z > 0.f ? v.z : -INFINITY; v.w = v.w > 0.f ? v.w : -INFINITY;
-        }
-        *reinterpret_cast<float4*>(zs + k) = v;
-        tmax = fmaxf(fmaxf(tmax, fmaxf(v.x, v.y)), fmaxf(v.z, v.w));
-      }
-    } else {
-      for (int k = tid; k < V; k += kT) {
-        float v = src[k];
-        if (a.dnb_linear) v = v > 0.f ? v : -INFINITY;
-        zs[k] = v; tmax = fmaxf(tmax, v);
-      }
-    }
-    if (tid == 0) s_nsurv = 0;
-    __syncthreads();
-  } else {
   // ---- the one pass over global memory
   if ((V & 3) == 0) {
     const int n4 = sl * V / 4;
@@ -151,14 +128,13 @@ __global__ void __launch_bounds__(kMaxT) scan_select_kernel(ScanSelectArgs a) {
     if (a.ldnb) a.ldnb[(long long)r * V + k] = out;
     tmax = fmaxf(tmax, out);
   }
-  }
   if (a.cand.n == nullptr) return;
   const int N = a.cand.N;
 
   // ---- a lower bound of the row's N-th best value: the N-th largest of 16 group maxima (each is a
   // distinct element of the row), so everything at or above it is a small superset of the answer
-  for (int o = (1 << gshift) >> 1; o > 0; o >>= 1) tmax = fmaxf(tmax, __shfl_xor_sync(0xffffffffu, tmax, o));
-  if ((tid & ((1 << gshift) - 1)) == 0) s_gmax[tid >> gshift] = tmax;
+  for (int o = 8; o > 0; o >>= 1) tmax = fmaxf(tmax, __shfl_xor_sync(0xffffffffu, tmax, o));
+  if ((tid & 15) == 0) s_gmax[tid >> 4] = tmax;
   __syncthreads();
   if (warp == 0) {
     for (int g = lane; g < ngroups; g += 32) {
@@ -192,7 +168,7 @@ __global__ void __launch_bounds__(kMaxT) scan_select_kernel(ScanSelectArgs a) {
         int rank = 0;
         for (int j = 0; j < ns; ++j) rank += cand_better(s_sv[j], s_sk[j], v, k);
         if (rank < N) {
-          a.cand.v[(long long)r * kMaxBeam + rank] = a.dnb_linear ? __logf(v) : v;
+          a.cand.v[(long long)r * kMaxBeam + rank] = v;
           a.cand.k[(long long)r * kMaxBeam + rank] = k;
         }
       }
@@ -227,7 +203,7 @@ __global__ void __launch_bounds__(kMaxT) scan_select_kernel(ScanSelectArgs a) {
       }
       bv = __shfl_sync(0xffffffffu, bv, 0); bk = __shfl_sync(0xffffffffu, bk, 0); bl = __shfl_sync(0xffffffffu, bl, 0);
       if (bv == -INFINITY) break;
-      if (lane == 0) { a.cand.v[(long long)r * kMaxBeam + j] = a.dnb_linear ? __logf(bv) : bv; a.cand.k[(long long)r * kMaxBeam + j] = bk; }
+      if (lane == 0) { a.cand.v[(long long)r * kMaxBeam + j] = bv; a.cand.k[(long long)r * kMaxBeam + j] = bk; }
       if (lane == bl) ++pos;
       ++cnt;
     }
@@ -249,10 +225,9 @@ int scan_select_setup() {
 
 void launch_scan_select(const ScanSelectArgs& a, bool fast_math, cudaStream_t st) {
   if (a.R_max <= 0) return;
-  const size_t smem = a.dnb_in ? scan_select_smem_bytes(1, a.V) : scan_select_smem_bytes(a.S, a.V);
+  const size_t smem = scan_select_smem_bytes(a.S, a.V);
   // a row that takes most of an SM's shared memory runs alone there: give it the whole SM's threads
-  // selection from a short row (delta_nb given): 128-thread CTAs, so that a whole batch of rows is resident at once
-  const int threads = smem > 96 * 1024 ? 1024 : (smem > 48 * 1024 ? 512 : ((a.dnb_in && smem <= 16 * 1024) ? 128 : 256));
+  const int threads = smem > 96 * 1024 ? 1024 : (smem > 48 * 1024 ? 512 : 256);
   if (fast_math) launch_pdl(scan_select_kernel<true>, dim3(a.R_max), dim3(threads), smem, st, a);
   else launch_pdl(scan_select_kernel<false>, dim3(a.R_max), dim3(threads), smem, st, a);
 }

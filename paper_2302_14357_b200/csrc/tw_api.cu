@@ -265,12 +265,12 @@ int build_bf16(tw_handle* h) {
       TW_CUDA(h, cudaMemcpy(&bound, bound_dev, sizeof(float), cudaMemcpyDeviceToHost));
       h->bf.no_max = (bound <= 40.f) && h->joiner_act == TW_ACT_TANH;   // the bound needs |act| <= 1
       h->bf.zbound = bound;
-      // two operand buffers: a step's operand is written while the previous step's is still read
-      for (Bf16Mat& a : h->bf.A_tiled)
-        TW_TRY(make_bf16_mat(h, &a, nullptr, &a == &h->bf.A_tiled[0] || h->S < 8 ? fused_joiner_A_rows(h->R_max, h->S) : 128, h->J, true, true));
+      // the steps that make their own rows (own_rows) have two operand buffers: one is written while the other is still read
+      const int buffers = h->pred_kind == TW_PRED_LSTM && h->S < 8 ? 2 : 1;
+      for (int i = 0; i < buffers; ++i)
+        TW_TRY(make_bf16_mat(h, &h->bf.A_tiled[i], nullptr, fused_joiner_A_rows(h->R_max, h->S), h->J, true, true));
       TW_TRY(dev_alloc(h, &h->bf.lse, (size_t)h->R_max * h->S));
       TW_TRY(dev_alloc(h, &h->bf.dmax, (size_t)h->R_max * (h->bf.Vp / 16)));
-      TW_TRY(scan_select_setup());
       h->bf.fused_ok = true;
       h->bf.fused_on = true;
     }
@@ -347,7 +347,7 @@ int build_workspace(tw_handle* h) {
   TW_TRY(dev_alloc(h, &hs.new_par, nb * kMaxBeam));
   TW_TRY(dev_alloc(h, &hs.new_tok, nb * kMaxBeam));
   TW_TRY(dev_alloc(h, &hs.new_row, nb * kMaxBeam));
-  int** per_row[] = {&hs.row_b, &hs.row_e0, &hs.row_p, &hs.row_slen, &hs.pw_new, &hs.pw_par, &hs.pw_tok, &hs.pw_bi,
+  int** per_row[] = {&hs.row_e0, &hs.row_p, &hs.row_slen, &hs.pw_new, &hs.pw_par, &hs.pw_tok, &hs.pw_bi,
                      &h->stage_e0, &h->stage_slen};
   for (int** p : per_row) TW_TRY(dev_alloc(h, p, R));
   TW_TRY(dev_alloc(h, &hs.row_ld, R * S));

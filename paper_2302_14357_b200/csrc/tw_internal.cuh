@@ -143,8 +143,6 @@ struct ScanSelectArgs {
   float* lse_out;      // [R, S] softmax normalisers: log J(t, k) = z[t, k] - lse[t]
   float *ldphi, *ldnb, *la; double *ldphi_d, *la_d;
   CandOut cand;
-  const float* dnb_in = nullptr;   // when set: [R, V] delta_nb values are given and only the selection runs
-  int dnb_linear = 0;              // dnb_in holds probabilities (0 = none), candidates are returned as logs
   StepWords words = {};
 };
 bool scan_select_fits(int S, int V);   // the row's S x V logits fit in shared memory
@@ -198,7 +196,7 @@ struct HypState {
   // new hypotheses of the current step, per utterance: [B][kMaxBeam] (global slot ids)
   int *new_slot, *new_par, *new_tok, *new_row;   // new_row: joiner row of the parent
   // compacted rows of the current step: [B*N]
-  int *row_b, *row_e0, *row_p, *row_slen; float* row_ld;   // row_ld [R][S]
+  int *row_e0, *row_p, *row_slen; float* row_ld;   // row_ld [R][S]
   int *row_off, *new_off;     // [B] first row / first work-list entry of each utterance
   // compacted predictor work list: [B*N]
   int *pw_new, *pw_par, *pw_tok;
