@@ -89,6 +89,8 @@ void gemm_bf16(tw_handle* h, const Bf16Mat& A, const Bf16Mat& B, const int* M_de
   launch_gemm_bf16(A.as_A, B.as_B128, B.as_B256, p, st, &B.as_B64);
 }
 
+bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0; }
+
 // UpdatePredictorOutput for n hypotheses: one predictor step on tok[i] from the state at row
 // (idx_in ? idx_in[i] : i) of hc_in, written to row (idx_out ? idx_out[i] : i) of hc_out; the projected
 // output W_p g goes to row (idx_out ? idx_out[i] : i) of Pp_out.  State rows are [L][2][Hd].
@@ -123,7 +125,9 @@ void enqueue_predictor(tw_handle* h, const int* tok, const float* hc_in, const i
       p.m_early = l > 0;                      // the row count is older than the layer below, which runs ahead of this one
       p.lstm = LstmEpi{hc_in, idx_in, hc_out, idx_out, L, l, Hd,
                        (l + 1 < L) ? h->bf.X[l + 1].ptr : h->bf.Htop.ptr, (l + 1 < L) ? 2LL * Hd : (long long)Hd};
-      if (!launch_gemm_lstm_wide(h->bf.X[l].as_A, h->bf.X[l].as_B32, h->bf.W_cat[l].as_B64, h->bf.W_cat[l].as_B32, p, st))
+      // the one-wave kernel moves a caller's states 16 bytes at a time, the tiled one element by element where it has to
+      const bool wide = aligned16(hc_in) && aligned16(hc_out);
+      if (!wide || !launch_gemm_lstm_wide(h->bf.X[l].as_A, h->bf.X[l].as_B32, h->bf.W_cat[l].as_B64, h->bf.W_cat[l].as_B32, p, st))
         launch_gemm_bf16(h->bf.X[l].as_A, h->bf.W_cat[l].as_B128, h->bf.W_cat[l].as_B256, p, st);
     }
     if (wo) {                             // the projection forms the joiner's operand too
