@@ -89,6 +89,7 @@ gemm_bf16_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
           tma_load_2d_hint(sB + s * C::kBBytes, &tmB, &full[s], kb * BK, n0, keep);
         }
       }
+      settle_copies(ok);
     }
   } else if (warp == 1) {
     if (lane == 0) {
@@ -116,6 +117,7 @@ gemm_bf16_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
         }
         if (ok) umma_commit(&acc_full[buf]);
       }
+      settle_copies(ok);
     }
   } else {
     const int ew = warp - 2;                 // 0..7

@@ -83,8 +83,8 @@ struct tw_handle {
   int graph_B = -1, graph_T = -1, graph_fused = -1, graph_launches = 0, graph_steps = 0;
   cudaEvent_t ev_poll = nullptr;
   // side branch of a decode step: the kernel that completes the new hypotheses' frame distributions and
-  // writes the rows' row_ld runs on aux_stream beside the next pass's predictor kernels (fork after the
-  // compaction kernel, join before the joiner's operand kernel)
+  // writes the rows' row_ld runs on aux_stream beside the next pass's predictor kernels (fork after
+  // hyp_step_kernel, join before the joiner's operand kernel)
   cudaStream_t aux_stream = nullptr;
   cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
   bool aux_ok = false, aux_pending = false;
