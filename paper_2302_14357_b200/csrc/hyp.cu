@@ -26,40 +26,34 @@ __device__ __forceinline__ unsigned long long hash_push(unsigned long long h, in
   return x;
 }
 
-// Starts the next segment of utterance b: A = ChooseNBest(B), B = [], t += S, d = (s, 0, ..., 0).
-// Precondition: list A is empty and frames remain.  Called by the whole CTA.
-__device__ void turn_over(const HypState& hs, int b) {
-  __shared__ double s_ls[kMaxBeam];
-  __syncthreads();
-  const int n = hs.nTop[b];                  // read by every thread before thread 0 clears it below
+// The list a segment starts with, ChooseNBest(B) of the one before, in shared memory: slots and scores, best first
+struct CarryList { int n; int slot[kMaxBeam]; double ls[kMaxBeam]; };
+
+// Starts the next segment of utterance b, at frame t0 with slen frames: A = ChooseNBest(B) (cl), B = [], d = (s, 0, ..., 0).
+// Called by the whole CTA, with cl visible to it.
+__device__ void turn_over(const HypState& hs, int b, const CarryList& cl, int t0, int slen) {
   if (threadIdx.x < kMaxBeam) {              // one thread per carried hypothesis
     const int i = threadIdx.x;
-    if (i < n) {
-      const int e = hs.B_top[b * kMaxBeam + i];
-      const int slot = hs.B_slot[(long long)b * hs.capB + e];
-      const double ls = hs.B_ls[(long long)b * hs.capB + e];
-      hs.A_slot[b * kMaxBeam + i] = slot;
-      hs.A_ls[b * kMaxBeam + i] = ls;
+    if (i < cl.n) {
+      hs.A_slot[b * kMaxBeam + i] = cl.slot[i];
+      hs.A_ls[b * kMaxBeam + i] = cl.ls[i];
       hs.A_done[b * kMaxBeam + i] = -INFINITY;
-      hs.carry[b * kMaxBeam + i] = slot;
-      s_ls[i] = ls;
+      hs.carry[b * kMaxBeam + i] = cl.slot[i];
     } else {
       hs.carry[b * kMaxBeam + i] = -1;
     }
   }
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    const int t0 = hs.t0[b] + hs.slen[b];
+  if (threadIdx.x == 32) {
     hs.t0[b] = t0;
-    hs.slen[b] = min(hs.S, hs.len[b] - t0);
-    hs.nA[b] = n;
+    hs.slen[b] = slen;
+    hs.nA[b] = cl.n;
     hs.nB[b] = 0;
     hs.nTop[b] = 0;
     hs.iters[b] = 0;
   }
-  for (int i = threadIdx.x; i < n * hs.S; i += blockDim.x) {
+  for (int i = threadIdx.x; i < cl.n * hs.S; i += blockDim.x) {
     const int a = i / hs.S, t = i - a * hs.S;
-    hs.A_ld[((long long)b * kMaxBeam + a) * hs.S + t] = (t == 0) ? s_ls[a] : -INFINITY;
+    hs.A_ld[((long long)b * kMaxBeam + a) * hs.S + t] = (t == 0) ? cl.ls[a] : -INFINITY;
   }
 }
 
@@ -70,38 +64,57 @@ __device__ __forceinline__ int pp_row(const HypState& hs, long long gs) {
   return ln > 0 ? hs.slot_tok[gs * hs.U_cap + ln - 1] : hs.empty_row;
 }
 
-// own_rows, behind a turn_over: claims the joiner rows of the carried hypotheses and writes their tables and operand rows.
-// Called by the whole CTA.
-__device__ void carry_rows(const HypState& hs, int b) {
-  __shared__ int s_r0;
-  __syncthreads();                           // what turn_over wrote
-  const int n = hs.nA[b], sl = hs.slen[b], t0 = hs.t0[b], S = hs.S, J = hs.J, per = J >> 3;
-  if (threadIdx.x == 0) { s_r0 = atomicAdd(hs.rows_next, n); hs.row_off[b] = s_r0; }
-  __syncthreads();
-  const int r0 = s_r0;
+// Eight operand values of row e_row of E and the hypothesis in slot `slot` of utterance b, from column x on
+__device__ __forceinline__ uint4 carry_operand(const HypState& hs, int b, long long e_row, int slot, int x) {
+  const float* e = hs.E + e_row * hs.J + x;
+  const float* pp = hs.slot_Pp + ((long long)b * hs.capSlot + slot) * hs.J + x;
+  return act8(*reinterpret_cast<const float4*>(e), *reinterpret_cast<const float4*>(e + 4), *reinterpret_cast<const float4*>(pp),
+              *reinterpret_cast<const float4*>(pp + 4), hs.act);
+}
+
+// own_rows, beside a turn_over: the tables and operand rows of the carried hypotheses' joiner rows r0 .. r0 + n - 1.  Called by
+// the whole CTA.  (own_rows == 1) of the first `done` operand rows, one per (hypothesis, frame), the first kEarlyCols columns
+// have been written.
+constexpr int kEarlyCols = 1024;             // four 16-byte pieces a lane, a warp per row
+__device__ void carry_rows(const HypState& hs, int b, const CarryList& cl, int t0, int sl, int r0, int done) {
+  const int n = cl.n, S = hs.S, J = hs.J, per = J >> 3, lane = threadIdx.x & 31;
+  if (threadIdx.x == 0) hs.row_off[b] = r0;
   if (threadIdx.x < n) hs.row_slen[r0 + threadIdx.x] = sl;
   if (hs.own_rows == 2 && threadIdx.x < n) {
     hs.row_e0[r0 + threadIdx.x] = b * hs.E_T + t0;
-    hs.row_p[r0 + threadIdx.x] = pp_row(hs, (long long)b * hs.capSlot + hs.A_slot[b * kMaxBeam + threadIdx.x]);
+    hs.row_p[r0 + threadIdx.x] = pp_row(hs, (long long)b * hs.capSlot + cl.slot[threadIdx.x]);
   }
   for (int i = threadIdx.x; i < n * S; i += blockDim.x) hs.row_ld[(long long)r0 * S + i] = (i % S) == 0 ? 0.f : -INFINITY;   // all mass on the first frame
   if (hs.own_rows == 2) return;
-  for (int c = threadIdx.x; c < n * sl * per; c += blockDim.x) {
-    const int pair = c / per, x = (c - pair * per) * 8, hh = pair / sl, t = pair - hh * sl;
-    const float* e = hs.E + ((long long)b * hs.E_T + t0 + t) * J + x;
-    const float* pp = hs.slot_Pp + ((long long)b * hs.capSlot + hs.A_slot[b * kMaxBeam + hh]) * J + x;
-    *reinterpret_cast<uint4*>(static_cast<__nv_bfloat16*>(hs.A_next) + operand_row(r0 + hh, t, S) * J + x) =
-        act8(*reinterpret_cast<const float4*>(e), *reinterpret_cast<const float4*>(e + 4), *reinterpret_cast<const float4*>(pp),
-             *reinterpret_cast<const float4*>(pp + 4), hs.act);
-  }
-  // padding frames of a short segment: zeros, whatever an older pass left there (see pred_out.cu)
-  if (__builtin_expect(sl < S, 0)) {
 #pragma unroll 1
-    for (int c = threadIdx.x; c < n * (S - sl) * per; c += blockDim.x) {
-      const int pair = c / per, x = (c - pair * per) * 8, hh = pair / (S - sl), t = sl + pair - hh * (S - sl);
-      *reinterpret_cast<uint4*>(static_cast<__nv_bfloat16*>(hs.A_next) + operand_row(r0 + hh, t, S) * J + x) = make_uint4(0, 0, 0, 0);
-    }
+  for (int pair = threadIdx.x >> 5; pair < n * S; pair += blockDim.x >> 5) {
+    const int hh = pair / S, t = pair - hh * S, first = pair < done ? kEarlyCols / 8 : 0;
+    __nv_bfloat16* dst = static_cast<__nv_bfloat16*>(hs.A_next) + operand_row(r0 + hh, t, S) * J;
+    // (padding frames of a short segment: zeros, whatever an older pass left there, see pred_out.cu)
+#pragma unroll 1
+    for (int c = first + lane; c < per; c += 32)
+      *reinterpret_cast<uint4*>(dst + c * 8) = t < sl ? carry_operand(hs, b, (long long)b * hs.E_T + t0 + t, cl.slot[hh], c * 8) : make_uint4(0, 0, 0, 0);
   }
+}
+
+// turn_over of an utterance whose list A is empty and that has frames left, from the lists in memory.  Called by the whole CTA.
+__device__ void next_segment(const HypState& hs, int b) {
+  __shared__ CarryList s_cl;
+  __shared__ int s_r0;
+  __syncthreads();
+  const int n = hs.nTop[b], t0 = hs.t0[b] + hs.slen[b], slen = min(hs.S, hs.len[b] - t0);
+  if (threadIdx.x < n) {
+    const int e = hs.B_top[b * kMaxBeam + threadIdx.x];
+    s_cl.slot[threadIdx.x] = hs.B_slot[(long long)b * hs.capB + e];
+    s_cl.ls[threadIdx.x] = hs.B_ls[(long long)b * hs.capB + e];
+  }
+  if (threadIdx.x == 0) {
+    s_cl.n = n;
+    if (hs.own_rows) s_r0 = atomicAdd(hs.rows_next, n);
+  }
+  __syncthreads();
+  turn_over(hs, b, s_cl, t0, slen);
+  if (hs.own_rows) carry_rows(hs, b, s_cl, t0, slen, s_r0, 0);
 }
 
 __global__ void __launch_bounds__(kThreads) hyp_init_kernel(HypState hs, const int* lengths, int T) {
@@ -128,14 +141,12 @@ __global__ void __launch_bounds__(kThreads) hyp_init_kernel(HypState hs, const i
     for (int i = threadIdx.x; i < hs.J; i += blockDim.x) hs.slot_Pp[gs * hs.J + i] = hs.init_Pp[i];
   }
   __syncthreads();
-  if (hs.len[b] > 0) {
-    turn_over(hs, b);
-    if (hs.own_rows) carry_rows(hs, b);
-  }
+  if (hs.len[b] > 0) next_segment(hs, b);
 }
 
 constexpr int kStepThreads = 512;   // 16 warps: one per hypothesis of list A
 constexpr int kSelCap = 64;         // survivors of a row's bound that are ranked directly
+constexpr int kKeyPitch = kMaxBeam + 1;   // rows of the candidate keys start in different banks
 
 __device__ __forceinline__ bool tok_better(float v1, int k1, float v2, int k2) { return v1 > v2 || (v1 == v2 && k1 < k2); }
 
@@ -146,33 +157,47 @@ __device__ __forceinline__ unsigned long long order_key(double x) {
   return (u >> 63) ? ~u : (u | 0x8000000000000000ull);
 }
 
+// The kernel is a chain of short phases, each as long as its slowest dependent accesses; it is organised to have few of them
+// behind the wait for the joiner kernel:
+//   ahead of the wait   lists A and B's best entries into shared memory, the search of list B, which of B's best entries are
+//                       merged into, the free slots of the ring
+//   1                   warp 0: the blank expansions into list B and the threshold (ChooseNthScore); warp 16 + h: the N best
+//                       tokens of row h
+//   2                   N best expansions (four threads a candidate) and the filter; the number kept comes with the barrier
+//   3                   work-list entries and rows claimed (atomics); beside that the new hypotheses' tokens, log J of the kept
+//                       expansions and the parents' h - or, with nothing kept, the next segment's list and operand rows
+//   4                   what goes to the claimed places
 // tok_cap: capacity (tokens) of the dynamic shared memory's [N] token sequences of list A's hypotheses, 0: they stay in
 // global memory.  Every new hypothesis is a child of one of these, whose tokens the search below reads anyway.
 constexpr int kTokStageMax = 24 * 1024;
 __global__ void __launch_bounds__(2 * kStepThreads) hyp_step_kernel(HypState hs, int tok_cap) {
   extern __shared__ int s_tok[];
-  __shared__ int s_hasthr, s_nkeep, s_wbase, s_rbase;
-  __shared__ int s_found[kMaxBeam], s_touched[kMaxBeam], s_carry[kMaxBeam];
-  __shared__ double s_Als[kMaxBeam], s_Adone[kMaxBeam];
+  __shared__ int s_found[kMaxBeam], s_fslot[kMaxBeam];   // the entry of list B that a hypothesis merges with (-1: none), its slot
+  __shared__ double s_Bls[kMaxBeam];                     // and score
+  __shared__ double s_Als[kMaxBeam];
   __shared__ int s_Aslot[kMaxBeam], s_Alen[kMaxBeam];
   __shared__ unsigned long long s_Ahash[kMaxBeam];
-  __shared__ double s_Bls[kMaxBeam];          // score of the entry of list B that a hypothesis merges with
+  __shared__ long long s_orow[kMaxBeam];                 // operand row of a hypothesis's first frame (own_rows == 1)
+  __shared__ int s_iters, s_nT0, s_Btop[kMaxBeam], s_Btopslot[kMaxBeam];   // list B's best entries as the previous pass left them
+  __shared__ double s_Btopls[kMaxBeam];
+  __shared__ int s_free[32];                             // the next free slots of the ring
+  __shared__ __align__(16) ulonglong2 s_ent[32];         // (key, index) of the entries that B's new best ones are chosen from
+  __shared__ CarryList s_cl;                             // B's new best entries
+  __shared__ int s_nB, s_hasthr, s_bad, s_nkeep, s_wbase, s_rbase;
   __shared__ double s_thr;
   __shared__ int s_ck[kMaxBeam * kMaxBeam];
   __shared__ double s_abs[kMaxBeam * kMaxBeam];
-  __shared__ unsigned long long s_key[kMaxBeam * kMaxBeam];
-  __shared__ unsigned long long s_nkey[32];
-  __shared__ int s_nidx[32];
-  __shared__ float s_lm[kMaxBeam][32], s_sv[kMaxBeam][kSelCap];   // in-kernel selection: lane maxima, survivors of a row
-  __shared__ int s_sk[kMaxBeam][kSelCap], s_cnt[kMaxBeam];
-  __shared__ int s_cursor, s_iters, s_nT0, s_Btop[kMaxBeam];     // per-utterance state fetched up front
-  __shared__ double s_Btopls[kMaxBeam], s_tval[kMaxBeam];         // scores of B's old best / of the entries touched now
-  __shared__ int s_sel[kMaxBeam];
-  __shared__ int s_keep_h[kMaxBeam], s_keep_k[kMaxBeam], s_keep_slot[kMaxBeam];
+  __shared__ unsigned long long s_key[kMaxBeam * kKeyPitch];
+  __shared__ __align__(16) float s_lm[kMaxBeam][32];     // in-kernel selection: lane maxima, survivors of a row, its chunks to look at
+  __shared__ float2 s_sv[kMaxBeam][kSelCap];
+  __shared__ unsigned char s_chunk[kMaxBeam][128];
+  __shared__ int s_cnt[kMaxBeam];
+  __shared__ int s_keep_h[kMaxBeam], s_keep_k[kMaxBeam];
   __shared__ double s_keep_ls[kMaxBeam];
+  __shared__ float s_rel[kMaxBeam * 8];                  // own_rows == 1 (S < 8): frame distributions relative to the scores
 
   const int b = blockIdx.x;
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nwarps = blockDim.x >> 5;
   // The lists and counters read below were written by the previous pass's kernels, all of which had finished before
   // the joiner kernel that runs ahead of this one began (and that kernel writes none of them): they are fetched
   // before the wait for it, under its tail.  Every first-round load is issued before the early exit, so that none
@@ -181,43 +206,56 @@ __global__ void __launch_bounds__(2 * kStepThreads) hyp_step_kernel(HypState hs,
   const int r0 = hs.row_off[b];
   const int slen = hs.slen[b];
   const int nB0 = hs.nB[b];
-  double ld_Als = 0.0, ld_Adone = -INFINITY;
-  int ld_Aslot = 0, ld_carry = -1;
-  if (tid < kMaxBeam) {                     // all kMaxBeam entries of the lists; those past H are never used
-    ld_Als = hs.A_ls[b * kMaxBeam + tid]; ld_Aslot = hs.A_slot[b * kMaxBeam + tid];
-    if (hs.mono) ld_Adone = hs.A_done[b * kMaxBeam + tid];
-    ld_carry = hs.carry[b * kMaxBeam + tid];
-  }
+  const int t0 = hs.t0[b], len = hs.len[b];
   const long long bB = (long long)b * hs.capB;
   const long long bS = (long long)b * hs.capSlot;
   // the search of list B (warp h looks for hypothesis h's tokens): its own slot and the first 32 entries of the list are
   // asked for now as well; the slot's hash and length follow as soon as the slot is there, still before the barriers
   int my_slot = 0, pre_len = -1, pre_slot = 0;
   unsigned long long pre_hash = 0;
-  if (warp < kMaxBeam) {
+  double my_ls = 0.0;
+  if (warp < kMaxBeam) {                    // all kMaxBeam entries of the lists; those past H are never used
     my_slot = hs.A_slot[b * kMaxBeam + warp];
+    my_ls = hs.A_ls[b * kMaxBeam + warp];
     if (lane < hs.capB) { pre_hash = hs.B_hash[bB + lane]; pre_len = hs.B_len[bB + lane]; pre_slot = hs.B_slot[bB + lane]; }
   }
-  unsigned long long my_hash = 0;
-  int my_len = 0;
-  if (warp < H) { my_hash = hs.slot_hash[bS + my_slot]; my_len = hs.slot_len[bS + my_slot]; }
-  if (warp == 15 && H > 0) {
+  const int N = hs.N, S = hs.S, V = hs.V;
+  const bool two_halves = hs.dnb_sel != nullptr;     // with in-kernel selection: 32 warps, the upper half selects
+  if (H == 0) {                              // idle (finished) utterance
+    pdl_wait();
+    pdl_trigger();
+    return;
+  }
+  if (warp == 15) {
     // ring cursor, pass counter and the best-N set of list B as the previous pass left it, by a warp that mostly has
     // nothing to do in the search
-    const int nT = hs.nTop[b];
-    if (lane == 0) { s_cursor = hs.cursor[b]; s_iters = hs.iters[b]; s_nT0 = nT; }
-    if (lane < kMaxBeam) {
+    const int nT = hs.nTop[b], cursor = hs.cursor[b], iters = hs.iters[b];
+    const int carry = lane < kMaxBeam ? hs.carry[b * kMaxBeam + lane] : -1;
+    if (lane < nT) {
       const int bt = hs.B_top[b * kMaxBeam + lane];
       s_Btop[lane] = bt;
-      if (lane < nT) s_Btopls[lane] = hs.B_ls[bB + bt];       // before this pass's merges; touched entries are patched below
+      s_Btopls[lane] = hs.B_ls[bB + bt];                      // before this pass's merges
+      s_Btopslot[lane] = hs.B_slot[bB + bt];
     }
+    // The ring's slots after the cursor; those still held by hypotheses carried into this segment are skipped.  At most
+    // N of them are, and at most N are wanted: 32 slots hold enough (a ring that is shorter starts over).
+    const int slot = (cursor + 1 + lane) % hs.capSlot;
+    bool busy = false;
+#pragma unroll 4
+    for (int q = 0; q < kMaxBeam; ++q) busy |= __shfl_sync(0xffffffffu, carry, q) == slot;
+    const unsigned free_mask = __ballot_sync(0xffffffffu, !busy);
+    if (!busy) s_free[__popc(free_mask & ((1u << lane) - 1u))] = slot;
+    if (lane == 0) { s_iters = iters; s_nT0 = nT; s_bad = 0; }
   }
+  if (tid < kMaxBeam && hs.own_rows == 1) s_orow[tid] = operand_row(r0 + tid, 0, S);
   // ---- AddAndMerge, search: warp h looks for the tokens of A_h among the entries already in B.  It needs the lists only,
   // so it runs ahead of the wait.  (Entries of A are distinct sequences, so two of them never merge with each other.)
-  if (warp < H) {
+  if (warp < H) {                            // (H <= kMaxBeam)
+    const unsigned long long my_hash = hs.slot_hash[bS + my_slot];
+    const int my_len = hs.slot_len[bS + my_slot];
     const int* ta = hs.slot_tok + (bS + my_slot) * hs.U_cap;
     if (tok_cap > 0) for (int i = lane; i < my_len; i += 32) s_tok[warp * tok_cap + i] = ta[i];
-    int found = -1;
+    int found = -1, fslot = my_slot;
     for (int base = 0; base < nB0 && found < 0; base += 32) {
       const int e = base + lane;
       const bool match = e < nB0 && (base == 0 ? (pre_hash == my_hash && pre_len == my_len)
@@ -232,49 +270,100 @@ __global__ void __launch_bounds__(2 * kStepThreads) hyp_step_kernel(HypState hs,
           const int* tb = hs.slot_tok + (bS + oslot) * hs.U_cap;
           for (int i = lane; i < my_len; i += 32) diff |= (ta[i] != tb[i]);
         }
-        if (!__any_sync(0xffffffffu, diff)) found = c;
+        if (!__any_sync(0xffffffffu, diff)) { found = c; fslot = oslot; }
       }
     }
     if (lane == 0) {
-      s_found[warp] = found; s_Alen[warp] = my_len; s_Ahash[warp] = my_hash;
+      s_found[warp] = found; s_fslot[warp] = fslot; s_Alen[warp] = my_len; s_Ahash[warp] = my_hash;
       s_Bls[warp] = found >= 0 ? hs.B_ls[bB + found] : 0.0;
     }
   }
-  if (tid < kMaxBeam) { s_Als[tid] = ld_Als; s_Aslot[tid] = ld_Aslot; s_Adone[tid] = ld_Adone; s_carry[tid] = ld_carry; }
+  if (warp < kMaxBeam && lane == 0) { s_Als[warp] = my_ls; s_Aslot[warp] = my_slot; }
+  __syncthreads();
+
+  // ---- warp 0, still ahead of the wait: lanes 0 .. 15 hold B's old best entries, lane 16 + h the entry that hypothesis h
+  // goes to.  m_src: the lane of the hypothesis that is merged into this old best entry.
+  int idx = -1, m_src = -1, m_slot = 0;
+  bool m_old = false, m_dup = false;
+  double score = -INFINITY, done = -INFINITY;
+  if (warp == 0) {
+    const int nT = s_nT0, h = lane - 16;
+    const int f = h >= 0 && h < H ? s_found[h] : 0;
+    const unsigned appended = __ballot_sync(0xffffffffu, f < 0);
+    if (lane == 0) s_nB = nB0 + __popc(appended);      // capB = N * I_max bounds this by construction
+    if (h < 0) {
+      if (lane < nT) {
+        idx = s_Btop[lane]; score = s_Btopls[lane]; m_slot = s_Btopslot[lane];
+#pragma unroll 4
+        for (int q = 0; q < H; ++q) if (s_found[q] == idx) m_src = 16 + q;
+      }
+    } else if (h < H) {
+      m_old = f >= 0;
+      idx = m_old ? f : nB0 + __popc(appended & ((1u << lane) - 1u));
+      m_slot = s_fslot[h];
+      if (hs.mono) done = hs.A_done[b * kMaxBeam + h];
+#pragma unroll 4
+      for (int i = 0; i < nT; ++i) m_dup |= s_Btop[i] == f;
+    }
+  }
   pdl_wait();                               // from here on: what the joiner kernel wrote (delta_phi, delta_nb, occupancies)
   pdl_trigger();
-  if (H == 0) return;                       // idle (finished) utterance
-  const int N = hs.N, S = hs.S, V = hs.V;
 
-  double dphi = 0.0;
-  if (tid < H) dphi = hs.ldphi_d ? hs.ldphi_d[r0 + tid] : (double)hs.ldphi[r0 + tid];
-  if (tid < kMaxBeam) s_sel[tid] = -1;
-  if (tid == 0) {
-    hs.calls[b] += 1; hs.joins[b] += slen;
+  if (warp == 0) {
+    // ---- AddAndMerge, apply: sum into the matching entry or append (appends keep the order of A)
+    const int h = lane - 16;
+    if (h >= 0 && h < H) {
+      const double dphi = hs.ldphi_d ? hs.ldphi_d[r0 + h] : (double)hs.ldphi[r0 + h];
+      double val = s_Als[h] + dphi;
+      if (hs.mono) val = logaddexp_d(val, done);       // plus what had already left the segment (else log 0)
+      if (m_old) {
+        val = logaddexp_d(s_Bls[h], val);              // (two hypotheses never merge with the same entry)
+      } else {
+        hs.B_slot[bB + idx] = s_Aslot[h];
+        hs.B_hash[bB + idx] = s_Ahash[h]; hs.B_len[bB + idx] = s_Alen[h];
+      }
+      hs.B_ls[bB + idx] = val;
+      score = val;
+    }
+    // ---- ChooseNthScore: the best N of B are among the previous best N and the entries touched now
+    const double merged = __shfl_sync(0xffffffffu, score, m_src & 31);
+    if (m_src >= 0) score = merged;
+    if (m_dup) idx = -1;                     // it stands among the old best entries
+    const unsigned long long key = order_key(score);
+    s_ent[lane] = make_ulonglong2(key, (unsigned long long)(long long)idx);
+    const int count = __popc(__ballot_sync(0xffffffffu, idx >= 0));
+    __syncwarp();
+    int rank = 0;
+#pragma unroll 8
+    for (int j = 0; j < 32; ++j) {          // all lanes read the same words: broadcasts, independent of each other
+      const ulonglong2 o = s_ent[j];
+      const int oi = (int)o.y;
+      rank += (oi >= 0 && (o.x > key || (o.x == key && oi < idx))) ? 1 : 0;
+    }
+    if (idx >= 0 && rank < N) {
+      hs.B_top[b * kMaxBeam + rank] = idx;
+      s_cl.slot[rank] = m_slot; s_cl.ls[rank] = score;
+      if (rank == N - 1) s_thr = score;
+    }
+    if (lane == 0) { s_cl.n = min(N, count); s_hasthr = count >= N; }
+  } else if (warp == 1 && lane == 0) {
+    atomicAdd(&hs.calls[b], 1);              // (nobody else writes these: additions without a round trip)
+    atomicAdd(&hs.joins[b], slen);
     if (hs.own_rows) {                      // totals of the pass
       atomicAdd(reinterpret_cast<unsigned long long*>(hs.rows_total), (unsigned long long)H);
       atomicAdd(reinterpret_cast<unsigned long long*>(hs.rows_total) + 1, (unsigned long long)(H * slen));
     }
   }
-  // With in-kernel selection the CTA has 32 warps: warps 16..31 select (one row each) while warps 0..15 merge the
-  // blank expansions into list B and find the threshold; the two halves meet at the barrier before the ranking.
-  // Until then the merging half synchronises on a named barrier of its own.
-  const bool two_halves = hs.dnb_sel != nullptr;
-  auto sync_merge = [&]() {
-    if (two_halves) asm volatile("bar.sync 1, 512;" ::: "memory");
-    else __syncthreads();
-  };
   if (two_halves && warp >= 16) {
     // ---- ChooseNBestExpansions, first stage, for the row of hypothesis warp - 16: its N best tokens by delta_nb,
     // order (value desc, token asc), straight into the candidate table of the second stage.
     const int h = warp - 16;
     if (lane < kMaxBeam) {
-      s_abs[h * kMaxBeam + lane] = -INFINITY; s_ck[h * kMaxBeam + lane] = -1; s_key[h * kMaxBeam + lane] = order_key(-INFINITY);
+      s_abs[h * kMaxBeam + lane] = -INFINITY; s_ck[h * kMaxBeam + lane] = -1; s_key[h * kKeyPitch + lane] = order_key(-INFINITY);
     }
-    __syncwarp();
     if (h < H) {
       const float* src = hs.dnb_sel + (long long)(r0 + h) * V;
-      const double base = hs.A_ls[b * kMaxBeam + h];
+      const double base = s_Als[h];
       // a lower bound of the N-th best value: the N-th largest of the 32 lane maxima (distinct elements)
       const int nchunk = V >> 5;
       const bool pairs = hs.dnb_chunk == 16;     // maxima of 16 columns: two make a chunk's
@@ -302,8 +391,14 @@ __global__ void __launch_bounds__(2 * kStepThreads) hyp_step_kernel(HypState hs,
       if (lane == 0) s_cnt[h] = 0;
       __syncwarp();
       int lrank = 0;
-#pragma unroll
-      for (int j = 0; j < 32; ++j) { const float o = s_lm[h][j]; lrank += (o > lmax || (o == lmax && j < lane)) ? 1 : 0; }
+#pragma unroll 2
+      for (int j = 0; j < 32; j += 4) {
+        const float4 o = *reinterpret_cast<const float4*>(&s_lm[h][j]);
+        lrank += (o.x > lmax || (o.x == lmax && j < lane)) ? 1 : 0;
+        lrank += (o.y > lmax || (o.y == lmax && j + 1 < lane)) ? 1 : 0;
+        lrank += (o.z > lmax || (o.z == lmax && j + 2 < lane)) ? 1 : 0;
+        lrank += (o.w > lmax || (o.w == lmax && j + 3 < lane)) ? 1 : 0;
+      }
       const unsigned who = __ballot_sync(0xffffffffu, lrank == N - 1);        // exactly one lane: the ranks are 0..31
       const float bound = __shfl_sync(0xffffffffu, lmax, __ffs(who) - 1);
       auto push4 = [&](const float4& v4, int k) {
@@ -312,38 +407,38 @@ __global__ void __launch_bounds__(2 * kStepThreads) hyp_step_kernel(HypState hs,
         for (int c = 0; c < 4; ++c) {
           if (vv[c] >= bound && vv[c] > 0.f) {
             const int i = atomicAdd(&s_cnt[h], 1);
-            if (i < kSelCap) { s_sv[h][i] = vv[c]; s_sk[h][i] = k + c; }
+            if (i < kSelCap) s_sv[h][i] = make_float2(vv[c], __int_as_float(k + c));
           }
         }
       };
       if (cmax != nullptr) {
-        // Only the chunks whose maximum reaches the bound can hold a survivor: a few 128-byte pieces of the row.  The
-        // warp takes them together, a lane per element and up to eight chunks per round, so that their loads (mostly
-        // from DRAM: a step moves more than L2 holds) are in flight at the same time.
-        unsigned qm[4];
+        // Only the chunks whose maximum reaches the bound can hold a survivor: a few 128-byte pieces of the row, N or some
+        // more of them.  They are listed, and the warp takes sixteen at a time, eight lanes to a piece, so that their loads
+        // (mostly from DRAM: a large step moves more than L2 holds) are in flight at the same time.
+        int total = 0;
 #pragma unroll
-        for (int u = 0; u < 4; ++u) qm[u] = __ballot_sync(0xffffffffu, m4[u] >= bound && m4[u] > 0.f);
-        int u = 0;
-        unsigned m = qm[0];
-        for (;;) {
-          int ids[8];
-          int n = 0;
+        for (int u = 0; u < 4; ++u) {
+          const bool in = m4[u] >= bound && m4[u] > 0.f;
+          const unsigned m = __ballot_sync(0xffffffffu, in);
+          if (in) s_chunk[h][total + __popc(m & ((1u << lane) - 1u))] = (unsigned char)(lane + 32 * u);
+          total += __popc(m);
+        }
+        __syncwarp();
+        const int k0 = (lane & 7) * 4;
+#pragma unroll 1
+        for (int c0 = lane >> 3; c0 - (lane >> 3) < total; c0 += 16) {
+          float4 v[4];
+          int id[4];
 #pragma unroll
-          for (int x = 0; x < 8; ++x) {
-            while (m == 0u && u < 3) { ++u; m = (u == 1) ? qm[1] : (u == 2 ? qm[2] : qm[3]); }
-            ids[x] = -1;
-            if (m != 0u) { ids[x] = (__ffs(m) - 1) + 32 * u; m &= m - 1; ++n; }
+          for (int x = 0; x < 4; ++x) {
+            const bool in = c0 + 4 * x < total;
+            id[x] = in ? (int)s_chunk[h][c0 + 4 * x] * 32 + k0 : 0;
+            v[x] = in ? __ldg(reinterpret_cast<const float4*>(src + id[x])) : make_float4(0.f, 0.f, 0.f, 0.f);
           }
-          if (n == 0) break;
-          float v[8];
 #pragma unroll
-          for (int x = 0; x < 8; ++x) v[x] = ids[x] >= 0 ? __ldg(src + ids[x] * 32 + lane) : 0.f;
-#pragma unroll
-          for (int x = 0; x < 8; ++x) {
-            if (v[x] >= bound && v[x] > 0.f) {
-              const int i = atomicAdd(&s_cnt[h], 1);
-              if (i < kSelCap) { s_sv[h][i] = v[x]; s_sk[h][i] = ids[x] * 32 + lane; }
-            }
+          for (int x = 0; x < 4; ++x) {
+            const float g = fmaxf(fmaxf(v[x].x, v[x].y), fmaxf(v[x].z, v[x].w));
+            if (g >= bound && g > 0.f) push4(v[x], id[x]);
           }
         }
       } else {
@@ -367,12 +462,14 @@ __global__ void __launch_bounds__(2 * kStepThreads) hyp_step_kernel(HypState hs,
       const int ns = s_cnt[h];
       if (ns <= kSelCap) {
         for (int i = lane; i < ns; i += 32) {
-          const float v = s_sv[h][i]; const int k = s_sk[h][i];
+          const float2 me = s_sv[h][i];
+          const float v = me.x; const int k = __float_as_int(me.y);
           int rank = 0;
-          for (int j = 0; j < ns; ++j) rank += tok_better(s_sv[h][j], s_sk[h][j], v, k) ? 1 : 0;
+#pragma unroll 4
+          for (int j = 0; j < ns; ++j) { const float2 o = s_sv[h][j]; rank += tok_better(o.x, __float_as_int(o.y), v, k) ? 1 : 0; }
           if (rank < N) {
             const double sc = base + (double)__logf(v);
-            s_abs[h * kMaxBeam + rank] = sc; s_ck[h * kMaxBeam + rank] = k; s_key[h * kMaxBeam + rank] = order_key(sc);
+            s_abs[h * kMaxBeam + rank] = sc; s_ck[h * kMaxBeam + rank] = k; s_key[h * kKeyPitch + rank] = order_key(sc);
           }
         }
       } else {
@@ -398,7 +495,7 @@ __global__ void __launch_bounds__(2 * kStepThreads) hyp_step_kernel(HypState hs,
           if (!(bv > 0.f)) break;
           if (lane == 0) {
             const double sc = base + (double)__logf(bv);
-            s_abs[h * kMaxBeam + j] = sc; s_ck[h * kMaxBeam + j] = bk; s_key[h * kMaxBeam + j] = order_key(sc);
+            s_abs[h * kMaxBeam + j] = sc; s_ck[h * kMaxBeam + j] = bk; s_key[h * kKeyPitch + j] = order_key(sc);
           }
           pv = bv; pk = bk;
         }
@@ -407,146 +504,134 @@ __global__ void __launch_bounds__(2 * kStepThreads) hyp_step_kernel(HypState hs,
   }
   if (!two_halves && tid >= kMaxBeam * kMaxBeam) {      // the rows' candidate lists, by the warps that merge nothing
     const int c = tid - kMaxBeam * kMaxBeam, h = c / kMaxBeam, j = c % kMaxBeam;
-    const bool valid = h < H && j < hs.cand_n[r0 + h];
-    s_abs[c] = valid ? hs.A_ls[b * kMaxBeam + h] + (double)hs.cand_v[(long long)(r0 + h) * kMaxBeam + j] : -INFINITY;
-    s_ck[c] = valid ? hs.cand_k[(long long)(r0 + h) * kMaxBeam + j] : -1;
-    s_key[c] = order_key(s_abs[c]);
-  }
-  if (warp < 16) sync_merge();
-  // ---- AddAndMerge, apply: sum into the matching entry or append (appends keep the order of A)
-  if (tid < H) {
-    const int h = tid;
-    const int slot = s_Aslot[h];
-    double val = s_Als[h] + dphi;
-    val = logaddexp_d(val, s_Adone[h]);       // monotonic: plus what had already left the segment (else log 0)
-    int e = s_found[h];
-    if (e >= 0) {
-      val = logaddexp_d(s_Bls[h], val);       // (two hypotheses never merge with the same entry)
-      hs.B_ls[bB + e] = val;
-    } else {
-      e = nB0;                              // capB = N * I_max bounds this by construction
-      for (int q = 0; q < h; ++q) e += (s_found[q] < 0);
-      hs.B_slot[bB + e] = slot; hs.B_ls[bB + e] = val;
-      hs.B_hash[bB + e] = s_Ahash[h]; hs.B_len[bB + e] = s_Alen[h];
+    int n = 0, k = -1;
+    float v = 0.f;
+    if (h < H) {
+      const long long at = (long long)(r0 + h) * kMaxBeam + j;
+      n = hs.cand_n[r0 + h]; v = hs.cand_v[at]; k = hs.cand_k[at];
     }
-    s_touched[h] = e;
-    s_tval[h] = val;
+    const double sc = j < n ? s_Als[h] + (double)v : -INFINITY;
+    s_abs[c] = sc;
+    s_ck[c] = j < n ? k : -1;
+    s_key[h * kKeyPitch + j] = order_key(sc);
   }
-  if (tid == 0) {
-    int nB = nB0;
-    for (int q = 0; q < H; ++q) nB += (s_found[q] < 0);
-    hs.nB[b] = nB;
-  }
-  if (warp < 16) sync_merge();
+  __syncthreads();
 
-  // ---- ChooseNthScore: the best N of B are among the previous best N and the entries touched now
-  if (warp == 0) {
-    const int nT = s_nT0;
-    int idx = -1;
-    double score = -INFINITY;
-    if (lane < nT) {
-      idx = s_Btop[lane];
-      score = s_Btopls[lane];
-      for (int q = 0; q < H; ++q) if (s_touched[q] == idx) score = s_tval[q];   // merged into in this pass
-    } else if (lane - nT < H) {
-      const int cand = s_touched[lane - nT];
-      bool dup = false;
-      for (int i = 0; i < nT; ++i) dup |= (s_Btop[i] == cand);
-      if (!dup) { idx = cand; score = s_tval[lane - nT]; }
-    }
-    const unsigned long long key = order_key(score);
-    s_nkey[lane] = key; s_nidx[lane] = idx;
-    __syncwarp();
-    int rank = 0;
-#pragma unroll
-    for (int j = 0; j < 32; ++j) {          // all lanes read the same word: broadcasts, independent of each other
-      const unsigned long long kj = s_nkey[j];
-      const int ij = s_nidx[j];
-      rank += (ij >= 0 && (kj > key || (kj == key && ij < idx))) ? 1 : 0;
-    }
-    const int count = __popc(__ballot_sync(0xffffffffu, idx >= 0));
-    __syncwarp();
-    if (idx >= 0 && rank < N) hs.B_top[b * kMaxBeam + rank] = idx;
-    if (idx >= 0 && rank == N - 1) s_thr = score;
-    if (lane == 0) { hs.nTop[b] = min(N, count); s_hasthr = (count >= N); }
-  }
   // ---- ChooseNBestExpansions, second stage: the N best (h, k) over the rows' candidate lists, in
   // float64; order (score desc, h asc, k asc).  The lists are sorted by (score desc, k asc).
-  __syncthreads();
-  if (tid < kMaxBeam * kMaxBeam && s_ck[tid] >= 0) {
-    const unsigned long long mine = s_key[tid];
-    const int h = tid / kMaxBeam, jj = tid % kMaxBeam;
-    // Rank = how many candidates come before this one in the order (score desc, h asc, k asc).  Every row's list is
-    // sorted that way and padded with the key of log 0, so the candidates of a row that come before this one are a
-    // prefix of its list: its length is found by bisection (four probes and a last one for a full list) instead of
-    // a look at all sixteen entries.  Rows before h count their ties with this score, rows after it do not, and in
-    // its own row exactly the jj entries ahead of it count.
-    int rank = jj;
-    for (int hh = 0; hh < H; ++hh) {
-      if (hh == h) continue;
-      const unsigned long long* key = s_key + hh * kMaxBeam;
-      const bool ties = hh < h;
-      int cnt = 0;
-#pragma unroll
-      for (int st = kMaxBeam / 2; st > 0; st >>= 1) {
-        const unsigned long long so = key[cnt + st - 1];
-        if (so > mine || (ties && so == mine)) cnt += st;
-      }
-      if (cnt == kMaxBeam - 1) { const unsigned long long so = key[cnt]; cnt += (so > mine || (ties && so == mine)) ? 1 : 0; }
-      rank += cnt;
-    }
-    if (rank < N) s_sel[rank] = tid;
-  }
-  __syncthreads();
+  // Rank = how many candidates come before this one in that order.  Every row's list is sorted and padded with the key of
+  // log 0, so the candidates of a row that come before this one are a prefix of its list: its length is found by bisection.
+  // Rows before h count their ties with this score, rows after it do not, and in its own row exactly the jj entries ahead of it
+  // count.  A candidate has 4 threads (2 in a CTA of 512), each with every fourth (second) row, four bisections at a time.
   const bool hasthr = s_hasthr != 0;
-  const double thr = hasthr ? s_thr : -INFINITY;
-
-  // ---- filter against the threshold, allocate slots: lane i of warp 0 takes the i-th best expansion
-  if (warp == 0) {
-    const int c = lane < N ? s_sel[lane] : -1;
-    const int h = c >= 0 ? c / kMaxBeam : 0;
-    const double sc = c >= 0 ? s_abs[c] : -INFINITY;
-    const bool pass = c >= 0 && (!hasthr || sc > thr);      // Length(B) < N or delta_nb > threshold
-    const bool capped = s_iters + 1 >= hs.I_max;
-    const bool fits = s_Alen[h] + 1 <= hs.U_cap;
-    const bool keep = pass && !capped && fits;
-    const unsigned passm = __ballot_sync(0xffffffffu, pass), keepm = __ballot_sync(0xffffffffu, keep);
-    const int nk = __popc(keepm), m = __popc(keepm & ((1u << lane) - 1u));
-    if (keep) {
-      // the (m + 1)-th free slot of the ring after the cursor: slots still held by hypotheses carried into
-      // this segment are skipped
-      int cur = s_cursor, need = m + 1;
-      while (need > 0) {
-        cur = (cur + 1 == hs.capSlot) ? 0 : cur + 1;
-        bool busy = false;
+  bool kept = false;
+  {
+    const int tpc = (int)blockDim.x / (kMaxBeam * kMaxBeam), c = tid / tpc, part = tid % tpc, h = c / kMaxBeam, jj = c % kMaxBeam;
+    int rank = 0;
+    if (s_ck[c] >= 0) {
+      const unsigned long long mine = s_key[h * kKeyPitch + jj];
+#pragma unroll 1
+      for (int hb = part; hb < H; hb += 4 * tpc) {
+        int cnt[4] = {0, 0, 0, 0};
+        int st = kMaxBeam / 2;
+#pragma unroll 1
+        for (int step = 0; step < 5; ++step) {               // 8, 4, 2, 1, and 1 for a full list
 #pragma unroll
-        for (int q = 0; q < kMaxBeam; ++q) busy |= (s_carry[q] == cur);
-        if (!busy) --need;
+          for (int u = 0; u < 4; ++u) {
+            const int hh = min(hb + u * tpc, H - 1);
+            const unsigned long long so = s_key[hh * kKeyPitch + cnt[u] + st - 1];
+            if (so > mine || (hh < h && so == mine)) cnt[u] += st;
+          }
+          st = max(st >> 1, 1);
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u) { const int hh = hb + u * tpc; if (hh < H) rank += hh == h ? jj : cnt[u]; }
       }
-      s_keep_h[m] = h; s_keep_k[m] = s_ck[c]; s_keep_ls[m] = sc; s_keep_slot[m] = cur;
-      if (m == nk - 1) hs.cursor[b] = cur;
     }
-    if (lane == 0) {
-      hs.iters[b] = s_iters + 1;
-      if (passm != 0 && (capped || (passm & ~keepm) != 0)) hs.status[b] = TW_ERR_LIMIT;   // pass cap or token capacity
-      s_nkeep = nk;
-      hs.nA[b] = nk; hs.n_new[b] = nk;
-      s_wbase = ((hs.inline_gather || hs.own_rows == 2) && nk > 0) ? atomicAdd(&hs.scalars[kScNPred], nk) : 0;   // this utterance's work-list entries
+    rank += __shfl_xor_sync(0xffffffffu, rank, 1);
+    if (tpc == 4) rank += __shfl_xor_sync(0xffffffffu, rank, 2);
+    // ---- filter against the threshold: Length(B) < N or delta_nb > threshold.  The scores fall with the rank, so the kept
+    // expansions are the first ones.
+    if (part == 0 && s_ck[c] >= 0 && rank < N && (!hasthr || s_abs[c] > s_thr)) {
+      kept = true;
+      s_keep_h[rank] = h; s_keep_k[rank] = s_ck[c]; s_keep_ls[rank] = s_abs[c];
+      if (s_Alen[h] + 1 > hs.U_cap) s_bad = 1;
     }
-    if (lane == 1 && hs.own_rows && nk > 0) { const int r = atomicAdd(hs.rows_next, nk); s_rbase = r; hs.row_off[b] = r; }
   }
-  __syncthreads();
-  const int nk = s_nkeep;
+  int nk = __syncthreads_count(kept);
+  if (nk > 0 && (s_iters + 1 >= hs.I_max || s_bad != 0)) {   // pass cap or token capacity: what does not fit is dropped
+    if (warp == 0) {
+      const int h = lane < nk ? s_keep_h[lane] : 0, k = lane < nk ? s_keep_k[lane] : 0;
+      const double ls = lane < nk ? s_keep_ls[lane] : 0.0;
+      const bool keep = lane < nk && s_iters + 1 < hs.I_max && s_Alen[h] + 1 <= hs.U_cap;
+      const unsigned m = __ballot_sync(0xffffffffu, keep);
+      if (keep) { const int i = __popc(m & ((1u << lane) - 1u)); s_keep_h[i] = h; s_keep_k[i] = k; s_keep_ls[i] = ls; }
+      if (lane == 0) { s_nkeep = __popc(m); hs.status[b] = TW_ERR_LIMIT; }
+    }
+    __syncthreads();
+    nk = s_nkeep;
+  }
+  // list A empty and frames left: this segment is done, the next one starts with ChooseNBest(B)
+  const bool turn = nk == 0 && t0 + slen < len;
+  const int t0n = t0 + slen, slen_n = min(S, len - t0n);
+
+  // ---- the places in the work list and among the joiner rows; everybody else goes on until the barrier below
+  if (warp == 0) {
+    const bool listed = (hs.inline_gather || hs.own_rows == 2) && nk > 0;
+    const int claim = turn ? s_cl.n : nk;
+    if (lane == 0) s_wbase = listed ? atomicAdd(&hs.scalars[kScNPred], nk) : 0;
+    if (lane == 1) s_rbase = hs.own_rows && claim > 0 ? atomicAdd(hs.rows_next, claim) : 0;
+  }
+  // the first pieces of the parents' h (or of the carried hypotheses' operand rows), a warp per row of up to kEarlyCols values:
+  // fetched here, written below
+  uint4 pk[4];
+  const int L = hs.L, Hd = hs.Hd;
+  const long long stride = (long long)L * 2 * Hd;
+  const bool vec = (Hd & 7) == 0 && (reinterpret_cast<uintptr_t>(hs.slot_hc) & 15) == 0;
+  const bool gather = hs.inline_gather && nk > 0;
+  auto h_src = [&](int i, int l) { return hs.slot_hc + (bS + s_Aslot[s_keep_h[i]]) * stride + (long long)l * 2 * Hd; };
+  auto h_piece = [&](const float* src) {
+    const float4 a = *reinterpret_cast<const float4*>(src), e = *reinterpret_cast<const float4*>(src + 4);
+    const __nv_bfloat162 p0 = __floats2bfloat162_rn(a.x, a.y), p1 = __floats2bfloat162_rn(a.z, a.w);
+    const __nv_bfloat162 p2 = __floats2bfloat162_rn(e.x, e.y), p3 = __floats2bfloat162_rn(e.z, e.w);
+    return make_uint4(*reinterpret_cast<const uint32_t*>(&p0), *reinterpret_cast<const uint32_t*>(&p1),
+                      *reinterpret_cast<const uint32_t*>(&p2), *reinterpret_cast<const uint32_t*>(&p3));
+  };
+  const bool early_op = turn && hs.own_rows == 1 && warp < s_cl.n * S;
+  const int o_h = early_op ? warp / S : 0, o_t = warp - o_h * S;
+  if (gather && vec && warp < nk * L) {
+    const int i = warp / L;
+    const float* src = h_src(i, warp - i * L);
+#pragma unroll
+    for (int u = 0; u < 4; ++u) { const int x = (lane + 32 * u) * 8; if (x < Hd) pk[u] = h_piece(src + x); }
+  } else if (early_op) {
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int x = (lane + 32 * u) * 8;
+      if (x < hs.J) pk[u] = o_t < slen_n ? carry_operand(hs, b, (long long)b * hs.E_T + t0n + o_t, s_cl.slot[o_h], x) : make_uint4(0, 0, 0, 0);
+    }
+  }
+
+  if (turn) {
+    turn_over(hs, b, s_cl, t0n, slen_n);
+    if (tid == 32) hs.n_new[b] = 0;
+  } else if (tid == 32) {
+    hs.nB[b] = s_nB;
+    hs.nTop[b] = s_cl.n;
+    hs.iters[b] = s_iters + 1;
+    hs.nA[b] = nk; hs.n_new[b] = nk;
+    if (nk > 0) hs.cursor[b] = s_free[nk - 1];
+  }
 
   // ---- own_rows: log J(t, k) of the kept expansions, a warp per (expansion, frame), the last warps first (the first ones
   // write the new lists below); their joiner rows' frame distributions relative to their scores
   if (hs.own_rows == 1) {
     const int J = hs.J;
-    for (int pair = (int)(blockDim.x >> 5) - 1 - warp; pair < nk * slen; pair += blockDim.x >> 5) {
+    for (int pair = nwarps - 1 - warp; pair < nk * slen; pair += nwarps) {
       const int i = pair / slen, t = pair - i * slen;
       const int h = s_keep_h[i], k = s_keep_k[i];
       const long long rt = (long long)(r0 + h) * S + t;
-      const __nv_bfloat16* arow = static_cast<const __nv_bfloat16*>(hs.A_cur) + operand_row(r0 + h, t, S) * J;
+      const __nv_bfloat16* arow = static_cast<const __nv_bfloat16*>(hs.A_cur) + (s_orow[h] + t) * J;
       const __nv_bfloat16* wrow = static_cast<const __nv_bfloat16*>(hs.W_out) + (long long)k * J;
       const float la = hs.la[rt], lse = hs.lse_j[rt], bias = hs.b_out[k];
       float acc = 0.f;
@@ -566,7 +651,7 @@ __global__ void __launch_bounds__(2 * kStepThreads) hyp_step_kernel(HypState hs,
       if (lane == 0) {
         const double d = s_Als[h] + (double)la + ((double)(acc + bias) - (double)lse), ls = s_keep_ls[i];
         const float rel = d == -INFINITY ? -INFINITY : (float)(d - ls);
-        float* out = hs.row_ld + (long long)(s_rbase + i) * S;
+        float* out = s_rel + i * 8;
         if (!hs.mono) {
           out[t] = rel;
         } else {                            // emitted at frame t: continues at t + 1, or has left the segment
@@ -577,13 +662,14 @@ __global__ void __launch_bounds__(2 * kStepThreads) hyp_step_kernel(HypState hs,
       }
     }
   }
-  if (hs.own_rows && tid < nk) hs.row_slen[s_rbase + tid] = slen;
 
   // ---- new list A (one warp per kept expansion): tokens, hash, frame distribution d_h(k) (Eq. 5)
+  long long gp = 0, gn = 0;
+  double d_t[2] = {-INFINITY, -INFINITY};             // the distribution at frames lane and lane + 32 (S <= 64)
   if (warp < nk) {
     const int i = warp;
-    const int h = s_keep_h[i], k = s_keep_k[i];
-    const long long gp = bS + s_Aslot[h], gn = bS + s_keep_slot[i];
+    const int h = s_keep_h[i], k = s_keep_k[i], slot = s_free[i];
+    gp = bS + s_Aslot[h]; gn = bS + slot;
     const int plen = s_Alen[h];
     const int* src = tok_cap > 0 ? s_tok + h * tok_cap : hs.slot_tok + gp * hs.U_cap;
     int* dst = hs.slot_tok + gn * hs.U_cap;
@@ -596,18 +682,15 @@ __global__ void __launch_bounds__(2 * kStepThreads) hyp_step_kernel(HypState hs,
       hs.new_par[b * kMaxBeam + i] = (int)gp;
       hs.new_tok[b * kMaxBeam + i] = k;
       hs.new_row[b * kMaxBeam + i] = r0 + h;
-      hs.A_slot[b * kMaxBeam + i] = s_keep_slot[i];
+      hs.A_slot[b * kMaxBeam + i] = slot;
       hs.A_ls[b * kMaxBeam + i] = s_keep_ls[i];
     }
-    if (hs.inline_gather && lane == 0) {           // the predictor's work-list entry of this hypothesis
+    if (hs.inline_gather && lane == 0) {           // what the predictor will read of this hypothesis's token and parent
       if (hs.pf_table != nullptr) sm100::prefetch_l2_bulk(hs.pf_table + (long long)k * hs.pf_row_bytes, (uint32_t)hs.pf_row_bytes);
-      if ((hs.Hd & 3) == 0) {
-        const float* pc = hs.slot_hc + gp * ((long long)hs.L * 2 * hs.Hd) + hs.Hd;      // the parent's c, layer by layer
-        for (int l = 0; l < hs.L; ++l) sm100::prefetch_l2_bulk(pc + (long long)l * 2 * hs.Hd, (uint32_t)hs.Hd * 4u);
+      if ((Hd & 3) == 0) {
+        const float* pc = hs.slot_hc + gp * stride + Hd;      // the parent's c, layer by layer
+        for (int l = 0; l < L; ++l) sm100::prefetch_l2_bulk(pc + (long long)l * 2 * Hd, (uint32_t)Hd * 4u);
       }
-      const int wrow = s_wbase + i;
-      if (wrow < hs.B * hs.N) { hs.pw_new[wrow] = (int)gn; hs.pw_par[wrow] = (int)gp; hs.pw_tok[wrow] = k; hs.pw_bi[wrow] = b * kMaxBeam + i; }
-      else hs.status[b] = TW_ERR_LIMIT;            // cannot happen: the list holds at most N entries per utterance
     }
     const long long r = r0 + h;
     // d_h(k) at frame t of the segment: occupancy times J(t, k)
@@ -622,57 +705,78 @@ __global__ void __launch_bounds__(2 * kStepThreads) hyp_step_kernel(HypState hs,
       }
       return v;
     };
-    if (hs.own_rows == 2 && lane == 0) {             // the joiner row's tables and the work-list entry
-      const int r = s_rbase + i, wrow = s_wbase + i;
-      hs.row_e0[r] = b * hs.E_T + hs.t0[b];
-      hs.row_p[r] = hs.stateless ? k : (int)gn;
-      hs.pw_new[wrow] = (int)gn; hs.pw_par[wrow] = (int)gp; hs.pw_tok[wrow] = k;
-    }
-    auto put_d = [&](int t, double d) {
-      if (hs.own_rows == 2) hs.row_ld[(long long)(s_rbase + i) * S + t] = d == -INFINITY ? -INFINITY : (float)(d - s_keep_ls[i]);
-      else hs.A_ld[((long long)b * kMaxBeam + i) * S + t] = d;
-    };
-    if (hs.own_rows == 1) {
-      // done above
-    } else if (!hs.mono) {
-      for (int t = lane; t < S; t += 32) put_d(t, d_at(t));
-    } else {
-      // emitted at frame t: the hypothesis continues at frame t + 1, or has left the segment
-      for (int t = lane; t < S; t += 32) put_d(t, t < slen ? d_at(t - 1) : -INFINITY);
-      if (lane == 0) hs.A_done[b * kMaxBeam + i] = d_at(slen - 1);
-    }
-  }
-  // ---- the parents' h of every layer as bf16 in the recurrent halves of the gate GEMMs' operand rows (all threads:
-  // 16-byte pieces, independent of each other)
-  if (hs.inline_gather && nk > 0 && s_wbase + nk <= hs.B * hs.N) {
-    const long long stride = (long long)hs.L * 2 * hs.Hd;
-    const bool vec = (hs.Hd & 7) == 0 && (reinterpret_cast<uintptr_t>(hs.slot_hc) & 15) == 0;
-    const int per = vec ? hs.Hd >> 3 : hs.Hd;                 // pieces per (hypothesis, layer)
-    const int total = nk * hs.L * per;
-    for (int c = threadIdx.x; c < total; c += blockDim.x) {
-      const int i = c / (hs.L * per), rem = c - i * (hs.L * per), l = rem / per, x = rem - l * per;
-      const long long gp = bS + s_Aslot[s_keep_h[i]];
-      const float* hsrc = hs.slot_hc + gp * stride + (long long)l * 2 * hs.Hd;
-      __nv_bfloat16* d = reinterpret_cast<__nv_bfloat16*>(hs.xg_dst[l]) + (long long)(s_wbase + i) * hs.xg_ld[l] + hs.xg_off[l];
-      if (vec && (reinterpret_cast<uintptr_t>(d) & 15) == 0) {
-        const float4 a = *reinterpret_cast<const float4*>(hsrc + x * 8), e = *reinterpret_cast<const float4*>(hsrc + x * 8 + 4);
-        __nv_bfloat162 p0 = __floats2bfloat162_rn(a.x, a.y), p1 = __floats2bfloat162_rn(a.z, a.w);
-        __nv_bfloat162 p2 = __floats2bfloat162_rn(e.x, e.y), p3 = __floats2bfloat162_rn(e.z, e.w);
-        uint4 pk;
-        pk.x = *reinterpret_cast<uint32_t*>(&p0); pk.y = *reinterpret_cast<uint32_t*>(&p1);
-        pk.z = *reinterpret_cast<uint32_t*>(&p2); pk.w = *reinterpret_cast<uint32_t*>(&p3);
-        *reinterpret_cast<uint4*>(d + x * 8) = pk;
-      } else if (vec) {
-        for (int u = 0; u < 8; ++u) d[x * 8 + u] = __float2bfloat16_rn(hsrc[x * 8 + u]);
-      } else {
-        d[x] = __float2bfloat16_rn(hsrc[x]);
+    if (hs.own_rows != 1) {
+      // (monotonic: emitted at frame t, the hypothesis continues at frame t + 1, or has left the segment)
+#pragma unroll
+      for (int u = 0; u < 2; ++u) {
+        const int t = lane + 32 * u;
+        if (t < S) d_t[u] = !hs.mono ? d_at(t) : (t < slen ? d_at(t - 1) : -INFINITY);
       }
+      if (hs.mono && lane == 0) hs.A_done[b * kMaxBeam + i] = d_at(slen - 1);
     }
   }
-  // ---- list A empty: this segment is done ------------------------------------------------------
-  if (nk == 0 && hs.t0[b] + slen < hs.len[b]) {
-    turn_over(hs, b);
-    if (hs.own_rows) carry_rows(hs, b);
+  __syncthreads();
+
+  // ---- what goes to the claimed places
+  const int wbase = s_wbase, rbase = s_rbase;
+  if (turn) {
+    if (early_op) {
+      __nv_bfloat16* dst = static_cast<__nv_bfloat16*>(hs.A_next) + operand_row(rbase + o_h, o_t, S) * hs.J;
+#pragma unroll
+      for (int u = 0; u < 4; ++u) { const int x = (lane + 32 * u) * 8; if (x < hs.J) *reinterpret_cast<uint4*>(dst + x) = pk[u]; }
+    }
+    if (hs.own_rows) carry_rows(hs, b, s_cl, t0n, slen_n, rbase, nwarps);
+    return;
+  }
+  if (nk == 0) return;
+  if (hs.own_rows) {
+    if (tid == 32) hs.row_off[b] = rbase;
+    if (tid < nk) hs.row_slen[rbase + tid] = slen;
+  }
+  if (hs.own_rows == 1) {
+    if (tid < nk * 8 && (tid & 7) < slen) hs.row_ld[(long long)(rbase + (tid >> 3)) * S + (tid & 7)] = s_rel[tid];
+  } else if (warp < nk) {
+#pragma unroll
+    for (int u = 0; u < 2; ++u) {
+      const int t = lane + 32 * u;
+      const double d = d_t[u];
+      if (t >= S) continue;
+      if (hs.own_rows == 2) hs.row_ld[(long long)(rbase + warp) * S + t] = d == -INFINITY ? -INFINITY : (float)(d - s_keep_ls[warp]);
+      else hs.A_ld[((long long)b * kMaxBeam + warp) * S + t] = d;
+    }
+  }
+  if (warp < nk && lane == 0 && (hs.inline_gather || hs.own_rows == 2)) {      // the predictor's work-list entry, the joiner row's tables
+    const int wrow = wbase + warp, k = s_keep_k[warp];
+    if (wrow < hs.B * hs.N) {
+      hs.pw_new[wrow] = (int)gn; hs.pw_par[wrow] = (int)gp; hs.pw_tok[wrow] = k;
+      if (hs.inline_gather) hs.pw_bi[wrow] = b * kMaxBeam + warp;
+    } else {
+      hs.status[b] = TW_ERR_LIMIT;                   // cannot happen: the list holds at most N entries per utterance
+    }
+    if (hs.own_rows == 2) {
+      hs.row_e0[rbase + warp] = b * hs.E_T + t0;
+      hs.row_p[rbase + warp] = hs.stateless ? k : (int)gn;
+    }
+  }
+  // the parents' h of every layer as bf16 in the recurrent halves of the gate GEMMs' operand rows
+  if (!gather || wbase + nk > hs.B * hs.N) return;
+#pragma unroll 1
+  for (int pair = warp; pair < nk * L; pair += nwarps) {
+    const int i = pair / L, l = pair - i * L;
+    const float* src = h_src(i, l);
+    __nv_bfloat16* d = reinterpret_cast<__nv_bfloat16*>(hs.xg_dst[l]) + (long long)(wbase + i) * hs.xg_ld[l] + hs.xg_off[l];
+    if (vec && (reinterpret_cast<uintptr_t>(d) & 15) == 0) {
+      int x = lane * 8;
+      if (pair == warp) {
+#pragma unroll
+        for (int u = 0; u < 4; ++u) { if (x + u * 256 < Hd) *reinterpret_cast<uint4*>(d + x + u * 256) = pk[u]; }
+        x += kEarlyCols;
+      }
+#pragma unroll 1
+      for (; x < Hd; x += 256) *reinterpret_cast<uint4*>(d + x) = h_piece(src + x);
+    } else {
+      for (int x = lane; x < Hd; x += 32) d[x] = __float2bfloat16_rn(src[x]);
+    }
   }
 }
 
@@ -778,10 +882,7 @@ __global__ void __launch_bounds__(kThreads) stream_advance_kernel(HypState hs, c
     s_go = (hs.nA[b] == 0 && hs.t0[b] + hs.slen[b] < len);
   }
   __syncthreads();
-  if (s_go) {
-    turn_over(hs, b);
-    if (hs.own_rows) carry_rows(hs, b);
-  }
+  if (s_go) next_segment(hs, b);
 }
 
 // ChooseNBest(B) at the end of the utterance, best first.
