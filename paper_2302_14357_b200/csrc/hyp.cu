@@ -50,6 +50,9 @@ __device__ void turn_over(const HypState& hs, int b, const CarryList& cl, int t0
     hs.nB[b] = 0;
     hs.nTop[b] = 0;
     hs.iters[b] = 0;
+    // only the carried hypotheses' slots are held now: the ring starts over, so that the few dozen slots of a segment are the
+    // same ones (in L2) again and not, one segment after the other, all N (I_max + 1) of them
+    hs.cursor[b] = hs.capSlot - 1;
   }
   for (int i = threadIdx.x; i < cl.n * hs.S; i += blockDim.x) {
     const int a = i / hs.S, t = i - a * hs.S;
