@@ -48,7 +48,7 @@ gemm_bf16_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
   uint64_t* acc_empty = acc_full + 2;          // [2]
   uint32_t* tmem_holder = reinterpret_cast<uint32_t*>(acc_empty + 2);
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = warp_uniform(threadIdx.x >> 5), lane = threadIdx.x & 31;
   const int num_kb = (p.K + BK - 1) / BK;
   const int M_pre = (p.m_early && p.M_dev) ? __ldcg(p.M_dev) : 0;   // under the set-up's latency (see m_early)
 
@@ -68,57 +68,57 @@ gemm_bf16_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
   // the set-up above touched only this CTA: it may overlap the tail of the kernel that produces A and M
   pdl_wait();
   pdl_trigger();
-  const int M = p.M_dev ? (p.m_early ? M_pre : *p.M_dev) : p.M;
+  const int M = warp_uniform(p.M_dev ? (p.m_early ? M_pre : *p.M_dev) : p.M);
   const int m_tiles = (M + BM - 1) / BM, n_tiles = (p.N + BN - 1) / BN;
   const int num_tiles = m_tiles * n_tiles;     // a CTA past the last tile runs no loop iteration below
 
   if (warp == 0) {
-    if (lane == 0) {
-      uint32_t it = 0;                       // k-block counter across tiles: the ring never restarts
-      bool ok = true;
-      const uint64_t keep = l2_policy_evict_last();        // B is a weight matrix in every use of this kernel
-      for (int tile = blockIdx.x; tile < num_tiles && ok; tile += gridDim.x) {
-        const int m0 = (tile / n_tiles) * BM, n0 = (tile % n_tiles) * BN;
-        for (int kb = 0; kb < num_kb; ++kb, ++it) {
-          const int s = it % C::kStages;
-          const uint32_t ph = (it / C::kStages) & 1;
-          ok = mbar_wait(&empty[s], ph ^ 1, p.err);
-          if (!ok) break;
+    uint32_t it = 0;                         // k-block counter across tiles: the ring never restarts
+    bool ok = true;
+    const uint64_t keep = l2_policy_evict_last();          // B is a weight matrix in every use of this kernel
+    for (int tile = blockIdx.x; tile < num_tiles && ok; tile += gridDim.x) {
+      const int m0 = (tile / n_tiles) * BM, n0 = (tile % n_tiles) * BN;
+      for (int kb = 0; kb < num_kb; ++kb, ++it) {
+        const int s = it % C::kStages;
+        const uint32_t ph = (it / C::kStages) & 1;
+        ok = mbar_wait_warp(&empty[s], ph ^ 1, p.err);
+        if (!ok) break;
+        if (elect_one()) {
           mbar_expect_tx(&full[s], C::kABytes + C::kBBytes);
           tma_load_2d(sA + s * C::kABytes, &tmA, &full[s], kb * BK, m0);
           tma_load_2d_hint(sB + s * C::kBBytes, &tmB, &full[s], kb * BK, n0, keep);
         }
       }
-      settle_copies(ok);
     }
+    settle_copies(ok);
   } else if (warp == 1) {
-    if (lane == 0) {
-      constexpr uint32_t idesc = make_idesc_bf16(BM, BN);
-      uint32_t it = 0, lt = 0;               // lt: tiles done by this CTA
-      bool ok = true;
-      for (int tile = blockIdx.x; tile < num_tiles && ok; tile += gridDim.x, ++lt) {
-        const uint32_t buf = lt & 1, aph = (lt >> 1) & 1;
-        ok = mbar_wait(&acc_empty[buf], aph ^ 1, p.err);      // epilogue has drained this buffer
+    constexpr uint32_t idesc = make_idesc_bf16(BM, BN);
+    uint32_t it = 0, lt = 0;                 // lt: tiles done by this CTA
+    bool ok = true;
+    for (int tile = blockIdx.x; tile < num_tiles && ok; tile += gridDim.x, ++lt) {
+      const uint32_t buf = lt & 1, aph = (lt >> 1) & 1;
+      ok = mbar_wait_warp(&acc_empty[buf], aph ^ 1, p.err);   // epilogue has drained this buffer
+      if (!ok) break;
+      tc_fence_after();
+      const uint32_t tmem_d = tmem_base + buf * BN;
+      for (int kb = 0; kb < num_kb; ++kb, ++it) {
+        const int s = it % C::kStages;
+        const uint32_t ph = (it / C::kStages) & 1;
+        ok = mbar_wait_warp(&full[s], ph, p.err);
         if (!ok) break;
         tc_fence_after();
-        const uint32_t tmem_d = tmem_base + buf * BN;
-        for (int kb = 0; kb < num_kb; ++kb, ++it) {
-          const int s = it % C::kStages;
-          const uint32_t ph = (it / C::kStages) & 1;
-          ok = mbar_wait(&full[s], ph, p.err);
-          if (!ok) break;
-          tc_fence_after();
-          const uint32_t a_addr = smem_u32(sA + s * C::kABytes), b_addr = smem_u32(sB + s * C::kBBytes);
+        const uint32_t a_addr = smem_u32(sA + s * C::kABytes), b_addr = smem_u32(sB + s * C::kBBytes);
+        if (elect_one()) {
 #pragma unroll
           for (int k = 0; k < BK / 16; ++k)
             umma_bf16(tmem_d, make_desc_k_sw128(a_addr + k * 32), make_desc_k_sw128(b_addr + k * 32), idesc,
                       (kb | k) != 0);
           umma_commit(&empty[s]);
         }
-        if (ok) umma_commit(&acc_full[buf]);
       }
-      settle_copies(ok);
+      if (ok && elect_one()) umma_commit(&acc_full[buf]);
     }
+    settle_copies(ok);
   } else {
     const int ew = warp - 2;                 // 0..7
     const int q = warp & 3;                  // TMEM lane quarter this warp may read
@@ -419,7 +419,7 @@ gemm_lstm_wide_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_cons
   uint64_t* acc_init = acc_full + 1;        // the epilogue warps have written the accumulators' initial values
   uint32_t* tmem_holder = reinterpret_cast<uint32_t*>(acc_init + 1);
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = warp_uniform(threadIdx.x >> 5), lane = threadIdx.x & 31;
   const int num_kb = (p.K + BK - 1) / BK;
   const int M_pre = (p.m_early && p.M_dev) ? __ldcg(p.M_dev) : 0;   // under the set-up's latency (see m_early)
 
@@ -444,7 +444,7 @@ gemm_lstm_wide_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_cons
   // writes the count (late), splits for the largest count: its tiles are narrow anyway, and so are known before the wait.
   const bool late = EPIW == 8 && p.M_dev != nullptr && !p.m_early;
   if (EPIW == 16) { pdl_wait(); pdl_trigger(); }      // the set-up touched only this CTA: it may overlap the tail of the kernel that produces A and M
-  const int M = (late || !p.M_dev) ? p.M : (p.m_early ? M_pre : *p.M_dev);
+  const int M = warp_uniform((late || !p.M_dev) ? p.M : (p.m_early ? M_pre : *p.M_dev));
   const int m_tiles = M > 0 ? (M + BM - 1) / BM : 1;
   const int units = p.N >> 5;
   int n_split = (int)gridDim.x / m_tiles;
@@ -464,7 +464,7 @@ gemm_lstm_wide_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_cons
     if (EPIW == 8) { pdl_wait(); pdl_trigger(); }
   } else if (warp == 0) {
     const uint64_t keep = l2_policy_evict_last();          // the gate weights: read again by every step
-    auto send_B = [&](int kb, int s, uint32_t more = 0) {
+    auto send_B = [&](int kb, int s, uint32_t more = 0) {    // by the elected lane
       mbar_expect_tx(&full[s], (uint32_t)w * (BK * 2) + more);
       uint8_t* bdst = smem + s * stage + kWideABytes;
       int r = 0;
@@ -476,55 +476,59 @@ gemm_lstm_wide_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_cons
       // the weights of the first stages ahead of the wait (with the wide tiles of a large step that measured slower: the
       // kernel ahead is still pulling its own through L2)
       npre = min(num_kb, nst);
-      if (lane == 0) for (int kb = 0; kb < npre; ++kb) send_B(kb, kb);
+      for (int kb = 0; kb < npre; ++kb) if (elect_one()) send_B(kb, kb);
       pdl_wait();
       pdl_trigger();
     }
-    if (lane == 0) {
-      const int rows = (late ? *p.M_dev : M) - m0;
+    {
+      const int rows = (late ? warp_uniform(*p.M_dev) : M) - m0;
       const int nq = EPIW == 8 && rows < BM ? (rows + 31) >> 5 : 4;      // lane quarters with rows in them (the large instance fetches all)
       const uint32_t a_bytes = (uint32_t)nq * (kWideABytes / 4);
       int s = 0;
       uint32_t ph = 0;
       if (rows <= 0)                                         // late: no rows after all; only the copies under way have to be waited for
-        for (int kb = 0; kb < npre; ++kb) { mbar_arrive(&full[kb]); mbar_wait(&full[kb], 0, p.err); }
+        for (int kb = 0; kb < npre; ++kb) { if (elect_one()) mbar_arrive(&full[kb]); mbar_wait_warp(&full[kb], 0, p.err); }
       for (int kb = 0; kb < num_kb && rows > 0; ++kb) {
         if (kb >= npre) {
-          ok = mbar_wait(&empty[s], ph ^ 1, p.err);
+          ok = mbar_wait_warp(&empty[s], ph ^ 1, p.err);
           if (!ok) break;
-          send_B(kb, s, EPIW == 8 ? 0 : a_bytes);
         }
-        if (EPIW == 8) mbar_expect_tx(&full[s], a_bytes);
-        uint8_t* adst = smem + s * stage;
-        if (nq == 4) tma_load_2d(adst, &tmA, &full[s], kb * BK, m0);
-        else for (int q = 0; q < nq; ++q) tma_load_2d(adst + q * (kWideABytes / 4), &tmA32, &full[s], kb * BK, m0 + 32 * q);
+        if (elect_one()) {
+          if (kb >= npre) send_B(kb, s, EPIW == 8 ? 0 : a_bytes);
+          if (EPIW == 8) mbar_expect_tx(&full[s], a_bytes);
+          uint8_t* adst = smem + s * stage;
+          if (nq == 4) tma_load_2d(adst, &tmA, &full[s], kb * BK, m0);
+          else for (int q = 0; q < nq; ++q) tma_load_2d(adst + q * (kWideABytes / 4), &tmA32, &full[s], kb * BK, m0 + 32 * q);
+        }
         if (++s == nst) { s = 0; ph ^= 1; }
       }
     }
   } else if (warp == 1) {
     if (EPIW == 8) { pdl_wait(); pdl_trigger(); }
-    if (lane == 0 && (!late || m0 < *p.M_dev)) {
+    if (!late || m0 < warp_uniform(*p.M_dev)) {
       const int n1 = w <= 256 ? w : ((w >> 1) + 15) & ~15, n2 = w - n1;    // wider than one MMA: two of about equal width
       const uint32_t idesc1 = make_idesc_bf16(BM, n1), idesc2 = make_idesc_bf16(BM, n2);
-      ok = mbar_wait(acc_init, 0, p.err);                  // the accumulators hold bias + addend: accumulate onto them
+      ok = mbar_wait_warp(acc_init, 0, p.err);             // the accumulators hold bias + addend: accumulate onto them
       int s = 0;
       uint32_t ph = 0;
       for (int kb = 0; kb < num_kb && ok; ++kb) {
-        ok = mbar_wait(&full[s], ph, p.err);
+        ok = mbar_wait_warp(&full[s], ph, p.err);
         if (!ok) break;
         tc_fence_after();
         const uint32_t a_addr = smem_u32(smem + s * stage), b_addr = a_addr + kWideABytes;
+        if (elect_one()) {
 #pragma unroll
-        for (int k = 0; k < BK / 16; ++k) {
-          const uint64_t da = make_desc_k_sw128(a_addr + k * 32);
-          umma_bf16(tmem_base, da, make_desc_k_sw128(b_addr + k * 32), idesc1, 1u);
-          if (n2 > 0)
-            umma_bf16(tmem_base + (uint32_t)n1, da, make_desc_k_sw128(b_addr + n1 * (BK * 2) + k * 32), idesc2, 1u);
+          for (int k = 0; k < BK / 16; ++k) {
+            const uint64_t da = make_desc_k_sw128(a_addr + k * 32);
+            umma_bf16(tmem_base, da, make_desc_k_sw128(b_addr + k * 32), idesc1, 1u);
+            if (n2 > 0)
+              umma_bf16(tmem_base + (uint32_t)n1, da, make_desc_k_sw128(b_addr + n1 * (BK * 2) + k * 32), idesc2, 1u);
+          }
+          umma_commit(&empty[s]);
         }
-        umma_commit(&empty[s]);
         if (++s == nst) { s = 0; ph ^= 1; }
       }
-      if (ok) umma_commit(acc_full);
+      if (ok && elect_one()) umma_commit(acc_full);
     }
   } else {
     if (EPIW == 8) { pdl_wait(); pdl_trigger(); }

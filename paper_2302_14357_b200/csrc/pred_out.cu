@@ -41,11 +41,11 @@ wp_operand_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
   uint64_t* acc_empty = acc_full + 2;          // [2]
   uint32_t* tmem_holder = reinterpret_cast<uint32_t*>(acc_empty + 2);
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = warp_uniform(threadIdx.x >> 5), lane = threadIdx.x & 31;
   const int num_kb = (p.K + BK - 1) / BK;
   // The work list is hyp_step_kernel's, which had finished before the last gate GEMM (the kernel ahead) began: the list and
   // the utterances' positions are read ahead of the wait.
-  const int M = __ldcg(p.M_dev);
+  const int M = warp_uniform(__ldcg(p.M_dev));
   // the joiner kernel that follows streams W_out, which a large step's other traffic has pushed out of L2: every CTA asks for
   // its share (a constant weight: nothing to wait for)
   if (p.pf_base != nullptr && threadIdx.x == 64) {
@@ -73,16 +73,18 @@ wp_operand_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
   if (warp == 0) {
     int npre = 0;                              // W_p is a constant: the first tile's first stages ahead of the wait
     const uint64_t keep = l2_policy_evict_last();
-    if (lane == 0 && (int)blockIdx.x < num_tiles) {
+    if ((int)blockIdx.x < num_tiles) {
       npre = num_kb < C::kStages ? num_kb : C::kStages;
       for (int kb = 0; kb < npre; ++kb) {
-        mbar_expect_tx(&full[kb], C::kBBytes);
-        tma_load_2d_hint(sB + kb * C::kBBytes, &tmB, &full[kb], kb * BK, ((int)blockIdx.x % n_tiles) * BN, keep);
+        if (elect_one()) {
+          mbar_expect_tx(&full[kb], C::kBBytes);
+          tma_load_2d_hint(sB + kb * C::kBBytes, &tmB, &full[kb], kb * BK, ((int)blockIdx.x % n_tiles) * BN, keep);
+        }
       }
     }
     pdl_wait();
     pdl_trigger();
-    if (lane == 0) {
+    {
       uint32_t it = 0;
       for (int tile = blockIdx.x; tile < num_tiles && ok; tile += gridDim.x) {
         const int m0 = (tile / n_tiles) * BM, n0 = (tile % n_tiles) * BN;
@@ -91,41 +93,47 @@ wp_operand_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
           const int s = it % C::kStages;
           const uint32_t ph = (it / C::kStages) & 1;
           if ((int)it >= npre) {
-            ok = mbar_wait(&empty[s], ph ^ 1, p.err);
+            ok = mbar_wait_warp(&empty[s], ph ^ 1, p.err);
             if (!ok) break;
-            mbar_expect_tx(&full[s], C::kBBytes);
-            tma_load_2d_hint(sB + s * C::kBBytes, &tmB, &full[s], kb * BK, n0, keep);
           }
-          mbar_expect_tx(&full[s], (uint32_t)nq * (C::kABytes / 4));
-          if (nq == 4) tma_load_2d(sA + s * C::kABytes, &tmA, &full[s], kb * BK, m0);
-          else for (int q = 0; q < nq; ++q) tma_load_2d(sA + s * C::kABytes + q * (C::kABytes / 4), &tmA32, &full[s], kb * BK, m0 + 32 * q);
+          if (elect_one()) {
+            if ((int)it >= npre) {
+              mbar_expect_tx(&full[s], C::kBBytes);
+              tma_load_2d_hint(sB + s * C::kBBytes, &tmB, &full[s], kb * BK, n0, keep);
+            }
+            mbar_expect_tx(&full[s], (uint32_t)nq * (C::kABytes / 4));
+            if (nq == 4) tma_load_2d(sA + s * C::kABytes, &tmA, &full[s], kb * BK, m0);
+            else for (int q = 0; q < nq; ++q) tma_load_2d(sA + s * C::kABytes + q * (C::kABytes / 4), &tmA32, &full[s], kb * BK, m0 + 32 * q);
+          }
         }
       }
     }
   } else if (warp == 1) {
     pdl_wait();
     pdl_trigger();
-    if (lane == 0) {
+    {
       constexpr uint32_t idesc = make_idesc_bf16(BM, BN);
       uint32_t it = 0, lt = 0;
       for (int tile = blockIdx.x; tile < num_tiles && ok; tile += gridDim.x, ++lt) {
         const uint32_t buf = lt & 1, aph = (lt >> 1) & 1;
-        ok = mbar_wait(&acc_empty[buf], aph ^ 1, p.err);
+        ok = mbar_wait_warp(&acc_empty[buf], aph ^ 1, p.err);
         if (!ok) break;
         tc_fence_after();
         const uint32_t tmem_d = tmem_base + buf * BN;
         for (int kb = 0; kb < num_kb; ++kb, ++it) {
           const int s = it % C::kStages;
-          ok = mbar_wait(&full[s], (it / C::kStages) & 1, p.err);
+          ok = mbar_wait_warp(&full[s], (it / C::kStages) & 1, p.err);
           if (!ok) break;
           tc_fence_after();
           const uint32_t a_addr = smem_u32(sA + s * C::kABytes), b_addr = smem_u32(sB + s * C::kBBytes);
+          if (elect_one()) {
 #pragma unroll
-          for (int k = 0; k < BK / 16; ++k)
-            umma_bf16(tmem_d, make_desc_k_sw128(a_addr + k * 32), make_desc_k_sw128(b_addr + k * 32), idesc, (kb | k) != 0);
-          umma_commit(&empty[s]);
+            for (int k = 0; k < BK / 16; ++k)
+              umma_bf16(tmem_d, make_desc_k_sw128(a_addr + k * 32), make_desc_k_sw128(b_addr + k * 32), idesc, (kb | k) != 0);
+            umma_commit(&empty[s]);
+          }
         }
-        if (ok) umma_commit(&acc_full[buf]);
+        if (ok && elect_one()) umma_commit(&acc_full[buf]);
       }
     }
   } else {

@@ -12,6 +12,8 @@ __device__ __forceinline__ uint32_t smem_u32(const void* p) {
   return static_cast<uint32_t>(__cvta_generic_to_shared(p));
 }
 
+// A value that is the same in all lanes, in a form in which the compiler knows it
+__device__ __forceinline__ int warp_uniform(int x) { return __shfl_sync(0xffffffffu, x, 0); }
 __device__ __forceinline__ bool elect_one() {
   uint32_t pred = 0;
   asm volatile(
@@ -60,6 +62,13 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, int* e
   }
   atomicExch(err, 1);
   return false;
+}
+
+// The same wait by a whole warp, with one answer.  The producer and MMA warps run their loops with all lanes and elect the lane
+// that issues inside them: with `if (lane == 0)` around a loop the compiler cannot know that the operands of the TMA and MMA
+// instructions, which take them from uniform registers, are the same for all active lanes.
+__device__ __forceinline__ bool mbar_wait_warp(uint64_t* bar, uint32_t parity, int* err) {
+  return __all_sync(0xffffffffu, mbar_wait(bar, parity, err));
 }
 
 // For a thread that leaves its loop because a wait gave up: copies that its CTA sent for may still be on their way into shared
