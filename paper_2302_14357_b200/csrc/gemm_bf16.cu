@@ -73,50 +73,50 @@ gemm_bf16_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
   const int num_tiles = m_tiles * n_tiles;     // a CTA past the last tile runs no loop iteration below
 
   if (warp == 0) {
-    uint32_t it = 0;                         // k-block counter across tiles: the ring never restarts
+    int s = 0;                               // stage and phase run on across tiles: the ring never restarts
+    uint32_t ph = 0;
     bool ok = true;
     const uint64_t keep = l2_policy_evict_last();          // B is a weight matrix in every use of this kernel
+    const uint32_t a0 = smem_u32(sA), b0 = smem_u32(sB), full0 = smem_u32(full), empty0 = smem_u32(empty);
     for (int tile = blockIdx.x; tile < num_tiles && ok; tile += gridDim.x) {
       const int m0 = (tile / n_tiles) * BM, n0 = (tile % n_tiles) * BN;
-      for (int kb = 0; kb < num_kb; ++kb, ++it) {
-        const int s = it % C::kStages;
-        const uint32_t ph = (it / C::kStages) & 1;
-        ok = mbar_wait_warp(&empty[s], ph ^ 1, p.err);
+      for (int kb = 0; kb < num_kb; ++kb) {
+        ok = mbar_wait_warp(empty0 + 8 * s, ph ^ 1, p.err);
         if (!ok) break;
         if (elect_one()) {
-          mbar_expect_tx(&full[s], C::kABytes + C::kBBytes);
-          tma_load_2d(sA + s * C::kABytes, &tmA, &full[s], kb * BK, m0);
-          tma_load_2d_hint(sB + s * C::kBBytes, &tmB, &full[s], kb * BK, n0, keep);
+          mbar_arrive_expect_a(full0 + 8 * s, C::kABytes + C::kBBytes);
+          tma_load_2d_a(a0 + s * C::kABytes, &tmA, full0 + 8 * s, kb * BK, m0);
+          tma_load_2d_hint_a(b0 + s * C::kBBytes, &tmB, full0 + 8 * s, kb * BK, n0, keep);
         }
+        if (++s == C::kStages) { s = 0; ph ^= 1; }
       }
     }
     settle_copies(ok);
   } else if (warp == 1) {
     constexpr uint32_t idesc = make_idesc_bf16(BM, BN);
-    uint32_t it = 0, lt = 0;                 // lt: tiles done by this CTA
+    int s = 0;
+    uint32_t ph = 0, lt = 0;                 // lt: tiles done by this CTA
     bool ok = true;
+    const uint32_t a_lo = desc_lo(smem_u32(sA)), b_lo = desc_lo(smem_u32(sB)), full0 = smem_u32(full), empty0 = smem_u32(empty);
     for (int tile = blockIdx.x; tile < num_tiles && ok; tile += gridDim.x, ++lt) {
       const uint32_t buf = lt & 1, aph = (lt >> 1) & 1;
-      ok = mbar_wait_warp(&acc_empty[buf], aph ^ 1, p.err);   // epilogue has drained this buffer
+      ok = mbar_wait_warp(smem_u32(acc_empty) + 8 * buf, aph ^ 1, p.err);   // epilogue has drained this buffer
       if (!ok) break;
       tc_fence_after();
       const uint32_t tmem_d = tmem_base + buf * BN;
-      for (int kb = 0; kb < num_kb; ++kb, ++it) {
-        const int s = it % C::kStages;
-        const uint32_t ph = (it / C::kStages) & 1;
-        ok = mbar_wait_warp(&full[s], ph, p.err);
+      for (int kb = 0; kb < num_kb; ++kb) {
+        ok = mbar_wait_warp(full0 + 8 * s, ph, p.err);
         if (!ok) break;
         tc_fence_after();
-        const uint32_t a_addr = smem_u32(sA + s * C::kABytes), b_addr = smem_u32(sB + s * C::kBBytes);
         if (elect_one()) {
+          const uint32_t al = a_lo + s * (C::kABytes >> 4), bl = b_lo + s * (C::kBBytes >> 4);
 #pragma unroll
-          for (int k = 0; k < BK / 16; ++k)
-            umma_bf16(tmem_d, make_desc_k_sw128(a_addr + k * 32), make_desc_k_sw128(b_addr + k * 32), idesc,
-                      (kb | k) != 0);
-          umma_commit(&empty[s]);
+          for (int k = 0; k < BK / 16; ++k) umma_bf16(tmem_d, desc_of(al + 2 * k), desc_of(bl + 2 * k), idesc, (kb | k) != 0);
+          umma_commit_a(empty0 + 8 * s);
         }
+        if (++s == C::kStages) { s = 0; ph ^= 1; }
       }
-      if (ok && elect_one()) umma_commit(&acc_full[buf]);
+      if (ok && elect_one()) umma_commit_a(smem_u32(acc_full) + 8 * buf);
     }
     settle_copies(ok);
   } else {
@@ -428,7 +428,7 @@ gemm_lstm_wide_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_cons
     if (EPIW == 8) prefetch_tensormap(&tmA32);
     prefetch_tensormap(&tmB64);
     prefetch_tensormap(&tmB32);
-    for (int s = 0; s < kWideMaxStages; ++s) { mbar_init(&full[s], EPIW == 8 ? 2 : 1); mbar_init(&empty[s], 1); }   // full, small instance: B's bytes and A's, each armed apart
+    for (int s = 0; s < kWideMaxStages; ++s) { mbar_init(&full[s], 1); mbar_init(&empty[s], 1); }
     mbar_init(acc_full, 1);
     mbar_init(acc_init, EPIW);
     fence_barrier_init();
@@ -464,19 +464,20 @@ gemm_lstm_wide_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_cons
     if (EPIW == 8) { pdl_wait(); pdl_trigger(); }
   } else if (warp == 0) {
     const uint64_t keep = l2_policy_evict_last();          // the gate weights: read again by every step
-    auto send_B = [&](int kb, int s, uint32_t more = 0) {    // by the elected lane
-      mbar_expect_tx(&full[s], (uint32_t)w * (BK * 2) + more);
-      uint8_t* bdst = smem + s * stage + kWideABytes;
+    const uint32_t smem0 = smem_u32(smem), full0 = smem_u32(full), empty0 = smem_u32(empty), b_bytes = (uint32_t)w * (BK * 2);
+    auto send_B = [&](int kb, int s) {                       // by the elected lane
+      const uint32_t bdst = smem0 + s * stage + kWideABytes;
       int r = 0;
-      for (; r + 64 <= w; r += 64) tma_load_2d_hint(bdst + r * (BK * 2), &tmB64, &full[s], kb * BK, n0 + r, keep);
-      if (r < w) tma_load_2d_hint(bdst + r * (BK * 2), &tmB32, &full[s], kb * BK, n0 + r, keep);
+      for (; r + 64 <= w; r += 64) tma_load_2d_hint_a(bdst + r * (BK * 2), &tmB64, full0 + 8 * s, kb * BK, n0 + r, keep);
+      if (r < w) tma_load_2d_hint_a(bdst + r * (BK * 2), &tmB32, full0 + 8 * s, kb * BK, n0 + r, keep);
     };
     int npre = 0;
     if (EPIW == 8) {
       // the weights of the first stages ahead of the wait (with the wide tiles of a large step that measured slower: the
       // kernel ahead is still pulling its own through L2)
       npre = min(num_kb, nst);
-      for (int kb = 0; kb < npre; ++kb) if (elect_one()) send_B(kb, kb);
+      for (int kb = 0; kb < npre; ++kb)
+        if (elect_one()) { mbar_expect_a(full0 + 8 * kb, b_bytes); send_B(kb, kb); }     // the arrival comes with A
       pdl_wait();
       pdl_trigger();
     }
@@ -487,18 +488,18 @@ gemm_lstm_wide_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_cons
       int s = 0;
       uint32_t ph = 0;
       if (rows <= 0)                                         // late: no rows after all; only the copies under way have to be waited for
-        for (int kb = 0; kb < npre; ++kb) { if (elect_one()) mbar_arrive(&full[kb]); mbar_wait_warp(&full[kb], 0, p.err); }
+        for (int kb = 0; kb < npre; ++kb) { if (elect_one()) mbar_arrive(&full[kb]); mbar_wait_warp(full0 + 8 * kb, 0, p.err); }
       for (int kb = 0; kb < num_kb && rows > 0; ++kb) {
         if (kb >= npre) {
-          ok = mbar_wait_warp(&empty[s], ph ^ 1, p.err);
+          ok = mbar_wait_warp(empty0 + 8 * s, ph ^ 1, p.err);
           if (!ok) break;
         }
         if (elect_one()) {
-          if (kb >= npre) send_B(kb, s, EPIW == 8 ? 0 : a_bytes);
-          if (EPIW == 8) mbar_expect_tx(&full[s], a_bytes);
-          uint8_t* adst = smem + s * stage;
-          if (nq == 4) tma_load_2d(adst, &tmA, &full[s], kb * BK, m0);
-          else for (int q = 0; q < nq; ++q) tma_load_2d(adst + q * (kWideABytes / 4), &tmA32, &full[s], kb * BK, m0 + 32 * q);
+          const uint32_t adst = smem0 + s * stage;
+          mbar_arrive_expect_a(full0 + 8 * s, kb < npre ? a_bytes : a_bytes + b_bytes);
+          if (kb >= npre) send_B(kb, s);
+          if (nq == 4) tma_load_2d_a(adst, &tmA, full0 + 8 * s, kb * BK, m0);
+          else for (int q = 0; q < nq; ++q) tma_load_2d_a(adst + q * (kWideABytes / 4), &tmA32, full0 + 8 * s, kb * BK, m0 + 32 * q);
         }
         if (++s == nst) { s = 0; ph ^= 1; }
       }
@@ -508,27 +509,34 @@ gemm_lstm_wide_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_cons
     if (!late || m0 < warp_uniform(*p.M_dev)) {
       const int n1 = w <= 256 ? w : ((w >> 1) + 15) & ~15, n2 = w - n1;    // wider than one MMA: two of about equal width
       const uint32_t idesc1 = make_idesc_bf16(BM, n1), idesc2 = make_idesc_bf16(BM, n2);
-      ok = mbar_wait_warp(acc_init, 0, p.err);             // the accumulators hold bias + addend: accumulate onto them
+      const uint32_t a_lo = desc_lo(smem_u32(smem)), full0 = smem_u32(full), empty0 = smem_u32(empty);
+      ok = mbar_wait_warp(smem_u32(acc_init), 0, p.err);   // the accumulators hold bias + addend: accumulate onto them
       int s = 0;
       uint32_t ph = 0;
       for (int kb = 0; kb < num_kb && ok; ++kb) {
-        ok = mbar_wait_warp(&full[s], ph, p.err);
+        ok = mbar_wait_warp(full0 + 8 * s, ph, p.err);
         if (!ok) break;
         tc_fence_after();
         const uint32_t a_addr = smem_u32(smem + s * stage), b_addr = a_addr + kWideABytes;
         if (elect_one()) {
+          if (EPIW == 8) {
+            const uint32_t al = a_lo + s * (stage >> 4), bl = al + (kWideABytes >> 4);
 #pragma unroll
-          for (int k = 0; k < BK / 16; ++k) {
-            const uint64_t da = make_desc_k_sw128(a_addr + k * 32);
-            umma_bf16(tmem_base, da, make_desc_k_sw128(b_addr + k * 32), idesc1, 1u);
-            if (n2 > 0)
-              umma_bf16(tmem_base + (uint32_t)n1, da, make_desc_k_sw128(b_addr + n1 * (BK * 2) + k * 32), idesc2, 1u);
+            for (int k = 0; k < BK / 16; ++k) umma_bf16(tmem_base, desc_of(al + 2 * k), desc_of(bl + 2 * k), idesc1, 1u);
+          } else {
+#pragma unroll
+            for (int k = 0; k < BK / 16; ++k) {
+              const uint64_t da = make_desc_k_sw128(a_addr + k * 32);
+              umma_bf16(tmem_base, da, make_desc_k_sw128(b_addr + k * 32), idesc1, 1u);
+              if (n2 > 0)
+                umma_bf16(tmem_base + (uint32_t)n1, da, make_desc_k_sw128(b_addr + n1 * (BK * 2) + k * 32), idesc2, 1u);
+            }
           }
-          umma_commit(&empty[s]);
+          umma_commit_a(empty0 + 8 * s);
         }
         if (++s == nst) { s = 0; ph ^= 1; }
       }
-      if (ok && elect_one()) umma_commit(acc_full);
+      if (ok && elect_one()) umma_commit_a(smem_u32(acc_full));
     }
   } else {
     if (EPIW == 8) { pdl_wait(); pdl_trigger(); }

@@ -56,7 +56,7 @@ wp_operand_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
     prefetch_tensormap(&tmA);
     prefetch_tensormap(&tmA32);
     prefetch_tensormap(&tmB);
-    for (int s = 0; s < C::kStages; ++s) { mbar_init(&full[s], 2); mbar_init(&empty[s], 1); }   // full: B's bytes and A's, each armed apart
+    for (int s = 0; s < C::kStages; ++s) { mbar_init(&full[s], 1); mbar_init(&empty[s], 1); }
     for (int i = 0; i < 2; ++i) { mbar_init(&acc_full[i], 1); mbar_init(&acc_empty[i], C::kEpiWarps); }
     fence_barrier_init();
     fence_proxy_async_smem();
@@ -73,38 +73,41 @@ wp_operand_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
   if (warp == 0) {
     int npre = 0;                              // W_p is a constant: the first tile's first stages ahead of the wait
     const uint64_t keep = l2_policy_evict_last();
+    const uint32_t a0 = smem_u32(sA), b0 = smem_u32(sB), full0 = smem_u32(full), empty0 = smem_u32(empty);
     if ((int)blockIdx.x < num_tiles) {
       npre = num_kb < C::kStages ? num_kb : C::kStages;
       for (int kb = 0; kb < npre; ++kb) {
         if (elect_one()) {
-          mbar_expect_tx(&full[kb], C::kBBytes);
-          tma_load_2d_hint(sB + kb * C::kBBytes, &tmB, &full[kb], kb * BK, ((int)blockIdx.x % n_tiles) * BN, keep);
+          mbar_expect_a(full0 + 8 * kb, C::kBBytes);         // the arrival comes with A
+          tma_load_2d_hint_a(b0 + kb * C::kBBytes, &tmB, full0 + 8 * kb, kb * BK, ((int)blockIdx.x % n_tiles) * BN, keep);
         }
       }
     }
     pdl_wait();
     pdl_trigger();
     {
-      uint32_t it = 0;
+      int s = 0;
+      uint32_t ph = 0;
       for (int tile = blockIdx.x; tile < num_tiles && ok; tile += gridDim.x) {
         const int m0 = (tile / n_tiles) * BM, n0 = (tile % n_tiles) * BN;
         const int nq = min(4, (M - m0 + 31) >> 5);           // lane quarters with rows in them
-        for (int kb = 0; kb < num_kb; ++kb, ++it) {
-          const int s = it % C::kStages;
-          const uint32_t ph = (it / C::kStages) & 1;
-          if ((int)it >= npre) {
-            ok = mbar_wait_warp(&empty[s], ph ^ 1, p.err);
+        const uint32_t a_bytes = (uint32_t)nq * (C::kABytes / 4);
+        for (int kb = 0; kb < num_kb; ++kb) {
+          const bool first = npre > 0;                       // B is on its way
+          if (!first) {
+            ok = mbar_wait_warp(empty0 + 8 * s, ph ^ 1, p.err);
             if (!ok) break;
+          } else {
+            --npre;
           }
           if (elect_one()) {
-            if ((int)it >= npre) {
-              mbar_expect_tx(&full[s], C::kBBytes);
-              tma_load_2d_hint(sB + s * C::kBBytes, &tmB, &full[s], kb * BK, n0, keep);
-            }
-            mbar_expect_tx(&full[s], (uint32_t)nq * (C::kABytes / 4));
-            if (nq == 4) tma_load_2d(sA + s * C::kABytes, &tmA, &full[s], kb * BK, m0);
-            else for (int q = 0; q < nq; ++q) tma_load_2d(sA + s * C::kABytes + q * (C::kABytes / 4), &tmA32, &full[s], kb * BK, m0 + 32 * q);
+            const uint32_t adst = a0 + s * C::kABytes;
+            mbar_arrive_expect_a(full0 + 8 * s, first ? a_bytes : a_bytes + C::kBBytes);
+            if (nq == 4) tma_load_2d_a(adst, &tmA, full0 + 8 * s, kb * BK, m0);
+            else for (int q = 0; q < nq; ++q) tma_load_2d_a(adst + q * (C::kABytes / 4), &tmA32, full0 + 8 * s, kb * BK, m0 + 32 * q);
+            if (!first) tma_load_2d_hint_a(b0 + s * C::kBBytes, &tmB, full0 + 8 * s, kb * BK, n0, keep);
           }
+          if (++s == C::kStages) { s = 0; ph ^= 1; }
         }
       }
     }
@@ -113,27 +116,28 @@ wp_operand_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
     pdl_trigger();
     {
       constexpr uint32_t idesc = make_idesc_bf16(BM, BN);
-      uint32_t it = 0, lt = 0;
+      int s = 0;
+      uint32_t ph = 0, lt = 0;
+      const uint32_t a_lo = desc_lo(smem_u32(sA)), b_lo = desc_lo(smem_u32(sB)), full0 = smem_u32(full), empty0 = smem_u32(empty);
       for (int tile = blockIdx.x; tile < num_tiles && ok; tile += gridDim.x, ++lt) {
         const uint32_t buf = lt & 1, aph = (lt >> 1) & 1;
-        ok = mbar_wait_warp(&acc_empty[buf], aph ^ 1, p.err);
+        ok = mbar_wait_warp(smem_u32(acc_empty) + 8 * buf, aph ^ 1, p.err);
         if (!ok) break;
         tc_fence_after();
         const uint32_t tmem_d = tmem_base + buf * BN;
-        for (int kb = 0; kb < num_kb; ++kb, ++it) {
-          const int s = it % C::kStages;
-          ok = mbar_wait_warp(&full[s], (it / C::kStages) & 1, p.err);
+        for (int kb = 0; kb < num_kb; ++kb) {
+          ok = mbar_wait_warp(full0 + 8 * s, ph, p.err);
           if (!ok) break;
           tc_fence_after();
-          const uint32_t a_addr = smem_u32(sA + s * C::kABytes), b_addr = smem_u32(sB + s * C::kBBytes);
           if (elect_one()) {
+            const uint32_t al = a_lo + s * (C::kABytes >> 4), bl = b_lo + s * (C::kBBytes >> 4);
 #pragma unroll
-            for (int k = 0; k < BK / 16; ++k)
-              umma_bf16(tmem_d, make_desc_k_sw128(a_addr + k * 32), make_desc_k_sw128(b_addr + k * 32), idesc, (kb | k) != 0);
-            umma_commit(&empty[s]);
+            for (int k = 0; k < BK / 16; ++k) umma_bf16(tmem_d, desc_of(al + 2 * k), desc_of(bl + 2 * k), idesc, (kb | k) != 0);
+            umma_commit_a(empty0 + 8 * s);
           }
+          if (++s == C::kStages) { s = 0; ph ^= 1; }
         }
-        if (ok && elect_one()) umma_commit(&acc_full[buf]);
+        if (ok && elect_one()) umma_commit_a(smem_u32(acc_full) + 8 * buf);
       }
     }
   } else {

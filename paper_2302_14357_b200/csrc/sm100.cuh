@@ -67,8 +67,36 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, int* e
 // The same wait by a whole warp, with one answer.  The producer and MMA warps run their loops with all lanes and elect the lane
 // that issues inside them: with `if (lane == 0)` around a loop the compiler cannot know that the operands of the TMA and MMA
 // instructions, which take them from uniform registers, are the same for all active lanes.
-__device__ __forceinline__ bool mbar_wait_warp(uint64_t* bar, uint32_t parity, int* err) {
-  return __all_sync(0xffffffffu, mbar_wait(bar, parity, err));
+// Those loops take shared-memory addresses and descriptor words that step by constants: a warp on its own issues an instruction
+// every 4 to 6 cycles, so that with addresses and descriptors made anew a K step's four MMAs took 540 cycles (of which the
+// tensor core works 40 to 160) and a stage's loads 350 to 450.
+__device__ __forceinline__ bool mbar_try_wait_a(uint32_t bar, uint32_t parity) {
+  uint32_t ok;
+  asm volatile(
+      "{\n\t.reg .pred P;\n\t"
+      "mbarrier.try_wait.parity.shared::cta.b64 P, [%1], %2;\n\t"
+      "selp.u32 %0, 1, 0, P;\n\t}"
+      : "=r"(ok)
+      : "r"(bar), "r"(parity)
+      : "memory");
+  return ok != 0;
+}
+__device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity, int* err) {
+  if (__all_sync(0xffffffffu, mbar_try_wait_a(bar, parity))) return true;
+#pragma unroll 1
+  for (uint32_t i = 0; i < kSpinLimit; ++i) {
+    if (__all_sync(0xffffffffu, mbar_try_wait_a(bar, parity))) return true;
+    if ((i & 1023u) == 1023u && __any_sync(0xffffffffu, *reinterpret_cast<volatile int*>(err) != 0)) return false;
+  }
+  atomicExch(err, 1);
+  return false;
+}
+__device__ __forceinline__ void mbar_arrive_expect_a(uint32_t bar, uint32_t bytes) {
+  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
+}
+// bytes to come, without an arrival: the phase stays open for the arrival that follows
+__device__ __forceinline__ void mbar_expect_a(uint32_t bar, uint32_t bytes) {
+  asm volatile("mbarrier.expect_tx.relaxed.cta.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
 }
 
 // For a thread that leaves its loop because a wait gave up: copies that its CTA sent for may still be on their way into shared
@@ -176,6 +204,11 @@ __device__ __forceinline__ void tma_load_2d(void* smem_dst, const CUtensorMap* m
       ::"r"(smem_u32(smem_dst)), "l"(reinterpret_cast<uint64_t>(m)), "r"(smem_u32(bar)), "r"(c0), "r"(c1)
       : "memory");
 }
+__device__ __forceinline__ void tma_load_2d_a(uint32_t smem_dst, const CUtensorMap* m, uint32_t bar, int c0, int c1) {
+  asm volatile(
+      "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4}], [%2];"
+      ::"r"(smem_dst), "l"(reinterpret_cast<uint64_t>(m)), "r"(bar), "r"(c0), "r"(c1) : "memory");
+}
 // a contiguous piece of global memory; both addresses and the size are multiples of 16 bytes
 __device__ __forceinline__ void bulk_load(void* smem_dst, const void* src, uint32_t bytes, uint64_t* bar) {
   asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
@@ -200,12 +233,10 @@ __device__ __forceinline__ void tma_prefetch_2d(const CUtensorMap* m, int c0, in
                : "memory");
 }
 // the same tile load with an L2 eviction policy
-__device__ __forceinline__ void tma_load_2d_hint(void* smem_dst, const CUtensorMap* m, uint64_t* bar, int c0, int c1,
-                                                 uint64_t policy) {
+__device__ __forceinline__ void tma_load_2d_hint_a(uint32_t smem_dst, const CUtensorMap* m, uint32_t bar, int c0, int c1, uint64_t policy) {
   asm volatile(
       "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint [%0], [%1, {%3, %4}], [%2], %5;"
-      ::"r"(smem_u32(smem_dst)), "l"(reinterpret_cast<uint64_t>(m)), "r"(smem_u32(bar)), "r"(c0), "r"(c1), "l"(policy)
-      : "memory");
+      ::"r"(smem_dst), "l"(reinterpret_cast<uint64_t>(m)), "r"(bar), "r"(c0), "r"(c1), "l"(policy) : "memory");
 }
 
 // ---- tcgen05 --------------------------------------------------------------------------------
@@ -234,9 +265,8 @@ __device__ __forceinline__ void umma_bf16(uint32_t tmem_d, uint64_t desc_a, uint
       : "memory");
 }
 // arrives on `bar` once every MMA this thread issued so far has completed
-__device__ __forceinline__ void umma_commit(uint64_t* bar) {
-  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(bar))
-               : "memory");
+__device__ __forceinline__ void umma_commit_a(uint32_t bar) {
+  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
 }
 
 // 32 consecutive fp32 columns of this thread's TMEM lane (warp w may touch lanes 32*(w%4) .. +31)
@@ -318,14 +348,18 @@ __device__ __forceinline__ void tmem_ld_wait16(uint32_t r[16]) {
 // Shared-memory operand descriptor for a K-major tile stored as rows of 64 bf16 (128 bytes) with the
 // 128-byte swizzle (what a TMA load with CU_TENSOR_MAP_SWIZZLE_128B writes): 8-row groups are 1024
 // bytes apart.  Stepping 16 elements along K inside the row adds 32 bytes to the start address.
+// The high word is a constant; stepping through stages and along K adds to the low one (shared-memory addresses have 18 bits, so
+// its 14-bit field of 16-byte units does not overflow).
+__device__ __forceinline__ uint32_t desc_lo(uint32_t smem_addr) { return (smem_addr >> 4) | (1u << 16); }
+__device__ __forceinline__ uint64_t desc_of(uint32_t lo) {
+  // stride between 8-row groups in 16-byte units; descriptor version of this architecture; layout type: 128-byte swizzle
+  return ((uint64_t)((1024u >> 4) | (1u << 14) | (2u << 29)) << 32) | lo;
+}
+// Descriptor of the operand at an address that the compiler may not fold into steps.  The MMAs of wide tiles (256 and 320 columns)
+// are issued with these: the few dozen cycles between two of them cost nothing there, and back to back they slow the operand
+// loads down (predictor and joiner stage calls of 1000 rows 110.6 against 108.8 us, 128 utterances 77.9 against 76.9 ms).
 __device__ __forceinline__ uint64_t make_desc_k_sw128(uint32_t smem_addr) {
-  uint64_t d = 0;
-  d |= (uint64_t)((smem_addr >> 4) & 0x3FFF);        // start address, 16-byte units
-  d |= (uint64_t)1 << 16;                            // leading byte offset (unused for swizzled K-major)
-  d |= (uint64_t)(1024 >> 4) << 32;                  // stride byte offset between 8-row groups
-  d |= (uint64_t)1 << 46;                            // descriptor version of this architecture
-  d |= (uint64_t)2 << 61;                            // layout type: 128-byte swizzle
-  return d;
+  return desc_of(((smem_addr >> 4) & 0x3FFF) | (1u << 16));
 }
 // Instruction descriptor: bf16 x bf16 -> fp32, both operands K-major, tile M x N
 __host__ __device__ constexpr uint32_t make_idesc_bf16(int M, int N) {
