@@ -149,9 +149,10 @@ __global__ void __launch_bounds__(kThreads) hyp_init_kernel(HypState hs, const i
 
 constexpr int kStepThreads = 512;   // 16 warps: one per hypothesis of list A
 constexpr int kSelCap = 64;         // survivors of a row's bound that are ranked directly
-constexpr int kKeyPitch = kMaxBeam + 1;   // rows of the candidate keys start in different banks
 
 __device__ __forceinline__ bool tok_better(float v1, int k1, float v2, int k2) { return v1 > v2 || (v1 == v2 && k1 < k2); }
+// (value desc, token asc) of a positive value as one integer, larger first
+__device__ __forceinline__ unsigned long long tok_key(float v, int k) { return ((unsigned long long)__float_as_uint(v) << 32) | (0xffffffffu - (unsigned)k); }
 
 // Order-preserving integer image of a score: a < b as doubles <=> order_key(a) < order_key(b) as unsigned
 // integers (-0 counts as +0; scores are never NaN).  The ranking loops compare these instead of doubles.
@@ -166,7 +167,7 @@ __device__ __forceinline__ unsigned long long order_key(double x) {
 //                       merged into, the free slots of the ring
 //   1                   warp 0: the blank expansions into list B and the threshold (ChooseNthScore); warp 16 + h: the N best
 //                       tokens of row h
-//   2                   N best expansions (four threads a candidate) and the filter; the number kept comes with the barrier
+//   2                   the expansions above the threshold listed, the N best of them
 //   3                   work-list entries and rows claimed (atomics); beside that the new hypotheses' tokens, log J of the kept
 //                       expansions and the parents' h - or, with nothing kept, the next segment's list and operand rows
 //   4                   what goes to the claimed places
@@ -184,15 +185,17 @@ __global__ void __launch_bounds__(2 * kStepThreads) hyp_step_kernel(HypState hs,
   __shared__ int s_iters, s_nT0, s_Btop[kMaxBeam], s_Btopslot[kMaxBeam];   // list B's best entries as the previous pass left them
   __shared__ double s_Btopls[kMaxBeam];
   __shared__ int s_free[32];                             // the next free slots of the ring
-  __shared__ __align__(16) ulonglong2 s_ent[32];         // (key, index) of the entries that B's new best ones are chosen from
+  __shared__ __align__(16) ulonglong2 s_ent[32];         // (key, index) of the entries that B's new best ones are chosen from,
+  __shared__ double s_els[32];                           // their scores
+  __shared__ int s_eslot[32];                            // and slots
   __shared__ CarryList s_cl;                             // B's new best entries
-  __shared__ int s_nB, s_hasthr, s_bad, s_nkeep, s_wbase, s_rbase;
+  __shared__ int s_nB, s_hasthr, s_bad, s_np, s_nkeep, s_wbase, s_rbase;
   __shared__ double s_thr;
   __shared__ int s_ck[kMaxBeam * kMaxBeam];
   __shared__ double s_abs[kMaxBeam * kMaxBeam];
-  __shared__ unsigned long long s_key[kMaxBeam * kKeyPitch];
-  __shared__ __align__(16) float s_lm[kMaxBeam][32];     // in-kernel selection: lane maxima, survivors of a row, its chunks to look at
-  __shared__ float2 s_sv[kMaxBeam][kSelCap];
+  __shared__ __align__(16) ulonglong2 s_pass[kMaxBeam * kMaxBeam];   // (key, place) of the candidates above the threshold
+  __shared__ __align__(16) unsigned s_lm[kMaxBeam][32];  // in-kernel selection: lane maxima, survivors of a row, its chunks to look at
+  __shared__ unsigned long long s_sv[kMaxBeam][kSelCap];
   __shared__ unsigned char s_chunk[kMaxBeam][128];
   __shared__ int s_cnt[kMaxBeam];
   __shared__ int s_keep_h[kMaxBeam], s_keep_k[kMaxBeam];
@@ -248,7 +251,7 @@ __global__ void __launch_bounds__(2 * kStepThreads) hyp_step_kernel(HypState hs,
     for (int q = 0; q < kMaxBeam; ++q) busy |= __shfl_sync(0xffffffffu, carry, q) == slot;
     const unsigned free_mask = __ballot_sync(0xffffffffu, !busy);
     if (!busy) s_free[__popc(free_mask & ((1u << lane) - 1u))] = slot;
-    if (lane == 0) { s_iters = iters; s_nT0 = nT; s_bad = 0; }
+    if (lane == 0) { s_iters = iters; s_nT0 = nT; s_bad = 0; s_np = 0; }
   }
   if (tid < kMaxBeam && hs.own_rows == 1) s_orow[tid] = operand_row(r0 + tid, 0, S);
   // ---- AddAndMerge, search: warp h looks for the tokens of A_h among the entries already in B.  It needs the lists only,
@@ -332,22 +335,9 @@ __global__ void __launch_bounds__(2 * kStepThreads) hyp_step_kernel(HypState hs,
     const double merged = __shfl_sync(0xffffffffu, score, m_src & 31);
     if (m_src >= 0) score = merged;
     if (m_dup) idx = -1;                     // it stands among the old best entries
-    const unsigned long long key = order_key(score);
-    s_ent[lane] = make_ulonglong2(key, (unsigned long long)(long long)idx);
+    s_ent[lane] = make_ulonglong2(order_key(score), (unsigned long long)(long long)idx);
+    s_els[lane] = score; s_eslot[lane] = m_slot;
     const int count = __popc(__ballot_sync(0xffffffffu, idx >= 0));
-    __syncwarp();
-    int rank = 0;
-#pragma unroll 8
-    for (int j = 0; j < 32; ++j) {          // all lanes read the same words: broadcasts, independent of each other
-      const ulonglong2 o = s_ent[j];
-      const int oi = (int)o.y;
-      rank += (oi >= 0 && (o.x > key || (o.x == key && oi < idx))) ? 1 : 0;
-    }
-    if (idx >= 0 && rank < N) {
-      hs.B_top[b * kMaxBeam + rank] = idx;
-      s_cl.slot[rank] = m_slot; s_cl.ls[rank] = score;
-      if (rank == N - 1) s_thr = score;
-    }
     if (lane == 0) { s_cl.n = min(N, count); s_hasthr = count >= N; }
   } else if (warp == 1 && lane == 0) {
     atomicAdd(&hs.calls[b], 1);              // (nobody else writes these: additions without a round trip)
@@ -357,17 +347,46 @@ __global__ void __launch_bounds__(2 * kStepThreads) hyp_step_kernel(HypState hs,
       atomicAdd(reinterpret_cast<unsigned long long*>(hs.rows_total) + 1, (unsigned long long)(H * slen));
     }
   }
+  if (warp < 16) {
+    if (!two_halves && warp >= 8) {                     // the rows' candidate lists, by the warps that merge nothing
+      const int c = tid - kMaxBeam * kMaxBeam, h = c / kMaxBeam, j = c % kMaxBeam;
+      int n = 0, k = -1;
+      float v = 0.f;
+      if (h < H) {
+        const long long at = (long long)(r0 + h) * kMaxBeam + j;
+        n = hs.cand_n[r0 + h]; v = hs.cand_v[at]; k = hs.cand_k[at];
+      }
+      s_abs[c] = j < n ? s_Als[h] + (double)v : -INFINITY;
+      s_ck[c] = j < n ? k : -1;
+    }
+    // the entries' ranks, two a warp: every lane compares with one of the others
+    asm volatile("bar.sync 1, 512;" ::: "memory");
+    const ulonglong2 o = s_ent[lane];
+#pragma unroll
+    for (int u = 0; u < 2; ++u) {
+      const int e = 2 * warp + u;
+      const ulonglong2 me = s_ent[e];
+      const int oi = (int)o.y, mi = (int)me.y;
+      const int rank = __popc(__ballot_sync(0xffffffffu, oi >= 0 && (o.x > me.x || (o.x == me.x && oi < mi))));
+      if (lane == 0 && mi >= 0 && rank < N) {
+        hs.B_top[b * kMaxBeam + rank] = mi;
+        s_cl.slot[rank] = s_eslot[e]; s_cl.ls[rank] = s_els[e];
+        if (rank == N - 1) s_thr = s_els[e];
+      }
+    }
+  }
   if (two_halves && warp >= 16) {
     // ---- ChooseNBestExpansions, first stage, for the row of hypothesis warp - 16: its N best tokens by delta_nb,
     // order (value desc, token asc), straight into the candidate table of the second stage.
     const int h = warp - 16;
     if (lane < kMaxBeam) {
-      s_abs[h * kMaxBeam + lane] = -INFINITY; s_ck[h * kMaxBeam + lane] = -1; s_key[h * kKeyPitch + lane] = order_key(-INFINITY);
+      s_abs[h * kMaxBeam + lane] = -INFINITY; s_ck[h * kMaxBeam + lane] = -1;
     }
     if (h < H) {
       const float* src = hs.dnb_sel + (long long)(r0 + h) * V;
       const double base = s_Als[h];
-      // a lower bound of the N-th best value: the N-th largest of the 32 lane maxima (distinct elements)
+      // a lower bound of the N-th best value: the N-th largest of the 32 lane maxima (distinct elements), whose last five bits
+      // make room for the lane
       const int nchunk = V >> 5;
       const bool pairs = hs.dnb_chunk == 16;     // maxima of 16 columns: two make a chunk's
       const float* cmax = (hs.dnb_max != nullptr && (V & 31) == 0 && nchunk <= 128) ? hs.dnb_max + (long long)(r0 + h) * (pairs ? 2 * nchunk : nchunk) : nullptr;
@@ -390,27 +409,25 @@ __global__ void __launch_bounds__(2 * kStepThreads) hyp_step_kernel(HypState hs,
           lmax = fmaxf(fmaxf(lmax, fmaxf(v.x, v.y)), fmaxf(v.z, v.w));
         }
       }
-      s_lm[h][lane] = lmax;
+      const unsigned lkey = (__float_as_uint(lmax) & ~31u) | (31u - lane);
+      s_lm[h][lane] = lkey;
       if (lane == 0) s_cnt[h] = 0;
       __syncwarp();
       int lrank = 0;
-#pragma unroll 2
+#pragma unroll
       for (int j = 0; j < 32; j += 4) {
-        const float4 o = *reinterpret_cast<const float4*>(&s_lm[h][j]);
-        lrank += (o.x > lmax || (o.x == lmax && j < lane)) ? 1 : 0;
-        lrank += (o.y > lmax || (o.y == lmax && j + 1 < lane)) ? 1 : 0;
-        lrank += (o.z > lmax || (o.z == lmax && j + 2 < lane)) ? 1 : 0;
-        lrank += (o.w > lmax || (o.w == lmax && j + 3 < lane)) ? 1 : 0;
+        const uint4 o = *reinterpret_cast<const uint4*>(&s_lm[h][j]);
+        lrank += (o.x > lkey) + (o.y > lkey) + (o.z > lkey) + (o.w > lkey);
       }
       const unsigned who = __ballot_sync(0xffffffffu, lrank == N - 1);        // exactly one lane: the ranks are 0..31
-      const float bound = __shfl_sync(0xffffffffu, lmax, __ffs(who) - 1);
+      const float bound = __uint_as_float(__shfl_sync(0xffffffffu, lkey, __ffs(who) - 1) & ~31u);
       auto push4 = [&](const float4& v4, int k) {
         const float vv[4] = {v4.x, v4.y, v4.z, v4.w};
 #pragma unroll
         for (int c = 0; c < 4; ++c) {
           if (vv[c] >= bound && vv[c] > 0.f) {
             const int i = atomicAdd(&s_cnt[h], 1);
-            if (i < kSelCap) s_sv[h][i] = make_float2(vv[c], __int_as_float(k + c));
+            if (i < kSelCap) s_sv[h][i] = tok_key(vv[c], k + c);
           }
         }
       };
@@ -465,14 +482,13 @@ __global__ void __launch_bounds__(2 * kStepThreads) hyp_step_kernel(HypState hs,
       const int ns = s_cnt[h];
       if (ns <= kSelCap) {
         for (int i = lane; i < ns; i += 32) {
-          const float2 me = s_sv[h][i];
-          const float v = me.x; const int k = __float_as_int(me.y);
+          const unsigned long long me = s_sv[h][i];
           int rank = 0;
 #pragma unroll 4
-          for (int j = 0; j < ns; ++j) { const float2 o = s_sv[h][j]; rank += tok_better(o.x, __float_as_int(o.y), v, k) ? 1 : 0; }
+          for (int j = 0; j < ns; ++j) rank += s_sv[h][j] > me ? 1 : 0;
           if (rank < N) {
-            const double sc = base + (double)__logf(v);
-            s_abs[h * kMaxBeam + rank] = sc; s_ck[h * kMaxBeam + rank] = k; s_key[h * kKeyPitch + rank] = order_key(sc);
+            s_abs[h * kMaxBeam + rank] = base + (double)__logf(__uint_as_float((unsigned)(me >> 32)));
+            s_ck[h * kMaxBeam + rank] = (int)(0xffffffffu - (unsigned)me);
           }
         }
       } else {
@@ -496,72 +512,46 @@ __global__ void __launch_bounds__(2 * kStepThreads) hyp_step_kernel(HypState hs,
             if (tok_better(ov, ok, bv, bk)) { bv = ov; bk = ok; }
           }
           if (!(bv > 0.f)) break;
-          if (lane == 0) {
-            const double sc = base + (double)__logf(bv);
-            s_abs[h * kMaxBeam + j] = sc; s_ck[h * kMaxBeam + j] = bk; s_key[h * kKeyPitch + j] = order_key(sc);
-          }
+          if (lane == 0) { s_abs[h * kMaxBeam + j] = base + (double)__logf(bv); s_ck[h * kMaxBeam + j] = bk; }
           pv = bv; pk = bk;
         }
       }
     }
   }
-  if (!two_halves && tid >= kMaxBeam * kMaxBeam) {      // the rows' candidate lists, by the warps that merge nothing
-    const int c = tid - kMaxBeam * kMaxBeam, h = c / kMaxBeam, j = c % kMaxBeam;
-    int n = 0, k = -1;
-    float v = 0.f;
-    if (h < H) {
-      const long long at = (long long)(r0 + h) * kMaxBeam + j;
-      n = hs.cand_n[r0 + h]; v = hs.cand_v[at]; k = hs.cand_k[at];
-    }
-    const double sc = j < n ? s_Als[h] + (double)v : -INFINITY;
-    s_abs[c] = sc;
-    s_ck[c] = j < n ? k : -1;
-    s_key[h * kKeyPitch + j] = order_key(sc);
-  }
   __syncthreads();
 
-  // ---- ChooseNBestExpansions, second stage: the N best (h, k) over the rows' candidate lists, in
-  // float64; order (score desc, h asc, k asc).  The lists are sorted by (score desc, k asc).
-  // Rank = how many candidates come before this one in that order.  Every row's list is sorted and padded with the key of
-  // log 0, so the candidates of a row that come before this one are a prefix of its list: its length is found by bisection.
-  // Rows before h count their ties with this score, rows after it do not, and in its own row exactly the jj entries ahead of it
-  // count.  A candidate has 4 threads (2 in a CTA of 512), each with every fourth (second) row, four bisections at a time.
-  const bool hasthr = s_hasthr != 0;
-  bool kept = false;
-  {
-    const int tpc = (int)blockDim.x / (kMaxBeam * kMaxBeam), c = tid / tpc, part = tid % tpc, h = c / kMaxBeam, jj = c % kMaxBeam;
-    int rank = 0;
-    if (s_ck[c] >= 0) {
-      const unsigned long long mine = s_key[h * kKeyPitch + jj];
-#pragma unroll 1
-      for (int hb = part; hb < H; hb += 4 * tpc) {
-        int cnt[4] = {0, 0, 0, 0};
-        int st = kMaxBeam / 2;
-#pragma unroll 1
-        for (int step = 0; step < 5; ++step) {               // 8, 4, 2, 1, and 1 for a full list
-#pragma unroll
-          for (int u = 0; u < 4; ++u) {
-            const int hh = min(hb + u * tpc, H - 1);
-            const unsigned long long so = s_key[hh * kKeyPitch + cnt[u] + st - 1];
-            if (so > mine || (hh < h && so == mine)) cnt[u] += st;
-          }
-          st = max(st >> 1, 1);
-        }
-#pragma unroll
-        for (int u = 0; u < 4; ++u) { const int hh = hb + u * tpc; if (hh < H) rank += hh == h ? jj : cnt[u]; }
-      }
+  // ---- ChooseNBestExpansions, second stage: the N best (h, k) over the rows' candidate lists, in float64; order (score desc, h
+  // asc, k asc), which within a row is the order of its list.  Only those above the threshold are ever kept (Length(B) < N or
+  // delta_nb > threshold), and all that rank before such a one are above it too: they are listed, mostly a handful, and
+  // ranked among themselves, a warp per candidate with a lane for each of the others.
+  if (tid < kMaxBeam * kMaxBeam) {
+    const double sc = s_abs[tid];
+    const bool pass = s_ck[tid] >= 0 && (s_hasthr == 0 || sc > s_thr);
+    const unsigned m = __ballot_sync(0xffffffffu, pass);
+    if (m != 0) {
+      int at = 0;
+      if (lane == 0) at = atomicAdd(&s_np, __popc(m));
+      at = __shfl_sync(0xffffffffu, at, 0) + __popc(m & ((1u << lane) - 1u));
+      if (pass) s_pass[at] = make_ulonglong2(order_key(sc), (unsigned long long)tid);
     }
-    rank += __shfl_xor_sync(0xffffffffu, rank, 1);
-    if (tpc == 4) rank += __shfl_xor_sync(0xffffffffu, rank, 2);
-    // ---- filter against the threshold: Length(B) < N or delta_nb > threshold.  The scores fall with the rank, so the kept
-    // expansions are the first ones.
-    if (part == 0 && s_ck[c] >= 0 && rank < N && (!hasthr || s_abs[c] > s_thr)) {
-      kept = true;
+  }
+  __syncthreads();
+  const int np = s_np;
+  for (int i = warp; i < np; i += nwarps) {
+    const ulonglong2 me = s_pass[i];
+    int rank = 0;
+    for (int j = 0; j < np; j += 32) {
+      const ulonglong2 o = j + lane < np ? s_pass[j + lane] : make_ulonglong2(0, 0);
+      rank += __popc(__ballot_sync(0xffffffffu, o.x > me.x || (o.x == me.x && o.y < me.y)));      // (no score has the key 0)
+    }
+    if (lane == 0 && rank < N) {
+      const int c = (int)me.y, h = c / kMaxBeam;
       s_keep_h[rank] = h; s_keep_k[rank] = s_ck[c]; s_keep_ls[rank] = s_abs[c];
       if (s_Alen[h] + 1 > hs.U_cap) s_bad = 1;
     }
   }
-  int nk = __syncthreads_count(kept);
+  __syncthreads();
+  int nk = min(np, N);
   if (nk > 0 && (s_iters + 1 >= hs.I_max || s_bad != 0)) {   // pass cap or token capacity: what does not fit is dropped
     if (warp == 0) {
       const int h = lane < nk ? s_keep_h[lane] : 0, k = lane < nk ? s_keep_k[lane] : 0;
@@ -579,11 +569,12 @@ __global__ void __launch_bounds__(2 * kStepThreads) hyp_step_kernel(HypState hs,
   const int t0n = t0 + slen, slen_n = min(S, len - t0n);
 
   // ---- the places in the work list and among the joiner rows; everybody else goes on until the barrier below
+  int claimed = 0;
   if (warp == 0) {
     const bool listed = (hs.inline_gather || hs.own_rows == 2) && nk > 0;
-    const int claim = turn ? s_cl.n : nk;
-    if (lane == 0) s_wbase = listed ? atomicAdd(&hs.scalars[kScNPred], nk) : 0;
-    if (lane == 1) s_rbase = hs.own_rows && claim > 0 ? atomicAdd(hs.rows_next, claim) : 0;
+    const int rows = turn ? s_cl.n : nk;
+    if (lane == 0 && listed) claimed = atomicAdd(&hs.scalars[kScNPred], nk);
+    if (lane == 1 && hs.own_rows && rows > 0) claimed = atomicAdd(hs.rows_next, rows);
   }
   // the first pieces of the parents' h (or of the carried hypotheses' operand rows), a warp per row of up to kEarlyCols values:
   // fetched here, written below
@@ -602,11 +593,18 @@ __global__ void __launch_bounds__(2 * kStepThreads) hyp_step_kernel(HypState hs,
   };
   const bool early_op = turn && hs.own_rows == 1 && warp < s_cl.n * S;
   const int o_h = early_op ? warp / S : 0, o_t = warp - o_h * S;
-  if (gather && vec && warp < nk * L) {
-    const int i = warp / L;
-    const float* src = h_src(i, warp - i * L);
+  // (the first nk warps write the new lists: the rows go to those behind them, the dot products to the last ones)
+  const int g_at = warp - nk;
+  const bool early_h = gather && vec && g_at >= 0 && g_at < nk * L;
+  __nv_bfloat16* g_dst = nullptr;            // this warp's destination, for work-list entry 0
+  int g_ld = 0;
+  if (early_h) {
+    const int i = g_at / L, l = g_at - i * L;
+    const float* src = h_src(i, l);
 #pragma unroll
     for (int u = 0; u < 4; ++u) { const int x = (lane + 32 * u) * 8; if (x < Hd) pk[u] = h_piece(src + x); }
+    g_ld = hs.xg_ld[l];
+    g_dst = reinterpret_cast<__nv_bfloat16*>(hs.xg_dst[l]) + (long long)i * g_ld + hs.xg_off[l];
   } else if (early_op) {
 #pragma unroll
     for (int u = 0; u < 4; ++u) {
@@ -718,6 +716,10 @@ __global__ void __launch_bounds__(2 * kStepThreads) hyp_step_kernel(HypState hs,
       if (hs.mono && lane == 0) hs.A_done[b * kMaxBeam + i] = d_at(slen - 1);
     }
   }
+  if (warp == 0) {
+    if (lane == 0) s_wbase = claimed;
+    if (lane == 1) s_rbase = claimed;
+  }
   __syncthreads();
 
   // ---- what goes to the claimed places
@@ -763,20 +765,24 @@ __global__ void __launch_bounds__(2 * kStepThreads) hyp_step_kernel(HypState hs,
   }
   // the parents' h of every layer as bf16 in the recurrent halves of the gate GEMMs' operand rows
   if (!gather || wbase + nk > hs.B * hs.N) return;
+  bool done_early = false;
+  if (early_h) {
+    __nv_bfloat16* d = g_dst + (long long)wbase * g_ld;
+    done_early = (reinterpret_cast<uintptr_t>(d) & 15) == 0 && Hd <= kEarlyCols;
+    if (done_early) {
+#pragma unroll
+      for (int u = 0; u < 4; ++u) { const int x = (lane + 32 * u) * 8; if (x < Hd) *reinterpret_cast<uint4*>(d + x) = pk[u]; }
+    }
+  }
+  // (rows that have not been fetched early, or not whole)
 #pragma unroll 1
-  for (int pair = warp; pair < nk * L; pair += nwarps) {
+  for (int pair = g_at; pair < nk * L; pair += nwarps) {
+    if (pair < 0 || (pair == g_at && done_early)) continue;
     const int i = pair / L, l = pair - i * L;
     const float* src = h_src(i, l);
     __nv_bfloat16* d = reinterpret_cast<__nv_bfloat16*>(hs.xg_dst[l]) + (long long)(wbase + i) * hs.xg_ld[l] + hs.xg_off[l];
     if (vec && (reinterpret_cast<uintptr_t>(d) & 15) == 0) {
-      int x = lane * 8;
-      if (pair == warp) {
-#pragma unroll
-        for (int u = 0; u < 4; ++u) { if (x + u * 256 < Hd) *reinterpret_cast<uint4*>(d + x + u * 256) = pk[u]; }
-        x += kEarlyCols;
-      }
-#pragma unroll 1
-      for (; x < Hd; x += 256) *reinterpret_cast<uint4*>(d + x) = h_piece(src + x);
+      for (int x = lane * 8; x < Hd; x += 256) *reinterpret_cast<uint4*>(d + x) = h_piece(src + x);
     } else {
       for (int x = lane; x < Hd; x += 32) d[x] = __float2bfloat16_rn(src[x]);
     }
