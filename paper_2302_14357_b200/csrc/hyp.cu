@@ -525,8 +525,11 @@ __global__ void __launch_bounds__(2 * kStepThreads) hyp_step_kernel(HypState hs,
   // delta_nb > threshold), and all that rank before such a one are above it too: they are listed, mostly a handful, and
   // ranked among themselves, a warp per candidate with a lane for each of the others.
   if (tid < kMaxBeam * kMaxBeam) {
-    const double sc = s_abs[tid];
-    const bool pass = s_ck[tid] >= 0 && (s_hasthr == 0 || sc > s_thr);
+    // (a row with N candidates bounds the N-th best score from below by its last one, log 0 where there is none: the first row,
+    // the best hypothesis's, leaves few to rank (one utterance, N = 10: 28.3 -> 27.6 ms); the largest of all rows' bounds leaves
+    // fewer and takes longer than it saves at N = 5)
+    const double sc = s_abs[tid], low = s_abs[N - 1];
+    const bool pass = s_ck[tid] >= 0 && !(sc < low) && (s_hasthr == 0 || sc > s_thr);
     const unsigned m = __ballot_sync(0xffffffffu, pass);
     if (m != 0) {
       int at = 0;
