@@ -260,10 +260,11 @@ gemm_bf16_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
 // Two instances: 16 epilogue warps for tiles of up to 320 columns, one CTA per SM; 8 for tiles of up to 128 columns (small
 // steps), which takes less than half of an SM's shared memory, registers and tensor memory, so that the next kernel's CTAs
 // are resident beside it, past their set-up and with their first weight tiles already in shared memory when it ends.
-// The ring's stages are as large as the CTA's own tile needs (128 rows of A, its columns of B).  A row tile whose last lane
+// The ring's stages are as large as the CTA's own tile needs (the rows of A, its columns of B; small instance: ring_quarters, and A
+// and B apart, so that an MMA that reads 128 rows of a smaller stage stays inside the ring).  A row tile whose last lane
 // quarters have no rows fetches, in the small instance, only the quarters that do (what the MMA makes of stale operand rows
 // stays in their lanes).
-constexpr int kWideMaxStages = 8;
+constexpr int kWideMaxStages = kMaxRingStages;
 constexpr uint32_t kWideABytes = BM * BK * 2;
 template <int EPIW>
 struct Wide {
@@ -456,17 +457,19 @@ gemm_lstm_wide_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_cons
   const int n0 = u0 * 32, w = nu * 32;                   // this CTA's columns [n0, n0 + w), w <= kMaxBN
   if (w > W::kMaxBN && threadIdx.x == 0) atomicExch(p.err, 1);     // the host sizes the grid so that this cannot happen
   const bool active = m0 < M && mt < m_tiles && w <= W::kMaxBN;    // an idle CTA skips the roles and only frees its TMEM
-  const uint32_t stage = kWideABytes + (uint32_t)w * (BK * 2);
-  const int nst = EPIW == 16 ? 4 : min((int)(W::kRing / stage), kWideMaxStages);
+  const uint32_t b_bytes = (uint32_t)w * (BK * 2), a_stage = EPIW == 16 ? kWideABytes : (uint32_t)ring_quarters(p.M) * (kWideABytes / 4);
+  const uint32_t stage = kWideABytes + b_bytes;          // large instance
+  const int nst = EPIW == 16 ? 4 : min((int)(W::kRing / (a_stage + b_bytes)), kWideMaxStages);
+  const uint32_t b_area = smem_u32(smem) + (EPIW == 16 ? kWideABytes : nst * a_stage), a_step = EPIW == 16 ? stage : a_stage, b_step = EPIW == 16 ? stage : b_bytes;
   bool ok = true;                                        // every wait of the ring so far has ended in time
 
   if (!active) {
     if (EPIW == 8) { pdl_wait(); pdl_trigger(); }
   } else if (warp == 0) {
     const uint64_t keep = l2_policy_evict_last();          // the gate weights: read again by every step
-    const uint32_t smem0 = smem_u32(smem), full0 = smem_u32(full), empty0 = smem_u32(empty), b_bytes = (uint32_t)w * (BK * 2);
+    const uint32_t smem0 = smem_u32(smem), full0 = smem_u32(full), empty0 = smem_u32(empty);
     auto send_B = [&](int kb, int s) {                       // by the elected lane
-      const uint32_t bdst = smem0 + s * stage + kWideABytes;
+      const uint32_t bdst = b_area + s * b_step;
       int r = 0;
       for (; r + 64 <= w; r += 64) tma_load_2d_hint_a(bdst + r * (BK * 2), &tmB64, full0 + 8 * s, kb * BK, n0 + r, keep);
       if (r < w) tma_load_2d_hint_a(bdst + r * (BK * 2), &tmB32, full0 + 8 * s, kb * BK, n0 + r, keep);
@@ -483,7 +486,7 @@ gemm_lstm_wide_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_cons
     }
     {
       const int rows = (late ? warp_uniform(*p.M_dev) : M) - m0;
-      const int nq = EPIW == 8 && rows < BM ? (rows + 31) >> 5 : 4;      // lane quarters with rows in them (the large instance fetches all)
+      const int nq = EPIW == 8 && rows <= 64 ? (rows + 31) >> 5 : 4;     // lane quarters with rows in them, three as four (the large instance fetches all)
       const uint32_t a_bytes = (uint32_t)nq * (kWideABytes / 4);
       int s = 0;
       uint32_t ph = 0;
@@ -495,7 +498,7 @@ gemm_lstm_wide_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_cons
           if (!ok) break;
         }
         if (elect_one()) {
-          const uint32_t adst = smem0 + s * stage;
+          const uint32_t adst = smem0 + s * a_step;
           mbar_arrive_expect_a(full0 + 8 * s, kb < npre ? a_bytes : a_bytes + b_bytes);
           if (kb >= npre) send_B(kb, s);
           if (nq == 4) tma_load_2d_a(adst, &tmA, full0 + 8 * s, kb * BK, m0);
@@ -520,7 +523,7 @@ gemm_lstm_wide_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_cons
         const uint32_t a_addr = smem_u32(smem + s * stage), b_addr = a_addr + kWideABytes;
         if (elect_one()) {
           if (EPIW == 8) {
-            const uint32_t al = a_lo + s * (stage >> 4), bl = al + (kWideABytes >> 4);
+            const uint32_t al = a_lo + s * (a_step >> 4), bl = desc_lo(b_area) + s * (b_step >> 4);
 #pragma unroll
             for (int k = 0; k < BK / 16; ++k) umma_bf16(tmem_base, desc_of(al + 2 * k), desc_of(bl + 2 * k), idesc1, 1u);
           } else {

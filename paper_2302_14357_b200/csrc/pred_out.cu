@@ -20,10 +20,12 @@ constexpr int BM = 128, BK = 64, kCols = 16;       // kCols: accumulator columns
 
 template <int BN>
 struct WpCfg {
-  static constexpr int kStages = BN == 64 ? 8 : 5;          // BN = 32: half an SM, to be resident beside a gate GEMM's CTA
+  // the ring: stages of 128 rows; BN = 32: half an SM, to be resident beside a gate GEMM's CTA
+  static constexpr int kFullStages = BN == 64 ? 8 : 5;
   static constexpr int kEpiWarps = 4 * (BN / kCols), kThreads = 64 + 32 * kEpiWarps;
   static constexpr uint32_t kABytes = BM * BK * 2, kBBytes = BN * BK * 2;
-  static constexpr size_t kSmem = (size_t)kStages * (kABytes + kBBytes) + 1024 + 256;
+  static constexpr uint32_t kRing = kFullStages * (kABytes + kBBytes);
+  static constexpr size_t kSmem = (size_t)kRing + 1024 + 256;
 };
 
 template <int BN>
@@ -33,11 +35,14 @@ wp_operand_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
   using C = WpCfg<BN>;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
+  // (A and B apart: an MMA that reads 128 rows of a smaller stage stays inside the ring)
+  const uint32_t a_stage = (uint32_t)ring_quarters(p.M) * (C::kABytes / 4);
+  const int nst = min((int)(C::kRing / (a_stage + C::kBBytes)), kMaxRingStages);
   uint8_t* sA = smem;
-  uint8_t* sB = smem + C::kStages * C::kABytes;
-  uint64_t* full = reinterpret_cast<uint64_t*>(sB + C::kStages * C::kBBytes);
-  uint64_t* empty = full + C::kStages;
-  uint64_t* acc_full = empty + C::kStages;     // [2]
+  uint8_t* sB = smem + nst * a_stage;
+  uint64_t* full = reinterpret_cast<uint64_t*>(smem + C::kRing);
+  uint64_t* empty = full + kMaxRingStages;
+  uint64_t* acc_full = empty + kMaxRingStages; // [2]
   uint64_t* acc_empty = acc_full + 2;          // [2]
   uint32_t* tmem_holder = reinterpret_cast<uint32_t*>(acc_empty + 2);
 
@@ -56,7 +61,7 @@ wp_operand_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
     prefetch_tensormap(&tmA);
     prefetch_tensormap(&tmA32);
     prefetch_tensormap(&tmB);
-    for (int s = 0; s < C::kStages; ++s) { mbar_init(&full[s], 1); mbar_init(&empty[s], 1); }
+    for (int s = 0; s < nst; ++s) { mbar_init(&full[s], 1); mbar_init(&empty[s], 1); }
     for (int i = 0; i < 2; ++i) { mbar_init(&acc_full[i], 1); mbar_init(&acc_empty[i], C::kEpiWarps); }
     fence_barrier_init();
     fence_proxy_async_smem();
@@ -75,7 +80,7 @@ wp_operand_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
     const uint64_t keep = l2_policy_evict_last();
     const uint32_t a0 = smem_u32(sA), b0 = smem_u32(sB), full0 = smem_u32(full), empty0 = smem_u32(empty);
     if ((int)blockIdx.x < num_tiles) {
-      npre = num_kb < C::kStages ? num_kb : C::kStages;
+      npre = num_kb < nst ? num_kb : nst;
       for (int kb = 0; kb < npre; ++kb) {
         if (elect_one()) {
           mbar_expect_a(full0 + 8 * kb, C::kBBytes);         // the arrival comes with A
@@ -90,7 +95,7 @@ wp_operand_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
       uint32_t ph = 0;
       for (int tile = blockIdx.x; tile < num_tiles && ok; tile += gridDim.x) {
         const int m0 = (tile / n_tiles) * BM, n0 = (tile % n_tiles) * BN;
-        const int nq = min(4, (M - m0 + 31) >> 5);           // lane quarters with rows in them
+        const int nq = M - m0 <= 64 ? (M - m0 + 31) >> 5 : 4;          // lane quarters with rows in them, three as four
         const uint32_t a_bytes = (uint32_t)nq * (C::kABytes / 4);
         for (int kb = 0; kb < num_kb; ++kb) {
           const bool first = npre > 0;                       // B is on its way
@@ -101,13 +106,13 @@ wp_operand_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
             --npre;
           }
           if (elect_one()) {
-            const uint32_t adst = a0 + s * C::kABytes;
+            const uint32_t adst = a0 + s * a_stage;
             mbar_arrive_expect_a(full0 + 8 * s, first ? a_bytes : a_bytes + C::kBBytes);
             if (nq == 4) tma_load_2d_a(adst, &tmA, full0 + 8 * s, kb * BK, m0);
             else for (int q = 0; q < nq; ++q) tma_load_2d_a(adst + q * (C::kABytes / 4), &tmA32, full0 + 8 * s, kb * BK, m0 + 32 * q);
             if (!first) tma_load_2d_hint_a(b0 + s * C::kBBytes, &tmB, full0 + 8 * s, kb * BK, n0, keep);
           }
-          if (++s == C::kStages) { s = 0; ph ^= 1; }
+          if (++s == nst) { s = 0; ph ^= 1; }
         }
       }
     }
@@ -130,12 +135,12 @@ wp_operand_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
           if (!ok) break;
           tc_fence_after();
           if (elect_one()) {
-            const uint32_t al = a_lo + s * (C::kABytes >> 4), bl = b_lo + s * (C::kBBytes >> 4);
+            const uint32_t al = a_lo + s * (a_stage >> 4), bl = b_lo + s * (C::kBBytes >> 4);
 #pragma unroll
             for (int k = 0; k < BK / 16; ++k) umma_bf16(tmem_d, desc_of(al + 2 * k), desc_of(bl + 2 * k), idesc, (kb | k) != 0);
             umma_commit_a(empty0 + 8 * s);
           }
-          if (++s == C::kStages) { s = 0; ph ^= 1; }
+          if (++s == nst) { s = 0; ph ^= 1; }
         }
         if (ok && elect_one()) umma_commit_a(smem_u32(acc_full) + 8 * buf);
       }
