@@ -444,7 +444,9 @@ gemm_lstm_wide_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_cons
   // CTAs, i.e. narrower and faster tiles (never wider than the host's bound).  The small instance, where the kernel ahead
   // writes the count (late), splits for the largest count: its tiles are narrow anyway, and so are known before the wait.
   const bool late = EPIW == 8 && p.M_dev != nullptr && !p.m_early;
-  if (EPIW == 16) { pdl_wait(); pdl_trigger(); }      // the set-up touched only this CTA: it may overlap the tail of the kernel that produces A and M
+  // (large instance: a row count that the kernel ahead does not write is read, and the split taken, ahead of the wait)
+  const bool known = EPIW == 16 && (p.m_early || !p.M_dev);
+  if (EPIW == 16 && !known) { pdl_wait(); pdl_trigger(); }      // the set-up touched only this CTA: it may overlap the tail of the kernel that produces A and M
   const int M = warp_uniform((late || !p.M_dev) ? p.M : (p.m_early ? M_pre : *p.M_dev));
   const int m_tiles = M > 0 ? (M + BM - 1) / BM : 1;
   const int units = p.N >> 5;
@@ -455,6 +457,7 @@ gemm_lstm_wide_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_cons
   const int ubase = units / n_split, urem = units - ubase * n_split;
   const int u0 = ns * ubase + (ns < urem ? ns : urem), nu = ubase + (ns < urem ? 1 : 0);
   const int n0 = u0 * 32, w = nu * 32;                   // this CTA's columns [n0, n0 + w), w <= kMaxBN
+  if (known) { pdl_wait(); pdl_trigger(); }
   if (w > W::kMaxBN && threadIdx.x == 0) atomicExch(p.err, 1);     // the host sizes the grid so that this cannot happen
   const bool active = m0 < M && mt < m_tiles && w <= W::kMaxBN;    // an idle CTA skips the roles and only frees its TMEM
   const uint32_t b_bytes = (uint32_t)w * (BK * 2), a_stage = EPIW == 16 ? kWideABytes : (uint32_t)ring_quarters(p.M) * (kWideABytes / 4);
