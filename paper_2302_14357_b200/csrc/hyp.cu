@@ -527,8 +527,9 @@ __global__ void __launch_bounds__(2 * kStepThreads) hyp_step_kernel(HypState hs,
   if (tid < kMaxBeam * kMaxBeam) {
     // (a row with N candidates bounds the N-th best score from below by its last one, log 0 where there is none: the first row,
     // the best hypothesis's, leaves few to rank (one utterance, N = 10: 28.3 -> 27.6 ms); the largest of all rows' bounds leaves
-    // fewer and takes longer than it saves at N = 5)
-    const double sc = s_abs[tid], low = s_abs[N - 1];
+    // fewer and takes longer than it saves at N = 5).  The rows are sorted by delta_nb, and the approximate logarithm may give two
+    // neighbours the wrong order, by less than 1e-6: the bound keeps well clear of that.
+    const double sc = s_abs[tid], low = s_abs[N - 1] - 1e-4;
     const bool pass = s_ck[tid] >= 0 && !(sc < low) && (s_hasthr == 0 || sc > s_thr);
     const unsigned m = __ballot_sync(0xffffffffu, pass);
     if (m != 0) {
@@ -545,7 +546,9 @@ __global__ void __launch_bounds__(2 * kStepThreads) hyp_step_kernel(HypState hs,
     int rank = 0;
     for (int j = 0; j < np; j += 32) {
       const ulonglong2 o = j + lane < np ? s_pass[j + lane] : make_ulonglong2(0, 0);
-      rank += __popc(__ballot_sync(0xffffffffu, o.x > me.x || (o.x == me.x && o.y < me.y)));      // (no score has the key 0)
+      // (no score has the key 0; candidates of one row keep the row's order)
+      const bool row = ((o.y ^ me.y) / kMaxBeam) == 0 && o.x != 0;
+      rank += __popc(__ballot_sync(0xffffffffu, row ? o.y < me.y : (o.x > me.x || (o.x == me.x && o.y < me.y))));
     }
     if (lane == 0 && rank < N) {
       const int c = (int)me.y, h = c / kMaxBeam;
