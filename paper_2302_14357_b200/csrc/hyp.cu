@@ -9,6 +9,7 @@
 #include <cuda_bf16.h>
 
 #include "operand.cuh"
+#include "rank_order.h"
 #include "sm100.cuh"
 
 namespace tw {
@@ -153,13 +154,6 @@ constexpr int kSelCap = 64;         // survivors of a row's bound that are ranke
 __device__ __forceinline__ bool tok_better(float v1, int k1, float v2, int k2) { return v1 > v2 || (v1 == v2 && k1 < k2); }
 // (value desc, token asc) of a positive value as one integer, larger first
 __device__ __forceinline__ unsigned long long tok_key(float v, int k) { return ((unsigned long long)__float_as_uint(v) << 32) | (0xffffffffu - (unsigned)k); }
-
-// Order-preserving integer image of a score: a < b as doubles <=> order_key(a) < order_key(b) as unsigned
-// integers (-0 counts as +0; scores are never NaN).  The ranking loops compare these instead of doubles.
-__device__ __forceinline__ unsigned long long order_key(double x) {
-  const unsigned long long u = (unsigned long long)__double_as_longlong(x + 0.0);
-  return (u >> 63) ? ~u : (u | 0x8000000000000000ull);
-}
 
 // The kernel is a chain of short phases, each as long as its slowest dependent accesses; it is organised to have few of them
 // behind the wait for the joiner kernel:
@@ -516,6 +510,10 @@ __global__ void __launch_bounds__(2 * kStepThreads) hyp_step_kernel(HypState hs,
           pv = bv; pk = bk;
         }
       }
+      // (hardly ever: neighbours whose logarithms are in the other order)
+      __syncwarp();
+      double* row = s_abs + h * kMaxBeam;
+      if (__any_sync(0xffffffffu, lane > 0 && lane < N && row[lane] > row[lane - 1]) && lane == 0) settle_row(row, N);
     }
   }
   __syncthreads();
@@ -527,9 +525,8 @@ __global__ void __launch_bounds__(2 * kStepThreads) hyp_step_kernel(HypState hs,
   if (tid < kMaxBeam * kMaxBeam) {
     // (a row with N candidates bounds the N-th best score from below by its last one, log 0 where there is none: the first row,
     // the best hypothesis's, leaves few to rank (one utterance, N = 10: 28.3 -> 27.6 ms); the largest of all rows' bounds leaves
-    // fewer and takes longer than it saves at N = 5).  The rows are sorted by delta_nb, and the approximate logarithm may give two
-    // neighbours the wrong order, by less than 1e-6: the bound keeps well clear of that.
-    const double sc = s_abs[tid], low = s_abs[N - 1] - 1e-4;
+    // fewer and takes longer than it saves at N = 5).  No score rises along its row.
+    const double sc = s_abs[tid], low = s_abs[N - 1];
     const bool pass = s_ck[tid] >= 0 && !(sc < low) && (s_hasthr == 0 || sc > s_thr);
     const unsigned m = __ballot_sync(0xffffffffu, pass);
     if (m != 0) {
@@ -545,10 +542,8 @@ __global__ void __launch_bounds__(2 * kStepThreads) hyp_step_kernel(HypState hs,
     const ulonglong2 me = s_pass[i];
     int rank = 0;
     for (int j = 0; j < np; j += 32) {
-      const ulonglong2 o = j + lane < np ? s_pass[j + lane] : make_ulonglong2(0, 0);
-      // (no score has the key 0; candidates of one row keep the row's order)
-      const bool row = ((o.y ^ me.y) / kMaxBeam) == 0 && o.x != 0;
-      rank += __popc(__ballot_sync(0xffffffffu, row ? o.y < me.y : (o.x > me.x || (o.x == me.x && o.y < me.y))));
+      const ulonglong2 o = j + lane < np ? s_pass[j + lane] : make_ulonglong2(0, ~0ull);     // ahead of nobody
+      rank += __popc(__ballot_sync(0xffffffffu, ranks_before(o.x, o.y, me.x, me.y)));
     }
     if (lane == 0 && rank < N) {
       const int c = (int)me.y, h = c / kMaxBeam;
