@@ -483,7 +483,7 @@ gemm_lstm_wide_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_cons
       // kernel ahead is still pulling its own through L2)
       npre = min(num_kb, nst);
       for (int kb = 0; kb < npre; ++kb)
-        if (elect_one()) { mbar_expect_a(full0 + 8 * kb, b_bytes); send_B(kb, kb); }     // the arrival comes with A
+        if (elect_one()) { mbar_expect_only_a(full0 + 8 * kb, b_bytes); send_B(kb, kb); }     // the arrival comes with A
       pdl_wait();
       pdl_trigger();
     }

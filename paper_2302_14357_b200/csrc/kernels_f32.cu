@@ -92,7 +92,7 @@ gemm_f32_kernel(const __grid_constant__ CUtensorMap tm0, const __grid_constant__
   __syncthreads();
   auto send_B = [&](int i) {               // one thread: the weights of block i
     const int blk = b_lo + i, s = i % kStagesF;
-    mbar_expect_tx(&full[s], (uint32_t)Sm::kB);
+    mbar_arrive_expect(&full[s], (uint32_t)Sm::kB);
     tma_load_2d(sB + s * Sm::kB, blk < nb0 ? &tm0 : &tm1, &full[s], (blk < nb0 ? blk : blk - nb0) * BK, n0);
   };
   const int pre = nb < kAhead ? nb : kAhead;
@@ -139,7 +139,7 @@ gemm_f32_kernel(const __grid_constant__ CUtensorMap tm0, const __grid_constant__
       fence_proxy_async_smem();
       __syncwarp();
     }
-    if (lane == 0) mbar_expect_tx(&full[s], (uint32_t)(min(TM, M - m0) * kn * 4));
+    if (lane == 0) mbar_arrive_expect(&full[s], (uint32_t)(min(TM, M - m0) * kn * 4));
     __syncwarp();
     if (lane < TM && arow != nullptr)
       bulk_load(sA + s * Sm::kA + lane * (BK * 4), (second ? prow : arow) + k, (uint32_t)kn * 4u, &full[s]);

@@ -86,7 +86,7 @@ wp_operand_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
       npre = num_kb < nst ? num_kb : nst;
       for (int kb = 0; kb < npre; ++kb) {
         if (elect_one()) {
-          mbar_expect_a(full0 + 8 * kb, C::kBBytes);         // the arrival comes with A
+          mbar_expect_only_a(full0 + 8 * kb, C::kBBytes);         // the arrival comes with A
           tma_load_2d_hint_a(b0 + kb * C::kBBytes, &tmB, full0 + 8 * kb, kb * BK, ((int)blockIdx.x % n_tiles) * BN, keep);
         }
       }
