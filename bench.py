@@ -55,7 +55,7 @@ def parse_args():
 # the running decode leaves them (--cache-control none); the commands are in profiles/.  Each
 # entry carries the digest of the kernel's sources at the time of the capture; once the sources differ the
 # counters no longer describe the kernel that runs and the bench reports null.
-KERNEL_SOURCES = ("fused_joiner.cu", "fused_joiner_kernel.inc", "fused_joiner_host.inc", "sm100.cuh")
+KERNEL_SOURCES = ("fused_joiner.cu", "fused_joiner_kernel.inc", "joiner_tile.inc", "fused_joiner_host.inc", "sm100.cuh")
 NCU_DRAM_BYTES_PER_LAUNCH = {
     # (workload, S): (source digest, cold bytes, warm bytes)
     ("c3", 3): ("62d81d70a8dc", 16909000, 19400000),      # cold: W_out + the A operand; warm: 3.9 MB read, 15.5 MB of delta_nb leaving L2

@@ -105,7 +105,7 @@ struct FusedJoinerParams {
                                      // launched, and not by it: it is read ahead of the wait)
   int S, V, K, blank, CL;            // K = J; CL = V / (columns per CTA) CTAs per cluster, filled in by launch_fused_joiner
   int no_max;                        // logits are bounded by zbound (at most 40): softmax sums need no maximum search
-  float zbound;                      // max_k (|W_out[k, :]|_1 + |b_out[k]|) >= |z| (tanh joiner); used when no_max
+  float zbound;                      // max_k (|W_out[k, :]|_1 + |b_out[k]|) >= |z| (tanh joiner) with no_max, else 0
   const float* bias;                 // b_out [V]
   const float* ld_old;               // [R][S]
   const int* row_slen;               // [R] (nullptr: S)

@@ -81,6 +81,7 @@ __device__ __forceinline__ float window_sum(float x) {
   return total;
 }
 
+#include "joiner_tile.inc"
 #include "fused_joiner_kernel.inc"
 
 }  // namespace
